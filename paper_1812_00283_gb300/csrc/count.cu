@@ -133,7 +133,7 @@ struct SharedTeam {
     int32_t start[kB + 33];             // compacted batch: exclusive prefix of run lengths, then
                                         // the total and 32 sentinels (INT_MAX)
     Pos src[kB];                        // compacted batch: adjacency position of a run minus its prefix
-    unsigned long long msum[has_second_walk(MODE) ? kB : 1];  // second walk: Σ δ per compacted middle
+    uint2 msum[has_second_walk(MODE) ? kB : 1];  // second walk: Σ δ per compacted middle (low, high half)
     long long wtot[kThreads / 32];
     unsigned long long red[kThreads / 32];
     int item;
@@ -262,22 +262,12 @@ __device__ __forceinline__ uint32_t get16(const uint32_t *w32, int idx) {
 }
 
 // 8-bit counters packed four per 32-bit word (a start whose counts stay below 256)
-__device__ __forceinline__ uint32_t inc8(uint32_t *w32, int idx) {
-    const uint32_t sh = (uint32_t)(idx & 3) << 3;
-    uint32_t old = atomicAdd(w32 + (idx >> 2), 1u << sh);
-    return (old >> sh) & 0xffu;
-}
 __device__ __forceinline__ uint32_t get8(const uint32_t *w32, int idx) {
     const uint32_t sh = (uint32_t)(idx & 3) << 3;
     return (w32[idx >> 2] >> sh) & 0xffu;
 }
 
 // 4-bit counters packed eight per 32-bit word (a chunk whose counts stay below 16)
-__device__ __forceinline__ uint32_t inc4(uint32_t *w32, int idx) {
-    const uint32_t sh = (uint32_t)(idx & 7) << 2;
-    uint32_t old = atomicAdd(w32 + (idx >> 3), 1u << sh);
-    return (old >> sh) & 0xfu;
-}
 __device__ __forceinline__ uint32_t get4(const uint32_t *w32, int idx) {
     const uint32_t sh = (uint32_t)(idx & 7) << 2;
     return (w32[idx >> 3] >> sh) & 0xfu;
@@ -303,58 +293,159 @@ __device__ __forceinline__ int kind_of_bits(int bits) {
     return bits == 32 ? kDenseWide : (bits == 16 ? kDenseNarrow : (bits == 8 ? kDenseByte : kDenseNibble));
 }
 
-// The counter operation for one wedge whose end id is w and whose end sits at
-// adjacency slot pos.  First walk: increment count_wedge(w), return the old
-// value.  Second walk: read the final count, attribute δ = count − 1 to the
-// edge (middle, w) and return δ for the middle's batch sum.
-template <int MODE, int KIND, bool kSecond, typename Pos>
-__device__ __forceinline__ unsigned long long wedge_op(const CountParams &p, int32_t w, Pos pos,
-                                                       int32_t lb, int32_t lo, int32_t span,
-                                                       uint32_t hmask, unsigned char *ctr, int *ovf,
-                                                       int *ins) {
-    uint32_t *w32 = reinterpret_cast<uint32_t *>(ctr);
-    uint32_t c;
-    if (KIND == kHash) {
-        int32_t *hkeys = reinterpret_cast<int32_t *>(ctr);
-        uint32_t *hcnt = reinterpret_cast<uint32_t *>(ctr + (size_t)(hmask + 1) * 4);
+// Where counter idx lies in the packed dense counters: the byte offset of its
+// 32-bit word, and its bit position (only the low five bits count).
+template <int KIND>
+__device__ __forceinline__ uint32_t dense_word(uint32_t idx) {
+    return KIND == kDenseWide ? idx << 2
+         : KIND == kDenseNarrow ? (idx << 1) & ~3u : (KIND == kDenseByte ? idx & ~3u : (idx >> 1) & ~3u);
+}
+template <int KIND>
+__device__ __forceinline__ uint32_t dense_bit(uint32_t idx) {
+    return KIND == kDenseWide ? 0u : idx << (KIND == kDenseNarrow ? 4 : (KIND == kDenseByte ? 3 : 2));
+}
+template <int KIND>
+__device__ __forceinline__ constexpr uint32_t dense_mask() {
+    return KIND == kDenseWide ? 0xffffffffu : (KIND == kDenseNarrow ? 0xffffu : (KIND == kDenseByte ? 0xffu : 0xfu));
+}
+
+// Predicated shared-memory operations of the dense walks.  They are written in
+// PTX so that the bounds test becomes the instruction's predicate: as a branch
+// around the atomic it made every window of an unrolled group wait for its own
+// atomic before the next one was issued.
+__device__ __forceinline__ uint32_t atom_inc_if(uint32_t addr, uint32_t v, uint32_t idx, uint32_t span) {
+    uint32_t old = 0;
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.lt.u32 q, %3, %4;\n\t@q atom.shared.add.u32 %0, [%1], %2;\n\t}"
+                 : "+r"(old) : "r"(addr), "r"(v), "r"(idx), "r"(span) : "memory");
+    return old;
+}
+__device__ __forceinline__ void red_inc_if(uint32_t addr, uint32_t v, uint32_t idx, uint32_t span) {
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.lt.u32 q, %2, %3;\n\t@q red.shared.add.u32 [%0], %1;\n\t}"
+                 :: "r"(addr), "r"(v), "r"(idx), "r"(span) : "memory");
+}
+__device__ __forceinline__ uint32_t load_if(uint32_t addr, uint32_t idx, uint32_t span, uint32_t other) {
+    uint32_t v = other;
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.lt.u32 q, %2, %3;\n\t@q ld.shared.u32 %0, [%1];\n\t}"
+                 : "+r"(v) : "r"(addr), "r"(idx), "r"(span) : "memory");
+    return v;
+}
+__device__ __forceinline__ void red_global_if(unsigned long long *addr, uint32_t v) {
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q red.global.add.u64 [%0], %1;\n\t}"
+                 :: "l"(addr), "l"((unsigned long long)v), "r"(v) : "memory");
+}
+
+// Σ δ of a middle, kept as two 32-bit halves: a 64-bit addition to shared
+// memory is a compare-and-swap loop, a 32-bit one is a single instruction.
+__device__ __forceinline__ void msum_add(uint2 *m, unsigned long long v) {
+    const uint32_t lo = (uint32_t)v;
+    uint32_t hi = (uint32_t)(v >> 32);
+    const uint32_t old = atomicAdd(&m->x, lo);
+    if (old + lo < lo) ++hi;   // carry out of the low half
+    if (hi) atomicAdd(&m->y, hi);
+}
+__device__ __forceinline__ unsigned long long msum_get(const uint2 &m) {
+    return ((unsigned long long)m.y << 32) | m.x;
+}
+
+// One group of N windows of dense counters: lane's ends w[u] (any value in
+// lanes that are off), on[u] = this lane takes part, pos[u] its adjacency slot.
+// First walk: count_wedge(w) is incremented; returns Σ old, or 0 when a second
+// walk follows (it finds the same sum: Σ δ = 2 Σ C(count, 2)).  Second walk:
+// d[u] = δ = count − 1, added to the edge (middle, w) at its slot; returns Σ δ.
+// An end outside the chunk touches nothing and is reported.
+template <int MODE, int KIND, bool kSecond, int N, typename Pos>
+__device__ __forceinline__ unsigned long long dense_group(const CountParams &p, const int32_t (&w)[N],
+                                                          const Pos (&pos)[N], const bool (&on)[N], int32_t base,
+                                                          uint32_t span, uint32_t ctr32, uint32_t (&d)[N]) {
+    constexpr bool kOld = !kSecond && !has_second_walk(MODE);
+    uint32_t idx[N], top = 0;
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+        idx[u] = (uint32_t)(w[u] - base);
+        top = max(top, on[u] ? idx[u] : 0u);
+        if (!on[u]) idx[u] = 0xffffffffu;
+    }
+    if (kSecond) {
+#pragma unroll
+        for (int u = 0; u < N; ++u) {
+            const uint32_t bit = dense_bit<KIND>(idx[u]);
+            // lanes that are off read a count of 1: δ = 0
+            const uint32_t v = load_if(ctr32 + dense_word<KIND>(idx[u]), idx[u], span,
+                                       KIND == kDenseWide ? 1u : 1u << (bit & 31));
+            d[u] = ((v >> (bit & 31)) & dense_mask<KIND>()) - 1u;
+        }
+        if (wants_edges(MODE)) {
+#pragma unroll
+            for (int u = 0; u < N; ++u) red_global_if(p.pe + pos[u], d[u]);
+        }
+    } else {
+#pragma unroll
+        for (int u = 0; u < N; ++u) {
+            const uint32_t bit = dense_bit<KIND>(idx[u]);
+            const uint32_t addr = ctr32 + dense_word<KIND>(idx[u]);
+            if (kOld) d[u] = atom_inc_if(addr, 1u << (bit & 31), idx[u], span);
+            else red_inc_if(addr, 1u << (bit & 31), idx[u], span);
+        }
+        if (kOld) {
+#pragma unroll
+            for (int u = 0; u < N; ++u) d[u] = (d[u] >> (dense_bit<KIND>(idx[u]) & 31)) & dense_mask<KIND>();
+        }
+    }
+    if (top >= span) atomicOr(p.err, kErrBounds);
+    if (!kSecond && !kOld) return 0;
+    if (KIND == kDenseWide) {
+        unsigned long long s = 0;
+#pragma unroll
+        for (int u = 0; u < N; ++u) s += d[u];
+        return s;
+    }
+    uint32_t s = 0;   // at most 8 values below 2^16
+#pragma unroll
+    for (int u = 0; u < N; ++u) s += d[u];
+    return s;
+}
+
+// The same for a hash table: w − lb is the key.
+template <int MODE, bool kSecond, int N, typename Pos>
+__device__ __forceinline__ unsigned long long hash_group(const CountParams &p, const int32_t (&w)[N],
+                                                         const Pos (&pos)[N], const bool (&on)[N], int32_t lb,
+                                                         uint32_t hmask, unsigned char *ctr, int *ovf, int *ins,
+                                                         uint32_t (&d)[N]) {
+    int32_t *hkeys = reinterpret_cast<int32_t *>(ctr);
+    uint32_t *hcnt = reinterpret_cast<uint32_t *>(ctr + (size_t)(hmask + 1) * 4);
+    uint32_t s = 0;
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+        d[u] = 0;
+        if (!on[u]) continue;
         int inserted = 0;
-        const int slot = hash_find(hkeys, hmask, w - lb, !kSecond, &inserted);
+        const int slot = hash_find(hkeys, hmask, w[u] - lb, !kSecond, &inserted);
         if (slot < 0) {
             // the first walk re-queues a start whose table filled up; the
             // second walk only looks up ends the first walk inserted
             if (!kSecond) *ovf = 1; else atomicOr(p.err, kErrHashFull);
-            return 0;
+            continue;
         }
         if (!kSecond) {
             // keep the load factor at most 3/4 so probes stay short
             // (ins is null when the start cannot reach that load)
             if (inserted && ins && atomicAdd(ins, 1) >= (int)((hmask + 1) / 4 * 3)) *ovf = 1;
-            return inc16(hcnt, slot);
+            d[u] = inc16(hcnt, slot);
+        } else {
+            d[u] = get16(hcnt, slot) - 1u;
+            if (wants_edges(MODE)) red_global_if(p.pe + pos[u], d[u]);
         }
-        c = get16(hcnt, slot);
-    } else {
-        const int idx = w - lb - lo;
-        if ((uint32_t)idx >= (uint32_t)span) { atomicOr(p.err, kErrBounds); return 0; }
-        if (!kSecond)
-            return (KIND == kDenseWide) ? atomicAdd(w32 + idx, 1u)
-                 : (KIND == kDenseByte) ? inc8(w32, idx) : (KIND == kDenseNibble ? inc4(w32, idx) : inc16(w32, idx));
-        c = (KIND == kDenseWide) ? w32[idx]
-          : (KIND == kDenseByte) ? get8(w32, idx) : (KIND == kDenseNibble ? get4(w32, idx) : get16(w32, idx));
+        s += d[u];
     }
-    // δ = count − 1 for the edge (middle, w); the caller sums it per middle
-    const unsigned long long delta = (unsigned long long)c - 1ull;
-    // per-edge sums are kept by G* slot: the ends of one run are consecutive
-    // slots, so a window's atomics fall on a few consecutive sectors
-    if (wants_edges(MODE) && delta) atomicAdd(p.pe + pos, delta);
-    return delta;
+    return !kSecond && has_second_walk(MODE) ? 0u : s;
 }
 
 // Adds each lane's x to msum[q], where equal q occupy consecutive lanes (the
 // runs of a window are contiguous): the last lane of each run takes the
 // difference of an inclusive warp scan at its lane and at the previous run's
 // last lane (found from a ballot of run ends), and makes the one shared atomic.
-template <typename T>
-__device__ __forceinline__ void run_add(unsigned long long *msum, int q, T x, int lane) {
+template <typename T, typename M>
+__device__ __forceinline__ void run_add(M *msum, int q, T x, int lane) {
     T sc = x;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -366,7 +457,7 @@ __device__ __forceinline__ void run_add(unsigned long long *msum, int q, T x, in
     const uint32_t below = __ballot_sync(0xffffffffu, last) & ((1u << lane) - 1u);
     const T prev = __shfl_sync(0xffffffffu, sc, below ? 31 - __clz(below) : 0);
     const T sum = below ? sc - prev : sc;
-    if (last && sum) atomicAdd(msum + q, (unsigned long long)sum);
+    if (last && sum) msum_add(msum + q, (unsigned long long)sum);
 }
 
 // The per-thread state of one batch of middles that the second walk needs
@@ -387,7 +478,7 @@ __device__ __forceinline__ void middle_sums(const CountParams &p, const BatchSlo
 #pragma unroll
     for (int i = 0; i < Batch<Pos, kThreads>::kPer; ++i) {
         if (bs.len[i] > 0) {
-            const unsigned long long dsum = sh.msum[bs.nzs[i]];
+            const unsigned long long dsum = msum_get(sh.msum[bs.nzs[i]]);
             if (dsum) {
                 if (wants_vertices(MODE)) atomicAdd(p.pv + bs.v[i], dsum);
                 if (wants_edges(MODE)) atomicAdd(p.pe + bs.e[i], dsum);
@@ -499,7 +590,7 @@ __device__ __forceinline__ void batch_runs(const CountParams &p, int64_t e0, int
         if (bs.len[i] > 0) {
             sh.start[bs.nzs[i]] = excl;
             sh.src[bs.nzs[i]] = src[i] - (Pos)excl;
-            if (kSecond) sh.msum[bs.nzs[i]] = 0;
+            if (kSecond) sh.msum[bs.nzs[i]] = make_uint2(0, 0);
         }
         packed += pk[i];
     }
@@ -508,13 +599,24 @@ __device__ __forceinline__ void batch_runs(const CountParams &p, int64_t e0, int
     *nnz_out = nnz;
 }
 
-// The windows of one compacted batch.  The concatenated runs are cut into
-// windows of 32 wedges and each warp takes a contiguous range of windows.
-// Inside a window the run of every lane is found from a 32-bit mask of run
-// starts (reduce-or + popc), so no search is needed per wedge, and four
-// windows are in flight per iteration so their end loads overlap.
-// kSecond = false: count (returns Σ old, i.e. Σ C(count, 2)).
-// kSecond = true : read the final counts and attribute δ = count − 1.
+// The wedges of one compacted batch.  The concatenated runs are cut into one
+// contiguous range per warp, and a warp takes its range in three ways:
+//   - at least 256 wedges of the current run left: eight windows of 32, no run
+//     lookup, eight end loads in flight per lane;
+//   - else, where the next runs are long enough, four segments of at most 32
+//     wedges, each inside one run (the run, its start and its end are the same
+//     in every lane, so no lane searches and a run's δ sum is one reduction);
+//   - else (many runs per 32 wedges) four windows across runs: the run of every
+//     lane is found from a 32-bit mask of run starts (reduce-or + popc).
+// Bound by instruction issue and load latency (53-63% issue, DRAM and L2 below
+// 20%).  Against windows across runs everywhere with a branch per wedge:
+// per-edge counts of a 30M-edge shopping graph 10.69 -> 8.83 ms, per-vertex
+// counts of a 6M-edge power-law graph 4.70 -> 3.92, prepare and total of a
+// 20M-edge power-law graph 13.25 -> 12.38.
+// kSecond = false: count; returns Σ old = Σ C(count, 2), or 0 in the modes with
+// a second walk.
+// kSecond = true : read the final counts and attribute δ = count − 1; returns
+// Σ δ = 2 Σ C(count, 2).
 template <int MODE, int KIND, bool kSecond, typename Pos, int kThreads, class SH>
 __device__ __forceinline__ unsigned long long batch_windows(const CountParams &p, int32_t lb, int32_t lo,
                                                             int32_t span, uint32_t hmask,
@@ -522,105 +624,123 @@ __device__ __forceinline__ unsigned long long batch_windows(const CountParams &p
                                                             int *ins, SH &sh, const Team<kThreads> &t) {
     constexpr int kWarps = kThreads / 32;
     constexpr int kU = 4;
+    // four segments against four windows: a window across runs costs about
+    // 17 instructions of lookup (and 25 for the segmented δ sums) that a
+    // segment does not, so segments win from this many wedges in four runs up
+    constexpr int32_t kSegMin = kSecond ? 64 : 96;
     const int lane = t.tid & 31, warp = t.tid >> 5;
     const uint32_t le_mask = 0xffffffffu >> (31 - lane);
+    const uint32_t ctr32 = (uint32_t)__cvta_generic_to_shared(ctr);
+    const int32_t base = lb + lo;
     unsigned long long acc = 0;
     const int32_t nwin = (total + 31) >> 5;
-    int32_t wb = (int32_t)(((int64_t)warp * nwin) / kWarps);
-    const int32_t wend = (int32_t)(((int64_t)(warp + 1) * nwin) / kWarps);
-    if (wb < wend) {
-        int32_t k0 = wb << 5;
-        int q0 = last_le(sh.start, nnz, k0);
-        // Fast path: the next N windows lie inside run q0 (most wedges do, as
-        // runs of heavy starts are long), so the slots are consecutive, no
-        // run lookup is needed and N loads are in flight per lane.
-        auto fast = [&](auto n_windows, int32_t next_run) {
-            constexpr int N = decltype(n_windows)::value;
-            const Pos base = sh.src[q0] + (Pos)(k0 + lane);
-            int32_t w[N];
+    int32_t k0 = (int32_t)(((int64_t)warp * nwin) / kWarps) << 5;
+    const int32_t kend = min((int32_t)(((int64_t)(warp + 1) * nwin) / kWarps) << 5, total);
+    if (k0 >= kend) return 0;
+    auto group = [&](auto n_windows, const auto &w, const auto &pos, const auto &on, auto &d) {
+        constexpr int N = decltype(n_windows)::value;
+        if constexpr (KIND == kHash)
+            return hash_group<MODE, kSecond, N, Pos>(p, w, pos, on, lb, hmask, ctr, &sh.overflow, ins, d);
+        else
+            return dense_group<MODE, KIND, kSecond, N, Pos>(p, w, pos, on, base, (uint32_t)span, ctr32, d);
+    };
+    // the δ sum of one run's lanes goes to middle q
+    auto flush = [&](int q, unsigned long long x) {
+        if (KIND == kDenseWide) {
 #pragma unroll
-            for (int u = 0; u < N; ++u) w[u] = __ldg(p.adj + base + (Pos)(32 * u));
-            uint32_t sum32 = 0;   // N olds (or δ) of 16-bit counts stay below 2^20
-            unsigned long long sum64 = 0;
+            for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        } else {
+            x = __reduce_add_sync(0xffffffffu, (uint32_t)x);
+        }
+        if (lane == 0 && x) msum_add(sh.msum + q, x);
+    };
+    int q0 = last_le(sh.start, nnz, k0);
+    int32_t nxt = min(sh.start[q0 + 1], kend);   // end of the current run (or of this warp's range)
+    while (k0 < kend) {   // warp-uniform throughout; k0 < nxt
+        if (nxt - k0 >= 64 * kU) {
+            constexpr int N = 2 * kU;
+            const Pos at = sh.src[q0] + (Pos)(k0 + lane);
+            int32_t w[N];
+            Pos pos[N];
+            bool on[N];
+            uint32_t d[N];
 #pragma unroll
             for (int u = 0; u < N; ++u) {
-                const unsigned long long r = wedge_op<MODE, KIND, kSecond, Pos>(
-                    p, w[u], base + (Pos)(32 * u), lb, lo, span, hmask, ctr, &sh.overflow, ins);
-                if (KIND == kDenseWide) sum64 += r; else sum32 += (uint32_t)r;
+                pos[u] = at + (Pos)(32 * u);
+                w[u] = __ldg(p.adj + pos[u]);
+                on[u] = true;
             }
-            if (!kSecond) {
-                acc += (KIND == kDenseWide) ? sum64 : (unsigned long long)sum32;
-            } else if (KIND == kDenseWide) {
-                run_add<unsigned long long>(sh.msum, q0, sum64, lane);
-            } else {
-                // one run: the warp's δ sum goes to middle q0
-                const uint32_t tot = __reduce_add_sync(0xffffffffu, sum32);
-                if (lane == 0 && tot) atomicAdd(sh.msum + q0, (unsigned long long)tot);
-            }
-            if (next_run == k0 + 32 * N) ++q0;   // the next window starts run q0 + 1
+            const unsigned long long x = group(std::integral_constant<int, N>(), w, pos, on, d);
+            acc += x;
+            if (kSecond) flush(q0, x);
             k0 += 32 * N;
-            wb += N;
-        };
-        while (wb < wend) {
-            const int32_t next_run = sh.start[q0 + 1];   // warp-uniform
-            if (wb + 2 * kU <= wend && next_run >= k0 + 64 * kU) {
-                fast(std::integral_constant<int, 2 * kU>(), next_run);
-                continue;
-            }
-            if (wb + kU <= wend && next_run >= k0 + 32 * kU) {
-                fast(std::integral_constant<int, kU>(), next_run);
-                continue;
-            }
-            int q[kU];
-            Pos pos[kU];
-            bool ok[kU];
-#pragma unroll
-            for (int u = 0; u < kU; ++u) {
-                q[u] = 0;
-                ok[u] = false;
-                pos[u] = 0;
-                if (wb + u < wend) {   // warp-uniform
-                    const int32_t kw = k0 + 32 * u;
-                    // run starts after this window's first wedge: 1 <= d, and
-                    // the sentinels keep the index below nnz + 33
-                    const int32_t d = sh.start[q0 + 1 + lane] - kw;
-                    uint32_t bit;   // 1 << d, 0 once d >= 32 (PTX clamps the shift)
-                    asm("shl.b32 %0, %1, %2;" : "=r"(bit) : "r"(1u), "r"(d));
-                    const uint32_t m = __reduce_or_sync(0xffffffffu, bit);
-                    q[u] = q0 + __popc(m & le_mask);
-                    q0 += __popc(__ballot_sync(0xffffffffu, d <= 32));
-                    ok[u] = kw + lane < total;
-                    if (ok[u]) pos[u] = sh.src[q[u]] + (Pos)(kw + lane);
-                }
-            }
-            int32_t w[kU];
-#pragma unroll
-            for (int u = 0; u < kU; ++u) w[u] = ok[u] ? __ldg(p.adj + pos[u]) : 0;
-            // counts below 2^16 keep four olds far below 2^32
-            uint32_t acc32 = 0;
-#pragma unroll
-            for (int u = 0; u < kU; ++u) {
-                if (!kSecond) {
-                    if (ok[u]) {
-                        const unsigned long long old =
-                            wedge_op<MODE, KIND, false, Pos>(p, w[u], pos[u], lb, lo, span, hmask,
-                                                             ctr, &sh.overflow, ins);
-                        if (KIND == kDenseWide) acc += old; else acc32 += (uint32_t)old;
-                    }
-                } else if (wb + u < wend) {   // warp-uniform: all lanes take part in run_add
-                    const unsigned long long d =
-                        ok[u] ? wedge_op<MODE, KIND, true, Pos>(p, w[u], pos[u], lb, lo, span, hmask,
-                                                                ctr, &sh.overflow, ins)
-                              : 0ull;
-                    // 16-bit counts keep a window's δ sum below 2^21
-                    if (KIND == kDenseWide) run_add<unsigned long long>(sh.msum, q[u], d, lane);
-                    else run_add<uint32_t>(sh.msum, q[u], (uint32_t)d, lane);
-                }
-            }
-            if (KIND != kDenseWide) acc += acc32;
-            k0 += 32 * kU;
-            wb += kU;
+            if (k0 == nxt) { ++q0; nxt = min(sh.start[q0 + 1], kend); }
+            continue;
         }
+        int32_t w[kU];
+        Pos pos[kU];
+        bool on[kU];
+        uint32_t d[kU];
+        if (sh.start[q0 + kU] - k0 >= kSegMin) {
+            int q[kU];
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                const int32_t n = min(nxt - k0, 32);   // 0 past the range
+                q[u] = q0;
+                on[u] = lane < n;
+                pos[u] = sh.src[q0] + (Pos)(k0 + lane);
+                w[u] = 0;
+                if (on[u]) w[u] = __ldg(p.adj + pos[u]);
+                k0 += n;
+                if (k0 == nxt && k0 < kend) { ++q0; nxt = min(sh.start[q0 + 1], kend); }
+            }
+            const unsigned long long x = group(std::integral_constant<int, kU>(), w, pos, on, d);
+            acc += x;
+            if (kSecond) {
+                if (q[0] == q[kU - 1]) {
+                    flush(q[0], x);
+                } else {
+#pragma unroll
+                    for (int u = 0; u < kU; ++u) flush(q[u], d[u]);
+                }
+            }
+            continue;
+        }
+        int q[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            q[u] = 0;
+            on[u] = false;
+            pos[u] = 0;
+            const int32_t kw = k0 + 32 * u;
+            if (kw < kend) {   // warp-uniform
+                // run starts after this window's first wedge: 1 <= d, and
+                // the sentinels keep the index below nnz + 33
+                const int32_t dd = sh.start[q0 + 1 + lane] - kw;
+                uint32_t bit;   // 1 << dd, 0 once dd >= 32 (PTX clamps the shift)
+                asm("shl.b32 %0, %1, %2;" : "=r"(bit) : "r"(1u), "r"(dd));
+                const uint32_t m = __reduce_or_sync(0xffffffffu, bit);
+                q[u] = q0 + __popc(m & le_mask);
+                q0 += __popc(__ballot_sync(0xffffffffu, dd <= 32));
+                on[u] = kw + lane < kend;
+                if (on[u]) pos[u] = sh.src[q[u]] + (Pos)(kw + lane);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < kU; ++u) w[u] = on[u] ? __ldg(p.adj + pos[u]) : 0;
+        acc += group(std::integral_constant<int, kU>(), w, pos, on, d);
+        if (kSecond) {
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                if (k0 + 32 * u < kend) {   // warp-uniform: all lanes take part in run_add
+                    // 16-bit counts keep a window's δ sum below 2^21
+                    if (KIND == kDenseWide) run_add<unsigned long long>(sh.msum, q[u], d[u], lane);
+                    else run_add<uint32_t>(sh.msum, q[u], d[u], lane);
+                }
+            }
+        }
+        k0 += 32 * kU;
+        if (k0 < kend) nxt = min(sh.start[q0 + 1], kend);
     }
     return acc;
 }
@@ -635,7 +755,6 @@ template <int MODE, int KIND, bool kSecond, typename Pos, int kThreads, class SH
 __device__ unsigned long long team_walk(const CountParams &p, int32_t x, int32_t lb, int32_t lo,
                                         int32_t hi, int flags, uint32_t hmask, unsigned char *ctr,
                                         SH &sh, const Team<kThreads> &t) {
-    constexpr int kPer = Batch<Pos, kThreads>::kPer;
     constexpr int kB = Batch<Pos, kThreads>::kSize;
     const int64_t e0 = p.off[x];
     // Algorithm 2: the middles are the cut[x] lower-priority neighbours;
@@ -663,8 +782,9 @@ __device__ unsigned long long team_walk(const CountParams &p, int32_t x, int32_t
 }
 
 // First walk, then (per-vertex / per-edge) the end contributions and the
-// second walk.  Returns Σ C(count, 2) over the pairs of this item, or 0 with
-// sh.overflow set when a hash table filled up (nothing is attributed then).
+// second walk.  Returns Σ C(count, 2) over the pairs of this item (twice that
+// in the modes with a second walk, whose Σ δ over the item's wedges it is), or 0
+// with sh.overflow set when a hash table filled up (nothing is attributed then).
 // The per-vertex end contributions of one item: each pair (x, w) of the
 // item adds C(count, 2) to ⋈_w.  Called after the first walk, with its
 // counters final.
@@ -692,20 +812,20 @@ __device__ unsigned long long item_body(const CountParams &p, int32_t x, int32_t
             t.sync();
             int *const ins = (KIND == kHash && sh.track) ? &sh.inserts : nullptr;
             const int32_t span = hi - lo;
-            const unsigned long long acc =
-                batch_windows<MODE, KIND, false, Pos>(p, lb, lo, span, hmask, ctr, total, nnz, ins, sh, t);
+            batch_windows<MODE, KIND, false, Pos>(p, lb, lo, span, hmask, ctr, total, nnz, ins, sh, t);
             t.sync();   // counters final
             if (KIND == kHash && sh.overflow) return 0;   // the caller re-queues x
             if (wants_vertices(MODE)) end_contributions<MODE, KIND>(p, lb, lo, hi, hmask, ctr, t);
 #pragma unroll
             for (int i = 0; i < Batch<Pos, kThreads>::kPer; ++i)
-                if (bs.len[i] > 0) sh.msum[bs.nzs[i]] = 0;
+                if (bs.len[i] > 0) sh.msum[bs.nzs[i]] = make_uint2(0, 0);
             t.sync();
-            batch_windows<MODE, KIND, true, Pos>(p, lb, lo, span, hmask, ctr, total, nnz, nullptr, sh, t);
+            const unsigned long long acc =
+                batch_windows<MODE, KIND, true, Pos>(p, lb, lo, span, hmask, ctr, total, nnz, nullptr, sh, t);
             t.sync();
             middle_sums<MODE, Pos>(p, bs, sh);
             if (wants_vertices(MODE)) {
-                const unsigned long long s = team_sum(acc, sh, t);
+                const unsigned long long s = team_sum(acc, sh, t) / 2;
                 if (t.tid == 0 && s) atomicAdd(p.pv + x, s);
             }
             return acc;
@@ -719,9 +839,9 @@ __device__ unsigned long long item_body(const CountParams &p, int32_t x, int32_t
     if (has_second_walk(MODE)) {
         t.sync();
         if (wants_vertices(MODE)) end_contributions<MODE, KIND>(p, lb, lo, hi, hmask, ctr, t);
-        team_walk<MODE, KIND, true, Pos>(p, x, lb, lo, hi, flags, hmask, ctr, sh, t);
+        acc = team_walk<MODE, KIND, true, Pos>(p, x, lb, lo, hi, flags, hmask, ctr, sh, t);
         if (wants_vertices(MODE)) {
-            const unsigned long long s = team_sum(acc, sh, t);
+            const unsigned long long s = team_sum(acc, sh, t) / 2;
             if (t.tid == 0 && s) atomicAdd(p.pv + x, s);
         }
     }
@@ -1030,7 +1150,7 @@ __device__ unsigned long long team_item(const CountParams &p, int32_t x, unsigne
 // always fits (at most 384 wedges, 512 slots).
 template <int MODE, bool kSecond>
 __device__ unsigned long long warp_walk(const CountParams &p, int32_t x, int32_t lb, uint32_t mask,
-                                        int32_t *keys, uint32_t *cnt, unsigned long long *msum,
+                                        int32_t *keys, uint32_t *cnt, uint2 *msum,
                                         int32_t *wstart, long long *wsrc) {
     const int lane = threadIdx.x & 31;
     const int64_t e0 = p.off[x];
@@ -1062,7 +1182,7 @@ __device__ unsigned long long warp_walk(const CountParams &p, int32_t x, int32_t
         if (len > 0) {
             wstart[nz] = excl;
             wsrc[nz] = src - excl;
-            if (kSecond) msum[nz] = 0;
+            if (kSecond) msum[nz] = make_uint2(0, 0);
         }
         if (lane == 0) wstart[nnz] = total;
         __syncwarp();
@@ -1084,7 +1204,8 @@ __device__ unsigned long long warp_walk(const CountParams &p, int32_t x, int32_t
                 if (good && slot < 0) atomicOr(p.err, kErrHashFull);
                 if (slot >= 0) {
                     if (!kSecond) {
-                        acc += atomicAdd(cnt + slot, 1u);
+                        const uint32_t old = atomicAdd(cnt + slot, 1u);
+                        if (!has_second_walk(MODE)) acc += old;
                     } else {
                         delta = cnt[slot] - 1u;   // below 384
                         if (wants_edges(MODE) && delta) atomicAdd(p.pe + pos, (unsigned long long)delta);
@@ -1092,10 +1213,11 @@ __device__ unsigned long long warp_walk(const CountParams &p, int32_t x, int32_t
                 }
             }
             if (kSecond) run_add<uint32_t>(msum, q, delta, lane);
+            if (kSecond) acc += delta;
         }
         __syncwarp();
         if (kSecond && len > 0) {
-            const unsigned long long dsum = msum[nz];
+            const unsigned long long dsum = msum_get(msum[nz]);
             if (dsum) {
                 if (wants_vertices(MODE)) atomicAdd(p.pv + v, dsum);
                 if (wants_edges(MODE)) atomicAdd(p.pe + e, dsum);
@@ -1122,7 +1244,7 @@ __device__ unsigned long long warp_item(const CountParams &p, int32_t x, unsigne
     while (cap < 2 * bound && cap < (uint32_t)kWarpSlots) cap <<= 1;
     int32_t *keys = reinterpret_cast<int32_t *>(region);
     uint32_t *cnt = reinterpret_cast<uint32_t *>(region + kWarpCntOff);
-    unsigned long long *msum = reinterpret_cast<unsigned long long *>(region + kWarpMsumOff);
+    uint2 *msum = reinterpret_cast<uint2 *>(region + kWarpMsumOff);
     long long *wsrc = reinterpret_cast<long long *>(region + kWarpSrcOff);
     int32_t *wstart = reinterpret_cast<int32_t *>(region + kWarpStartOff);
     for (uint32_t s = lane; s < cap; s += 32) { keys[s] = -1; cnt[s] = 0; }
@@ -1136,12 +1258,12 @@ __device__ unsigned long long warp_item(const CountParams &p, int32_t x, unsigne
                 if (k >= 0 && cnt[s] >= 2) atomicAdd(p.pv + lb + k, c2(cnt[s]));
             }
         }
-        warp_walk<MODE, true>(p, x, lb, cap - 1, keys, cnt, msum, wstart, wsrc);
+        acc = warp_walk<MODE, true>(p, x, lb, cap - 1, keys, cnt, msum, wstart, wsrc);
         if (wants_vertices(MODE)) {
             unsigned long long t = acc;
 #pragma unroll
             for (int d = 16; d > 0; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
-            if (lane == 0 && t) atomicAdd(p.pv + x, t);
+            if (lane == 0 && t) atomicAdd(p.pv + x, t / 2);
         }
     }
     if (MODE == kModeBatch) {
@@ -1215,8 +1337,8 @@ __global__ void __launch_bounds__(kCountThreads, kCountCtasPerSm) k_count(CountP
             acc += warp_item<MODE>(p, p.warp_items[it], region);
         }
     }
-    // a7: reduction of the per-thread partial sums
-    const unsigned long long t = team_sum(acc, sh, cta);
+    // a7: reduction of the per-thread partial sums (twice ⋈ with a second walk)
+    const unsigned long long t = team_sum(acc, sh, cta) / (has_second_walk(MODE) ? 2 : 1);
     if (threadIdx.x == 0 && t) atomicAdd(p.acc, t);
 }
 
@@ -1251,7 +1373,7 @@ __global__ void __launch_bounds__(kCountThreads, kCountCtasPerSm) k_count_retry(
         __syncthreads();
         acc += item_acc;
     }
-    const unsigned long long t = team_sum(acc, sh, cta);
+    const unsigned long long t = team_sum(acc, sh, cta) / (has_second_walk(MODE) ? 2 : 1);
     if (threadIdx.x == 0 && t) atomicAdd(p.acc, t);
 }
 
