@@ -132,7 +132,7 @@ struct SharedTeam {
     static constexpr int kB = Batch<Pos, kThreads>::kSize;
     int32_t start[kB + 33];             // compacted batch: exclusive prefix of run lengths, then
                                         // the total and 32 sentinels (INT_MAX)
-    Pos src[kB];                        // compacted batch: adjacency position of a run minus its prefix
+    Pos src[kB + 1];                    // compacted batch: adjacency position of a run minus its prefix
     uint2 msum[has_second_walk(MODE) ? kB : 1];  // second walk: Σ δ per compacted middle (low, high half)
     long long wtot[kThreads / 32];
     unsigned long long red[kThreads / 32];
@@ -347,23 +347,22 @@ __device__ __forceinline__ unsigned long long msum_get(const uint2 &m) {
     return ((unsigned long long)m.y << 32) | m.x;
 }
 
-// One group of N windows of dense counters: lane's ends w[u] (any value in
-// lanes that are off), on[u] = this lane takes part, pos[u] its adjacency slot.
+// One group of N windows of dense counters: lane's ends w[u] (-1 in lanes that
+// take no part), pos[u] their adjacency slots.
 // First walk: count_wedge(w) is incremented; returns Σ old, or 0 when a second
 // walk follows (it finds the same sum: Σ δ = 2 Σ C(count, 2)).  Second walk:
 // d[u] = δ = count − 1, added to the edge (middle, w) at its slot; returns Σ δ.
 // An end outside the chunk touches nothing and is reported.
 template <int MODE, int KIND, bool kSecond, int N, typename Pos>
 __device__ __forceinline__ unsigned long long dense_group(const CountParams &p, const int32_t (&w)[N],
-                                                          const Pos (&pos)[N], const bool (&on)[N], int32_t base,
-                                                          uint32_t span, uint32_t ctr32, uint32_t (&d)[N]) {
+                                                          const Pos (&pos)[N], int32_t base, uint32_t span,
+                                                          uint32_t ctr32, uint32_t (&d)[N]) {
     constexpr bool kOld = !kSecond && !has_second_walk(MODE);
     uint32_t idx[N], top = 0;
 #pragma unroll
     for (int u = 0; u < N; ++u) {
-        idx[u] = (uint32_t)(w[u] - base);
-        top = max(top, on[u] ? idx[u] : 0u);
-        if (!on[u]) idx[u] = 0xffffffffu;
+        idx[u] = (uint32_t)(w[u] - base);   // w = -1: at least 2^31, past any span
+        if (w[u] >= 0) top = max(top, idx[u]);
     }
     if (kSecond) {
 #pragma unroll
@@ -408,7 +407,7 @@ __device__ __forceinline__ unsigned long long dense_group(const CountParams &p, 
 // The same for a hash table: w − lb is the key.
 template <int MODE, bool kSecond, int N, typename Pos>
 __device__ __forceinline__ unsigned long long hash_group(const CountParams &p, const int32_t (&w)[N],
-                                                         const Pos (&pos)[N], const bool (&on)[N], int32_t lb,
+                                                         const Pos (&pos)[N], int32_t lb,
                                                          uint32_t hmask, unsigned char *ctr, int *ovf, int *ins,
                                                          uint32_t (&d)[N]) {
     int32_t *hkeys = reinterpret_cast<int32_t *>(ctr);
@@ -417,7 +416,7 @@ __device__ __forceinline__ unsigned long long hash_group(const CountParams &p, c
 #pragma unroll
     for (int u = 0; u < N; ++u) {
         d[u] = 0;
-        if (!on[u]) continue;
+        if (w[u] < 0) continue;
         int inserted = 0;
         const int slot = hash_find(hkeys, hmask, w[u] - lb, !kSecond, &inserted);
         if (slot < 0) {
@@ -603,8 +602,8 @@ __device__ __forceinline__ void batch_runs(const CountParams &p, int64_t e0, int
 // contiguous range per warp, and a warp takes its range in three ways:
 //   - at least 256 wedges of the current run left: eight windows of 32, no run
 //     lookup, eight end loads in flight per lane;
-//   - else, where the next runs are long enough, four segments of at most 32
-//     wedges, each inside one run (the run, its start and its end are the same
+//   - else, where the next runs are long enough, eight segments of at most 32
+//     wedges (four of a hash table), each inside one run (the run, its start and its end are the same
 //     in every lane, so no lane searches and a run's δ sum is one reduction);
 //   - else (many runs per 32 wedges) four windows across runs: the run of every
 //     lane is found from a 32-bit mask of run starts (reduce-or + popc).
@@ -628,6 +627,11 @@ __device__ __forceinline__ unsigned long long batch_windows(const CountParams &p
     // 17 instructions of lookup (and 25 for the segmented δ sums) that a
     // segment does not, so segments win from this many wedges in four runs up
     constexpr int32_t kSegMin = kSecond ? 64 : 96;
+    constexpr int kSegRuns = 4;
+    // segments in flight per warp (eight of the second walk's slots and sums do
+    // not fit the registers beside a team's or 64-bit positions)
+    constexpr int kSeg = KIND == kHash || (kSecond && wants_edges(MODE) && (sizeof(Pos) == 8 || kThreads != kCountThreads))
+                             ? 4 : 8;
     const int lane = t.tid & 31, warp = t.tid >> 5;
     const uint32_t le_mask = 0xffffffffu >> (31 - lane);
     const uint32_t ctr32 = (uint32_t)__cvta_generic_to_shared(ctr);
@@ -637,12 +641,12 @@ __device__ __forceinline__ unsigned long long batch_windows(const CountParams &p
     int32_t k0 = (int32_t)(((int64_t)warp * nwin) / kWarps) << 5;
     const int32_t kend = min((int32_t)(((int64_t)(warp + 1) * nwin) / kWarps) << 5, total);
     if (k0 >= kend) return 0;
-    auto group = [&](auto n_windows, const auto &w, const auto &pos, const auto &on, auto &d) {
+    auto group = [&](auto n_windows, const auto &w, const auto &pos, auto &d) {
         constexpr int N = decltype(n_windows)::value;
         if constexpr (KIND == kHash)
-            return hash_group<MODE, kSecond, N, Pos>(p, w, pos, on, lb, hmask, ctr, &sh.overflow, ins, d);
+            return hash_group<MODE, kSecond, N, Pos>(p, w, pos, lb, hmask, ctr, &sh.overflow, ins, d);
         else
-            return dense_group<MODE, KIND, kSecond, N, Pos>(p, w, pos, on, base, (uint32_t)span, ctr32, d);
+            return dense_group<MODE, KIND, kSecond, N, Pos>(p, w, pos, base, (uint32_t)span, ctr32, d);
     };
     // the δ sum of one run's lanes goes to middle q
     auto flush = [&](int q, unsigned long long x) {
@@ -662,56 +666,55 @@ __device__ __forceinline__ unsigned long long batch_windows(const CountParams &p
             const Pos at = sh.src[q0] + (Pos)(k0 + lane);
             int32_t w[N];
             Pos pos[N];
-            bool on[N];
             uint32_t d[N];
 #pragma unroll
             for (int u = 0; u < N; ++u) {
                 pos[u] = at + (Pos)(32 * u);
                 w[u] = __ldg(p.adj + pos[u]);
-                on[u] = true;
             }
-            const unsigned long long x = group(std::integral_constant<int, N>(), w, pos, on, d);
+            const unsigned long long x = group(std::integral_constant<int, N>(), w, pos, d);
             acc += x;
             if (kSecond) flush(q0, x);
             k0 += 32 * N;
             if (k0 == nxt) { ++q0; nxt = min(sh.start[q0 + 1], kend); }
             continue;
         }
-        int32_t w[kU];
-        Pos pos[kU];
-        bool on[kU];
-        uint32_t d[kU];
-        if (sh.start[q0 + kU] - k0 >= kSegMin) {
-            int q[kU];
+        if (sh.start[q0 + kSegRuns] - k0 >= kSegMin) {
+            int32_t w[kSeg];
+            Pos pos[kSeg];
+            uint32_t d[kSeg];
+            int q[kSeg];
 #pragma unroll
-            for (int u = 0; u < kU; ++u) {
+            for (int u = 0; u < kSeg; ++u) {
                 const int32_t n = min(nxt - k0, 32);   // 0 past the range
                 q[u] = q0;
-                on[u] = lane < n;
                 pos[u] = sh.src[q0] + (Pos)(k0 + lane);
-                w[u] = 0;
-                if (on[u]) w[u] = __ldg(p.adj + pos[u]);
+                w[u] = -1;
+                if (lane < n) w[u] = __ldg(p.adj + pos[u]);
                 k0 += n;
-                if (k0 == nxt && k0 < kend) { ++q0; nxt = min(sh.start[q0 + 1], kend); }
+                q0 += k0 == nxt;   // at the range's end: a run past it, never read from
+                nxt = min(sh.start[q0 + 1], kend);
             }
-            const unsigned long long x = group(std::integral_constant<int, kU>(), w, pos, on, d);
+            const unsigned long long x = group(std::integral_constant<int, kSeg>(), w, pos, d);
             acc += x;
             if (kSecond) {
-                if (q[0] == q[kU - 1]) {
+                if (q[0] == q[kSeg - 1]) {
                     flush(q[0], x);
                 } else {
 #pragma unroll
-                    for (int u = 0; u < kU; ++u) flush(q[u], d[u]);
+                    for (int u = 0; u < kSeg; ++u) flush(q[u], d[u]);
                 }
             }
             continue;
         }
+        int32_t w[kU];
+        Pos pos[kU];
+        uint32_t d[kU];
         int q[kU];
 #pragma unroll
         for (int u = 0; u < kU; ++u) {
             q[u] = 0;
-            on[u] = false;
-            pos[u] = 0;
+            pos[u] = -1;
             const int32_t kw = k0 + 32 * u;
             if (kw < kend) {   // warp-uniform
                 // run starts after this window's first wedge: 1 <= d, and
@@ -722,13 +725,12 @@ __device__ __forceinline__ unsigned long long batch_windows(const CountParams &p
                 const uint32_t m = __reduce_or_sync(0xffffffffu, bit);
                 q[u] = q0 + __popc(m & le_mask);
                 q0 += __popc(__ballot_sync(0xffffffffu, dd <= 32));
-                on[u] = kw + lane < kend;
-                if (on[u]) pos[u] = sh.src[q[u]] + (Pos)(kw + lane);
+                if (kw + lane < kend) pos[u] = sh.src[q[u]] + (Pos)(kw + lane);
             }
         }
 #pragma unroll
-        for (int u = 0; u < kU; ++u) w[u] = on[u] ? __ldg(p.adj + pos[u]) : 0;
-        acc += group(std::integral_constant<int, kU>(), w, pos, on, d);
+        for (int u = 0; u < kU; ++u) w[u] = pos[u] >= 0 ? __ldg(p.adj + pos[u]) : -1;
+        acc += group(std::integral_constant<int, kU>(), w, pos, d);
         if (kSecond) {
 #pragma unroll
             for (int u = 0; u < kU; ++u) {
@@ -1129,15 +1131,37 @@ __device__ unsigned long long dense_stream(const CountParams &p, int64_t &it, un
 }
 
 // ---- phase B: team items ----------------------------------------------------------
+// A start whose whole end range fits the team's memory as 8- or 16-bit
+// counters (Algorithm 2: the ends are the x - lb vertices below x; a count is
+// at most min(cut[x], degree of the last end, work[x])) is counted with those:
+// clearing them costs less than probing a table.  Otherwise a hash table (and
+// always above 3,072 wedges, which only a caller's own team bound brings here:
+// those starts may be re-queued).
 template <int MODE, typename Pos, class SH>
-__device__ unsigned long long team_item(const CountParams &p, int32_t x, unsigned char *table,
+__device__ unsigned long long team_item(const CountParams &p, int32_t x, unsigned char *table, int dense_bytes,
                                         SH &sh, const Team<kTeamThreads> &t) {
-    unsigned long long acc = hash_item<MODE, Pos>(p, x, table, kTeamSlots, sh, t);
-    if (sh.overflow) {
-        // a CTA table next
-        if (t.tid == 0) push_retry(p, x);
+    unsigned long long acc;
+    int32_t R = 0, lb = 0;
+    bool narrow = true;
+    if (!p.orient && p.work[x] <= (uint64_t)kTeamFitWork) {
+        lb = range_lo(p, x);
+        R = x - lb;
+        const int64_t last = R > 0 ? p.off[x] - p.off[x - 1] : 0;
+        narrow = min(min((int64_t)p.cut[x], last), (int64_t)p.work[x]) > (int64_t)kByteMaxCut;
+    }
+    if (R > 0 && (narrow ? 2 * (int64_t)R : (int64_t)R) <= dense_bytes) {
+        team_fill(table, narrow ? 2 * R : R, 0u, t);
         t.sync();
-        return 0;
+        acc = narrow ? item_body<MODE, kDenseNarrow, Pos>(p, x, lb, 0, R, 0, 0, table, sh, t)
+                     : item_body<MODE, kDenseByte, Pos>(p, x, lb, 0, R, 0, 0, table, sh, t);
+    } else {
+        acc = hash_item<MODE, Pos>(p, x, table, kTeamSlots, sh, t);
+        if (sh.overflow) {
+            // a CTA table next
+            if (t.tid == 0) push_retry(p, x);
+            t.sync();
+            return 0;
+        }
     }
     if (MODE == kModeBatch) add_to_graph(p, x, acc, sh, t);
     t.sync();
@@ -1303,25 +1327,30 @@ __global__ void __launch_bounds__(kCountThreads, kCountCtasPerSm) k_count(CountP
         __syncthreads();
     }
     // phase B: team items.  Team k owns warps 8k..8k+7 and the 48 KB of shared
-    // memory that are their warp regions; its table is followed by its batch
+    // memory that are their warp regions; its counters are followed by its batch
     // arrays.  A team leaves together (its item index is read before its
     // barrier), so none of its warps is still using the region when the
     // first one starts phase C in its own part of it.
     const int64_t n_team = n_team_items(p);
     if (n_team > 0) {
         typedef SharedTeam<MODE, Pos, kTeamThreads> TS;
-        static_assert(kTeamTableBytes + sizeof(TS) <= kTeamRegion, "team region overflow");
+        constexpr int kDenseBytes = (int)(kTeamRegion - sizeof(TS)) & ~15;
+        static_assert(kTeamTableBytes <= kDenseBytes, "team region overflow");
         const int k = threadIdx.x / kTeamThreads;
         const Team<kTeamThreads> team{(int)(threadIdx.x % kTeamThreads), 1 + k};
         unsigned char *table = ctr + (size_t)k * kTeamRegion;
-        TS &tsh = *reinterpret_cast<TS *>(table + kTeamTableBytes);
+        TS &tsh = *reinterpret_cast<TS *>(table + kDenseBytes);
+        // four items at a time where there are many per team: one queue
+        // access (and its latency) for four
+        const int grab = n_team >= (int64_t)gridDim.x * kTeams * 16 ? 4 : 1;
         for (;;) {
-            if (team.tid == 0) tsh.item = atomicAdd(p.cursors + 4, 1);
+            if (team.tid == 0) tsh.item = atomicAdd(p.cursors + 4, grab);
             team.sync();
             const int64_t it = tsh.item;
             team.sync();
             if (it >= n_team) break;
-            acc += team_item<MODE, Pos>(p, p.team_items[it], table, tsh, team);
+            for (int64_t j = it; j < min(it + grab, n_team); ++j)
+                acc += team_item<MODE, Pos>(p, p.team_items[j], table, kDenseBytes, tsh, team);
         }
     }
     // phase C: warp items

@@ -529,11 +529,22 @@ __global__ void k_chunk_counts(const int32_t *__restrict__ order, int64_t n_dens
     nch[i] = dense_chunks(x, l, cut[x], off, vbase);
 }
 
+// A start of the CTA-hash bin whose whole end range is one chunk of dense
+// counters gets those instead of a table (Algorithm 2 only): clearing at most
+// 192 KB costs a CTA about 1,500 clocks, a table with as many wedges 70 clocks
+// per 32 of them against about 10.
+__device__ __forceinline__ int2 hash_or_dense_item(int32_t x, int32_t l, int32_t cut, const int64_t *off,
+                                                   const int32_t *vbase) {
+    const int32_t lb = vbase ? vbase[x] : (x >= l ? l : 0);
+    int bits;
+    return make_int2(x, dense_chunk_end(0, x - lb, cut, off, lb, &bits) == x - lb ? 0 : -1);
+}
+
 // starts in descending work order: dense (chunked), CTA hash, team, warp
 __global__ void k_emit_items(const int32_t *__restrict__ order, int64_t n_dense, int64_t n_hash,
                              int64_t n_team, int64_t n_warp, const int64_t *__restrict__ nch_scan,
                              int32_t l, const int32_t *__restrict__ cut, const int64_t *__restrict__ off,
-                             const int32_t *__restrict__ vbase, int2 *cta_items,
+                             const int32_t *__restrict__ vbase, int ends_above, int2 *cta_items,
                              int32_t *team_items, int32_t *warp_items) {
     const int64_t total_dense = nch_scan[n_dense];
     const int64_t all = n_dense + n_hash + n_team + n_warp;
@@ -543,7 +554,8 @@ __global__ void k_emit_items(const int32_t *__restrict__ order, int64_t n_dense,
         if (i < n_dense) {
             dense_chunks(x, l, cut[x], off, vbase, cta_items + nch_scan[i]);
         } else if (i < n_dense + n_hash) {
-            cta_items[total_dense + (i - n_dense)] = make_int2(x, -1);
+            cta_items[total_dense + (i - n_dense)] =
+                ends_above ? make_int2(x, -1) : hash_or_dense_item(x, l, cut[x], off, vbase);
         } else if (i < n_dense + n_hash + n_team) {
             team_items[i - n_dense - n_hash] = x;
         } else {
@@ -824,7 +836,7 @@ static int schedule_graph(Graph *g, cudaStream_t s, int32_t warp_max_work, int32
         GET(g->mem, g->warp_items, std::max<int64_t>(n_warp, 1));
         if (n_dense + n_hash + n_team + n_warp > 0) {
             k_emit_items<<<grid_stride_blocks(n_dense + n_hash + n_team + n_warp), kT, 0, s>>>(
-                order, n_dense, n_hash, n_team, n_warp, nch_scan, l, g->cut, g->off, g->vbase, g->cta_items,
+                order, n_dense, n_hash, n_team, n_warp, nch_scan, l, g->cut, g->off, g->vbase, vpp ? 1 : 0, g->cta_items,
                 g->team_items, g->warp_items); note_launch();
             BFC_CUDA(cudaGetLastError());
         }
@@ -1347,7 +1359,8 @@ __global__ void k_sched_keys_plan(const uint64_t *__restrict__ work, int32_t n, 
 }
 
 // the item lists from the sorted order and the bin sizes on the device: a
-// dense start is one chunk, so the lists follow the order directly
+// dense start is one chunk (and so is one of the CTA-hash bin, which gets dense
+// counters too), so the lists follow the order directly
 __global__ void k_emit_items_plan(const int32_t *__restrict__ order,
                                   const unsigned long long *__restrict__ counts, int2 *cta_items,
                                   int32_t *team_items, int32_t *warp_items, const int *guard) {
@@ -1357,8 +1370,7 @@ __global__ void k_emit_items_plan(const int32_t *__restrict__ order,
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nd + nh + nt + nw;
          i += (int64_t)gridDim.x * blockDim.x) {
         const int32_t x = order[i];
-        if (i < nd) cta_items[i] = make_int2(x, 0);
-        else if (i < nd + nh) cta_items[i] = make_int2(x, -1);
+        if (i < nd + nh) cta_items[i] = make_int2(x, 0);
         else if (i < nd + nh + nt) team_items[i - nd - nh] = x;
         else warp_items[i - nd - nh - nt] = x;
     }
