@@ -515,7 +515,7 @@ int bfc_count_all_host(int32_t num_u, int32_t num_l, int64_t num_edges, const in
  * num_edges <= 1,048,576; larger graphs return BFC_ERR_INVALID_ARGUMENT
  * before any GPU work.
  *
- * All working memory is one fixed array of about 4.8 MB that every GPU which
+ * All working memory is one fixed array of about 5.8 MB that every GPU which
  * loads the library holds until the process exits; no call allocates.  The
  * first call on a device looks up that array's device address and sets the
  * kernel's attributes, so make one call per device before any stream capture.

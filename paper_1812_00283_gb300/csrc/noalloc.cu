@@ -13,9 +13,11 @@
 // file-scope __device__ array of fixed size (below), which every GPU that
 // loads the library holds until the process exits.  The caller passes only
 // inputs and outputs.  The whole count is one cooperative kernel: it clears
-// the scratch it uses, checks the CSR, builds the L-side lists, and counts
-// with Algorithm 2's priority filters (no sorted lists; each neighbour is
-// tested against the start's priority).
+// the scratch it uses, checks the CSR, ranks all vertices by Definition 3,
+// writes both sides' lists as 16-bit ranks (the filter p(w) < p(x) is then one
+// comparison, with no degree lookup per wedge) and counts with Algorithm 2:
+// a start with at most 768 possible wedges by one warp with a hash table, a
+// heavier one by a CTA with dense 16-bit counters.
 #include <cooperative_groups.h>
 
 #include <mutex>
@@ -29,152 +31,369 @@ namespace {
 
 constexpr int kNaThreads = 1024;                  // one CTA of 32 warps per SM
 constexpr int kNaWarps = kNaThreads / 32;
-constexpr int kNaSmemBytes = 192 * 1024;          // dynamic shared memory: the dense counters
-constexpr int32_t kNaMaxVertices = 65536;        // |U| + |L|
-constexpr int32_t kNaMaxLayer = kNaSmemBytes / 4; // 49,152 per layer (one dense 32-bit counter array)
-constexpr int64_t kNaMaxEdges = 1 << 20;         // 1,048,576 edges
-// words: [0,2) 64-bit accumulator | [2] error flags | [3] pad | deg[n] | loff[l+1] | lfill[l] | ladj[m]
-constexpr int64_t kNaWords = 4 + 3ll * kNaMaxVertices + 1 + kNaMaxEdges;
+constexpr int kNaSmemBytes = 192 * 1024;          // dynamic shared memory: counters, tables, sorts
+constexpr int32_t kNaMaxVertices = 65536;         // |U| + |L|: ranks fit 16 bits
+constexpr int32_t kNaMaxLayer = 49152;
+constexpr int64_t kNaMaxEdges = 1 << 20;          // 1,048,576 edges
+constexpr int kNaTiles = kNaMaxVertices / kNaThreads;
+constexpr int kNaDigits = 256;                    // rank classes: degrees 0..254 and "255 or more"
+// the degrees add up to 2m, so at most 2m / 255 vertices are in the last class
+constexpr int kNaMaxHigh = 8224;
+static_assert(2 * kNaMaxEdges / 255 <= kNaMaxHigh, "high-degree list too small");
+constexpr int kNaSlots = 1024;                    // hash slots per warp
+constexpr int32_t kNaLightWork = kNaSlots / 4 * 3;
+constexpr int kNaBigList = 512;                   // a middle's list above this is read by the whole CTA
+constexpr int kNaMaxBig = (int)(2 * kNaMaxEdges / kNaBigList);
+constexpr int kNaCntBytes = kNaMaxVertices * 2;   // 16-bit counters by rank
+static_assert(kNaCntBytes + kNaMaxBig * 2 <= kNaSmemBytes, "counters and big-list queue");
+static_assert(kNaWarps * kNaSlots * 4 <= kNaSmemBytes, "warp tables");
+static_assert(16384 * 8 <= kNaSmemBytes && kNaMaxHigh <= 16384, "high-degree sort");
+static_assert(kNaWarps * kNaDigits * 4 <= kNaSmemBytes, "per-warp digit counts");
+// words: header | deg[n] | rank[n] | vstart[n] | vdeg[n] | items[n] | lpos[l] |
+// tile histograms | high-degree list | lists as 16-bit ranks [2m]
+constexpr int kNaHeader = 16;
+constexpr int64_t kNaWords = kNaHeader + 5ll * kNaMaxVertices + kNaMaxLayer + kNaTiles * kNaDigits + kNaMaxHigh +
+                             kNaMaxEdges;
 
 }  // namespace
 }  // namespace bfc
 
-// The shared scratch of bfc_count_small_noalloc (about 4.8 MB).
+// The shared scratch of bfc_count_small_noalloc (about 5.8 MB).
 static __device__ __align__(256) int32_t g_noalloc_scratch[bfc::kNaWords];
 
 namespace bfc {
 namespace {
 
-// p(a) < p(b) in Definition 3's order, ids in the global id space
-// (L vertex v -> v, U vertex u -> l + u)
-__device__ __forceinline__ bool lower_priority(const int32_t *deg, int32_t a, int32_t b) {
-    const int32_t da = deg[a], db = deg[b];
-    return da < db || (da == db && a < b);
+// Where the scratch's parts begin.
+struct NaScratch {
+    unsigned long long *acc;
+    int32_t *err, *cursor, *n_heavy, *n_light, *q_heavy, *q_light;
+    int32_t *deg;      // [n] by global id (L vertex v -> v, U vertex u -> l + u)
+    int32_t *rank;     // [n] by global id: position in Definition 3's order
+    int32_t *vstart;   // [n] by rank: where the vertex's list starts in `adj`
+    int32_t *vdeg;     // [n] by rank: its length
+    int32_t *items;    // [n] heavy starts from the front, light ones from the back
+    int32_t *lpos;     // [l] next free position of each L list
+    int32_t *thist;    // [tiles][256]
+    int32_t *high;     // vertices of degree 255 or more, ascending global id
+    uint16_t *adj;     // [2m] neighbours' ranks: L lists, then U lists at m + off_u
+    __device__ NaScratch(int32_t *s, int32_t n, int32_t l) {
+        acc = reinterpret_cast<unsigned long long *>(s);
+        err = s + 2; cursor = s + 3; n_heavy = s + 4; n_light = s + 5; q_heavy = s + 6; q_light = s + 7;
+        deg = s + kNaHeader;
+        rank = deg + n;
+        vstart = rank + n;
+        vdeg = vstart + n;
+        items = vdeg + n;
+        lpos = items + n;
+        thist = lpos + l;
+        high = thist + kNaTiles * kNaDigits;
+        adj = reinterpret_cast<uint16_t *>(high + kNaMaxHigh);
+    }
+};
+
+// The wedges through up to 32 middles, lane i's being the list [s, s + d)
+// (d = 0: none): eight lanes per middle, four middles at a time; op(w) for
+// every end rank w below rx.  Called by whole warps.
+template <class Op>
+__device__ __forceinline__ void na_middles(const uint16_t *adj, int32_t s, int32_t d, int32_t rx,
+                                           int lane, Op op) {
+    const int g = lane >> 3, j = lane & 7;
+    uint32_t left = __ballot_sync(0xffffffffu, d > 0);
+    while (left) {
+        // the four lowest lanes still to do, one per group
+        int src = -1;
+        uint32_t m = left;
+        for (int k = 0; k < 4; ++k) {
+            const int f = __ffs((int)m) - 1;   // -1 when none is left
+            if (k == g) src = f;
+            m &= m - 1;
+        }
+        left = m;
+        const int32_t gs = __shfl_sync(0xffffffffu, s, src & 31);
+        int32_t gd = __shfl_sync(0xffffffffu, d, src & 31);
+        if (src < 0) gd = 0;
+        for (int32_t k = j; __any_sync(0xffffffffu, k < gd); k += 32) {
+            int32_t w[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) w[u] = k + 8 * u < gd ? (int32_t)adj[gs + k + 8 * u] : 0x7fffffff;
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (w[u] < rx) op(w[u]);
+        }
+    }
 }
 
+// What bounds it: latency.  A small graph is a chain of dependent passes over a
+// few hundred KB with a grid barrier between them, then starts of a few
+// microseconds each.  On 12,007 x 8,001 vertices with 150,001 edges 129 us; 521 us
+// when each row's list was built by one thread and every start took a CTA.
 __global__ void __launch_bounds__(kNaThreads, 1)
 k_count_noalloc(int32_t r, int32_t l, int32_t m, const int32_t *__restrict__ off_u,
                 const int32_t *__restrict__ adj_u, int32_t *scratch,
                 unsigned long long *total_out, int32_t *status_out) {
     cg::grid_group grid = cg::this_grid();
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    uint32_t *cnt = reinterpret_cast<uint32_t *>(smem_raw);
     __shared__ unsigned long long red[32];
-    __shared__ int32_t carry;
+    __shared__ int32_t sh_item, sh_nbig, sh_part[32], sh_base[kNaDigits];
 
     const int32_t n = r + l;
-    unsigned long long *acc_g = reinterpret_cast<unsigned long long *>(scratch);
-    int32_t *err = scratch + 2;
-    int32_t *deg = scratch + 4;
-    int32_t *loff = deg + n;
-    int32_t *lfill = loff + l + 1;
-    int32_t *ladj = lfill + l;
-    const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t gstride = (int64_t)gridDim.x * blockDim.x;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const NaScratch S(scratch, n, l);
+    const int32_t gtid = (int32_t)(blockIdx.x * blockDim.x + threadIdx.x);
+    const int32_t gstride = (int32_t)(gridDim.x * blockDim.x);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int32_t gwarp = gtid >> 5, gwarps = gstride >> 5;
+    const uint32_t lt = (1u << lane) - 1u;
 
     // clear what must start at zero (the scratch keeps the previous call's contents)
-    if (gtid == 0) { *acc_g = 0; *err = 0; }
-    for (int64_t i = gtid; i < n; i += gstride) deg[i] = 0;
-    for (int64_t i = gtid; i < l; i += gstride) lfill[i] = 0;
+    if (gtid < kNaHeader) scratch[gtid] = 0;
+    for (int32_t i = gtid; i < l; i += gstride) S.deg[i] = 0;
     grid.sync();
 
-    // the CSR must be a CSR before anything indexes with it
-    for (int64_t u = gtid; u <= r; u += gstride) {
-        if (u == 0 && off_u[0] != 0) atomicOr(err, 1);
-        if (u < r && off_u[u + 1] < off_u[u]) atomicOr(err, 1);
-        if (u == r && off_u[r] != m) atomicOr(err, 1);
-    }
-    for (int64_t k = gtid; k < m; k += gstride) {
-        const int32_t v = adj_u[k];
-        if (v < 0 || v >= l) atomicOr(err, 2);
-    }
-    grid.sync();
-    const bool bad = *((volatile int32_t *)err) != 0;
-
-    // degrees, in the global id space
-    if (!bad) {
-        for (int64_t u = gtid; u < r; u += gstride) deg[l + u] = off_u[u + 1] - off_u[u];
-        for (int64_t k = gtid; k < m; k += gstride) atomicAdd(&deg[adj_u[k]], 1);
-    }
-    grid.sync();
-
-    // L-side offsets: one block scans deg[0, l)
-    if (!bad && blockIdx.x == 0) {
-        if (threadIdx.x == 0) carry = 0;
-        __syncthreads();
-        for (int32_t base = 0; base < l; base += kNaThreads) {
-            const int32_t i = base + threadIdx.x;
-            int32_t x = i < l ? deg[i] : 0;
-            int32_t v = x;
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                int32_t o = __shfl_up_sync(0xffffffffu, v, d);
-                if (lane >= d) v += o;
-            }
-            __shared__ int32_t wsum[32];
-            if (lane == 31) wsum[warp] = v;
-            __syncthreads();
-            if (warp == 0) {
-                int32_t w = wsum[lane];
-#pragma unroll
-                for (int d = 1; d < 32; d <<= 1) {
-                    int32_t o = __shfl_up_sync(0xffffffffu, w, d);
-                    if (lane >= d) w += o;
-                }
-                wsum[lane] = w;
-            }
-            __syncthreads();
-            const int32_t incl = v + (warp > 0 ? wsum[warp - 1] : 0);
-            if (i < l) loff[i] = carry + incl - x;
-            __syncthreads();
-            if (threadIdx.x == kNaThreads - 1) carry += incl;
-            __syncthreads();
+    // the CSR must be a CSR before anything indexes with it; degrees
+    for (int32_t u = gtid; u <= r; u += gstride) {
+        const int32_t o = off_u[u];
+        if (u == 0 && o != 0) atomicOr(S.err, 1);
+        if (u == r && o != m) atomicOr(S.err, 1);
+        if (u < r) {
+            const int32_t d = off_u[u + 1] - o;
+            if (off_u[u + 1] < o) atomicOr(S.err, 1);
+            S.deg[l + u] = d;
         }
-        if (threadIdx.x == 0) loff[l] = carry;
+    }
+    for (int32_t k = gtid; k < m; k += gstride) {
+        const int32_t v = adj_u[k];
+        if (v < 0 || v >= l) atomicOr(S.err, 2);
+        else atomicAdd(&S.deg[v], 1);
     }
     grid.sync();
+    if (*((volatile int32_t *)S.err) != 0) {   // the same in every thread of the grid
+        if (gtid == 0) {
+            *total_out = 0ull;
+            if (status_out) *status_out = BFC_ERR_INVALID_GRAPH;
+        }
+        return;
+    }
 
-    // L-side lists (any order: every neighbour is tested against the filter)
-    if (!bad) {
-        for (int64_t u = gtid; u < r; u += gstride)
-            for (int32_t k = off_u[u]; k < off_u[u + 1]; ++k) {
-                const int32_t v = adj_u[k];
-                ladj[loff[v] + atomicAdd(&lfill[v], 1)] = (int32_t)u;
+    // ranks: vertices in (degree, global id) order.  One stable counting pass
+    // over 256 classes (degrees 0..254 exactly, the rest in the last class),
+    // 1,024 vertices per CTA; then the few vertices of the last class are
+    // sorted by one CTA.
+    uint32_t *const wcnt = reinterpret_cast<uint32_t *>(smem_raw);   // [32 warps][256]
+    const int tiles = (n + kNaThreads - 1) / kNaThreads;
+    int32_t digit = 0, before = 0;   // this thread's class and its place among its warp's
+    const int32_t id = (int32_t)blockIdx.x * kNaThreads + tid;
+    if ((int)blockIdx.x < tiles) {
+        for (int i = tid; i < kNaWarps * kNaDigits; i += kNaThreads) wcnt[i] = 0;
+        __syncthreads();
+        digit = id < n ? min(S.deg[id], kNaDigits - 1) : kNaDigits;
+        const uint32_t peers = __match_any_sync(0xffffffffu, digit);
+        before = __popc(peers & lt);
+        if (id < n && before == 0) wcnt[warp * kNaDigits + digit] = __popc(peers);
+        __syncthreads();
+        if (tid < kNaDigits) {   // prefix over the warps, tile totals
+            uint32_t run = 0;
+            for (int w = 0; w < kNaWarps; ++w) {
+                const uint32_t c = wcnt[w * kNaDigits + tid];
+                wcnt[w * kNaDigits + tid] = run;
+                run += c;
             }
+            S.thist[blockIdx.x * kNaDigits + tid] = (int32_t)run;
+        }
+    }
+    // L lists: 32 at a time take their room from one cursor (any order)
+    for (int32_t v0 = gwarp * 32; v0 < l; v0 += gwarps * 32) {
+        const int32_t v = v0 + lane, d = v < l ? S.deg[v] : 0;
+        int32_t incl = d;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        int32_t at = 0;
+        if (lane == 31) at = atomicAdd(S.cursor, incl);
+        at = __shfl_sync(0xffffffffu, at, 31) + incl - d;
+        if (v < l) S.lpos[v] = at;
+    }
+    grid.sync();
+    if ((int)blockIdx.x < tiles) {
+        // class starts: all tiles of the lower classes, and the lower tiles of this one
+        int32_t all = 0, mine = 0;
+        if (tid < kNaDigits)
+            for (int t = 0; t < tiles; ++t) {
+                const int32_t c = S.thist[t * kNaDigits + tid];
+                if (t < (int)blockIdx.x) mine += c;
+                all += c;
+            }
+        int32_t incl = all;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        if (lane == 31) sh_part[warp] = incl;
+        __syncthreads();
+        if (tid < kNaDigits) {
+            int32_t lower = 0;
+            for (int w = 0; w < warp; ++w) lower += sh_part[w];
+            sh_base[tid] = lower + incl - all + mine;
+            if (tid == kNaDigits - 1) sh_item = lower + incl - all;   // first rank of the last class
+        }
+        __syncthreads();
+        if (id < n) {
+            const int32_t rk = sh_base[digit] + (int32_t)wcnt[warp * kNaDigits + digit] + before;
+            if (digit == kNaDigits - 1) {
+                S.high[rk - sh_item] = id;
+            } else {
+                S.rank[id] = rk;
+                S.vstart[rk] = id < l ? S.lpos[id] : m + off_u[id - l];
+                S.vdeg[rk] = S.deg[id];
+            }
+        }
+    }
+    grid.sync();
+    if (blockIdx.x == 0) {   // the last class: ascending (degree, id) by a bitonic sort
+        const int32_t first = n > 0 ? sh_item : 0, nh = n - first;
+        uint64_t *const buf = reinterpret_cast<uint64_t *>(smem_raw);
+        int np = 1;
+        while (np < nh) np <<= 1;
+        if (nh > 0) {
+            for (int i = tid; i < np; i += kNaThreads)
+                buf[i] = i < nh ? ((uint64_t)(uint32_t)S.deg[S.high[i]] << 32) | (uint32_t)S.high[i] : ~0ull;
+            __syncthreads();
+            for (int k = 2; k <= np; k <<= 1)
+                for (int j = k >> 1; j > 0; j >>= 1) {
+                    for (int i = tid; i < np; i += kNaThreads) {
+                        const int ij = i ^ j;
+                        if (ij > i) {
+                            const uint64_t a = buf[i], c = buf[ij];
+                            if ((a > c) == ((i & k) == 0)) { buf[i] = c; buf[ij] = a; }
+                        }
+                    }
+                    __syncthreads();
+                }
+            for (int i = tid; i < nh; i += kNaThreads) {
+                const int32_t v = (int32_t)(uint32_t)buf[i], rk = first + i;
+                S.rank[v] = rk;
+                S.vstart[rk] = v < l ? S.lpos[v] : m + off_u[v - l];
+                S.vdeg[rk] = S.deg[v];
+            }
+        }
     }
     grid.sync();
 
-    // Algorithm 2: for every start x, middles v with p(v) < p(x), ends w with
-    // p(w) < p(x); Σ old over the increments of count_wedge(w) = Σ C(count, 2)
+    // both sides' lists as ranks; an edge finds its row by a binary search
+    for (int32_t k = gtid; k < m; k += gstride) {
+        const int32_t v = adj_u[k];
+        int32_t lo = 0, hi = r;   // last u with off_u[u] <= k (the one with a non-empty row)
+        while (hi - lo > 1) {
+            const int32_t mid = (lo + hi) >> 1;
+            if (off_u[mid] <= k) lo = mid; else hi = mid;
+        }
+        S.adj[m + k] = (uint16_t)S.rank[v];
+        S.adj[atomicAdd(&S.lpos[v], 1)] = (uint16_t)S.rank[l + lo];
+    }
+    grid.sync();
+
+    // starts: one with at most one possible wedge closes no butterfly; a light
+    // one has at most 768
+    for (int32_t i = gwarp; i < n; i += gwarps) {
+        const int32_t x = n - 1 - i, s = S.vstart[x], d = S.vdeg[x];
+        if (d < 2) continue;
+        int32_t bound = 0;
+        bool heavy = d > 1024;
+        for (int32_t j = lane; !heavy && j - lane < d; j += 32) {
+            const int32_t v = j < d ? (int32_t)S.adj[s + j] : 0x7fffffff;
+            const int32_t b = v < x ? min(S.vdeg[v] - 1, kNaLightWork + 1) : 0;
+            bound += (int32_t)__reduce_add_sync(0xffffffffu, (unsigned)b);
+            heavy = bound > kNaLightWork;   // the same in every lane
+        }
+        if (!heavy && bound < 2) continue;
+        if (lane == 0) {
+            if (heavy) S.items[atomicAdd(S.n_heavy, 1)] = x;
+            else S.items[n - 1 - atomicAdd(S.n_light, 1)] = x;
+        }
+    }
+    grid.sync();
+
+    // Algorithm 2: Σ old over the increments of count_wedge(w) = Σ C(count, 2)
     unsigned long long acc = 0;
-    if (!bad) {
-        for (int32_t x = blockIdx.x; x < n; x += gridDim.x) {
-            const bool in_u = x >= l;
-            const int32_t layer = in_u ? r : l;
-            const int32_t mb = in_u ? off_u[x - l] : loff[x];
-            const int32_t me = in_u ? off_u[x - l + 1] : loff[x + 1];
-            // a start none of whose neighbours has lower priority has no
-            // wedges: skip its clear and its walk (most light starts)
-            bool any = false;
-            for (int32_t j = mb + threadIdx.x; j < me && !any; j += kNaThreads)
-                any = lower_priority(deg, in_u ? adj_u[j] : l + ladj[j], x);
-            if (!__syncthreads_or(any)) continue;
-            uint4 *c4 = reinterpret_cast<uint4 *>(cnt);
-            for (int32_t i = threadIdx.x; i < (layer + 3) / 4; i += kNaThreads)
-                c4[i] = make_uint4(0, 0, 0, 0);
+    const int32_t n_heavy = *((volatile int32_t *)S.n_heavy), n_light = *((volatile int32_t *)S.n_light);
+    {
+        uint32_t *const cnt = reinterpret_cast<uint32_t *>(smem_raw);   // 16-bit counters, two per word
+        uint16_t *const big = reinterpret_cast<uint16_t *>(smem_raw + kNaCntBytes);
+        for (;;) {
             __syncthreads();
-            for (int32_t j = mb + warp; j < me; j += kNaWarps) {
-                const int32_t v = in_u ? adj_u[j] : l + ladj[j];       // middle, global id
-                if (!lower_priority(deg, v, x)) continue;
-                const int32_t eb = in_u ? loff[v] : off_u[v - l];
-                const int32_t ee = in_u ? loff[v + 1] : off_u[v - l + 1];
-                for (int32_t k = eb + lane; k < ee; k += 32) {
-                    const int32_t w = in_u ? l + ladj[k] : adj_u[k];   // end, global id
-                    if (lower_priority(deg, w, x)) acc += atomicAdd(&cnt[in_u ? w - l : w], 1u);
+            if (tid == 0) { sh_item = atomicAdd(S.q_heavy, 1); sh_nbig = 0; }
+            __syncthreads();
+            const int32_t it = sh_item;
+            if (it >= n_heavy) break;
+            const int32_t x = S.items[it], s = S.vstart[x], d = S.vdeg[x];
+            uint4 *const c4 = reinterpret_cast<uint4 *>(smem_raw);
+            for (int32_t i = tid; i < (x + 7) / 8; i += kNaThreads) c4[i] = make_uint4(0, 0, 0, 0);
+            __syncthreads();
+            auto op = [&](int32_t w) {
+                const uint32_t sh = (uint32_t)(w & 1) << 4;
+                acc += (atomicAdd(cnt + (w >> 1), 1u << sh) >> sh) & 0xffffu;
+            };
+            for (int32_t j0 = warp * 32; j0 < d; j0 += kNaThreads) {
+                const int32_t v = j0 + lane < d ? (int32_t)S.adj[s + j0 + lane] : 0x7fffffff;
+                int32_t vs = 0, vd = 0;
+                if (v < x) { vs = S.vstart[v]; vd = S.vdeg[v]; }
+                if (vd > kNaBigList) {
+                    const int at = atomicAdd(&sh_nbig, 1);
+                    if (at < kNaMaxBig) { big[at] = (uint16_t)v; vd = 0; }   // else this warp reads it
+                }
+                na_middles(S.adj, vs, vd, x, lane, op);
+            }
+            __syncthreads();
+            const int nbig = min(sh_nbig, kNaMaxBig);
+            for (int b = 0; b < nbig; ++b) {
+                const int32_t v = big[b], vs = S.vstart[v], vd = S.vdeg[v];
+                for (int32_t k = tid; k < vd; k += kNaThreads) {
+                    const int32_t w = S.adj[vs + k];
+                    if (w < x) op(w);
                 }
             }
-            __syncthreads();
+        }
+    }
+    {
+        // light starts: a table of (rank, count) words per warp; a rank below
+        // x is never 65,535, so all ones marks an empty slot
+        uint32_t *const tab = reinterpret_cast<uint32_t *>(smem_raw) + warp * kNaSlots;
+        for (;;) {
+            int32_t it = 0;
+            if (lane == 0) it = atomicAdd(S.q_light, 1);
+            it = __shfl_sync(0xffffffffu, it, 0);
+            if (it >= n_light) break;
+            const int32_t x = S.items[n - 1 - it], s = S.vstart[x], d = S.vdeg[x];
+            uint4 *const t4 = reinterpret_cast<uint4 *>(tab);
+            for (int i = lane; i < kNaSlots / 4; i += 32) t4[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
+            __syncwarp();
+            auto op = [&](int32_t w) {
+                uint32_t h = ((uint32_t)w * 0x9E3779B1u) >> 22;   // 10 bits
+                static_assert(kNaSlots == 1024, "ten hash bits");
+                for (int probe = 0; probe < kNaSlots; ++probe) {
+                    uint32_t e = *((volatile uint32_t *)(tab + h));
+                    if (e == ~0u) {
+                        e = atomicCAS(tab + h, ~0u, ((uint32_t)w << 16) | 1u);
+                        if (e == ~0u) return;
+                    }
+                    if ((e >> 16) == (uint32_t)w) {
+                        acc += atomicAdd(tab + h, 1u) & 0xffffu;
+                        return;
+                    }
+                    h = (h + 1) & (kNaSlots - 1);
+                }
+                atomicOr(S.err, 4);   // cannot happen: at most 768 distinct ends
+            };
+            for (int32_t j0 = 0; j0 < d; j0 += 32) {
+                const int32_t v = j0 + lane < d ? (int32_t)S.adj[s + j0 + lane] : 0x7fffffff;
+                int32_t vs = 0, vd = 0;
+                if (v < x) { vs = S.vstart[v]; vd = S.vdeg[v]; }
+                na_middles(S.adj, vs, vd, x, lane, op);
+            }
+            __syncwarp();
         }
     }
 #pragma unroll
@@ -185,12 +404,13 @@ k_count_noalloc(int32_t r, int32_t l, int32_t m, const int32_t *__restrict__ off
         unsigned long long t = red[lane];
 #pragma unroll
         for (int d = 16; d > 0; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
-        if (lane == 0 && t) atomicAdd(acc_g, t);
+        if (lane == 0 && t) atomicAdd(S.acc, t);
     }
     grid.sync();
     if (gtid == 0) {
-        *total_out = bad ? 0ull : *((volatile unsigned long long *)acc_g);
-        if (status_out) *status_out = bad ? BFC_ERR_INVALID_GRAPH : BFC_OK;
+        const bool full = (*((volatile int32_t *)S.err) & 4) != 0;
+        *total_out = *((volatile unsigned long long *)S.acc);
+        if (status_out) *status_out = full ? BFC_ERR_INTERNAL : BFC_OK;
     }
 }
 
@@ -219,7 +439,7 @@ int noalloc_setup(int dev, int32_t **ptr, int *grid) {
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_count_noalloc, kNaThreads,
                                                           kNaSmemBytes);
         if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
-        if (per_sm < 1) { set_last_error("k_count_noalloc does not fit on an SM"); return BFC_ERR_CUDA; }
+        if (per_sm < 1 || sms * per_sm < kNaTiles) { set_last_error("k_count_noalloc does not fit on the device"); return BFC_ERR_CUDA; }
         g_na_grid[dev] = sms * per_sm;
         g_na_ptr[dev] = static_cast<int32_t *>(p);
     }
