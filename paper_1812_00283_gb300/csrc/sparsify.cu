@@ -50,54 +50,114 @@ __global__ void k_sp_check_offsets(const int32_t *__restrict__ off, int32_t r, i
     }
 }
 
-// One warp per row (j, u) of the union: lanes draw for the row's slots, a
-// ballot gives the kept slots.  kWrite = false: the kept count of the row
-// (and, for sample 0, a check of the L ids, bit 1 of *bad); kWrite = true:
-// the kept L ids, shifted to sample j's range, at the row's offset.
-template <bool kWrite>
-__global__ void k_sp_rows(const int32_t *__restrict__ off, const int32_t *__restrict__ adj, int32_t r,
-                          int32_t l, int64_t m, int32_t samples, SampleRule rule, int64_t *__restrict__ cnt,
-                          const int64_t *__restrict__ uoff, int32_t *__restrict__ uoff32,
-                          int32_t *__restrict__ uadj, int *bad) {
-    const int lane = threadIdx.x & 31;
+// The union's edges in order are the kept slots of sample 0, then of sample
+// 1, ...: a stream compaction over the linear index (sample, slot), with no row
+// in it.  Slots are taken 32 at a time: sample j has m / 32 + 1 words, bit i of
+// word w = slot 32 w + i is kept (the last word reaches past slot m - 1, so that
+// every row offset lies in a word of its sample).  The masks and their prefixes
+// (8 bytes per word) are held for as many samples at a time as fit 2 GB; when
+// that is not all of them the masks are drawn twice.
+// Before: two passes of one warp per (sample, row), whose rows average 20 slots,
+// 5.7 ms for 16 samples of a 20M-edge graph.
+constexpr int kSpWords = kT;   // words per CTA: 32 per warp
+constexpr int64_t kSpGroupBytes = 1ll << 31;
+
+// Pass 1: the keep masks and the kept slots per CTA (and, for sample 0, a
+// check of the L ids, bit 1 of *bad).  Bound by the draws' 64-bit integer
+// multiplications.
+__global__ void __launch_bounds__(kT) k_sp_masks(const int32_t *__restrict__ adj, int32_t l, int64_t m,
+                                                 int32_t j0, int64_t words, int64_t all_words, SampleRule rule,
+                                                 uint32_t *__restrict__ mask, int64_t *__restrict__ cnt, int *bad) {
+    __shared__ int32_t part[kT / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t w0 = (int64_t)blockIdx.x * kSpWords + warp * 32;
+    uint32_t mine = 0;
+    int64_t j = j0 + w0 / words, wj = w0 % words;   // sample, word of it
+    for (int k = 0; k < 32 && w0 + k < all_words; ++k) {   // warp-uniform
+        const int64_t e = wj * 32 + lane;
+        const bool in = e < m;
+        if (j == 0 && in) {
+            const int32_t v = adj[e];
+            if (v < 0 || v >= l) atomicOr(bad, 2);
+        }
+        const bool keep = in && (rule.keep_all ||
+                                 splitmix64_at(rule.seed, (uint64_t)j * (uint64_t)m + 1 + (uint64_t)e) < rule.threshold);
+        const uint32_t b = __ballot_sync(0xffffffffu, keep);
+        if (k == lane) mine = b;
+        if (++wj == words) { wj = 0; ++j; }
+    }
+    if (w0 + lane < all_words) mask[w0 + lane] = mine;
+    const int32_t c = (int32_t)__reduce_add_sync(0xffffffffu, (unsigned)__popc(mine));
+    if (lane == 0) part[warp] = c;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int32_t t = 0;
+        for (int w = 0; w < kT / 32; ++w) t += part[w];
+        cnt[blockIdx.x] = t;
+    }
+}
+
+// Pass 2: the kept L ids, shifted to their sample's range, in order; per word
+// the kept slots before it.  The id check has passed, the union fits 32 bits.
+__global__ void __launch_bounds__(kT) k_sp_compact(const int32_t *__restrict__ adj, int32_t l, int32_t j0,
+                                                   int64_t words, int64_t all_words, const uint32_t *__restrict__ mask,
+                                                   const int64_t *__restrict__ cnt_scan,
+                                                   int32_t *__restrict__ wpre, int32_t *__restrict__ uadj) {
+    __shared__ int32_t part[kT / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t w0 = (int64_t)blockIdx.x * kSpWords + warp * 32;
+    const uint32_t mine = w0 + lane < all_words ? mask[w0 + lane] : 0;
+    const int32_t c = __popc(mine);
+    int32_t incl = c;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int32_t o = __shfl_up_sync(0xffffffffu, incl, d);
+        if (lane >= d) incl += o;
+    }
+    if (lane == 31) part[warp] = incl;
+    __syncthreads();
+    int32_t at = (int32_t)cnt_scan[blockIdx.x] + incl - c;
+    for (int w = 0; w < warp; ++w) at += part[w];
+    if (w0 + lane < all_words) wpre[w0 + lane] = at;
     const uint32_t lt = (1u << lane) - 1u;
-    const int64_t rows = (int64_t)samples * r;
-    const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t row = w0; row < rows; row += nw) {
-        const int64_t j = row / r;
-        const int32_t u = (int32_t)(row - j * r);
-        const int32_t e0 = off[u], e1 = off[u + 1];
-        const uint64_t k0 = (uint64_t)j * (uint64_t)m + 1;   // draw number of slot 0
-        const int32_t shift = (int32_t)(j * l);
-        int64_t at = kWrite ? uoff[row] : 0;
-        int32_t kept = 0;
-        for (int64_t b = e0; b < e1; b += 32) {   // warp-uniform
-            const int64_t e = b + lane;
-            const bool in = e < e1;
-            const int32_t v = in ? adj[e] : 0;
-            const bool keep = in && (rule.keep_all || splitmix64_at(rule.seed, k0 + (uint64_t)e) < rule.threshold);
-            if (!kWrite && j == 0 && in && (v < 0 || v >= l)) atomicOr(bad, 2);
-            const uint32_t bal = __ballot_sync(0xffffffffu, keep);
-            if (kWrite && keep) uadj[at + kept + __popc(bal & lt)] = v + shift;
-            kept += __popc(bal);
+    int64_t j = j0 + w0 / words, wj = w0 % words;
+    for (int k = 0; k < 32 && w0 + k < all_words; ++k) {   // warp-uniform
+        const uint32_t b = __shfl_sync(0xffffffffu, mine, k);
+        const int32_t p = __shfl_sync(0xffffffffu, at, k);
+        if ((b >> lane) & 1u) uadj[p + __popc(b & lt)] = adj[wj * 32 + lane] + (int32_t)(j * l);
+        if (++wj == words) { wj = 0; ++j; }
+    }
+}
+
+// Pass 3: the union's row offsets: row (j, u) starts after the kept slots
+// of sample j below off[u] (and all of the samples before it); and where each
+// sample starts.
+__global__ void k_sp_offsets(const int32_t *__restrict__ off, int32_t r, int32_t j0, int32_t group, int64_t words,
+                             const uint32_t *__restrict__ mask, const int32_t *__restrict__ wpre,
+                             int32_t *__restrict__ uoff, int32_t *__restrict__ sstart) {
+    const int64_t rows = (int64_t)group * r;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < rows + group;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        if (i >= rows) {
+            sstart[j0 + (i - rows)] = wpre[(i - rows) * words];
+            continue;
         }
-        if (lane == 0) {
-            if (kWrite) uoff32[row] = (int32_t)at;
-            else cnt[row] = kept;
-        }
+        const int64_t j = i / r;
+        const int32_t e = off[i - j * r];
+        const int64_t w = j * words + (e >> 5);
+        uoff[(int64_t)j0 * r + i] = wpre[w] + __popc(mask[w] & ((1u << (e & 31)) - 1u));
     }
 }
 
 // the union's last offset, the sample ranges and the kept edges per sample
-__global__ void k_sp_ranges(const int64_t *__restrict__ uoff, int32_t r, int32_t l, int32_t samples,
-                            int32_t *uoff32, int32_t *us, int32_t *ls, uint64_t *sample_edges) {
+__global__ void k_sp_ranges(const int32_t *__restrict__ sstart, int32_t kept, int32_t r, int32_t l,
+                            int32_t samples, int32_t *uoff, int32_t *us, int32_t *ls, uint64_t *sample_edges) {
     for (int32_t j = blockIdx.x * blockDim.x + threadIdx.x; j <= samples; j += gridDim.x * blockDim.x) {
         us[j] = (int32_t)((int64_t)j * r);
         ls[j] = (int32_t)((int64_t)j * l);
-        if (j == samples) uoff32[(int64_t)samples * r] = (int32_t)uoff[(int64_t)samples * r];
+        if (j == samples) uoff[(int64_t)samples * r] = kept;
         if (sample_edges && j < samples)
-            sample_edges[j] = (uint64_t)(uoff[(int64_t)(j + 1) * r] - uoff[(int64_t)j * r]);
+            sample_edges[j] = (uint64_t)((j + 1 < samples ? sstart[j + 1] : kept) - sstart[j]);
     }
 }
 
@@ -160,15 +220,30 @@ extern "C" int bfc_prepare_sparsified(int32_t num_u, int32_t num_l, int64_t num_
     a.stream = s;
     struct Guard { bfc::Allocs *a; ~Guard() { a->release(); } } guard{&a};
     const int64_t rows = (int64_t)num_samples * num_u;
+    const int64_t words = num_edges / 32 + 1;
+    const int32_t group = (int32_t)std::min<int64_t>(num_samples, std::max<int64_t>(bfc::kSpGroupBytes / (8 * words), 1));
+    const int32_t groups = (num_samples + group - 1) / group;
+    const int64_t gctas = (group * words + bfc::kSpWords - 1) / bfc::kSpWords;   // per group
     int *bad;
-    int64_t *cnt, *uoff, *scan_tmp;
-    int32_t *uoff32, *us, *ls;
-    if (a.get(&bad, 1) || a.get(&cnt, rows + 1) || a.get(&uoff, rows + 1) ||
-        a.get(&scan_tmp, bfc::scan_tmp_elems<int64_t>(rows)) || a.get(&uoff32, rows + 1) ||
-        a.get(&us, (size_t)num_samples + 1) || a.get(&ls, (size_t)num_samples + 1)) {
+    int64_t *cnt, *cnt_scan, *scan_tmp;
+    uint32_t *mask;
+    int32_t *wpre, *uoff, *us, *ls, *sstart;
+    if (a.get(&bad, 1) || a.get(&cnt, gctas * groups) || a.get(&cnt_scan, gctas * groups + 1) ||
+        a.get(&scan_tmp, bfc::scan_tmp_elems<int64_t>(gctas * groups)) || a.get(&mask, group * words) ||
+        a.get(&wpre, group * words) || a.get(&uoff, rows + 1) || a.get(&us, (size_t)num_samples + 1) ||
+        a.get(&ls, (size_t)num_samples + 1) || a.get(&sstart, num_samples)) {
         bfc::set_last_error("device allocation failed: sample offsets");
         return BFC_ERR_OUT_OF_MEMORY;
     }
+    // the masks of group g (every group but the last is full; a CTA past the
+    // last one's words counts 0)
+    auto draw = [&](int32_t g) {
+        const int64_t all = std::min(group, num_samples - g * group) * words;
+        bfc::k_sp_masks<<<(unsigned)gctas, bfc::kT, 0, s>>>(adj_u_dev, num_l, num_edges, g * group, words, all, rule,
+                                                             mask, cnt + g * gctas, bad);
+        bfc::note_launch();
+        return cudaGetLastError();
+    };
     BFC_CUDA(cudaMemsetAsync(bad, 0, sizeof(int), s));
     bfc::k_sp_check_offsets<<<bfc::grid_for((int64_t)num_u + 1), bfc::kT, 0, s>>>(off_u_dev, num_u, num_edges, bad);
     bfc::note_launch();
@@ -177,16 +252,10 @@ extern "C" int bfc_prepare_sparsified(int32_t num_u, int32_t num_l, int64_t num_
     BFC_CUDA(cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
     BFC_CUDA(cudaStreamSynchronize(s));
     if (hbad) { bfc::set_last_error("offsets are not a CSR of num_edges slots"); return BFC_ERR_INVALID_GRAPH; }
-    const unsigned rgrid = bfc::grid_for(rows * 32);
-    if (rows > 0) {
-        bfc::k_sp_rows<false><<<rgrid, bfc::kT, 0, s>>>(off_u_dev, adj_u_dev, num_u, num_l, num_edges, num_samples,
-                                                        rule, cnt, nullptr, nullptr, nullptr, bad);
-        bfc::note_launch();
-        BFC_CUDA(cudaGetLastError());
-    }
-    BFC_CUDA(bfc::scan_exclusive<int64_t>(cnt, uoff, rows, scan_tmp, s));
+    for (int32_t g = 0; g < groups; ++g) BFC_CUDA(draw(g));
+    BFC_CUDA(bfc::scan_exclusive<int64_t>(cnt, cnt_scan, gctas * groups, scan_tmp, s));
     int64_t kept = 0;
-    BFC_CUDA(cudaMemcpyAsync(&kept, uoff + rows, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+    BFC_CUDA(cudaMemcpyAsync(&kept, cnt_scan + gctas * groups, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     BFC_CUDA(cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
     BFC_CUDA(cudaStreamSynchronize(s));
     if (hbad) { bfc::set_last_error("an L id lies outside [0, num_l)"); return BFC_ERR_INVALID_GRAPH; }
@@ -199,17 +268,23 @@ extern "C" int bfc_prepare_sparsified(int32_t num_u, int32_t num_l, int64_t num_
         bfc::set_last_error("device allocation failed: sampled edges");
         return BFC_ERR_OUT_OF_MEMORY;
     }
-    if (rows > 0) {
-        bfc::k_sp_rows<true><<<rgrid, bfc::kT, 0, s>>>(off_u_dev, adj_u_dev, num_u, num_l, num_edges, num_samples,
-                                                       rule, nullptr, uoff, uoff32, uadj, bad);
+    for (int32_t g = 0; g < groups; ++g) {
+        const int32_t j0 = g * group, gs = std::min(group, num_samples - j0);
+        if (groups > 1) BFC_CUDA(draw(g));
+        bfc::k_sp_compact<<<(unsigned)gctas, bfc::kT, 0, s>>>(adj_u_dev, num_l, j0, words, gs * words, mask,
+                                                               cnt_scan + g * gctas, wpre, uadj);
+        bfc::note_launch();
+        BFC_CUDA(cudaGetLastError());
+        bfc::k_sp_offsets<<<bfc::grid_for((int64_t)gs * num_u + gs), bfc::kT, 0, s>>>(off_u_dev, num_u, j0, gs, words,
+                                                                                       mask, wpre, uoff, sstart);
         bfc::note_launch();
         BFC_CUDA(cudaGetLastError());
     }
     bfc::k_sp_ranges<<<bfc::grid_for((int64_t)num_samples + 1), bfc::kT, 0, s>>>(
-        uoff, num_u, num_l, num_samples, uoff32, us, ls, sample_edges_dev);
+        sstart, (int32_t)kept, num_u, num_l, num_samples, uoff, us, ls, sample_edges_dev);
     bfc::note_launch();
     BFC_CUDA(cudaGetLastError());
-    const bfc_csr u{(int32_t)rows, (int32_t)((int64_t)num_samples * num_l), kept, uoff32, uadj};
+    const bfc_csr u{(int32_t)rows, (int32_t)((int64_t)num_samples * num_l), kept, uoff, uadj};
     const bfc_batch b{num_samples, us, ls};
     // the union's arrays go back to the pool in stream order after the prepare
     return bfc_prepare_batch(&u, &b, opt, stream, out);
