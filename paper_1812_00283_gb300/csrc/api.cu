@@ -14,6 +14,7 @@ namespace bfc {
 
 int gather_vertices(Graph *g, cudaStream_t s, uint64_t *per_u, uint64_t *per_l);
 int gather_edges(Graph *g, cudaStream_t s, uint64_t *per_edge);
+int export_eid(const Graph *g, cudaStream_t s, int32_t *out);
 
 namespace {
 thread_local std::string g_last_error;
@@ -594,7 +595,7 @@ int bfc_export(const bfc_graph *h, int which, void *dst, void *stream) {
         case BFC_RANK_L: src = g->rank_l; bytes = 4 * (size_t)g->l; break;
         case BFC_PROJ_OFF: src = g->off; bytes = 8 * ((size_t)g->n + 1); break;
         case BFC_PROJ_ADJ: src = g->adj; bytes = 4 * (size_t)(2 * g->m); break;
-        case BFC_PROJ_EID: src = g->eid; bytes = 4 * (size_t)(2 * g->m); break;
+        case BFC_PROJ_EID: return bfc::export_eid(g, s, static_cast<int32_t *>(dst));
         case BFC_CUT: src = g->cut; bytes = 4 * (size_t)g->n; break;
         case BFC_WORK: src = g->work; bytes = 8 * (size_t)g->n; break;
         case BFC_RETRIES: src = g->cursors + 2; bytes = 4; break;

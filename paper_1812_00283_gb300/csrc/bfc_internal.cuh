@@ -158,7 +158,7 @@ struct Graph {
     int32_t *rank_u = nullptr, *rank_l = nullptr;  // original id -> rank in layer
     int64_t *off = nullptr;   // [n+1] CSR of G*
     int32_t *adj = nullptr;   // [2m]
-    int32_t *eid = nullptr;   // [2m]
+    int32_t *eid = nullptr;   // [2m] U-side slots: edge id; L-side slots: the edge's U-side position (slot - m)
     int32_t *plen = nullptr;  // [2m] wedges through each middle slot (0 if not a middle slot)
     int32_t *cut = nullptr;   // [n]
     uint64_t *work = nullptr; // [n]
@@ -236,15 +236,15 @@ cudaError_t max_scan_inclusive_i64(const int64_t *in, int64_t *out, int64_t n, i
 // Stable LSD radix sort of (uint64 key, int32 value) pairs on key bits
 // [begin_bit, end_bit).  Ping-pongs between (k0, v0) and (k1, v1); returns
 // 0 if the result is in (k0, v0), 1 if in (k1, v1).  `hist` needs
-// radix_hist_elems(n) uint32 and `scan_tmp` scan_tmp_elems<uint32_t>(..).
+// radix_hist_elems(n) uint32 and `scan_tmp` scan_tmp_elems<uint32_t>(..).  With
+// index_values the values are the keys' indexes before the sort (v0 is not read).
 size_t radix_hist_elems(int64_t n);
 cudaError_t radix_sort_pairs(uint64_t *k0, int32_t *v0, uint64_t *k1, int32_t *v1, int64_t n,
                              int begin_bit, int end_bit, uint32_t *hist, uint32_t *scan_tmp,
-                             cudaStream_t s, int *which);
+                             cudaStream_t s, int *which, bool index_values = false);
 
-// Device-wide max / sum reductions into one element (result in device memory).
+// Device-wide maximum into one element (result in device memory).
 cudaError_t reduce_max_i32(const int32_t *in, int64_t n, int32_t *out, cudaStream_t s);
-cudaError_t reduce_max_u64(const uint64_t *in, int64_t n, unsigned long long *out, cudaStream_t s);
 
 // ---------------------------------------------------------------------------
 // Prepare and count (prepare.cu, count.cu)
@@ -273,7 +273,7 @@ struct BatchPlan {
     uint64_t team_max = 0;         // team bin bound (at most 3,072: no retry pass)
     uint64_t *k0 = nullptr, *k1 = nullptr;
     int32_t *v0 = nullptr, *v1 = nullptr, *deg_u = nullptr, *deg_l = nullptr, *deg_star = nullptr;
-    int32_t *rows = nullptr, *heads = nullptr, *rows_star = nullptr, *tier_rows = nullptr, *tier_n = nullptr;
+    int32_t *rows_star = nullptr, *tier_rows = nullptr, *tier_n = nullptr, *big = nullptr, *n_big = nullptr;
     uint32_t *hist = nullptr, *hist_tmp = nullptr;
     int64_t *scan64_tmp = nullptr, *deg64 = nullptr;
     unsigned long long *red = nullptr;   // [0] W, [4..8) bin sizes

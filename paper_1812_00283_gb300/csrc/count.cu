@@ -469,8 +469,16 @@ struct BatchSlots {
     int nzs[kPer];
 };
 
+// Where a middle's Σ δ goes: the U-side slot of the edge (x, v).  An L start's
+// slots hold that position, so its sums skip the L-side slots, whose additions
+// would all have to be carried over to the U side after the walk.
+__device__ __forceinline__ int64_t edge_slot(const CountParams &p, int64_t e) {
+    const int64_t m = p.adj_len >> 1;
+    return e < m ? m + __ldg(p.eid + e) : e;
+}
+
 // The per-middle sums of a second-walk batch: Σ δ over each middle's ends
-// goes to the middle (per-vertex) and to the edge (x, v) at its slot.
+// goes to the middle (per-vertex) and to the edge (x, v) at its U-side slot.
 template <int MODE, typename Pos, int kThreads, class SH>
 __device__ __forceinline__ void middle_sums(const CountParams &p, const BatchSlots<Pos, kThreads> &bs,
                                             const SH &sh) {
@@ -480,7 +488,7 @@ __device__ __forceinline__ void middle_sums(const CountParams &p, const BatchSlo
             const unsigned long long dsum = msum_get(sh.msum[bs.nzs[i]]);
             if (dsum) {
                 if (wants_vertices(MODE)) atomicAdd(p.pv + bs.v[i], dsum);
-                if (wants_edges(MODE)) atomicAdd(p.pe + bs.e[i], dsum);
+                if (wants_edges(MODE)) atomicAdd(p.pe + edge_slot(p, bs.e[i]), dsum);
             }
         }
     }
@@ -1244,7 +1252,7 @@ __device__ unsigned long long warp_walk(const CountParams &p, int32_t x, int32_t
             const unsigned long long dsum = msum_get(msum[nz]);
             if (dsum) {
                 if (wants_vertices(MODE)) atomicAdd(p.pv + v, dsum);
-                if (wants_edges(MODE)) atomicAdd(p.pe + e, dsum);
+                if (wants_edges(MODE)) atomicAdd(p.pe + edge_slot(p, e), dsum);
             }
         }
         __syncwarp();
@@ -1415,27 +1423,32 @@ __global__ void k_gather_vertices(const unsigned long long *__restrict__ pv,
     if (i < l && per_l) per_l[i] = pv[rank_l[i]];
 }
 
-// ⋈_e from the two G* slots of every edge: the U-side slots [m, 2m) hold
-// each edge once, in rows that are permutations of the caller's rows (so
-// the stores stay inside one row), then the L-side slots [0, m) add theirs,
-// at edge ids in no useful order.  Every edge id occurs once per side, so the
-// second pass needs no atomicity; it adds with reductions anyway, which the
-// L2 carries out without returning the old value to the SM, so no thread
-// waits on the scattered reads.  The second runs after the first on the same
-// stream.
+// ⋈_e from the two G* slots of every edge.  First the L-side slots [0, m) add
+// theirs to the edge's U-side slot (scattered, and only where they are not zero:
+// they hold the δ of wedges whose middle is an L vertex, the fewer the more
+// skewed the L side is); every edge occurs once per side, so this needs no
+// atomicity, but as reductions the L2 carries the additions out and no thread
+// waits.  Then the U-side slots are stored at their edge ids; the U-side rows
+// are permutations of the caller's, so those stores stay inside one row.
+__global__ void k_edges_from_slots_l(unsigned long long *pe_slot, const int32_t *__restrict__ eid, int64_t m) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += stride) {
+        const unsigned long long x = pe_slot[i];
+        if (x) atomicAdd(pe_slot + m + __ldg(eid + i), x);
+    }
+}
 __global__ void k_edges_from_slots_u(const unsigned long long *__restrict__ pe_slot,
                                      const int32_t *__restrict__ eid, int64_t m, uint64_t *per_edge) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += stride)
         per_edge[__ldg(eid + m + i)] = pe_slot[m + i];
 }
-__global__ void k_edges_from_slots_l(const unsigned long long *__restrict__ pe_slot,
-                                     const int32_t *__restrict__ eid, int64_t m, uint64_t *per_edge) {
+
+// the edge id of every slot (an L-side slot holds the edge's U-side position)
+__global__ void k_export_eid(const int32_t *__restrict__ eid, int64_t m, int32_t *out) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += stride) {
-        const unsigned long long x = pe_slot[i];
-        if (x) atomicAdd(reinterpret_cast<unsigned long long *>(per_edge) + __ldg(eid + i), x);
-    }
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < 2 * m; i += stride)
+        out[i] = i < m ? eid[m + eid[i]] : eid[i];
 }
 
 template <int MODE, typename Pos>
@@ -1546,10 +1559,19 @@ int launch_count(Graph *g, cudaStream_t s, int mode, unsigned long long *pv_proj
 int gather_edges(Graph *g, cudaStream_t s, uint64_t *per_edge) {
     if (g->m == 0) return BFC_OK;
     const unsigned blocks = (unsigned)std::min<int64_t>((g->m + 255) / 256, (int64_t)g->num_sms * 16);
+    k_edges_from_slots_l<<<blocks, 256, 0, s>>>(g->pe_slot, g->eid, g->m);
+    note_launch();
+    BFC_CUDA(cudaGetLastError());
     k_edges_from_slots_u<<<blocks, 256, 0, s>>>(g->pe_slot, g->eid, g->m, per_edge);
     note_launch();
     BFC_CUDA(cudaGetLastError());
-    k_edges_from_slots_l<<<blocks, 256, 0, s>>>(g->pe_slot, g->eid, g->m, per_edge);
+    return BFC_OK;
+}
+
+int export_eid(const Graph *g, cudaStream_t s, int32_t *out) {
+    if (g->m == 0) return BFC_OK;
+    k_export_eid<<<(unsigned)std::min<int64_t>((2 * g->m + 255) / 256, (int64_t)g->num_sms * 16), 256, 0, s>>>(
+        g->eid, g->m, out);
     note_launch();
     BFC_CUDA(cudaGetLastError());
     return BFC_OK;

@@ -40,32 +40,23 @@ __global__ void k_check_offsets(const int32_t *__restrict__ off, int32_t r, int6
     if (u == r && (int64_t)off[r] != m) atomicOr(err, kErrBadOffsets);
 }
 
-__global__ void k_check_ids(const int32_t *__restrict__ adj, int64_t m, int32_t l, int *err) {
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < m;
-         k += (int64_t)gridDim.x * blockDim.x) {
-        int32_t v = adj[k];
-        if (v < 0 || v >= l) atomicOr(err, kErrBadId);
-    }
-}
-
 // ----- a1: degrees -----------------------------------------------------------
 __global__ void k_deg_u(const int32_t *__restrict__ off, int32_t r, int32_t *deg_u,
-                        int32_t *heads,
     const int *guard = nullptr) {
     if (aborted(guard)) return;
     int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (u >= r) return;
-    int32_t d = off[u + 1] - off[u];
-    deg_u[u] = d;
-    if (heads && d > 0) heads[off[u]] = (int32_t)u;   // row owning slot off[u]; rows via max-scan
+    deg_u[u] = off[u + 1] - off[u];
 }
 
-__global__ void k_deg_l(const int32_t *__restrict__ adj, int64_t m, int32_t *deg_l,
-    const int *guard = nullptr) {
-    if (aborted(guard)) return;
+// L degrees; an id outside [0, l) is reported and counted nowhere
+__global__ void k_deg_l(const int32_t *__restrict__ adj, int64_t m, int32_t l, int32_t *deg_l, int *err) {
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < m;
-         k += (int64_t)gridDim.x * blockDim.x)
-        atomicAdd(&deg_l[adj[k]], 1);
+         k += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t v = adj[k];
+        if (v < 0 || v >= l) atomicOr(err, kErrBadId);
+        else atomicAdd(&deg_l[v], 1);
+    }
 }
 
 // ----- a2: priority ranks ----------------------------------------------------
@@ -120,7 +111,8 @@ __global__ void k_ranks(const uint64_t *__restrict__ sorted_deg, const int32_t *
 //   d > 4,096          (a few hundred rows) one radix sort of their edges.
 // Each tier also writes the swapped key (rank_l, rank_u) at the U-side
 // position; U-side order is ascending in rank_u, so the stable sort of those
-// keys on the rank_l bits yields the L side.
+// keys on the rank_l bits yields the L side.  The sort carries each key's
+// U-side position (its index before the sort).
 constexpr int kRowWarpMax = 32;
 constexpr int kRowWarpSortMax = 256;
 constexpr int kRowCtaMax = 4096;
@@ -133,7 +125,6 @@ struct URowOut {
     const int64_t *off_star;
     int32_t *adj_star, *eid_star, *rows_star;
     uint64_t *keys2;
-    int32_t *vals2;
     int *err;
     int check_dup;   // flag duplicate edges (validate)
     __device__ __forceinline__ void put(int32_t ru, int64_t pos, int32_t rl, int32_t slot) const {
@@ -142,7 +133,6 @@ struct URowOut {
         eid_star[m + k] = slot;
         rows_star[m + k] = l + ru;
         keys2[k] = ((uint64_t)(uint32_t)rl << bu) | (uint64_t)(uint32_t)ru;
-        vals2[k] = slot;
     }
 };
 
@@ -326,18 +316,41 @@ __global__ void k_large_emit(const uint64_t *__restrict__ keys, const int32_t *_
     }
 }
 
+// L-side slot i = (v, u): v's list in ascending U rank, with the edge's
+// U-side position k.  Algorithm 2's runs come from the two positions of the
+// edge, with no search: where v is the start (u has fewer neighbours than v) the
+// run through u is the prefix of N(u) before v, which is as long as v's position
+// in that list; where u is the start the run through v is as long as u's
+// position in N(v).  The second kind is scattered to the U-side slot, whose
+// plen the caller has set to zero.  Reads `off` at random (L2-resident: 8 bytes
+// per vertex), writes 4 bytes at random for the U starts' middles only; a
+// binary search of the middle's list per slot took 15.8 ms on a 300M-edge
+// shopping graph.
+template <bool kRuns>
 __global__ void k_emit_l_side(const uint64_t *__restrict__ keys2, const int32_t *__restrict__ vals2,
-                              int64_t m, int bu, int32_t l, int32_t *adj_star, int32_t *eid_star,
-                              int32_t *rows_star,
+                              int64_t m, int bu, int32_t l, const int64_t *__restrict__ off, int32_t *adj_star,
+                              int32_t *eid_star, int32_t *rows_star, int32_t *plen, int64_t *sbeg,
     const int *guard = nullptr) {
     if (aborted(guard)) return;
     const uint64_t mask_u = (1ull << bu) - 1ull;
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < m;
-         k += (int64_t)gridDim.x * blockDim.x) {
-        uint64_t key = keys2[k];
-        adj_star[k] = l + (int32_t)(key & mask_u);
-        eid_star[k] = vals2[k];
-        rows_star[k] = (int32_t)(key >> bu);
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const uint64_t key = keys2[i];
+        const int32_t k = vals2[i], v = (int32_t)(key >> bu), u = l + (int32_t)(key & mask_u);
+        adj_star[i] = u;
+        eid_star[i] = k;
+        rows_star[i] = v;
+        if (kRuns) {
+            const int64_t bv = off[v], bu0 = off[u];
+            // equal degrees: the U vertex has the higher priority
+            if (off[u + 1] - bu0 < off[v + 1] - bv) {
+                plen[i] = (int32_t)(m + k - bu0);
+                sbeg[i] = bu0;
+            } else {
+                plen[i] = 0;
+                plen[m + k] = (int32_t)(i - bv);
+            }
+        }
     }
 }
 
@@ -372,35 +385,6 @@ __global__ void k_cut(const int64_t *__restrict__ off, const int32_t *__restrict
     cut[x] = (int32_t)lo;
 }
 
-// plen[e] for a middle slot e = (x, v): the number of ends w in N(v) with
-// p(w) < p(x), i.e. the prefix of v's ascending list below x; sbeg[e] = the
-// position where that prefix starts (off[v]), so the count kernel reads it
-// with the slot instead of after the slot's neighbour id.
-__global__ void k_plen(const int64_t *__restrict__ off, const int32_t *__restrict__ adj,
-                       const int32_t *__restrict__ rows, const int32_t *__restrict__ cut,
-                       int64_t slots, int32_t *plen, int64_t *sbeg,
-    const int *guard = nullptr) {
-    if (aborted(guard)) return;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < slots;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t x = rows[e];
-        int32_t out = 0;
-        int64_t b = 0;
-        if (e - off[x] < cut[x]) {
-            const int32_t v = adj[e];
-            b = off[v];
-            int64_t lo = 0, hi = off[v + 1] - b;
-            while (lo < hi) {
-                int64_t mid = (lo + hi) >> 1;
-                if (adj[b + mid] < x) lo = mid + 1; else hi = mid;
-            }
-            out = (int32_t)lo;
-        }
-        plen[e] = out;
-        sbeg[e] = b;
-    }
-}
-
 // Algorithm 3: for slot e = (x, v) the ends are the w in N(v) with
 // p(w) > p(x) and p(w) > p(v).  N(v) ascends in priority, so they form the
 // suffix that starts after both x (x is in N(v)) and v's cut.
@@ -424,27 +408,142 @@ __global__ void k_slen(const int64_t *__restrict__ off, const int32_t *__restric
 }
 
 // work[x] = Σ plen over x's middle slots (the first cut[x] slots for
-// Algorithm 2, every slot for Algorithm 3); one warp per start.
-__global__ void k_work(const int64_t *__restrict__ off, const int32_t *__restrict__ cut,
-                       const int32_t *__restrict__ plen, int32_t n, int all_slots, uint64_t *work,
-                       unsigned long long *total,
+// Algorithm 2, every slot for Algorithm 3).  For Algorithm 2 the U-side middle
+// slots (at or past `fill_from`) also get the start of their run, off[middle].
+// A warp takes 32 starts and each lane walks its own where there are at most
+// 24 slots (neighbouring lists share their sectors); the longer ones go to a
+// queue that k_work_long takes 32 at a time per CTA, one per warp, or one after
+// another by the whole CTA above 4,096 slots.  With one warp per start the
+// millions of one-slot starts of a sparse batch and the longest list of a skewed
+// graph each took 2.5 ms.
+constexpr int kWorkLane = 24;
+constexpr int kWorkWarp = 4096;
+
+__device__ __forceinline__ unsigned slot_work(const int64_t *off, const int32_t *adj, const int32_t *plen,
+                                              int64_t e, bool fill, int64_t *sbeg) {
+    if (fill) sbeg[e] = off[adj[e]];
+    return (unsigned)plen[e];
+}
+
+__global__ void k_work(const int64_t *__restrict__ off, const int32_t *__restrict__ adj,
+                       const int32_t *__restrict__ cut, const int32_t *__restrict__ plen, int32_t n, int all_slots,
+                       int64_t fill_from, int64_t *sbeg, uint64_t *work, int32_t *queue, int32_t *queued,
     const int *guard = nullptr) {
     if (aborted(guard)) return;
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    unsigned long long tot = 0;
-    for (int64_t x = warp; x < n; x += nwarps) {
-        const int64_t b = off[x];
-        const int64_t c = all_slots ? off[x + 1] - b : (int64_t)cut[x];
+    for (int64_t x0 = warp * 32; x0 < n; x0 += nwarps * 32) {
+        const int64_t x = x0 + lane;
+        int64_t b = 0;
+        int32_t c = 0;
+        if (x < n) {
+            b = off[x];
+            c = all_slots ? (int32_t)(off[x + 1] - b) : cut[x];
+        }
         unsigned long long s = 0;
-        for (int64_t j = lane; j < c; j += 32) s += (unsigned)plen[b + j];
-#pragma unroll
-        for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
-        if (lane == 0) work[x] = s;
-        tot += s;
+        if (c <= kWorkLane) {
+            const bool fill = b >= fill_from;
+            for (int32_t j = 0; j < c; ++j) s += slot_work(off, adj, plen, b + j, fill, sbeg);
+            if (x < n) work[x] = s;
+        }
+        const uint32_t todo = __ballot_sync(0xffffffffu, c > kWorkLane);
+        int32_t at = 0;
+        if (lane == 0 && todo) at = atomicAdd(queued, __popc(todo));
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (c > kWorkLane) queue[at + __popc(todo & ((1u << lane) - 1u))] = (int32_t)x;
     }
-    if (lane == 0 && tot) atomicAdd(total, tot);
+}
+
+__global__ void __launch_bounds__(1024) k_work_long(const int64_t *__restrict__ off, const int32_t *__restrict__ adj,
+                                                    const int32_t *__restrict__ cut, const int32_t *__restrict__ plen,
+                                                    int all_slots, int64_t fill_from, int64_t *sbeg, uint64_t *work,
+                                                    const int32_t *__restrict__ queue,
+                                                    const int32_t *__restrict__ queued,
+    const int *guard = nullptr) {
+    if (aborted(guard)) return;
+    __shared__ unsigned long long part[32];
+    const int n = *queued, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int i0 = blockIdx.x * 32; i0 < n; i0 += gridDim.x * 32) {
+        if (i0 + warp < n) {
+            const int32_t x = queue[i0 + warp];
+            const int64_t b = off[x];
+            const int32_t c = all_slots ? (int32_t)(off[x + 1] - b) : cut[x];
+            if (c <= kWorkWarp) {
+                const bool fill = b >= fill_from;
+                unsigned long long t = 0;
+#pragma unroll 4
+                for (int32_t j = lane; j < c; j += 32) t += slot_work(off, adj, plen, b + j, fill, sbeg);
+#pragma unroll
+                for (int d = 16; d > 0; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
+                if (lane == 0) work[x] = t;
+            }
+        }
+        for (int k = 0; k < 32 && i0 + k < n; ++k) {   // uniform over the CTA
+            const int32_t x = queue[i0 + k];
+            const int64_t b = off[x];
+            const int32_t c = all_slots ? (int32_t)(off[x + 1] - b) : cut[x];
+            if (c <= kWorkWarp) continue;
+            const bool fill = b >= fill_from;
+            unsigned long long t = 0;
+#pragma unroll 8
+            for (int32_t j = threadIdx.x; j < c; j += 1024) t += slot_work(off, adj, plen, b + j, fill, sbeg);
+#pragma unroll
+            for (int d = 16; d > 0; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
+            if (lane == 0) part[warp] = t;
+            __syncthreads();
+            if (warp == 0) {
+                t = part[lane];
+#pragma unroll
+                for (int d = 16; d > 0; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
+                if (lane == 0) work[x] = t;
+            }
+            __syncthreads();
+        }
+    }
+}
+
+// stats[0] += Σ work, stats[1] = max work, stats[2] += starts above `heavy`;
+// of a batch, gwork[g] += the work of graph g (one addition per warp where its
+// vertices lie in one graph, which all but a few warps' do)
+__global__ void k_work_stats(const uint64_t *__restrict__ work, int32_t n, uint64_t heavy,
+                             const int32_t *__restrict__ gstar, unsigned long long *stats, unsigned long long *gwork,
+    const int *guard = nullptr) {
+    if (aborted(guard)) return;
+    const int lane = threadIdx.x & 31;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    unsigned long long sum = 0, top = 0, above = 0;
+    for (int64_t x0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); x0 < n; x0 += stride) {
+        const int64_t x = x0 + lane;
+        const unsigned long long w = x < n ? work[x] : 0;
+        sum += w;
+        top = w > top ? w : top;
+        above += w > heavy ? 1 : 0;
+        if (gwork) {
+            const int32_t g = x < n ? gstar[x] : -1;
+            const int32_t g0 = __shfl_sync(0xffffffffu, g, 0);
+            if (__all_sync(0xffffffffu, g == g0)) {
+                unsigned long long t = w;
+#pragma unroll
+                for (int d = 16; d > 0; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
+                if (lane == 0 && t) atomicAdd(gwork + g0, t);
+            } else if (w) {
+                atomicAdd(gwork + g, w);
+            }
+        }
+    }
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+        sum += __shfl_xor_sync(0xffffffffu, sum, d);
+        above += __shfl_xor_sync(0xffffffffu, above, d);
+        const unsigned long long o = __shfl_xor_sync(0xffffffffu, top, d);
+        top = o > top ? o : top;
+    }
+    if (lane == 0) {
+        if (sum) atomicAdd(stats, sum);
+        if (top) atomicMax(stats + 1, top);
+        if (above) atomicAdd(stats + 2, above);
+    }
 }
 
 // ----- a5: bins and schedule ---------------------------------------------------
@@ -465,18 +564,6 @@ __global__ void k_sched_keys(const uint64_t *__restrict__ work, int32_t n, uint6
     // ascending key = descending work; zero work last; forced dense starts first
     keys[x] = forced_dense((int32_t)x, l, core_lo_u, core_lo_l, work[x]) ? 0 : maxw - work[x];
     vals[x] = (int32_t)x;
-}
-
-// starts with more than `bound` wedges (the dense bin's size before any core)
-__global__ void k_count_heavy(const uint64_t *__restrict__ work, int32_t n, uint64_t bound,
-                              unsigned long long *count) {
-    unsigned long long c = 0;
-    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n;
-         x += (int64_t)gridDim.x * blockDim.x)
-        c += work[x] > bound ? 1 : 0;
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) c += __shfl_xor_sync(0xffffffffu, c, d);
-    if ((threadIdx.x & 31) == 0 && c) atomicAdd(count, c);
 }
 
 // counts[0] = dense starts, [1] = hash starts, [2] = warp starts
@@ -706,16 +793,41 @@ __global__ void k_check_starts(const int32_t *__restrict__ start, int32_t num_gr
     }
 }
 
-// every edge must join a U and an L vertex of the same graph
-__global__ void k_check_batch_edges(const int32_t *__restrict__ rows, const int32_t *__restrict__ adj,
-                                    int64_t m, const int32_t *__restrict__ gu,
-                                    const int32_t *__restrict__ gl, int32_t num_graphs, int *err,
+// every edge must join a U and an L vertex of the same graph: one lookup of
+// the row's graph, then its L ids against that graph's range.  A warp takes 32
+// rows (lanes on their own up to 24 neighbours, the warp together above).
+__global__ void k_check_batch_rows(const int32_t *__restrict__ off, const int32_t *__restrict__ adj, int32_t r,
+                                   const int32_t *__restrict__ gu, const int32_t *__restrict__ gl,
+                                   int32_t num_graphs, int *err,
     const int *guard = nullptr) {
     if (aborted(guard)) return;
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < m;
-         k += (int64_t)gridDim.x * blockDim.x)
-        if (graph_of(gu, num_graphs, rows[k]) != graph_of(gl, num_graphs, adj[k]))
-            atomicOr(err, kErrBadId);
+    const int lane = threadIdx.x & 31;
+    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    bool bad = false;
+    for (int64_t u0 = warp * 32; u0 < r; u0 += nwarps * 32) {
+        const int64_t u = u0 + lane;
+        int32_t b = 0, d = 0, lo = 0, hi = 0;
+        if (u < r) {
+            b = off[u];
+            d = off[u + 1] - b;
+            const int32_t g = graph_of(gu, num_graphs, (int32_t)u);
+            lo = gl[g];
+            hi = gl[g + 1];
+        }
+        if (d <= kWorkLane)
+            for (int32_t j = 0; j < d; ++j) { const int32_t v = adj[b + j]; bad |= v < lo || v >= hi; }
+        uint32_t todo = __ballot_sync(0xffffffffu, d > kWorkLane);
+        while (todo) {
+            const int k = __ffs((int)todo) - 1;
+            todo &= todo - 1;
+            const int32_t bk = __shfl_sync(0xffffffffu, b, k), dk = __shfl_sync(0xffffffffu, d, k);
+            const int32_t lk = __shfl_sync(0xffffffffu, lo, k), hk = __shfl_sync(0xffffffffu, hi, k);
+#pragma unroll 8
+            for (int32_t j = lane; j < dk; j += 32) { const int32_t v = adj[bk + j]; bad |= v < lk || v >= hk; }
+        }
+    }
+    if (bad) atomicOr(err, kErrBadId);
 }
 
 // graph-major ranks: vertex x of G* belongs to the graph whose rank range
@@ -739,15 +851,6 @@ __global__ void k_graph_star(int32_t r, int32_t l, const int32_t *__restrict__ g
             vend[x] = l + gu[gg + 1];
         }
     }
-}
-
-__global__ void k_graph_work(const uint64_t *__restrict__ work, const int32_t *__restrict__ gstar,
-                             int32_t n, unsigned long long *gwork,
-    const int *guard = nullptr) {
-    if (aborted(guard)) return;
-    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n;
-         x += (int64_t)gridDim.x * blockDim.x)
-        if (work[x]) atomicAdd(gwork + gstar[x], (unsigned long long)work[x]);
 }
 
 // slot -> owning vertex of G*, one warp per vertex
@@ -957,6 +1060,22 @@ int rebin_graph(Graph *g, cudaStream_t s, int32_t warp_max_work, int32_t team_ma
     return rc;
 }
 
+// work per start, the runs of the U-side middle slots (Algorithm 2), and
+// stats[0] = W, [1] = the heaviest start, [2] = starts beyond the CTA-hash bin
+static void launch_work(Graph *g, int32_t *big, int32_t *n_big, unsigned long long *gwork, unsigned long long *stats,
+                        cudaStream_t s, const int *guard) {
+    const int vpp = g->opt.orientation;
+    const int64_t fill_from = vpp ? 2 * g->m + 1 : g->m;
+    k_work<<<grid_stride_blocks(g->n), kT, 0, s>>>(g->off, g->adj, g->cut, g->plen, g->n, vpp, fill_from, g->sbeg,
+                                                   g->work, big, n_big, guard); note_launch();
+    if (2 * g->m > kWorkLane) {
+        k_work_long<<<(unsigned)std::min<int64_t>(2 * g->m / kWorkLane / 32 + 1, 152 * 2), 1024, 0, s>>>(
+            g->off, g->adj, g->cut, g->plen, vpp, fill_from, g->sbeg, g->work, big, n_big, guard); note_launch();
+    }
+    k_work_stats<<<(unsigned)std::min<int64_t>(blocks_for(g->n), 152 * 8), kT, 0, s>>>(
+        g->work, g->n, (uint64_t)g->opt.hash_max_work, g->gstar, stats, gwork, guard); note_launch();
+}
+
 int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Graph *g,
                   int32_t num_graphs, const int32_t *graph_u_start, const int32_t *graph_l_start) {
     const int32_t r = csr->num_u, l = csr->num_l;
@@ -988,6 +1107,7 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
     GET(g->mem, g->adj, 2 * m);
     GET(g->mem, g->eid, 2 * m);
     GET(g->mem, g->plen, 2 * m);
+    GET(g->mem, g->sbeg, std::max<int64_t>(2 * m, 1));
     GET(g->mem, g->cut, n);
     GET(g->mem, g->work, n);
     GET(g->mem, g->cursors, 8);
@@ -1002,14 +1122,6 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
     BFC_CUDA(cudaMemcpyAsync(&herr, g->err, sizeof(int), cudaMemcpyDeviceToHost, s));
     BFC_CUDA(cudaStreamSynchronize(s));
     if (herr) { set_last_error("off_u is not a CSR offset array of num_edges entries"); return BFC_ERR_INVALID_GRAPH; }
-    if (m > 0) {
-        k_check_ids<<<grid_stride_blocks(m), kT, 0, s>>>(csr->adj_u, m, l, g->err); note_launch();
-        BFC_CUDA(cudaGetLastError());
-        BFC_CUDA(cudaMemcpyAsync(&herr, g->err, sizeof(int), cudaMemcpyDeviceToHost, s));
-        BFC_CUDA(cudaStreamSynchronize(s));
-        if (herr) { set_last_error("adj_u holds an id outside [0, num_l)"); return BFC_ERR_INVALID_GRAPH; }
-    }
-
     if (num_graphs > 0) {
         k_check_starts<<<blocks_for((int64_t)num_graphs + 1), kT, 0, s>>>(graph_u_start, num_graphs, r, g->err); note_launch();
         k_check_starts<<<blocks_for((int64_t)num_graphs + 1), kT, 0, s>>>(graph_l_start, num_graphs, l, g->err); note_launch();
@@ -1028,7 +1140,7 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
     // ---- temporaries
     const int64_t nsort = std::max<int64_t>({(int64_t)r, (int64_t)l, m, (int64_t)n, 1});
     uint64_t *k0, *k1;
-    int32_t *v0, *v1, *deg_u, *deg_l, *deg_star, *rows, *rows_star, *heads, *order_u, *order_l;
+    int32_t *v0, *v1, *deg_u, *deg_l, *deg_star, *rows_star, *heads, *big, *n_big;
     uint32_t *hist, *hist_tmp;
     int64_t *scan64_tmp, *deg64;
     int32_t *maxdeg;
@@ -1036,8 +1148,8 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
     GET(tmp, k0, nsort + 1); GET(tmp, k1, nsort + 1);
     GET(tmp, v0, nsort); GET(tmp, v1, nsort);
     GET(tmp, deg_u, r); GET(tmp, deg_l, l); GET(tmp, deg_star, n);
-    GET(tmp, rows, m); GET(tmp, heads, m); GET(tmp, rows_star, 2 * m);
-    GET(tmp, order_u, r); GET(tmp, order_l, l);
+    GET(tmp, rows_star, 2 * m);
+    GET(tmp, big, std::min<int64_t>(2 * m / kWorkLane, n) + 1); GET(tmp, n_big, 1);
     GET(tmp, hist, radix_hist_elems(nsort));
     GET(tmp, hist_tmp, scan_tmp_elems<uint32_t>((int64_t)radix_hist_elems(nsort)));
     GET(tmp, scan64_tmp, std::max(scan_tmp_elems<int64_t>((int64_t)n + 1),
@@ -1046,20 +1158,18 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
     GET(tmp, maxdeg, 4);
     GET(tmp, red, 8);
 
-    // ---- a1: degrees (and the head of each U row for the slot -> row map)
+    // ---- a1: degrees (and the check of the L ids)
     BFC_CUDA(cudaMemsetAsync(deg_l, 0, sizeof(int32_t) * std::max<int64_t>(l, 1), s));
-    // the row of every input slot is only needed to check a batch's edges
-    if (num_graphs > 0) BFC_CUDA(cudaMemsetAsync(heads, 0, sizeof(int32_t) * std::max<int64_t>(m, 1), s));
-    if (r > 0) {
-        k_deg_u<<<blocks_for(r), kT, 0, s>>>(csr->off_u, r, deg_u, num_graphs > 0 ? heads : nullptr); note_launch();
-    }
-    if (m > 0) { k_deg_l<<<grid_stride_blocks(m), kT, 0, s>>>(csr->adj_u, m, deg_l); note_launch(); }
+    if (r > 0) { k_deg_u<<<blocks_for(r), kT, 0, s>>>(csr->off_u, r, deg_u); note_launch(); }
+    if (m > 0) { k_deg_l<<<grid_stride_blocks(m), kT, 0, s>>>(csr->adj_u, m, l, deg_l, g->err); note_launch(); }
     BFC_CUDA(cudaGetLastError());
     BFC_CUDA(reduce_max_i32(deg_u, r, maxdeg, s));
     BFC_CUDA(reduce_max_i32(deg_l, l, maxdeg + 1, s));
     int32_t hmax[2] = {0, 0};
     BFC_CUDA(cudaMemcpyAsync(hmax, maxdeg, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    BFC_CUDA(cudaMemcpyAsync(&herr, g->err, sizeof(int), cudaMemcpyDeviceToHost, s));
     BFC_CUDA(cudaStreamSynchronize(s));
+    if (herr) { set_last_error("adj_u holds an id outside [0, num_l)"); return BFC_ERR_INVALID_GRAPH; }
     g->info.max_deg_u = hmax[0];
     g->info.max_deg_l = hmax[1];
 
@@ -1078,7 +1188,6 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
                                   hist_tmp, s, &which));
         const uint64_t *ks = which ? k1 : k0;
         const int32_t *vs = which ? v1 : v0;
-        BFC_CUDA(cudaMemcpyAsync(order_u, vs, sizeof(int32_t) * r, cudaMemcpyDeviceToDevice, s));
         k_ranks<<<blocks_for(r), kT, 0, s>>>(ks, vs, r, g->rank_u, deg_star, l, (1ull << bits_for((uint64_t)hmax[0])) - 1); note_launch();
         BFC_CUDA(cudaGetLastError());
     }
@@ -1095,7 +1204,6 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
                                   hist_tmp, s, &which));
         const uint64_t *ks = which ? k1 : k0;
         const int32_t *vs = which ? v1 : v0;
-        BFC_CUDA(cudaMemcpyAsync(order_l, vs, sizeof(int32_t) * l, cudaMemcpyDeviceToDevice, s));
         k_ranks<<<blocks_for(l), kT, 0, s>>>(ks, vs, l, g->rank_l, deg_star, 0, (1ull << bits_for((uint64_t)hmax[1])) - 1); note_launch();
         BFC_CUDA(cudaGetLastError());
     }
@@ -1116,17 +1224,16 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
     const int bl = bits_for(l > 0 ? (uint64_t)(l - 1) : 0);
     if (m > 0) {
         if (num_graphs > 0) {
-            BFC_CUDA(max_scan_inclusive(heads, rows, m, (int32_t *)scan64_tmp, s));
-            k_check_batch_edges<<<grid_stride_blocks(m), kT, 0, s>>>(rows, csr->adj_u, m, graph_u_start,
-                                                                     graph_l_start, num_graphs, g->err); note_launch();
+            k_check_batch_rows<<<grid_stride_blocks(r), kT, 0, s>>>(csr->off_u, csr->adj_u, r, graph_u_start,
+                                                                    graph_l_start, num_graphs, g->err); note_launch();
             BFC_CUDA(cudaGetLastError());
             BFC_CUDA(cudaMemcpyAsync(&herr, g->err, sizeof(int), cudaMemcpyDeviceToHost, s));
             BFC_CUDA(cudaStreamSynchronize(s));
             if (herr) { set_last_error("an edge joins vertices of two different graphs of the batch"); return BFC_ERR_INVALID_GRAPH; }
         }
         // U side row by row (warp / CTA tiers, radix sort for the largest rows);
-        // the swapped keys for the L side land in (k1, v1)
-        const URowOut uo{m, l, bu, g->off, g->adj, g->eid, rows_star, k1, v1, g->err, opt->validate};
+        // the swapped keys for the L side land in k1
+        const URowOut uo{m, l, bu, g->off, g->adj, g->eid, rows_star, k1, g->err, opt->validate};
         k_u_rows_warp<<<grid_stride_blocks((int64_t)r * 32), kT, 0, s>>>(csr->off_u, csr->adj_u, g->rank_u,
                                                                          g->rank_l, r, uo); note_launch();
         BFC_CUDA(cudaGetLastError());
@@ -1167,7 +1274,7 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
             if (nlarge > 0) {
                 uint64_t *ka;
                 int32_t *va, *rowf;
-                GET(tmp, ka, nlarge); GET(tmp, va, nlarge); GET(tmp, rowf, nlarge);
+                GET(tmp, ka, nlarge); GET(tmp, va, nlarge); GET(tmp, rowf, nlarge); GET(tmp, heads, nlarge);
                 k_large_keys<<<(unsigned)std::min<int32_t>(nl, 1024), kT, 0, s>>>(csr->off_u, csr->adj_u, g->rank_u,
                                                                                    g->rank_l, large_rows, loff, nl, bl,
                                                                                    k0, v0); note_launch();
@@ -1190,11 +1297,17 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
         // stable sort of the (rank_l, rank_u) keys on the rank_l bits only:
         // the input is already ascending in rank_u within each rank_l
         int which2 = 0;
-        BFC_CUDA(radix_sort_pairs(ko, vo, ks, vs, m, bu, bu + bl, hist, hist_tmp, s, &which2));
+        BFC_CUDA(radix_sort_pairs(ko, vo, ks, vs, m, bu, bu + bl, hist, hist_tmp, s, &which2, true));
         const uint64_t *k2 = which2 ? ks : ko;
         const int32_t *v2 = which2 ? vs : vo;
-        k_emit_l_side<<<grid_stride_blocks(m), kT, 0, s>>>(k2, v2, m, bu, l, g->adj, g->eid,
-                                                            rows_star); note_launch();
+        if (opt->orientation == 0) {
+            BFC_CUDA(cudaMemsetAsync(g->plen + m, 0, sizeof(int32_t) * (size_t)m, s));
+            k_emit_l_side<true><<<grid_stride_blocks(m), kT, 0, s>>>(k2, v2, m, bu, l, g->off, g->adj, g->eid,
+                                                                      rows_star, g->plen, g->sbeg); note_launch();
+        } else {
+            k_emit_l_side<false><<<grid_stride_blocks(m), kT, 0, s>>>(k2, v2, m, bu, l, g->off, g->adj, g->eid,
+                                                                       rows_star, nullptr, nullptr); note_launch();
+        }
         BFC_CUDA(cudaGetLastError());
         if (opt->validate) {
             BFC_CUDA(cudaMemcpyAsync(&herr, g->err, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -1209,30 +1322,15 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
         k_cut<<<blocks_for(n), kT, 0, s>>>(g->off, g->adj, deg_star, n, l, g->cut); note_launch();
         BFC_CUDA(cudaGetLastError());
     }
-    GET(g->mem, g->sbeg, std::max<int64_t>(2 * m, 1));
-    if (m > 0 && opt->orientation == 0) {
-        k_plen<<<grid_stride_blocks(2 * m), kT, 0, s>>>(g->off, g->adj, rows_star, g->cut, 2 * m,
-                                                         g->plen, g->sbeg); note_launch();
-        BFC_CUDA(cudaGetLastError());
-    }
     if (m > 0 && opt->orientation == 1) {
         k_slen<<<grid_stride_blocks(2 * m), kT, 0, s>>>(g->off, g->adj, rows_star, g->cut, 2 * m,
                                                          g->plen, g->sbeg); note_launch();
         BFC_CUDA(cudaGetLastError());
     }
-    if (n > 0) {
-        k_work<<<grid_stride_blocks((int64_t)n * 32), kT, 0, s>>>(g->off, g->cut, g->plen, n,
-                                                                   opt->orientation, g->work, red); note_launch();
-        BFC_CUDA(cudaGetLastError());
-        BFC_CUDA(reduce_max_u64(g->work, n, red + 1, s));
-    }
-    if (num_graphs > 0 && n > 0) {
-        k_graph_work<<<grid_stride_blocks(n), kT, 0, s>>>(g->work, g->gstar, n, g->gwork); note_launch();
-        BFC_CUDA(cudaGetLastError());
-    }
     const bool core_auto = opt->core_vertices < 0 && opt->orientation == 0 && num_graphs == 0;
-    if (core_auto && n > 0) {
-        k_count_heavy<<<grid_stride_blocks(n), kT, 0, s>>>(g->work, n, (uint64_t)opt->hash_max_work, red + 2); note_launch();
+    if (n > 0) {
+        BFC_CUDA(cudaMemsetAsync(n_big, 0, sizeof(int32_t), s));
+        launch_work(g, big, n_big, num_graphs > 0 ? g->gwork : nullptr, red, s, nullptr);
         BFC_CUDA(cudaGetLastError());
     }
     unsigned long long hred[3] = {0, 0, 0};
@@ -1414,7 +1512,7 @@ int batch_plan_create(BatchPlan *pl, cudaStream_t s) {
     const int64_t nsort = std::max<int64_t>({(int64_t)r, (int64_t)l, m, (int64_t)n, 1});
     GET(pl->k0, nsort + 1); GET(pl->k1, nsort + 1); GET(pl->v0, nsort); GET(pl->v1, nsort);
     GET(pl->deg_u, r); GET(pl->deg_l, l); GET(pl->deg_star, n);
-    GET(pl->rows, m); GET(pl->heads, m); GET(pl->rows_star, 2 * m);
+    GET(pl->rows_star, 2 * m); GET(pl->big, std::min<int64_t>(2 * m / kWorkLane, n) + 1); GET(pl->n_big, 1);
     GET(pl->tier_rows, 3 * (int64_t)std::max(r, 1)); GET(pl->tier_n, 4);
     GET(pl->hist, radix_hist_elems(nsort));
     GET(pl->hist_tmp, scan_tmp_elems<uint32_t>((int64_t)radix_hist_elems(nsort)));
@@ -1449,15 +1547,13 @@ int batch_plan_run(BatchPlan *pl, const int32_t *off_u, const int32_t *adj_u, co
     BFC_CUDA(cudaMemsetAsync(g->err, 0, 4 * sizeof(int), s));
     // ---- checks: the CSR, the graph start arrays, edges inside their graph
     k_check_offsets<<<blocks_for((int64_t)r + 1), kT, 0, s>>>(off_u, r, m, g->err); note_launch();
-    if (m > 0) { k_check_ids<<<grid_stride_blocks(m), kT, 0, s>>>(adj_u, m, l, g->err); note_launch(); }
     k_check_starts<<<blocks_for((int64_t)G + 1), kT, 0, s>>>(gu, G, r, g->err, pl->max_layer); note_launch();
     k_check_starts<<<blocks_for((int64_t)G + 1), kT, 0, s>>>(gl, G, l, g->err, pl->max_layer); note_launch();
     BFC_CUDA(cudaGetLastError());
-    // ---- a1: degrees
+    // ---- a1: degrees (and the check of the L ids)
     BFC_CUDA(cudaMemsetAsync(pl->deg_l, 0, sizeof(int32_t) * std::max<int64_t>(l, 1), s));
-    BFC_CUDA(cudaMemsetAsync(pl->heads, 0, sizeof(int32_t) * std::max<int64_t>(m, 1), s));
-    if (r > 0) { k_deg_u<<<blocks_for(r), kT, 0, s>>>(off_u, r, pl->deg_u, pl->heads, guard); note_launch(); }
-    if (m > 0) { k_deg_l<<<grid_stride_blocks(m), kT, 0, s>>>(adj_u, m, pl->deg_l, guard); note_launch(); }
+    if (m > 0) { k_deg_l<<<grid_stride_blocks(m), kT, 0, s>>>(adj_u, m, l, pl->deg_l, g->err); note_launch(); }
+    if (r > 0) { k_deg_u<<<blocks_for(r), kT, 0, s>>>(off_u, r, pl->deg_u, guard); note_launch(); }
     BFC_CUDA(cudaGetLastError());
     // ---- a2: graph-major ranks; a degree is below 2^bdeg (at most the other layer)
     const int bdeg = bits_for((uint64_t)pl->max_layer);
@@ -1488,9 +1584,8 @@ int batch_plan_run(BatchPlan *pl, const int32_t *off_u, const int32_t *adj_u, co
     const int bu = bits_for(r > 0 ? (uint64_t)(r - 1) : 0);
     const int bl = bits_for(l > 0 ? (uint64_t)(l - 1) : 0);
     if (m > 0) {
-        BFC_CUDA(max_scan_inclusive(pl->heads, pl->rows, m, (int32_t *)pl->scan64_tmp, s));
-        k_check_batch_edges<<<grid_stride_blocks(m), kT, 0, s>>>(pl->rows, adj_u, m, gu, gl, G, g->err, guard); note_launch();
-        const URowOut uo{m, l, bu, g->off, g->adj, g->eid, pl->rows_star, pl->k1, pl->v1, g->err, opt->validate};
+        k_check_batch_rows<<<grid_stride_blocks(r), kT, 0, s>>>(off_u, adj_u, r, gu, gl, G, g->err, guard); note_launch();
+        const URowOut uo{m, l, bu, g->off, g->adj, g->eid, pl->rows_star, pl->k1, g->err, opt->validate};
         k_u_rows_warp<<<grid_stride_blocks((int64_t)r * 32), kT, 0, s>>>(off_u, adj_u, g->rank_u, g->rank_l, r, uo,
                                                                          guard); note_launch();
         BFC_CUDA(cudaMemsetAsync(pl->tier_n, 0, 4 * sizeof(int32_t), s));
@@ -1505,25 +1600,21 @@ int batch_plan_run(BatchPlan *pl, const int32_t *off_u, const int32_t *adj_u, co
         BFC_CUDA(cudaGetLastError());
         // L side: stable sort of the swapped keys on their rank_l bits
         int which2 = 0;
-        BFC_CUDA(radix_sort_pairs(pl->k1, pl->v1, pl->k0, pl->v0, m, bu, bu + bl, pl->hist, pl->hist_tmp, s, &which2));
+        BFC_CUDA(radix_sort_pairs(pl->k1, pl->v1, pl->k0, pl->v0, m, bu, bu + bl, pl->hist, pl->hist_tmp, s, &which2, true));
         const uint64_t *k2 = which2 ? pl->k0 : pl->k1;
         const int32_t *v2 = which2 ? pl->v0 : pl->v1;
-        k_emit_l_side<<<grid_stride_blocks(m), kT, 0, s>>>(k2, v2, m, bu, l, g->adj, g->eid, pl->rows_star,
-                                                            guard); note_launch();
+        BFC_CUDA(cudaMemsetAsync(g->plen + m, 0, sizeof(int32_t) * (size_t)m, s));
+        k_emit_l_side<true><<<grid_stride_blocks(m), kT, 0, s>>>(k2, v2, m, bu, l, g->off, g->adj, g->eid,
+                                                                  pl->rows_star, g->plen, g->sbeg, guard); note_launch();
         BFC_CUDA(cudaGetLastError());
     }
     // ---- a4: cut, runs, work
     BFC_CUDA(cudaMemsetAsync(pl->red, 0, 8 * sizeof(unsigned long long), s));
     if (n > 0) { k_cut<<<blocks_for(n), kT, 0, s>>>(g->off, g->adj, pl->deg_star, n, l, g->cut, guard); note_launch(); }
-    if (m > 0) {
-        k_plen<<<grid_stride_blocks(2 * m), kT, 0, s>>>(g->off, g->adj, pl->rows_star, g->cut, 2 * m, g->plen,
-                                                         g->sbeg, guard); note_launch();
-    }
     if (n > 0) {
-        k_work<<<grid_stride_blocks((int64_t)n * 32), kT, 0, s>>>(g->off, g->cut, g->plen, n, 0, g->work, pl->red,
-                                                                   guard); note_launch();
         BFC_CUDA(cudaMemsetAsync(g->gwork, 0, sizeof(unsigned long long) * G, s));
-        k_graph_work<<<grid_stride_blocks(n), kT, 0, s>>>(g->work, g->gstar, n, g->gwork, guard); note_launch();
+        BFC_CUDA(cudaMemsetAsync(pl->n_big, 0, sizeof(int32_t), s));
+        launch_work(g, pl->big, pl->n_big, g->gwork, pl->red, s, guard);
         BFC_CUDA(cudaGetLastError());
     }
     // ---- a5: heaviest first, bins from device counts

@@ -3,6 +3,7 @@
 // These are the building blocks of the degree ranking (Definition 3 via the
 // bin sort named in the proof of Theorem 2), the renumbering of Definition 4
 // and the per-start work prefix sums.
+#include <algorithm>
 #include <climits>
 
 #include "bfc_internal.cuh"
@@ -213,7 +214,7 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(
         int64_t k = base + i * 32 + lane;
         bool valid = k < n;
         key[i] = valid ? kin[k] : 0;
-        val[i] = valid ? vin[k] : 0;
+        val[i] = valid ? (vin ? vin[k] : (int32_t)k) : 0;
     }
 #pragma unroll
     for (int i = 0; i < kSortItems; ++i) {
@@ -269,22 +270,16 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(
     }
 }
 
+__global__ void k_index_values(int32_t *v, int64_t n) {
+    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
+        v[k] = (int32_t)k;
+}
+
 __global__ void k_reduce_max_i32(const int32_t *__restrict__ in, int64_t n, int32_t *out) {
     int32_t m = 0;
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
          k += (int64_t)gridDim.x * blockDim.x)
         m = max(m, in[k]);
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, d));
-    if ((threadIdx.x & 31) == 0 && m > 0) atomicMax(out, m);
-}
-
-__global__ void k_reduce_max_u64(const uint64_t *__restrict__ in, int64_t n,
-                                 unsigned long long *out) {
-    unsigned long long m = 0;
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
-         k += (int64_t)gridDim.x * blockDim.x)
-        m = max(m, (unsigned long long)in[k]);
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, d));
     if ((threadIdx.x & 31) == 0 && m > 0) atomicMax(out, m);
@@ -334,9 +329,15 @@ size_t radix_hist_elems(int64_t n) {
 
 cudaError_t radix_sort_pairs(uint64_t *k0, int32_t *v0, uint64_t *k1, int32_t *v1, int64_t n,
                              int begin_bit, int end_bit, uint32_t *hist, uint32_t *scan_tmp,
-                             cudaStream_t s, int *which) {
+                             cudaStream_t s, int *which, bool index_values) {
     *which = 0;
-    if (n <= 1 || end_bit <= begin_bit) return cudaSuccess;
+    if (n <= 1 || end_bit <= begin_bit) {
+        if (index_values && n > 0) {   // nothing to sort: the values still have to be written
+            k_index_values<<<(unsigned)std::min<int64_t>((n + 255) / 256, 4096), 256, 0, s>>>(v0, n); note_launch();
+            return cudaGetLastError();
+        }
+        return cudaSuccess;
+    }
     const int64_t ntiles = (n + kSortTile - 1) / kSortTile;
     {
         static bool attr_set[64] = {false};
@@ -353,14 +354,16 @@ cudaError_t radix_sort_pairs(uint64_t *k0, int32_t *v0, uint64_t *k1, int32_t *v
     }
     uint64_t *ki = k0, *ko = k1;
     int32_t *vi = v0, *vo = v1;
+    bool from_index = index_values;   // the first pass's values are the keys' indexes
     for (int shift = begin_bit; shift < end_bit; shift += 8) {
         k_radix_hist<<<(unsigned)ntiles, kSortThreads, 0, s>>>(ki, n, shift, hist, ntiles); note_launch();
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         e = scan_impl<uint32_t, OpSum, false>(hist, hist, 256 * ntiles, scan_tmp, s);
         if (e != cudaSuccess) return e;
-        k_radix_scatter<<<(unsigned)ntiles, kSortThreads, kScatterSmem, s>>>(ki, vi, ko, vo, n, shift,
-                                                                              hist, ntiles); note_launch();
+        k_radix_scatter<<<(unsigned)ntiles, kSortThreads, kScatterSmem, s>>>(ki, from_index ? nullptr : vi, ko, vo, n,
+                                                                              shift, hist, ntiles); note_launch();
+        from_index = false;
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         uint64_t *tk = ki; ki = ko; ko = tk;
@@ -376,16 +379,6 @@ cudaError_t reduce_max_i32(const int32_t *in, int64_t n, int32_t *out, cudaStrea
     int blocks = (int)((n + 255) / 256);
     if (blocks > 4096) blocks = 4096;
     k_reduce_max_i32<<<blocks, 256, 0, s>>>(in, n, out); note_launch();
-    return cudaGetLastError();
-}
-
-cudaError_t reduce_max_u64(const uint64_t *in, int64_t n, unsigned long long *out,
-                           cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(out, 0, sizeof(unsigned long long), s);
-    if (e != cudaSuccess || n <= 0) return e;
-    int blocks = (int)((n + 255) / 256);
-    if (blocks > 4096) blocks = 4096;
-    k_reduce_max_u64<<<blocks, 256, 0, s>>>(in, n, out); note_launch();
     return cudaGetLastError();
 }
 
