@@ -100,12 +100,30 @@ __global__ void k_ranks(const uint64_t *__restrict__ sorted_deg, const int32_t *
     deg_star[base + i] = (int32_t)(sorted_deg[i] & deg_mask);   // low bits: the degree
 }
 
+__device__ __forceinline__ int32_t graph_of(const int32_t *start, int32_t num_graphs, int32_t id) {
+    int32_t lo = 0, hi = num_graphs;   // last g with start[g] <= id
+    while (hi - lo > 1) {
+        const int32_t mid = (lo + hi) >> 1;
+        if (start[mid] <= id) lo = mid; else hi = mid;
+    }
+    return lo;
+}
+
 // ----- a3: projection + sorted adjacency -------------------------------------
 // ---- U side row by row.  Row u of the caller's CSR becomes G* row l + rank_u[u]
 // (its slots start at off_star[l + rank_u[u]]); inside the row the neighbours
 // go in ascending L rank.  The ranks of a row are distinct (E is a set), so
-// any ordering method gives the same layout.  Three tiers by degree:
-//   d <= 32            one warp, each lane's position = the lanes below it;
+// any ordering method gives the same layout.  Tiers by degree:
+//   d <= 32            one warp (eight lanes up to 8 neighbours), each lane's
+//                      position = the lanes below it;
+//   32 < d <= 256      one warp, bitonic sort of 32-bit (rank, index) keys in
+//                      registers where the ranks have at most 24 bits;
+//   256 < d            one CTA (256 threads up to 4,096 neighbours, 1,024 above),
+//                      a bitmap of the L ranks of the row's graph, whose prefix
+//                      popcounts are the positions, where that range is at most
+//                      524,288 ranks (64 KB) and duplicate edges are rejected
+//                      anyway (a repeated bit has no position of its own).
+// Otherwise (wider ranges, validate = 0):
 //   32 < d <= 256      one warp, bitonic sort of (rank, slot) in its shared memory;
 //   256 < d <= 4,096   one CTA, bitonic sort of (rank, slot) in shared memory;
 //   d > 4,096          (a few hundred rows) one radix sort of their edges.
@@ -117,6 +135,8 @@ constexpr int kRowWarpMax = 32;
 constexpr int kRowWarpSortMax = 256;
 constexpr int kRowCtaMax = 4096;
 constexpr int kRowCtaThreads = 256;
+constexpr int32_t kRowBitmapMax = 1 << 19;   // L ranks of one bitmap
+constexpr int kRowTiers = 5;   // warp sort, bitmap (256 threads), bitmap (1,024), CTA sort, radix
 
 struct URowOut {
     int64_t m;
@@ -136,30 +156,155 @@ struct URowOut {
     }
 };
 
+// A warp takes 32 rows (their offsets and ranks are one load per lane), then
+// four rows of at most 8 neighbours at a time, then the longer ones one by one.
 __global__ void k_u_rows_warp(const int32_t *__restrict__ off_u, const int32_t *__restrict__ adj_u,
                               const int32_t *__restrict__ rank_u, const int32_t *__restrict__ rank_l,
                               int32_t r, URowOut o,
     const int *guard = nullptr) {
     if (aborted(guard)) return;
     const int lane = threadIdx.x & 31;
+    const int g = lane >> 3, j = lane & 7;
     const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t u = w0; u < r; u += nw) {
-        const int32_t b = off_u[u], d = off_u[u + 1] - b;
-        if (d == 0 || d > kRowWarpMax) continue;   // warp-uniform
-        const int32_t rl = lane < d ? rank_l[adj_u[b + lane]] : 0x7fffffff;
-        int pos = 0;
-        bool dup = false;
-        for (int k = 0; k < d; ++k) {
-            const int32_t ok = __shfl_sync(0xffffffffu, rl, k);
-            // ties (duplicate edges) are broken by lane, so positions stay distinct
-            pos += (ok < rl || (ok == rl && k < lane)) ? 1 : 0;
-            dup |= ok == rl && k != lane;
+    for (int64_t u0 = w0 * 32; u0 < r; u0 += nw * 32) {
+        const int64_t u = u0 + lane;
+        int32_t b = 0, d = 0, ru = 0;
+        if (u < r) {
+            b = off_u[u];
+            d = off_u[u + 1] - b;
+            if (d > 0 && d <= kRowWarpMax) ru = rank_u[u];
         }
-        if (lane < d) {
-            if (dup && o.check_dup) atomicOr(o.err, kErrDuplicate);
-            o.put(rank_u[u], pos, rl, b + lane);
+        uint32_t left = __ballot_sync(0xffffffffu, d > 0 && d <= 8);
+        while (left) {   // four short rows, one per group of eight lanes
+            int src = 32;
+            for (int k = 0; k < 4; ++k) {
+                if (k == g && left) src = __ffs((int)left) - 1;
+                left &= left - 1;
+            }
+            const int32_t bk = __shfl_sync(0xffffffffu, b, src & 31), rk = __shfl_sync(0xffffffffu, ru, src & 31);
+            int32_t dk = __shfl_sync(0xffffffffu, d, src & 31);
+            if (src > 31) dk = 0;
+            const int32_t rl = j < dk ? rank_l[adj_u[bk + j]] : 0x7fffffff;
+            int pos = 0;
+            bool dup = false;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const int32_t ok = __shfl_sync(0xffffffffu, rl, (g << 3) + k);
+                // ties (duplicate edges) are broken by lane, so positions stay distinct
+                pos += (ok < rl || (ok == rl && k < j)) ? 1 : 0;
+                dup |= ok == rl && k != j;
+            }
+            if (j < dk) {
+                if (dup && o.check_dup) atomicOr(o.err, kErrDuplicate);
+                o.put(rk, pos, rl, bk + j);
+            }
         }
+        left = __ballot_sync(0xffffffffu, d > 8 && d <= kRowWarpMax);
+        while (left) {
+            const int src = __ffs((int)left) - 1;
+            left &= left - 1;
+            const int32_t bk = __shfl_sync(0xffffffffu, b, src), dk = __shfl_sync(0xffffffffu, d, src);
+            const int32_t rk = __shfl_sync(0xffffffffu, ru, src);
+            const int32_t rl = lane < dk ? rank_l[adj_u[bk + lane]] : 0x7fffffff;
+            int pos = 0;
+            bool dup = false;
+            for (int k = 0; k < dk; ++k) {
+                const int32_t ok = __shfl_sync(0xffffffffu, rl, k);
+                pos += (ok < rl || (ok == rl && k < lane)) ? 1 : 0;
+                dup |= ok == rl && k != lane;
+            }
+            if (lane < dk) {
+                if (dup && o.check_dup) atomicOr(o.err, kErrDuplicate);
+                o.put(rk, pos, rl, bk + lane);
+            }
+        }
+    }
+}
+
+// Ascending bitonic sort of 32 * R keys held by a warp, key lane * R + r in
+// register r: strides below R are exchanges inside a lane, the others one
+// shuffle per key.
+template <int R>
+__device__ __forceinline__ void warp_sort(uint32_t (&key)[R], int lane) {
+#pragma unroll
+    for (int k = 2; k <= 32 * R; k <<= 1) {
+#pragma unroll
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            if (j >= R) {
+                // ascending where bit k of the index is clear; the lower of a
+                // pair keeps the smaller key there
+                const bool keep_min = ((lane * R) & k) == 0 ? ((lane * R) & j) == 0 : ((lane * R) & j) != 0;
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const uint32_t o = __shfl_xor_sync(0xffffffffu, key[r], j / R);
+                    key[r] = keep_min ? min(key[r], o) : max(key[r], o);
+                }
+            } else {
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    if ((r & j) == 0) {
+                        const bool up = k < R ? (r & k) == 0 : ((lane * R) & k) == 0;
+                        const uint32_t a = key[r], c = key[r | j];
+                        key[r] = up ? min(a, c) : max(a, c);
+                        key[r | j] = up ? max(a, c) : min(a, c);
+                    }
+                }
+            }
+        }
+    }
+}
+
+// one row of at most 32 * R neighbours; `buf` (32 * R keys of this warp) turns
+// the sorted order back into consecutive lanes for the stores
+template <int R>
+__device__ __forceinline__ void warp_sort_row(const int32_t *adj_u, const int32_t *rank_l, int32_t b, int32_t d,
+                                              int32_t ru, int32_t base, uint32_t *buf, int lane, const URowOut &o) {
+    uint32_t key[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int i = r * 32 + lane;
+        key[r] = i < d ? ((uint32_t)(rank_l[adj_u[b + i]] - base) << 8) | (uint32_t)i : 0xffffffffu;
+    }
+    warp_sort<R>(key, lane);
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < R; ++r) buf[lane * R + r] = key[r];
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int i = r * 32 + lane;
+        if (i < d) {
+            const uint32_t k = buf[i];
+            if (o.check_dup && i > 0 && (buf[i - 1] >> 8) == (k >> 8)) atomicOr(o.err, kErrDuplicate);
+            o.put(ru, i, base + (int32_t)(k >> 8), b + (int32_t)(k & 0xffu));
+        }
+    }
+}
+
+// rows of 33 to 256 neighbours, L ranks (within a batch's graph) of at most 24
+// bits (a rank of all ones in 24 bits with index 255 equals the padding key, and
+// then no key is padding)
+__global__ void __launch_bounds__(kRowCtaThreads) k_u_rows_warp_reg(
+    const int32_t *__restrict__ off_u, const int32_t *__restrict__ adj_u,
+    const int32_t *__restrict__ rank_u, const int32_t *__restrict__ rank_l,
+    const int32_t *__restrict__ rows, const int32_t *__restrict__ nrows_dev,
+    const int32_t *__restrict__ gl, const int32_t *__restrict__ gu, int32_t num_graphs, URowOut o,
+    const int *guard = nullptr) {
+    if (aborted(guard)) return;
+    __shared__ uint32_t buf[kRowCtaThreads / 32][kRowWarpSortMax];
+    const int lane = threadIdx.x & 31;
+    uint32_t *wb = buf[threadIdx.x >> 5];
+    const int32_t nrows = *nrows_dev;
+    const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t i0 = w0; i0 < nrows; i0 += nw) {
+        const int32_t u = rows[i0];
+        const int32_t b = off_u[u], d = off_u[u + 1] - b, ru = rank_u[u];
+        const int32_t base = gl ? gl[graph_of(gu, num_graphs, u)] : 0;
+        if (d <= 64) warp_sort_row<2>(adj_u, rank_l, b, d, ru, base, wb, lane, o);
+        else if (d <= 128) warp_sort_row<4>(adj_u, rank_l, b, d, ru, base, wb, lane, o);
+        else warp_sort_row<8>(adj_u, rank_l, b, d, ru, base, wb, lane, o);
     }
 }
 
@@ -182,10 +327,10 @@ __device__ __forceinline__ void warp_bitonic(uint64_t *buf, int np, int lane) {
 __global__ void __launch_bounds__(kRowCtaThreads) k_u_rows_warp_sort(
     const int32_t *__restrict__ off_u, const int32_t *__restrict__ adj_u,
     const int32_t *__restrict__ rank_u, const int32_t *__restrict__ rank_l,
-    const int32_t *__restrict__ rows, int32_t nrows, URowOut o,
-    const int *guard = nullptr, const int32_t *nrows_dev = nullptr) {
+    const int32_t *__restrict__ rows, const int32_t *__restrict__ nrows_dev, URowOut o,
+    const int *guard = nullptr) {
     if (aborted(guard)) return;
-    if (nrows_dev) nrows = *nrows_dev;
+    const int32_t nrows = *nrows_dev;
     __shared__ uint64_t buf[kRowCtaThreads / 32][kRowWarpSortMax];
     const int lane = threadIdx.x & 31;
     uint64_t *wb = buf[threadIdx.x >> 5];
@@ -214,10 +359,7 @@ __global__ void __launch_bounds__(kRowCtaThreads) k_u_rows_warp_sort(
 __global__ void __launch_bounds__(kRowCtaThreads) k_u_rows_cta(
     const int32_t *__restrict__ off_u, const int32_t *__restrict__ adj_u,
     const int32_t *__restrict__ rank_u, const int32_t *__restrict__ rank_l,
-    const int32_t *__restrict__ rows, int32_t nrows, URowOut o,
-    const int *guard = nullptr, const int32_t *nrows_dev = nullptr) {
-    if (aborted(guard)) return;
-    if (nrows_dev) nrows = *nrows_dev;
+    const int32_t *__restrict__ rows, int32_t nrows, URowOut o) {
     __shared__ uint64_t buf[kRowCtaMax];
     for (int64_t i0 = blockIdx.x; i0 < nrows; i0 += gridDim.x) {
         const int32_t u = rows[i0];
@@ -251,27 +393,121 @@ __global__ void __launch_bounds__(kRowCtaThreads) k_u_rows_cta(
     }
 }
 
-// lists of the rows of the CTA tier and of the largest rows (any order: every
-// row is written to its own slots); one atomic per warp and list
-__global__ void k_row_tiers(const int32_t *__restrict__ off_u, int32_t r, int32_t *lists,
-                            int32_t *counts,
+// lists of the rows of every tier above 32 neighbours (any order: every row
+// is written to its own slots); one atomic per warp and list.  lists[t * r ...]:
+// tier 0 warp sort, 1 and 2 bitmap, 3 CTA sort, 4 radix.  `range`: the L ranks of
+// a single graph (a batch's row: its graph's); bitmaps only where `bitmaps`.
+__global__ void k_row_tiers(const int32_t *__restrict__ off_u, int32_t r, int32_t range,
+                            const int32_t *__restrict__ gu, const int32_t *__restrict__ gl, int32_t num_graphs,
+                            int bitmaps, int32_t *lists, int32_t *counts,
     const int *guard = nullptr) {
     if (aborted(guard)) return;
-    // lists[t * r ...]: rows of tier t (0: warp sort, 1: CTA sort, 2: radix)
     const int lane = threadIdx.x & 31;
     const uint32_t lt = (1u << lane) - 1u;
     for (int64_t u0 = (int64_t)blockIdx.x * blockDim.x; u0 < r; u0 += (int64_t)gridDim.x * blockDim.x) {
         const int64_t u = u0 + threadIdx.x;
         const int32_t d = u < r ? off_u[u + 1] - off_u[u] : 0;
-        const int tier = d <= kRowWarpMax ? -1 : d <= kRowWarpSortMax ? 0 : d <= kRowCtaMax ? 1 : 2;
+        int tier = d <= kRowWarpMax ? -1 : 0;
+        if (d > kRowWarpSortMax) {
+            int32_t len = range;
+            if (gl) {
+                const int32_t g = graph_of(gu, num_graphs, (int32_t)u);
+                len = gl[g + 1] - gl[g];
+            }
+            tier = (bitmaps && len <= kRowBitmapMax) ? (d <= kRowCtaMax ? 1 : 2) : (d <= kRowCtaMax ? 3 : 4);
+        }
+        if (!__any_sync(0xffffffffu, tier >= 0)) continue;
 #pragma unroll
-        for (int t = 0; t < 3; ++t) {
+        for (int t = 0; t < kRowTiers; ++t) {
             const uint32_t bm = __ballot_sync(0xffffffffu, tier == t);
             int32_t o = 0;
             if (lane == 0 && bm) o = atomicAdd(counts + t, __popc(bm));
             o = __shfl_sync(0xffffffffu, o, 0);
             if (tier == t) lists[(int64_t)t * r + o + __popc(bm & lt)] = (int32_t)u;
         }
+    }
+}
+
+// U rows of more than 256 neighbours, one CTA per row: one bit per neighbour's
+// L rank in a bitmap of its graph's L rank range (all L ranks of a single
+// graph); a neighbour's position is the number of set bits below its rank.  A
+// bit that is already set is a duplicate edge: it is reported, and one of the
+// positions past the distinct ranks is written for it, so that every position
+// of the row holds a valid id.  Replaces a bitonic sort (78 stages with a barrier each at 4,096
+// neighbours) and, above 4,096, a radix sort of all such rows' edges.
+template <int kThreads>
+__global__ void __launch_bounds__(kThreads) k_u_rows_bitmap(
+    const int32_t *__restrict__ off_u, const int32_t *__restrict__ adj_u,
+    const int32_t *__restrict__ rank_u, const int32_t *__restrict__ rank_l,
+    const int32_t *__restrict__ rows, const int32_t *__restrict__ nrows_dev, int32_t range,
+    const int32_t *__restrict__ gl, const int32_t *__restrict__ gu, int32_t num_graphs, URowOut o,
+    const int *guard = nullptr) {
+    if (aborted(guard)) return;
+    extern __shared__ __align__(16) uint32_t bm_smem[];   // bits[words], then prefix of each 4 words
+    __shared__ int32_t part[kThreads / 32];
+    __shared__ int32_t n_dup;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int32_t nrows = *nrows_dev;
+    for (int64_t i0 = blockIdx.x; i0 < nrows; i0 += gridDim.x) {
+        const int32_t u = rows[i0];
+        const int32_t b = off_u[u], d = off_u[u + 1] - b, ru = rank_u[u];
+        int32_t base = 0, len = range;
+        if (gl) {
+            const int32_t g = graph_of(gu, num_graphs, u);
+            base = gl[g];   // the graph's L ranks: [gl[g], gl[g + 1])
+            len = gl[g + 1] - base;
+        }
+        // every edge stays inside its graph (checked), so 0 <= rank - base < len
+        const int quads = (len + 127) / 128;   // 16-byte units of the bitmap
+        uint4 *const q4 = reinterpret_cast<uint4 *>(bm_smem);
+        int32_t *const qpre = reinterpret_cast<int32_t *>(q4 + quads);
+        for (int i = tid; i < quads; i += kThreads) q4[i] = make_uint4(0, 0, 0, 0);
+        if (tid == 0) n_dup = 0;
+        __syncthreads();
+#pragma unroll 4
+        for (int32_t i = tid; i < d; i += kThreads) {
+            const int32_t rl = rank_l[adj_u[b + i]], k = rl - base;
+            const uint32_t bit = 1u << (k & 31);
+            if (atomicOr(&bm_smem[k >> 5], bit) & bit) {
+                if (o.check_dup) atomicOr(o.err, kErrDuplicate);
+                o.put(ru, d - 1 - atomicAdd(&n_dup, 1), rl, b + i);
+            }
+        }
+        __syncthreads();
+        // exclusive prefix of the quads' popcounts: a contiguous share per thread
+        const int per = (quads + kThreads - 1) / kThreads;
+        const int f = min(tid * per, quads), e = min(f + per, quads);
+        int32_t sum = 0;
+        for (int i = f; i < e; ++i) {
+            const uint4 q = q4[i];
+            qpre[i] = sum;
+            sum += __popc(q.x) + __popc(q.y) + __popc(q.z) + __popc(q.w);
+        }
+        int32_t incl = sum;
+#pragma unroll
+        for (int dd = 1; dd < 32; dd <<= 1) {
+            const int32_t t = __shfl_up_sync(0xffffffffu, incl, dd);
+            if (lane >= dd) incl += t;
+        }
+        if (lane == 31) part[warp] = incl;
+        __syncthreads();
+        int32_t before = incl - sum;
+        for (int w = 0; w < warp; ++w) before += part[w];
+        for (int i = f; i < e; ++i) qpre[i] += before;
+        __syncthreads();
+#pragma unroll 4
+        for (int32_t i = tid; i < d; i += kThreads) {
+            const int32_t rl = rank_l[adj_u[b + i]], k = rl - base;
+            const uint4 q = q4[k >> 7];
+            const int w = (k >> 5) & 3;
+            const uint32_t mine = w == 0 ? q.x : (w == 1 ? q.y : (w == 2 ? q.z : q.w));
+            int32_t pos = qpre[k >> 7] + __popc(mine & ((1u << (k & 31)) - 1u));
+            if (w > 0) pos += __popc(q.x);
+            if (w > 1) pos += __popc(q.y);
+            if (w > 2) pos += __popc(q.z);
+            o.put(ru, pos, rl, b + i);
+        }
+        __syncthreads();   // the bitmap is reused by the next row
     }
 }
 
@@ -773,22 +1009,15 @@ unsigned grid_stride_blocks(int64_t n) {
 }
 
 // ----- batches prepared as one disjoint union ------------------------------------
-__device__ __forceinline__ int32_t graph_of(const int32_t *start, int32_t num_graphs, int32_t id) {
-    int32_t lo = 0, hi = num_graphs;   // last g with start[g] <= id
-    while (hi - lo > 1) {
-        const int32_t mid = (lo + hi) >> 1;
-        if (start[mid] <= id) lo = mid; else hi = mid;
-    }
-    return lo;
-}
-
 __global__ void k_check_starts(const int32_t *__restrict__ start, int32_t num_graphs,
-                               int32_t total, int *err, int32_t max_len = 0x7fffffff) {
+                               int32_t total, int *err, int32_t max_len = 0x7fffffff,
+                               int *longest = nullptr) {
     for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g <= num_graphs;
          g += (int64_t)gridDim.x * blockDim.x) {
         if (g == 0 && start[0] != 0) atomicOr(err, kErrBadOffsets);
         if (g < num_graphs && (start[g + 1] < start[g] || start[g + 1] - start[g] > max_len))
             atomicOr(err, kErrBadOffsets);
+        if (longest && g < num_graphs) atomicMax(longest, start[g + 1] - start[g]);
         if (g == num_graphs && start[g] != total) atomicOr(err, kErrBadOffsets);
     }
 }
@@ -1060,6 +1289,62 @@ int rebin_graph(Graph *g, cudaStream_t s, int32_t warp_max_work, int32_t team_ma
     return rc;
 }
 
+// shared memory of a bitmap over `range` L ranks
+static int bitmap_bytes(int32_t range) { return (std::min(range, kRowBitmapMax) + 127) / 128 * 20; }
+
+static int rows_smem_setup(int device) {
+    static bool done[64] = {false};
+    if (device < 0 || device >= 64) return BFC_ERR_INVALID_ARGUMENT;
+    if (done[device]) return BFC_OK;
+    BFC_CUDA(cudaFuncSetAttribute(k_u_rows_bitmap<kRowCtaThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  bitmap_bytes(kRowBitmapMax)));
+    BFC_CUDA(cudaFuncSetAttribute(k_u_rows_bitmap<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  bitmap_bytes(kRowBitmapMax)));
+    done[device] = true;
+    return BFC_OK;
+}
+
+// The U side of G*: every tier that needs no size on the host.  `range`: the L
+// ranks of a single graph, or of a batch's largest graph; `max_deg` bounds the
+// row lengths (tiers above it are not launched).
+static int launch_u_rows(const int32_t *off_u, const int32_t *adj_u, Graph *g, int32_t range, const int32_t *gu,
+                         const int32_t *gl, int32_t num_graphs, int32_t max_deg, int bitmaps, const URowOut &uo,
+                         int32_t *tier_rows, int32_t *tier_n, cudaStream_t s, const int *guard) {
+    const int32_t r = g->r;
+    const int64_t m = g->m;
+    int rc = rows_smem_setup(g->device);
+    if (rc) return rc;
+    k_u_rows_warp<<<grid_stride_blocks(r), kT, 0, s>>>(off_u, adj_u, g->rank_u, g->rank_l, r, uo, guard); note_launch();
+    BFC_CUDA(cudaGetLastError());
+    if (max_deg <= kRowWarpMax || m <= kRowWarpMax) return BFC_OK;
+    BFC_CUDA(cudaMemsetAsync(tier_n, 0, kRowTiers * sizeof(int32_t), s));
+    k_row_tiers<<<grid_stride_blocks(r), kT, 0, s>>>(off_u, r, range, gu, gl, num_graphs, bitmaps, tier_rows, tier_n,
+                                                     guard); note_launch();
+    const unsigned wg = (unsigned)std::min<int64_t>(m / (kRowWarpMax + 1) * 32 / kRowCtaThreads + 1, 152 * 8);
+    if (range <= 1 << 24) {
+        k_u_rows_warp_reg<<<wg, kRowCtaThreads, 0, s>>>(off_u, adj_u, g->rank_u, g->rank_l, tier_rows, tier_n, gl, gu,
+                                                        num_graphs, uo, guard); note_launch();
+    } else {
+        k_u_rows_warp_sort<<<wg, kRowCtaThreads, 0, s>>>(off_u, adj_u, g->rank_u, g->rank_l, tier_rows, tier_n, uo,
+                                                         guard); note_launch();
+    }
+    if (bitmaps && max_deg > kRowWarpSortMax && m > kRowWarpSortMax) {
+        k_u_rows_bitmap<kRowCtaThreads>
+            <<<(unsigned)std::min<int64_t>(m / kRowWarpSortMax, 152 * 8), kRowCtaThreads, bitmap_bytes(range), s>>>(
+                off_u, adj_u, g->rank_u, g->rank_l, tier_rows + r, tier_n + 1, range, gl, gu, num_graphs, uo, guard);
+        note_launch();
+    }
+    if (bitmaps && max_deg > kRowCtaMax && m > kRowCtaMax) {
+        k_u_rows_bitmap<1024>
+            <<<(unsigned)std::min<int64_t>(m / kRowCtaMax, 152 * 2), 1024, bitmap_bytes(range), s>>>(
+                off_u, adj_u, g->rank_u, g->rank_l, tier_rows + 2 * (int64_t)r, tier_n + 2, range, gl, gu, num_graphs, uo,
+                guard);
+        note_launch();
+    }
+    BFC_CUDA(cudaGetLastError());
+    return BFC_OK;
+}
+
 // work per start, the runs of the U-side middle slots (Algorithm 2), and
 // stats[0] = W, [1] = the heaviest start, [2] = starts beyond the CTA-hash bin
 static void launch_work(Graph *g, int32_t *big, int32_t *n_big, unsigned long long *gwork, unsigned long long *stats,
@@ -1122,12 +1407,16 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
     BFC_CUDA(cudaMemcpyAsync(&herr, g->err, sizeof(int), cudaMemcpyDeviceToHost, s));
     BFC_CUDA(cudaStreamSynchronize(s));
     if (herr) { set_last_error("off_u is not a CSR offset array of num_edges entries"); return BFC_ERR_INVALID_GRAPH; }
+    int32_t l_range = l;
     if (num_graphs > 0) {
         k_check_starts<<<blocks_for((int64_t)num_graphs + 1), kT, 0, s>>>(graph_u_start, num_graphs, r, g->err); note_launch();
-        k_check_starts<<<blocks_for((int64_t)num_graphs + 1), kT, 0, s>>>(graph_l_start, num_graphs, l, g->err); note_launch();
+        k_check_starts<<<blocks_for((int64_t)num_graphs + 1), kT, 0, s>>>(graph_l_start, num_graphs, l, g->err, 0x7fffffff, g->err + 1); note_launch();
         BFC_CUDA(cudaGetLastError());
-        BFC_CUDA(cudaMemcpyAsync(&herr, g->err, sizeof(int), cudaMemcpyDeviceToHost, s));
+        int hstart[2] = {0, 0};
+        BFC_CUDA(cudaMemcpyAsync(hstart, g->err, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
         BFC_CUDA(cudaStreamSynchronize(s));
+        herr = hstart[0];
+        l_range = hstart[1];   // the largest L layer of one graph
         if (herr) { set_last_error("graph start arrays are not prefix sums of the layer sizes"); return BFC_ERR_INVALID_GRAPH; }
         g->num_graphs = num_graphs;
         GET(g->mem, g->gstar, std::max<int64_t>(n, 1));
@@ -1234,32 +1523,27 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
         // U side row by row (warp / CTA tiers, radix sort for the largest rows);
         // the swapped keys for the L side land in k1
         const URowOut uo{m, l, bu, g->off, g->adj, g->eid, rows_star, k1, g->err, opt->validate};
-        k_u_rows_warp<<<grid_stride_blocks((int64_t)r * 32), kT, 0, s>>>(csr->off_u, csr->adj_u, g->rank_u,
-                                                                         g->rank_l, r, uo); note_launch();
-        BFC_CUDA(cudaGetLastError());
+        int32_t *tier_rows = nullptr, *tier_n = nullptr;
+        GET(tmp, tier_rows, kRowTiers * std::max<int64_t>(r, 1));
+        GET(tmp, tier_n, kRowTiers);
         {
-            int32_t *tier_rows, *tier_n;
-            GET(tmp, tier_rows, 3 * std::max<int64_t>(r, 1));
-            GET(tmp, tier_n, 4);
-            BFC_CUDA(cudaMemsetAsync(tier_n, 0, 4 * sizeof(int32_t), s));
-            k_row_tiers<<<grid_stride_blocks(r), kT, 0, s>>>(csr->off_u, r, tier_rows, tier_n); note_launch();
-            BFC_CUDA(cudaGetLastError());
-            int32_t hn[3] = {0, 0, 0};
-            BFC_CUDA(cudaMemcpyAsync(hn, tier_n, 3 * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+            int rc = launch_u_rows(csr->off_u, csr->adj_u, g, l_range, graph_u_start, graph_l_start, num_graphs,
+                                   hmax[0], opt->validate, uo, tier_rows, tier_n, s, nullptr);
+            if (rc) return rc;
+        }
+        // rows that no bitmap takes (see the tiers): CTA sorts, and a radix sort
+        // of the largest rows' edges
+        if (hmax[0] > kRowWarpSortMax && (!opt->validate || l_range > kRowBitmapMax)) {
+            int32_t hn[2] = {0, 0};
+            BFC_CUDA(cudaMemcpyAsync(hn, tier_n + 3, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
             BFC_CUDA(cudaStreamSynchronize(s));
             if (hn[0] > 0) {
-                const int64_t warps = std::min<int64_t>(hn[0], 152 * 64);
-                k_u_rows_warp_sort<<<(unsigned)((warps * 32 + kRowCtaThreads - 1) / kRowCtaThreads), kRowCtaThreads, 0, s>>>(
-                    csr->off_u, csr->adj_u, g->rank_u, g->rank_l, tier_rows, hn[0], uo); note_launch();
+                k_u_rows_cta<<<(unsigned)std::min<int32_t>(hn[0], 152 * 16), kRowCtaThreads, 0, s>>>(
+                    csr->off_u, csr->adj_u, g->rank_u, g->rank_l, tier_rows + 3 * (int64_t)r, hn[0], uo); note_launch();
                 BFC_CUDA(cudaGetLastError());
             }
-            if (hn[1] > 0) {
-                k_u_rows_cta<<<(unsigned)std::min<int32_t>(hn[1], 152 * 16), kRowCtaThreads, 0, s>>>(
-                    csr->off_u, csr->adj_u, g->rank_u, g->rank_l, tier_rows + r, hn[1], uo); note_launch();
-                BFC_CUDA(cudaGetLastError());
-            }
-            const int32_t *large_rows = tier_rows + 2 * (int64_t)r;
-            const int32_t nl = hn[2];
+            const int32_t *large_rows = tier_rows + 4 * (int64_t)r;
+            const int32_t nl = hn[1];
             int64_t *ldeg, *loff;
             GET(tmp, ldeg, (int64_t)nl + 1);
             GET(tmp, loff, (int64_t)nl + 1);
@@ -1378,73 +1662,6 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
 // ----------------------------------------------------------------------------
 namespace {
 
-constexpr int32_t kPlanMaxLayer = 65535;
-constexpr int kBitmapWords = (kPlanMaxLayer + 1) / 32;   // 2,048 words, 8 KB
-
-// U rows of more than 4,096 neighbours, one CTA per row.  The row's L ranks
-// are distinct and lie in its graph's L rank range, so a bitmap of that range
-// gives every neighbour its position: the number of set bits below its rank.
-// A bit that is already set is a duplicate edge.
-__global__ void __launch_bounds__(kRowCtaThreads) k_u_rows_bitmap(
-    const int32_t *__restrict__ off_u, const int32_t *__restrict__ adj_u,
-    const int32_t *__restrict__ rank_u, const int32_t *__restrict__ rank_l,
-    const int32_t *__restrict__ rows, const int32_t *__restrict__ nrows_dev,
-    const int32_t *__restrict__ gl, const int32_t *__restrict__ gu, int32_t num_graphs, URowOut o,
-    const int *guard) {
-    if (aborted(guard)) return;
-    __shared__ uint32_t bits[kBitmapWords];
-    __shared__ int32_t wpre[kBitmapWords];
-    __shared__ int32_t part[kRowCtaThreads / 32];
-    constexpr int kPerThread = kBitmapWords / kRowCtaThreads;   // 8 words
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int32_t nrows = *nrows_dev;
-    for (int64_t i0 = blockIdx.x; i0 < nrows; i0 += gridDim.x) {
-        const int32_t u = rows[i0];
-        const int32_t b = off_u[u], d = off_u[u + 1] - b;
-        const int32_t g = graph_of(gu, num_graphs, u);
-        const int32_t base = gl[g];   // the graph's L ranks: [gl[g], gl[g + 1])
-        for (int i = tid; i < kBitmapWords; i += kRowCtaThreads) bits[i] = 0;
-        __syncthreads();
-        for (int32_t i = tid; i < d; i += kRowCtaThreads) {
-            // every edge stays inside its graph (checked), so 0 <= k < 65,536
-            const int32_t k = rank_l[adj_u[b + i]] - base;
-            const uint32_t bit = 1u << (k & 31);
-            const uint32_t old = atomicOr(&bits[k >> 5], bit);
-            if ((old & bit) && o.check_dup) atomicOr(o.err, kErrDuplicate);
-        }
-        __syncthreads();
-        // exclusive prefix of the words' popcounts: 8 words per thread
-        int32_t loc[kPerThread], sum = 0;
-#pragma unroll
-        for (int j = 0; j < kPerThread; ++j) {
-            loc[j] = sum;
-            sum += __popc(bits[tid * kPerThread + j]);
-        }
-        int32_t incl = sum;
-#pragma unroll
-        for (int dd = 1; dd < 32; dd <<= 1) {
-            const int32_t t = __shfl_up_sync(0xffffffffu, incl, dd);
-            if (lane >= dd) incl += t;
-        }
-        if (lane == 31) part[warp] = incl;
-        __syncthreads();
-        int32_t before = 0;
-        for (int w = 0; w < warp; ++w) before += part[w];
-        before += incl - sum;
-#pragma unroll
-        for (int j = 0; j < kPerThread; ++j) wpre[tid * kPerThread + j] = before + loc[j];
-        __syncthreads();
-        const int32_t ru = rank_u[u];
-        for (int32_t i = tid; i < d; i += kRowCtaThreads) {
-            const int32_t rl = rank_l[adj_u[b + i]];
-            const int32_t k = rl - base;
-            const int32_t pos = wpre[k >> 5] + __popc(bits[k >> 5] & ((1u << (k & 31)) - 1u));
-            o.put(ru, pos, rl, b + i);
-        }
-        __syncthreads();   // the bitmap is reused by the next row
-    }
-}
-
 // heaviest first by exact work, 32 key bits (work saturated at 2^32 - 1)
 __global__ void k_sched_keys_plan(const uint64_t *__restrict__ work, int32_t n, uint64_t *keys,
                                   int32_t *vals, const int *guard) {
@@ -1513,7 +1730,7 @@ int batch_plan_create(BatchPlan *pl, cudaStream_t s) {
     GET(pl->k0, nsort + 1); GET(pl->k1, nsort + 1); GET(pl->v0, nsort); GET(pl->v1, nsort);
     GET(pl->deg_u, r); GET(pl->deg_l, l); GET(pl->deg_star, n);
     GET(pl->rows_star, 2 * m); GET(pl->big, std::min<int64_t>(2 * m / kWorkLane, n) + 1); GET(pl->n_big, 1);
-    GET(pl->tier_rows, 3 * (int64_t)std::max(r, 1)); GET(pl->tier_n, 4);
+    GET(pl->tier_rows, kRowTiers * (int64_t)std::max(r, 1)); GET(pl->tier_n, kRowTiers);
     GET(pl->hist, radix_hist_elems(nsort));
     GET(pl->hist_tmp, scan_tmp_elems<uint32_t>((int64_t)radix_hist_elems(nsort)));
     GET(pl->scan64_tmp, std::max(scan_tmp_elems<int64_t>((int64_t)n + 1), max_scan_tmp_elems(m)));
@@ -1531,6 +1748,7 @@ int batch_plan_create(BatchPlan *pl, cudaStream_t s) {
     int which = 0;
     BFC_CUDA(radix_sort_pairs(pl->k0, pl->v0, pl->k1, pl->v1, 2, 0, 8, pl->hist, pl->hist_tmp, s, &which));
     int rc = count_smem_setup(g->device);
+    if (rc == BFC_OK) rc = rows_smem_setup(g->device);
     if (rc) return rc;
     BFC_CUDA(cudaStreamSynchronize(s));
     return BFC_OK;
@@ -1586,18 +1804,9 @@ int batch_plan_run(BatchPlan *pl, const int32_t *off_u, const int32_t *adj_u, co
     if (m > 0) {
         k_check_batch_rows<<<grid_stride_blocks(r), kT, 0, s>>>(off_u, adj_u, r, gu, gl, G, g->err, guard); note_launch();
         const URowOut uo{m, l, bu, g->off, g->adj, g->eid, pl->rows_star, pl->k1, g->err, opt->validate};
-        k_u_rows_warp<<<grid_stride_blocks((int64_t)r * 32), kT, 0, s>>>(off_u, adj_u, g->rank_u, g->rank_l, r, uo,
-                                                                         guard); note_launch();
-        BFC_CUDA(cudaMemsetAsync(pl->tier_n, 0, 4 * sizeof(int32_t), s));
-        k_row_tiers<<<grid_stride_blocks(r), kT, 0, s>>>(off_u, r, pl->tier_rows, pl->tier_n, guard); note_launch();
-        k_u_rows_warp_sort<<<152 * 8, kRowCtaThreads, 0, s>>>(off_u, adj_u, g->rank_u, g->rank_l, pl->tier_rows, 0,
-                                                              uo, guard, pl->tier_n); note_launch();
-        k_u_rows_cta<<<152 * 16, kRowCtaThreads, 0, s>>>(off_u, adj_u, g->rank_u, g->rank_l, pl->tier_rows + r, 0,
-                                                         uo, guard, pl->tier_n + 1); note_launch();
-        k_u_rows_bitmap<<<152 * 4, kRowCtaThreads, 0, s>>>(off_u, adj_u, g->rank_u, g->rank_l,
-                                                           pl->tier_rows + 2 * (int64_t)r, pl->tier_n + 2, gl, gu,
-                                                           G, uo, guard); note_launch();
-        BFC_CUDA(cudaGetLastError());
+        int rc = launch_u_rows(off_u, adj_u, g, pl->max_layer, gu, gl, G, pl->max_layer, 1, uo, pl->tier_rows,
+                               pl->tier_n, s, guard);
+        if (rc) return rc;
         // L side: stable sort of the swapped keys on their rank_l bits
         int which2 = 0;
         BFC_CUDA(radix_sort_pairs(pl->k1, pl->v1, pl->k0, pl->v0, m, bu, bu + bl, pl->hist, pl->hist_tmp, s, &which2, true));

@@ -187,6 +187,7 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_hist(const uint64_t *__r
 // each digit's keys are consecutive (coalesced) rather than one per key.
 constexpr int kScatterSmem = (kSortThreads / 32) * 256 * 4 + 2 * 256 * 4 + kSortTile * (8 + 4);
 
+template <bool kIndexValues>
 __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(
     const uint64_t *__restrict__ kin, const int32_t *__restrict__ vin, uint64_t *__restrict__ kout,
     int32_t *__restrict__ vout, int64_t n, int shift, const uint32_t *__restrict__ hist_scan,
@@ -214,7 +215,7 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(
         int64_t k = base + i * 32 + lane;
         bool valid = k < n;
         key[i] = valid ? kin[k] : 0;
-        val[i] = valid ? (vin ? vin[k] : (int32_t)k) : 0;
+        val[i] = kIndexValues ? (int32_t)k : (valid ? vin[k] : 0);
     }
 #pragma unroll
     for (int i = 0; i < kSortItems; ++i) {
@@ -346,8 +347,11 @@ cudaError_t radix_sort_pairs(uint64_t *k0, int32_t *v0, uint64_t *k1, int32_t *v
         if (e != cudaSuccess) return e;
         if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
         if (!attr_set[dev]) {
-            e = cudaFuncSetAttribute(k_radix_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            e = cudaFuncSetAttribute(k_radix_scatter<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      kScatterSmem);
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(k_radix_scatter<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         kScatterSmem);
             if (e != cudaSuccess) return e;
             attr_set[dev] = true;
         }
@@ -361,8 +365,13 @@ cudaError_t radix_sort_pairs(uint64_t *k0, int32_t *v0, uint64_t *k1, int32_t *v
         if (e != cudaSuccess) return e;
         e = scan_impl<uint32_t, OpSum, false>(hist, hist, 256 * ntiles, scan_tmp, s);
         if (e != cudaSuccess) return e;
-        k_radix_scatter<<<(unsigned)ntiles, kSortThreads, kScatterSmem, s>>>(ki, from_index ? nullptr : vi, ko, vo, n,
-                                                                              shift, hist, ntiles); note_launch();
+        if (from_index)
+            k_radix_scatter<true><<<(unsigned)ntiles, kSortThreads, kScatterSmem, s>>>(ki, vi, ko, vo, n, shift, hist,
+                                                                                       ntiles);
+        else
+            k_radix_scatter<false><<<(unsigned)ntiles, kSortThreads, kScatterSmem, s>>>(ki, vi, ko, vo, n, shift, hist,
+                                                                                        ntiles);
+        note_launch();
         from_index = false;
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
