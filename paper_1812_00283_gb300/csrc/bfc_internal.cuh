@@ -98,8 +98,14 @@ void pool_free(void *p, cudaStream_t s);
 // (reset to zero first when reset_high).
 cudaError_t pool_usage(int64_t *current, int64_t *high, bool reset_high);
 
-// A list of pool allocations released together.
+// A list of pool allocations released together.  Requests of at most 128 KB
+// are carved from 512 KB slabs (a prepare makes about forty of them, and each
+// pool call costs the host about a microsecond); a carved piece goes back with
+// its slab.
 struct Allocs {
+    static constexpr size_t kSlab = 512 << 10, kCarve = 128 << 10;
+    char *slab = nullptr;
+    size_t slab_left = 0;
     static constexpr int kMax = 64;
     void *ptr[kMax];
     size_t bytes[kMax];
@@ -112,6 +118,15 @@ struct Allocs {
         size_t b = count * sizeof(T);
         if (b == 0) b = 16;
         b = (b + 255) & ~size_t(255);
+        if (b <= kCarve && b <= slab_left) {
+            *p = reinterpret_cast<T *>(slab);
+            slab += b;
+            slab_left -= b;
+            return cudaSuccess;
+        }
+        const bool carve = b <= kCarve;
+        const size_t want = b;
+        if (carve) b = kSlab;
         void *q = nullptr;
         cudaError_t e = pool_alloc(&q, b, stream);
         if (e != cudaSuccess) return e;
@@ -119,14 +134,18 @@ struct Allocs {
         bytes[n] = b;
         ++n;
         total += b;
+        if (carve) {
+            slab = static_cast<char *>(q) + want;
+            slab_left = b - want;
+        }
         *p = static_cast<T *>(q);
         return cudaSuccess;
     }
-    // frees one allocation of the list (no-op for null or unknown pointers)
+    // frees one allocation of the list (no-op for null, unknown and carved pointers)
     void drop(void *p) {
         if (!p) return;
         for (int i = 0; i < n; ++i)
-            if (ptr[i] == p) {
+            if (ptr[i] == p && bytes[i] != kSlab) {
                 pool_free(p, stream);
                 total -= bytes[i];
                 for (int j = i + 1; j < n; ++j) { ptr[j - 1] = ptr[j]; bytes[j - 1] = bytes[j]; }
@@ -138,6 +157,8 @@ struct Allocs {
         for (int i = n - 1; i >= 0; --i) pool_free(ptr[i], stream);
         n = 0;
         total = 0;
+        slab = nullptr;
+        slab_left = 0;
     }
 };
 
@@ -146,6 +167,7 @@ struct Allocs {
 // ---------------------------------------------------------------------------
 struct Graph {
     int32_t r = 0, l = 0, n = 0;
+    int32_t max_range = 0;         // the larger layer (of a batch: of any one graph)
     int64_t m = 0;
     bfc_options opt{};
     bfc_info info{};
@@ -169,7 +191,7 @@ struct Graph {
     int32_t team_max = 0;          // effective team bound of the current schedule
     bool may_retry = false;        // the schedule can re-queue starts (retry pass launched)
     int *cursors = nullptr;        // [8] work-queue cursors of the count kernels
-    unsigned long long *acc = nullptr;  // [1] device accumulator for ⋈_G
+    unsigned long long *acc = nullptr;  // [1] device accumulator for ⋈_G (after the cursors)
     unsigned long long *pv = nullptr;   // [n] per-vertex scratch in G* ids (allocated on demand? no: in prepare)
     int *err = nullptr;            // device error word
     // chunk-boundary table: for vertex v of G*, entry c is the position in
@@ -243,9 +265,6 @@ cudaError_t radix_sort_pairs(uint64_t *k0, int32_t *v0, uint64_t *k1, int32_t *v
                              int begin_bit, int end_bit, uint32_t *hist, uint32_t *scan_tmp,
                              cudaStream_t s, int *which, bool index_values = false);
 
-// Device-wide maximum into one element (result in device memory).
-cudaError_t reduce_max_i32(const int32_t *in, int64_t n, int32_t *out, cudaStream_t s);
-
 // ---------------------------------------------------------------------------
 // Prepare and count (prepare.cu, count.cu)
 // ---------------------------------------------------------------------------
@@ -274,9 +293,10 @@ struct BatchPlan {
     uint64_t *k0 = nullptr, *k1 = nullptr;
     int32_t *v0 = nullptr, *v1 = nullptr, *deg_u = nullptr, *deg_l = nullptr, *deg_star = nullptr;
     int32_t *rows_star = nullptr, *tier_rows = nullptr, *tier_n = nullptr, *big = nullptr, *n_big = nullptr;
+    int32_t *heavy = nullptr;
     uint32_t *hist = nullptr, *hist_tmp = nullptr;
     int64_t *scan64_tmp = nullptr, *deg64 = nullptr;
-    unsigned long long *red = nullptr;   // [0] W, [4..8) bin sizes
+    unsigned long long *red = nullptr;   // [0] W, [3..8) bin sizes, [8], [9] largest degrees
 };
 int batch_plan_create(BatchPlan *pl, cudaStream_t s);
 int batch_plan_run(BatchPlan *pl, const int32_t *off_u, const int32_t *adj_u, const int32_t *gu,

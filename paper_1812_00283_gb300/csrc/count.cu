@@ -1537,8 +1537,7 @@ int launch_count(Graph *g, cudaStream_t s, int mode, unsigned long long *pv_proj
         int rc2 = core_product(g, s);
         if (rc2) return rc2;
     }
-    BFC_CUDA(cudaMemsetAsync(g->cursors, 0, 8 * sizeof(int), s));
-    BFC_CUDA(cudaMemsetAsync(g->acc, 0, sizeof(unsigned long long), s));
+    BFC_CUDA(cudaMemsetAsync(g->cursors, 0, 8 * sizeof(int) + sizeof(unsigned long long), s));   // and acc
     const int grid = g->grid;
     // 32-bit adjacency positions whenever G* has fewer than 2^31 slots
     const bool narrow_pos = 2 * g->m <= 0x7fffffffll && !g->opt.wide_positions;

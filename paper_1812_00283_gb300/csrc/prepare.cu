@@ -32,23 +32,21 @@ __device__ __forceinline__ bool aborted(const int *guard) {
 }
 
 // ----- validation (always on: every later index depends on it) -------------
-__global__ void k_check_offsets(const int32_t *__restrict__ off, int32_t r, int64_t m, int *err) {
+// (and the U degrees, which are only read once the offsets have passed)
+__global__ void k_check_offsets(const int32_t *__restrict__ off, int32_t r, int64_t m, int32_t *deg_u, int *err) {
     int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (u > r) return;
-    if (u == 0 && off[0] != 0) atomicOr(err, kErrBadOffsets);
-    if (u < r && off[u + 1] < off[u]) atomicOr(err, kErrBadOffsets);
-    if (u == r && (int64_t)off[r] != m) atomicOr(err, kErrBadOffsets);
+    const int32_t o = off[u];
+    if (u == 0 && o != 0) atomicOr(err, kErrBadOffsets);
+    if (u < r) {
+        const int32_t e = off[u + 1];
+        if (e < o) atomicOr(err, kErrBadOffsets);
+        deg_u[u] = e - o;
+    }
+    if (u == r && (int64_t)o != m) atomicOr(err, kErrBadOffsets);
 }
 
 // ----- a1: degrees -----------------------------------------------------------
-__global__ void k_deg_u(const int32_t *__restrict__ off, int32_t r, int32_t *deg_u,
-    const int *guard = nullptr) {
-    if (aborted(guard)) return;
-    int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (u >= r) return;
-    deg_u[u] = off[u + 1] - off[u];
-}
-
 // L degrees; an id outside [0, l) is reported and counted nowhere
 __global__ void k_deg_l(const int32_t *__restrict__ adj, int64_t m, int32_t l, int32_t *deg_l, int *err) {
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < m;
@@ -60,46 +58,12 @@ __global__ void k_deg_l(const int32_t *__restrict__ adj, int64_t m, int32_t l, i
 }
 
 // ----- a2: priority ranks ----------------------------------------------------
-// keys = degree, values = vertex id (ascending), so a stable sort by degree
-// orders each layer by (deg, id): Definition 3 restricted to one layer.
-__global__ void k_iota_keys(const int32_t *__restrict__ deg, int32_t n, uint64_t *keys,
-                            int32_t *vals) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    keys[i] = (uint64_t)(uint32_t)deg[i];
-    vals[i] = (int32_t)i;
-}
-
-// batch of graphs: rank graph-major (graph id above the degree bits), so each
-// graph's vertices keep Definition 3's order among themselves and occupy the
-// contiguous rank range [start[g], start[g+1]) of their layer
-__global__ void k_iota_keys_batch(const int32_t *__restrict__ deg, int32_t n,
-                                  const int32_t *__restrict__ start, int32_t num_graphs, int bdeg,
-                                  uint64_t *keys, int32_t *vals,
-    const int *guard = nullptr) {
-    if (aborted(guard)) return;
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int32_t lo = 0, hi = num_graphs;
-    while (hi - lo > 1) {
-        const int32_t mid = (lo + hi) >> 1;
-        if (start[mid] <= (int32_t)i) lo = mid; else hi = mid;
-    }
-    keys[i] = ((uint64_t)lo << bdeg) | (uint64_t)(uint32_t)deg[i];
-    vals[i] = (int32_t)i;
-}
-
-// rank[order[i]] = i; degree of G* vertex (base + i) = sorted key
-__global__ void k_ranks(const uint64_t *__restrict__ sorted_deg, const int32_t *__restrict__ order,
-                        int32_t n, int32_t *rank, int32_t *deg_star, int32_t base, uint64_t deg_mask,
-    const int *guard = nullptr) {
-    if (aborted(guard)) return;
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    rank[order[i]] = (int32_t)i;
-    deg_star[base + i] = (int32_t)(sorted_deg[i] & deg_mask);   // low bits: the degree
-}
-
+// Both layers in one sort: the key is (layer, graph of a batch, degree), the
+// value the global id (L vertex v -> v, U vertex u -> l + u, ascending before the
+// sort), so the stable sort's positions are the ids of G*: L first, each layer
+// (each graph's part of it) by (degree, id), Definition 3's order.  A degree
+// that does not fit its bits belongs to a row with duplicate edges; it is cut
+// off in the key only.
 __device__ __forceinline__ int32_t graph_of(const int32_t *start, int32_t num_graphs, int32_t id) {
     int32_t lo = 0, hi = num_graphs;   // last g with start[g] <= id
     while (hi - lo > 1) {
@@ -107,6 +71,46 @@ __device__ __forceinline__ int32_t graph_of(const int32_t *start, int32_t num_gr
         if (start[mid] <= id) lo = mid; else hi = mid;
     }
     return lo;
+}
+
+__global__ void k_rank_keys(const int32_t *__restrict__ deg_l, const int32_t *__restrict__ deg_u, int32_t l,
+                            int32_t n, const int32_t *__restrict__ gl, const int32_t *__restrict__ gu,
+                            int32_t num_graphs, int bdeg, int blayer, uint64_t *keys,
+    const int *guard = nullptr) {
+    if (aborted(guard)) return;
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const bool in_u = i >= l;
+    const int32_t id = in_u ? (int32_t)(i - l) : (int32_t)i;
+    const uint64_t d = (uint64_t)(uint32_t)(in_u ? deg_u[id] : deg_l[id]), top = (1ull << bdeg) - 1;
+    uint64_t key = (d < top ? d : top) | ((uint64_t)(in_u ? 1 : 0) << blayer);
+    if (gl) key |= (uint64_t)graph_of(in_u ? gu : gl, num_graphs, id) << bdeg;
+    keys[i] = key;
+}
+
+// ranks, the degree of every G* vertex (32 bits, and 64 for the offsets' scan)
+// and the largest degree of each layer: top[0] L, top[1] U
+__global__ void __launch_bounds__(kT) k_ranks(const int32_t *__restrict__ order, const int32_t *__restrict__ deg_l,
+                                              const int32_t *__restrict__ deg_u, int32_t l, int32_t n,
+                                              int32_t *rank_l, int32_t *rank_u, int32_t *deg_star, int64_t *deg64,
+                                              unsigned long long *top,
+    const int *guard = nullptr) {
+    if (aborted(guard)) return;
+    __shared__ int32_t best[2];
+    if (threadIdx.x < 2) best[threadIdx.x] = 0;
+    __syncthreads();
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) {
+        const int32_t id = order[i];
+        const bool in_u = id >= l;
+        const int32_t d = in_u ? deg_u[id - l] : deg_l[id];
+        if (in_u) rank_u[id - l] = (int32_t)(i - l); else rank_l[id] = (int32_t)i;
+        deg_star[i] = d;
+        deg64[i] = d;
+        if (d > best[in_u]) atomicMax(&best[in_u], d);
+    }
+    __syncthreads();
+    if (threadIdx.x < 2 && best[threadIdx.x] > 0) atomicMax(top + threadIdx.x, (unsigned long long)best[threadIdx.x]);
 }
 
 // ----- a3: projection + sorted adjacency -------------------------------------
@@ -160,20 +164,29 @@ struct URowOut {
 // four rows of at most 8 neighbours at a time, then the longer ones one by one.
 __global__ void k_u_rows_warp(const int32_t *__restrict__ off_u, const int32_t *__restrict__ adj_u,
                               const int32_t *__restrict__ rank_u, const int32_t *__restrict__ rank_l,
-                              int32_t r, URowOut o,
+                              int32_t r, const int32_t *__restrict__ gl, const int32_t *__restrict__ gu,
+                              int32_t num_graphs, URowOut o,
     const int *guard = nullptr) {
     if (aborted(guard)) return;
     const int lane = threadIdx.x & 31;
     const int g = lane >> 3, j = lane & 7;
+    bool cross = false;   // a batch: an L rank outside the row's graph
     const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t u0 = w0 * 32; u0 < r; u0 += nw * 32) {
         const int64_t u = u0 + lane;
-        int32_t b = 0, d = 0, ru = 0;
+        int32_t b = 0, d = 0, ru = 0, lo = 0, hi = o.l;
         if (u < r) {
             b = off_u[u];
             d = off_u[u + 1] - b;
-            if (d > 0 && d <= kRowWarpMax) ru = rank_u[u];
+            if (d > 0 && d <= kRowWarpMax) {
+                ru = rank_u[u];
+                if (gl) {
+                    const int32_t gg = graph_of(gu, num_graphs, (int32_t)u);
+                    lo = gl[gg];
+                    hi = gl[gg + 1];
+                }
+            }
         }
         uint32_t left = __ballot_sync(0xffffffffu, d > 0 && d <= 8);
         while (left) {   // four short rows, one per group of eight lanes
@@ -185,7 +198,9 @@ __global__ void k_u_rows_warp(const int32_t *__restrict__ off_u, const int32_t *
             const int32_t bk = __shfl_sync(0xffffffffu, b, src & 31), rk = __shfl_sync(0xffffffffu, ru, src & 31);
             int32_t dk = __shfl_sync(0xffffffffu, d, src & 31);
             if (src > 31) dk = 0;
+            const int32_t lok = __shfl_sync(0xffffffffu, lo, src & 31), hik = __shfl_sync(0xffffffffu, hi, src & 31);
             const int32_t rl = j < dk ? rank_l[adj_u[bk + j]] : 0x7fffffff;
+            cross |= j < dk && (rl < lok || rl >= hik);
             int pos = 0;
             bool dup = false;
 #pragma unroll
@@ -206,7 +221,9 @@ __global__ void k_u_rows_warp(const int32_t *__restrict__ off_u, const int32_t *
             left &= left - 1;
             const int32_t bk = __shfl_sync(0xffffffffu, b, src), dk = __shfl_sync(0xffffffffu, d, src);
             const int32_t rk = __shfl_sync(0xffffffffu, ru, src);
+            const int32_t lok = __shfl_sync(0xffffffffu, lo, src), hik = __shfl_sync(0xffffffffu, hi, src);
             const int32_t rl = lane < dk ? rank_l[adj_u[bk + lane]] : 0x7fffffff;
+            cross |= lane < dk && (rl < lok || rl >= hik);
             int pos = 0;
             bool dup = false;
             for (int k = 0; k < dk; ++k) {
@@ -220,6 +237,7 @@ __global__ void k_u_rows_warp(const int32_t *__restrict__ off_u, const int32_t *
             }
         }
     }
+    if (cross) atomicOr(o.err, kErrBadId);
 }
 
 // Ascending bitonic sort of 32 * R keys held by a warp, key lane * R + r in
@@ -259,12 +277,15 @@ __device__ __forceinline__ void warp_sort(uint32_t (&key)[R], int lane) {
 // the sorted order back into consecutive lanes for the stores
 template <int R>
 __device__ __forceinline__ void warp_sort_row(const int32_t *adj_u, const int32_t *rank_l, int32_t b, int32_t d,
-                                              int32_t ru, int32_t base, uint32_t *buf, int lane, const URowOut &o) {
+                                              int32_t ru, int32_t base, int32_t len, uint32_t *buf, int lane,
+                                              const URowOut &o) {
     uint32_t key[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const int i = r * 32 + lane;
-        key[r] = i < d ? ((uint32_t)(rank_l[adj_u[b + i]] - base) << 8) | (uint32_t)i : 0xffffffffu;
+        const uint32_t k = i < d ? (uint32_t)(rank_l[adj_u[b + i]] - base) : 0xffffffu;
+        if (i < d && k >= (uint32_t)len) atomicOr(o.err, kErrBadId);   // an edge to another graph of the batch
+        key[r] = i < d ? (k << 8) | (uint32_t)i : 0xffffffffu;
     }
     warp_sort<R>(key, lane);
     __syncwarp();
@@ -301,10 +322,15 @@ __global__ void __launch_bounds__(kRowCtaThreads) k_u_rows_warp_reg(
     for (int64_t i0 = w0; i0 < nrows; i0 += nw) {
         const int32_t u = rows[i0];
         const int32_t b = off_u[u], d = off_u[u + 1] - b, ru = rank_u[u];
-        const int32_t base = gl ? gl[graph_of(gu, num_graphs, u)] : 0;
-        if (d <= 64) warp_sort_row<2>(adj_u, rank_l, b, d, ru, base, wb, lane, o);
-        else if (d <= 128) warp_sort_row<4>(adj_u, rank_l, b, d, ru, base, wb, lane, o);
-        else warp_sort_row<8>(adj_u, rank_l, b, d, ru, base, wb, lane, o);
+        int32_t base = 0, len = o.l;
+        if (gl) {
+            const int32_t g = graph_of(gu, num_graphs, u);
+            base = gl[g];
+            len = gl[g + 1] - base;
+        }
+        if (d <= 64) warp_sort_row<2>(adj_u, rank_l, b, d, ru, base, len, wb, lane, o);
+        else if (d <= 128) warp_sort_row<4>(adj_u, rank_l, b, d, ru, base, len, wb, lane, o);
+        else warp_sort_row<8>(adj_u, rank_l, b, d, ru, base, len, wb, lane, o);
     }
 }
 
@@ -396,10 +422,11 @@ __global__ void __launch_bounds__(kRowCtaThreads) k_u_rows_cta(
 // lists of the rows of every tier above 32 neighbours (any order: every row
 // is written to its own slots); one atomic per warp and list.  lists[t * r ...]:
 // tier 0 warp sort, 1 and 2 bitmap, 3 CTA sort, 4 radix.  `range`: the L ranks of
-// a single graph (a batch's row: its graph's); bitmaps only where `bitmaps`.
+// a single graph (a batch's row: its graph's); bitmaps only where `bitmaps`, and
+// tier 2 only where `wide_tier`.
 __global__ void k_row_tiers(const int32_t *__restrict__ off_u, int32_t r, int32_t range,
                             const int32_t *__restrict__ gu, const int32_t *__restrict__ gl, int32_t num_graphs,
-                            int bitmaps, int32_t *lists, int32_t *counts,
+                            int bitmaps, int wide_tier, int32_t *lists, int32_t *counts,
     const int *guard = nullptr) {
     if (aborted(guard)) return;
     const int lane = threadIdx.x & 31;
@@ -414,7 +441,7 @@ __global__ void k_row_tiers(const int32_t *__restrict__ off_u, int32_t r, int32_
                 const int32_t g = graph_of(gu, num_graphs, (int32_t)u);
                 len = gl[g + 1] - gl[g];
             }
-            tier = (bitmaps && len <= kRowBitmapMax) ? (d <= kRowCtaMax ? 1 : 2) : (d <= kRowCtaMax ? 3 : 4);
+            tier = (bitmaps && len <= kRowBitmapMax) ? (d <= kRowCtaMax || !wide_tier ? 1 : 2) : (d <= kRowCtaMax ? 3 : 4);
         }
         if (!__any_sync(0xffffffffu, tier >= 0)) continue;
 #pragma unroll
@@ -457,7 +484,6 @@ __global__ void __launch_bounds__(kThreads) k_u_rows_bitmap(
             base = gl[g];   // the graph's L ranks: [gl[g], gl[g + 1])
             len = gl[g + 1] - base;
         }
-        // every edge stays inside its graph (checked), so 0 <= rank - base < len
         const int quads = (len + 127) / 128;   // 16-byte units of the bitmap
         uint4 *const q4 = reinterpret_cast<uint4 *>(bm_smem);
         int32_t *const qpre = reinterpret_cast<int32_t *>(q4 + quads);
@@ -467,6 +493,10 @@ __global__ void __launch_bounds__(kThreads) k_u_rows_bitmap(
 #pragma unroll 4
         for (int32_t i = tid; i < d; i += kThreads) {
             const int32_t rl = rank_l[adj_u[b + i]], k = rl - base;
+            if ((uint32_t)k >= (uint32_t)len) {   // an edge to another graph of the batch
+                atomicOr(o.err, kErrBadId);
+                continue;
+            }
             const uint32_t bit = 1u << (k & 31);
             if (atomicOr(&bm_smem[k >> 5], bit) & bit) {
                 if (o.check_dup) atomicOr(o.err, kErrDuplicate);
@@ -498,6 +528,7 @@ __global__ void __launch_bounds__(kThreads) k_u_rows_bitmap(
 #pragma unroll 4
         for (int32_t i = tid; i < d; i += kThreads) {
             const int32_t rl = rank_l[adj_u[b + i]], k = rl - base;
+            if ((uint32_t)k >= (uint32_t)len) continue;
             const uint4 q = q4[k >> 7];
             const int w = (k >> 5) & 3;
             const uint32_t mine = w == 0 ? q.x : (w == 1 ? q.y : (w == 2 ? q.z : q.w));
@@ -590,13 +621,6 @@ __global__ void k_emit_l_side(const uint64_t *__restrict__ keys2, const int32_t 
     }
 }
 
-__global__ void k_deg_to_i64(const int32_t *__restrict__ d, int32_t n, int64_t *out,
-    const int *guard = nullptr) {
-    if (aborted(guard)) return;
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = d[i];
-}
-
 // ----- a4: orientation cut and per-start work ---------------------------------
 // cut[x] = |{y in N(x): p(y) < p(x)}|.  Lists are ascending in priority and
 // the degree of G* ids is non-decreasing inside a layer, so the cut is a
@@ -626,7 +650,8 @@ __global__ void k_cut(const int64_t *__restrict__ off, const int32_t *__restrict
 // suffix that starts after both x (x is in N(v)) and v's cut.
 __global__ void k_slen(const int64_t *__restrict__ off, const int32_t *__restrict__ adj,
                        const int32_t *__restrict__ rows, const int32_t *__restrict__ cut,
-                       int64_t slots, int32_t *slen, int64_t *sbeg) {
+                       int64_t slots, int32_t *slen, int64_t *sbeg, const int *guard) {
+    if (aborted(guard)) return;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < slots;
          e += (int64_t)gridDim.x * blockDim.x) {
         const int32_t x = rows[e];
@@ -790,41 +815,85 @@ __device__ __forceinline__ bool forced_dense(int32_t x, int32_t l, int32_t core_
     return w > 0 && (x >= l ? x >= core_lo_u : x >= core_lo_l);
 }
 
-__global__ void k_sched_keys(const uint64_t *__restrict__ work, int32_t n, uint64_t maxw,
-                             int32_t l, int32_t core_lo_u, int32_t core_lo_l, uint64_t *keys,
-                             int32_t *vals,
+// Bins of a6: 0 dense (work > hash_max), 1 CTA hash (team_max < work <=
+// hash_max), 2 team (warp_max < work <= team_max), 3 warp (0 < work <= warp_max).
+struct BinBounds {
+    uint64_t warp_max, team_max, hash_max;
+    int32_t l, core_lo_u, core_lo_l;
+    __device__ __forceinline__ int of(int32_t x, uint64_t w) const {
+        if (w > hash_max || forced_dense(x, l, core_lo_u, core_lo_l, w)) return 0;
+        return w > team_max ? 1 : (w > warp_max ? 2 : (w > 0 ? 3 : 4));
+    }
+};
+
+// The starts of each bin: counts[b], the warp bin's starts in `warp_items` and
+// the others' in `heavy` (in no order; only the heavy ones, a few per cent of
+// the starts with work, are then sorted).  A CTA takes 2,048 starts and reserves
+// their room with one addition per list.
+constexpr int kBinTile = 8 * kT;
+__global__ void __launch_bounds__(kT) k_bin_starts(const uint64_t *__restrict__ work, int32_t n, BinBounds bb,
+                                                   unsigned long long *counts, int32_t *heavy, int32_t *warp_items,
     const int *guard = nullptr) {
     if (aborted(guard)) return;
-    int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= n) return;
-    // ascending key = descending work; zero work last; forced dense starts first
-    keys[x] = forced_dense((int32_t)x, l, core_lo_u, core_lo_l, work[x]) ? 0 : maxw - work[x];
-    vals[x] = (int32_t)x;
+    __shared__ int32_t cnt[4], at_heavy, at_warp;
+    const int lane = threadIdx.x & 31;
+    const uint32_t lt = (1u << lane) - 1u;
+    for (int64_t x0 = (int64_t)blockIdx.x * kBinTile; x0 < n; x0 += (int64_t)gridDim.x * kBinTile) {
+        if (threadIdx.x < 4) cnt[threadIdx.x] = 0;
+        __syncthreads();
+        int bin[8], place[8];   // place: among the tile's heavy, or warp, starts
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int64_t x = x0 + i * kT + threadIdx.x;
+            bin[i] = x < n ? bb.of((int32_t)x, work[x]) : 4;
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                const uint32_t m = __ballot_sync(0xffffffffu, bin[i] == b);
+                if (b == 3) {
+                    int o = 0;
+                    if (lane == 0 && m) o = atomicAdd(&cnt[3], __popc(m));
+                    o = __shfl_sync(0xffffffffu, o, 0);
+                    if (bin[i] == 3) place[i] = o + __popc(m & lt);
+                } else if (lane == 0 && m) {
+                    atomicAdd(&cnt[b], __popc(m));
+                }
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            const int32_t h = cnt[0] + cnt[1] + cnt[2];
+            at_heavy = h ? (int32_t)atomicAdd(counts + 4, (unsigned long long)h) : 0;
+            at_warp = cnt[3] ? (int32_t)atomicAdd(counts + 3, (unsigned long long)cnt[3]) : 0;
+            for (int b = 0; b < 3; ++b)
+                if (cnt[b]) atomicAdd(counts + b, (unsigned long long)cnt[b]);
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) cnt[0] = 0;   // now the place among the heavy ones
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int32_t x = (int32_t)(x0 + i * kT + threadIdx.x);
+            const uint32_t m = __ballot_sync(0xffffffffu, bin[i] < 3);
+            int o = 0;
+            if (lane == 0 && m) o = atomicAdd(&cnt[0], __popc(m));
+            o = __shfl_sync(0xffffffffu, o, 0);
+            if (bin[i] < 3) heavy[at_heavy + o + __popc(m & lt)] = x;
+            if (bin[i] == 3) warp_items[at_warp + place[i]] = x;
+        }
+        __syncthreads();
+    }
 }
 
-// counts[0] = dense starts, [1] = hash starts, [2] = warp starts
-// Bins of a6: [0] dense (work > hash_max), [1] CTA hash (team_max < work <=
-// hash_max), [2] team (warp_max < work <= team_max), [3] warp (0 < work <= warp_max).
-__global__ void k_classify(const uint64_t *__restrict__ work, int32_t n, uint64_t warp_max,
-                           uint64_t team_max, uint64_t hash_max, int32_t l, int32_t core_lo_u,
-                           int32_t core_lo_l, unsigned long long *counts,
-    const int *guard = nullptr) {
-    if (aborted(guard)) return;
-    unsigned long long c[4] = {0, 0, 0, 0};
-    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n;
-         x += (int64_t)gridDim.x * blockDim.x) {
-        uint64_t w = work[x];
-        if (w > hash_max || forced_dense((int32_t)x, l, core_lo_u, core_lo_l, w)) ++c[0];
-        else if (w > team_max) ++c[1];
-        else if (w > warp_max) ++c[2];
-        else if (w > 0) ++c[3];
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-#pragma unroll
-        for (int d = 16; d > 0; d >>= 1) c[k] += __shfl_xor_sync(0xffffffffu, c[k], d);
-        if ((threadIdx.x & 31) == 0 && c[k]) atomicAdd(&counts[k], c[k]);
-    }
+// ascending key = descending work; forced dense starts first
+__global__ void k_sched_keys(const uint64_t *__restrict__ work, const int32_t *__restrict__ heavy, int64_t n_heavy,
+                             uint64_t maxw, int32_t l, int32_t core_lo_u, int32_t core_lo_l, uint64_t *keys) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n_heavy) return;
+    const int32_t x = heavy[i];
+    keys[i] = forced_dense(x, l, core_lo_u, core_lo_l, work[x]) ? 0 : maxw - work[x];
 }
 
 // the dense chunks of start x (dense_chunk_end from offset 0 up); with `out`,
@@ -863,26 +932,26 @@ __device__ __forceinline__ int2 hash_or_dense_item(int32_t x, int32_t l, int32_t
     return make_int2(x, dense_chunk_end(0, x - lb, cut, off, lb, &bits) == x - lb ? 0 : -1);
 }
 
-// starts in descending work order: dense (chunked), CTA hash, team, warp
+// starts in descending work order: dense (chunked; nch_scan null: one chunk
+// each), CTA hash, team
 __global__ void k_emit_items(const int32_t *__restrict__ order, int64_t n_dense, int64_t n_hash,
-                             int64_t n_team, int64_t n_warp, const int64_t *__restrict__ nch_scan,
+                             int64_t n_team, const int64_t *__restrict__ nch_scan,
                              int32_t l, const int32_t *__restrict__ cut, const int64_t *__restrict__ off,
                              const int32_t *__restrict__ vbase, int ends_above, int2 *cta_items,
-                             int32_t *team_items, int32_t *warp_items) {
-    const int64_t total_dense = nch_scan[n_dense];
-    const int64_t all = n_dense + n_hash + n_team + n_warp;
+                             int32_t *team_items) {
+    const int64_t total_dense = nch_scan ? nch_scan[n_dense] : n_dense;
+    const int64_t all = n_dense + n_hash + n_team;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < all;
          i += (int64_t)gridDim.x * blockDim.x) {
         int32_t x = order[i];
         if (i < n_dense) {
-            dense_chunks(x, l, cut[x], off, vbase, cta_items + nch_scan[i]);
+            if (nch_scan) dense_chunks(x, l, cut[x], off, vbase, cta_items + nch_scan[i]);
+            else cta_items[i] = make_int2(x, 0);
         } else if (i < n_dense + n_hash) {
             cta_items[total_dense + (i - n_dense)] =
                 ends_above ? make_int2(x, -1) : hash_or_dense_item(x, l, cut[x], off, vbase);
-        } else if (i < n_dense + n_hash + n_team) {
-            team_items[i - n_dense - n_hash] = x;
         } else {
-            warp_items[i - n_dense - n_hash - n_team] = x;
+            team_items[i - n_dense - n_hash] = x;
         }
     }
 }
@@ -1022,9 +1091,11 @@ __global__ void k_check_starts(const int32_t *__restrict__ start, int32_t num_gr
     }
 }
 
-// every edge must join a U and an L vertex of the same graph: one lookup of
-// the row's graph, then its L ids against that graph's range.  A warp takes 32
-// rows (lanes on their own up to 24 neighbours, the warp together above).
+// Every edge must join a U and an L vertex of the same graph.  The row kernels
+// that know their row's graph check its L ranks as they read them; this pass is
+// for the tiers that do not (ranges above 524,288 ranks, validate = 0): one
+// lookup of the row's graph, then its L ids against that graph's range.  A warp
+// takes 32 rows (lanes on their own up to 24 neighbours, the warp together above).
 __global__ void k_check_batch_rows(const int32_t *__restrict__ off, const int32_t *__restrict__ adj, int32_t r,
                                    const int32_t *__restrict__ gu, const int32_t *__restrict__ gl,
                                    int32_t num_graphs, int *err,
@@ -1093,12 +1164,47 @@ __global__ void k_rows_from_off(const int64_t *__restrict__ off, int32_t n, int3
 
 }  // namespace
 
+// the bin bounds that a schedule's three limits stand for
+static BinBounds bin_bounds(const Graph *g, int32_t warp_max_work, int32_t team_max_work, int32_t hash_max_work) {
+    const bool vpp = g->opt.orientation == 1;
+    BinBounds bb;
+    bb.warp_max = (uint64_t)warp_max_work;
+    // Algorithm 3: ends concentrate on few high-priority vertices, so no start
+    // gets dense counters up front; every start beyond the warp bin gets a
+    // team or CTA hash table and one whose table fills up is re-queued
+    bb.hash_max = vpp ? ~0ull : (uint64_t)hash_max_work;
+    const int32_t team_req = team_max_work >= 0 ? team_max_work : (vpp ? kTeamMaxWork : kTeamFitWork);
+    bb.team_max = std::max<uint64_t>((uint64_t)team_req, bb.warp_max);
+    if (!vpp) bb.team_max = std::min<uint64_t>(bb.team_max, bb.hash_max);
+    if (vpp && hash_max_work == 0) bb.team_max = bb.warp_max;   // all of them to the dense pass
+    // without a core the bounds lie past every id
+    bb.l = g->l;
+    bb.core_lo_u = g->core_u > 0 ? g->core_lo_u : g->n;
+    bb.core_lo_l = g->core_l > 0 ? g->core_lo_l : g->n;
+    return bb;
+}
+
+// Starts the binning of all starts on s: counts[0..4] (zeroed here) = dense,
+// hash, team, warp, and all but the warp bin together; g->warp_items is filled.
+static int bin_starts(Graph *g, cudaStream_t s, const BinBounds &bb, unsigned long long *counts, int32_t *heavy,
+                      const int *guard) {
+    BFC_CUDA(cudaMemsetAsync(counts, 0, 5 * sizeof(unsigned long long), s));
+    if (g->n == 0) return BFC_OK;
+    k_bin_starts<<<(unsigned)std::min<int64_t>(((int64_t)g->n + kBinTile - 1) / kBinTile, 152 * 8), kT, 0, s>>>(
+        g->work, g->n, bb, counts, heavy, g->warp_items, guard); note_launch();
+    BFC_CUDA(cudaGetLastError());
+    return BFC_OK;
+}
+
 // Step a5: order the starts by descending exact work and split them into the
 // warp, CTA-hash and CTA-dense bins (dense starts into end-range chunks);
 // builds the chunk-boundary table when a dense start has several chunks.
 // `rows_star` (slot -> vertex of G*) may be null; it is rebuilt when needed.
+// hc[0..4] and `heavy` are bin_starts' results with the bounds bb.  Only reads
+// memory of the library.
 static int schedule_graph(Graph *g, cudaStream_t s, int32_t warp_max_work, int32_t team_max_work,
-                          int32_t hash_max_work, const int32_t *rows_star) {
+                          int32_t hash_max_work, const int32_t *rows_star, const BinBounds &bb,
+                          const unsigned long long *hc, int32_t *heavy) {
     const int32_t r = g->r, l = g->l, n = g->n;
     const int64_t m = g->m;
     const bool vpp = g->opt.orientation == 1;
@@ -1113,63 +1219,50 @@ static int schedule_graph(Graph *g, cudaStream_t s, int32_t warp_max_work, int32
             return BFC_ERR_OUT_OF_MEMORY;                                             \
         }                                                                             \
     } while (0)
-    const uint64_t warp_max = (uint64_t)warp_max_work;
-    // Algorithm 3: ends concentrate on few high-priority vertices, so no start
-    // gets dense counters up front; every start beyond the warp bin gets a
-    // team or CTA hash table and one whose table fills up is re-queued
-    const uint64_t hash_max = vpp ? ~0ull : (uint64_t)hash_max_work;
-    const int32_t team_req = team_max_work >= 0 ? team_max_work : (vpp ? kTeamMaxWork : kTeamFitWork);
-    uint64_t team_max = std::max<uint64_t>((uint64_t)team_req, warp_max);
-    if (!vpp) team_max = std::min<uint64_t>(team_max, hash_max);
-    if (vpp && hash_max_work == 0) team_max = warp_max;   // all of them to the dense pass
-    const uint64_t maxw = g->info.max_start_work;
+    const uint64_t maxw = g->info.max_start_work, team_max = bb.team_max;
     int64_t n_dense = 0, n_hash = 0, n_team = 0, n_warp = 0, n_items = 0, h_dense_items = 0;
     if (n > 0 && g->info.wedges > 0) {
-        const int64_t nn = (int64_t)n + 1;
-        uint64_t *k0, *k1;
-        int32_t *v0, *v1;
-        uint32_t *hist, *hist_tmp;
-        int64_t *scan64_tmp, *nch;
-        unsigned long long *red;
-        GET(tmp, k0, nn); GET(tmp, k1, nn); GET(tmp, v0, nn); GET(tmp, v1, nn);
-        GET(tmp, hist, radix_hist_elems(n));
-        GET(tmp, hist_tmp, scan_tmp_elems<uint32_t>((int64_t)radix_hist_elems(n)));
-        GET(tmp, scan64_tmp, scan_tmp_elems<int64_t>(nn));
-        GET(tmp, nch, nn);
-        GET(tmp, red, 4);
-        BFC_CUDA(cudaMemsetAsync(red, 0, 4 * sizeof(unsigned long long), s));
-        int which = 0;
-        // without a core the bounds lie past every id
-        const int32_t clo_u = g->core_u > 0 ? g->core_lo_u : n, clo_l = g->core_l > 0 ? g->core_lo_l : n;
-        k_sched_keys<<<blocks_for(n), kT, 0, s>>>(g->work, n, maxw, l, clo_u, clo_l, k0, v0); note_launch();
-        BFC_CUDA(cudaGetLastError());
-        BFC_CUDA(radix_sort_pairs(k0, v0, k1, v1, n, 0, bits_for(maxw), hist, hist_tmp, s, &which));
-        const int32_t *order = which ? v1 : v0;
-        k_classify<<<grid_stride_blocks(n), kT, 0, s>>>(g->work, n, warp_max, team_max, hash_max, l, clo_u,
-                                                        clo_l, red); note_launch();
-        BFC_CUDA(cudaGetLastError());
-        unsigned long long hc[4];
-        BFC_CUDA(cudaMemcpyAsync(hc, red, 4 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
-        BFC_CUDA(cudaStreamSynchronize(s));
         n_dense = (int64_t)hc[0]; n_hash = (int64_t)hc[1]; n_team = (int64_t)hc[2]; n_warp = (int64_t)hc[3];
-        if (n_dense > 0) {
+        const int64_t n_heavy = n_dense + n_hash + n_team;
+        uint64_t *k0 = nullptr, *k1 = nullptr;
+        int32_t *v1 = nullptr;
+        uint32_t *hist, *hist_tmp;
+        int64_t *scan64_tmp = nullptr, *nch = nullptr;
+        const int32_t *order = heavy;
+        if (n_heavy > 0) {
+            GET(tmp, k0, n_heavy + 1); GET(tmp, k1, n_heavy + 1); GET(tmp, v1, n_heavy);
+            GET(tmp, hist, radix_hist_elems(n_heavy));
+            GET(tmp, hist_tmp, scan_tmp_elems<uint32_t>((int64_t)radix_hist_elems(n_heavy)));
+            int which = 0;
+            k_sched_keys<<<blocks_for(n_heavy), kT, 0, s>>>(g->work, heavy, n_heavy, maxw, l, bb.core_lo_u,
+                                                            bb.core_lo_l, k0); note_launch();
+            BFC_CUDA(cudaGetLastError());
+            BFC_CUDA(radix_sort_pairs(k0, heavy, k1, v1, n_heavy, 0, bits_for(maxw), hist, hist_tmp, s, &which));
+            order = which ? v1 : heavy;
+            GET(tmp, scan64_tmp, scan_tmp_elems<int64_t>(std::max<int64_t>(n_dense, n) + 1));
+        }
+        // a layer (a batch's graph's) this small is one chunk of any counters,
+        // or of 16-bit ones where no degree can pass 65,535
+        const bool one_chunk = g->max_range <= kDense32 || (g->max_range <= kDense16 && g->max_range <= (int32_t)kNarrowMaxCut);
+        int64_t *nch_scan = nullptr;
+        h_dense_items = n_dense;
+        if (n_dense > 0 && !one_chunk) {
+            GET(tmp, nch, n_dense + 1);
+            GET(tmp, nch_scan, n_dense + 1);
             k_chunk_counts<<<blocks_for(n_dense), kT, 0, s>>>(order, n_dense, l, g->cut, g->off, g->vbase, nch); note_launch();
             BFC_CUDA(cudaGetLastError());
+            BFC_CUDA(scan_exclusive<int64_t>(nch, nch_scan, n_dense, scan64_tmp, s));
+            BFC_CUDA(cudaMemcpyAsync(&h_dense_items, nch_scan + n_dense, sizeof(int64_t),
+                                     cudaMemcpyDeviceToHost, s));
+            BFC_CUDA(cudaStreamSynchronize(s));
         }
-        // the sorted keys are no longer needed; the other key buffer holds the scan
-        int64_t *nch_scan = reinterpret_cast<int64_t *>(which ? k0 : k1);
-        BFC_CUDA(scan_exclusive<int64_t>(nch, nch_scan, n_dense, scan64_tmp, s));
-        BFC_CUDA(cudaMemcpyAsync(&h_dense_items, nch_scan + n_dense, sizeof(int64_t),
-                                 cudaMemcpyDeviceToHost, s));
-        BFC_CUDA(cudaStreamSynchronize(s));
         n_items = h_dense_items + n_hash;
         GET(g->mem, g->cta_items, std::max<int64_t>(n_items, 1));
         GET(g->mem, g->team_items, std::max<int64_t>(n_team, 1));
-        GET(g->mem, g->warp_items, std::max<int64_t>(n_warp, 1));
-        if (n_dense + n_hash + n_team + n_warp > 0) {
-            k_emit_items<<<grid_stride_blocks(n_dense + n_hash + n_team + n_warp), kT, 0, s>>>(
-                order, n_dense, n_hash, n_team, n_warp, nch_scan, l, g->cut, g->off, g->vbase, vpp ? 1 : 0, g->cta_items,
-                g->team_items, g->warp_items); note_launch();
+        if (n_heavy > 0) {
+            k_emit_items<<<grid_stride_blocks(n_heavy), kT, 0, s>>>(
+                order, n_dense, n_hash, n_team, nch_scan, l, g->cut, g->off, g->vbase, vpp ? 1 : 0, g->cta_items,
+                g->team_items); note_launch();
             BFC_CUDA(cudaGetLastError());
         }
         // chunk boundaries of every list, so dense items read them instead of searching
@@ -1239,7 +1332,6 @@ static int schedule_graph(Graph *g, cudaStream_t s, int32_t warp_max_work, int32
     } else {
         GET(g->mem, g->cta_items, 1);
         GET(g->mem, g->team_items, 1);
-        GET(g->mem, g->warp_items, 1);
     }
     g->n_cta_items = n_items;
     g->n_team_items = n_team;
@@ -1270,7 +1362,6 @@ static int schedule_graph(Graph *g, cudaStream_t s, int32_t warp_max_work, int32
     g->opt.warp_max_work = warp_max_work;
     g->opt.team_max_work = team_max_work;
     g->opt.hash_max_work = hash_max_work;
-    BFC_CUDA(cudaStreamSynchronize(s));
 #undef GET
     return BFC_OK;
 }
@@ -1280,13 +1371,60 @@ int rebin_graph(Graph *g, cudaStream_t s, int32_t warp_max_work, int32_t team_ma
     g->mem.stream = s;
     g->mem.drop(g->cta_items);
     g->mem.drop(g->team_items);
-    g->mem.drop(g->warp_items);
     g->cta_items = nullptr;
     g->team_items = nullptr;
-    g->warp_items = nullptr;
-    int rc = schedule_graph(g, s, warp_max_work, team_max_work, hash_max_work, nullptr);
+    Allocs tmp;
+    tmp.stream = s;
+    struct TmpGuard { Allocs *a; ~TmpGuard() { a->release(); } } guard{&tmp};
+    int32_t *heavy;
+    unsigned long long *counts, hc[5] = {0, 0, 0, 0, 0};
+    if (tmp.get(&heavy, (size_t)std::max(g->n, 1)) || tmp.get(&counts, 5)) {
+        set_last_error("device allocation failed: bins");
+        return BFC_ERR_OUT_OF_MEMORY;
+    }
+    const BinBounds bb = bin_bounds(g, warp_max_work, team_max_work, hash_max_work);
+    int rc = bin_starts(g, s, bb, counts, heavy, nullptr);
+    if (rc) return rc;
+    BFC_CUDA(cudaMemcpyAsync(hc, counts, sizeof(hc), cudaMemcpyDeviceToHost, s));
+    BFC_CUDA(cudaStreamSynchronize(s));
+    rc = schedule_graph(g, s, warp_max_work, team_max_work, hash_max_work, nullptr, bb, hc, heavy);
+    if (rc == BFC_OK) BFC_CUDA(cudaStreamSynchronize(s));
     g->info.device_bytes = (int64_t)g->mem.total;
     return rc;
+}
+
+// what an error word says about the caller's arrays (BFC_OK: nothing)
+static int input_error(int err, int32_t num_graphs) {
+    if (err & kErrBadOffsets) { set_last_error("off_u is not a CSR offset array of num_edges entries"); return BFC_ERR_INVALID_GRAPH; }
+    if (err & kErrBadId) {
+        set_last_error(num_graphs > 0 ? "an L id lies outside [0, num_l), or an edge joins vertices of two different "
+                                        "graphs of the batch"
+                                      : "adj_u holds an id outside [0, num_l)");
+        return BFC_ERR_INVALID_GRAPH;
+    }
+    if (err & kErrDuplicate) { set_last_error("duplicate edge"); return BFC_ERR_INVALID_GRAPH; }
+    return BFC_OK;
+}
+
+// Step a2: one sort of both layers' vertices; `max_range` = the largest layer
+// (of one graph), which bounds every degree of a simple graph.
+static int launch_ranks(Graph *g, const int32_t *deg_l, const int32_t *deg_u, const int32_t *gl, const int32_t *gu,
+                        int32_t max_range, uint64_t *k0, int32_t *v0, uint64_t *k1, int32_t *v1, uint32_t *hist,
+                        uint32_t *hist_tmp, int32_t *deg_star, int64_t *deg64, unsigned long long *top,
+                        cudaStream_t s, const int *guard) {
+    const int32_t n = g->n;
+    if (n == 0) return BFC_OK;
+    const int bdeg = bits_for((uint64_t)max_range);
+    const int blayer = bdeg + (g->num_graphs > 0 ? bits_for((uint64_t)(g->num_graphs - 1)) : 0);
+    k_rank_keys<<<blocks_for(n), kT, 0, s>>>(deg_l, deg_u, g->l, n, gl, gu, g->num_graphs, bdeg, blayer, k0, guard); note_launch();
+    BFC_CUDA(cudaGetLastError());
+    int which = 0;
+    BFC_CUDA(radix_sort_pairs(k0, v0, k1, v1, n, 0, blayer + (g->r > 0 && g->l > 0 ? 1 : 0), hist, hist_tmp, s, &which,
+                              true));
+    k_ranks<<<blocks_for(n), kT, 0, s>>>(which ? v1 : v0, deg_l, deg_u, g->l, n, g->rank_l, g->rank_u, deg_star, deg64,
+                                         top, guard); note_launch();
+    BFC_CUDA(cudaGetLastError());
+    return BFC_OK;
 }
 
 // shared memory of a bitmap over `range` L ranks
@@ -1305,20 +1443,22 @@ static int rows_smem_setup(int device) {
 }
 
 // The U side of G*: every tier that needs no size on the host.  `range`: the L
-// ranks of a single graph, or of a batch's largest graph; `max_deg` bounds the
-// row lengths (tiers above it are not launched).
+// ranks of a single graph, or of a batch's largest graph.
 static int launch_u_rows(const int32_t *off_u, const int32_t *adj_u, Graph *g, int32_t range, const int32_t *gu,
-                         const int32_t *gl, int32_t num_graphs, int32_t max_deg, int bitmaps, const URowOut &uo,
+                         const int32_t *gl, int32_t num_graphs, int bitmaps, const URowOut &uo,
                          int32_t *tier_rows, int32_t *tier_n, cudaStream_t s, const int *guard) {
     const int32_t r = g->r;
     const int64_t m = g->m;
     int rc = rows_smem_setup(g->device);
     if (rc) return rc;
-    k_u_rows_warp<<<grid_stride_blocks(r), kT, 0, s>>>(off_u, adj_u, g->rank_u, g->rank_l, r, uo, guard); note_launch();
+    k_u_rows_warp<<<grid_stride_blocks(r), kT, 0, s>>>(off_u, adj_u, g->rank_u, g->rank_l, r, gl, gu,
+                                                       num_graphs, uo, guard); note_launch();
     BFC_CUDA(cudaGetLastError());
-    if (max_deg <= kRowWarpMax || m <= kRowWarpMax) return BFC_OK;
+    if (m <= kRowWarpMax) return BFC_OK;
+    const int wide_tier = range > kRowCtaMax ? 1 : 0;   // a valid row is no longer than the range
     BFC_CUDA(cudaMemsetAsync(tier_n, 0, kRowTiers * sizeof(int32_t), s));
-    k_row_tiers<<<grid_stride_blocks(r), kT, 0, s>>>(off_u, r, range, gu, gl, num_graphs, bitmaps, tier_rows, tier_n,
+    k_row_tiers<<<grid_stride_blocks(r), kT, 0, s>>>(off_u, r, range, gu, gl, num_graphs, bitmaps, wide_tier, tier_rows,
+                                                     tier_n,
                                                      guard); note_launch();
     const unsigned wg = (unsigned)std::min<int64_t>(m / (kRowWarpMax + 1) * 32 / kRowCtaThreads + 1, 152 * 8);
     if (range <= 1 << 24) {
@@ -1328,13 +1468,13 @@ static int launch_u_rows(const int32_t *off_u, const int32_t *adj_u, Graph *g, i
         k_u_rows_warp_sort<<<wg, kRowCtaThreads, 0, s>>>(off_u, adj_u, g->rank_u, g->rank_l, tier_rows, tier_n, uo,
                                                          guard); note_launch();
     }
-    if (bitmaps && max_deg > kRowWarpSortMax && m > kRowWarpSortMax) {
+    if (bitmaps && m > kRowWarpSortMax) {
         k_u_rows_bitmap<kRowCtaThreads>
             <<<(unsigned)std::min<int64_t>(m / kRowWarpSortMax, 152 * 8), kRowCtaThreads, bitmap_bytes(range), s>>>(
                 off_u, adj_u, g->rank_u, g->rank_l, tier_rows + r, tier_n + 1, range, gl, gu, num_graphs, uo, guard);
         note_launch();
     }
-    if (bitmaps && max_deg > kRowCtaMax && m > kRowCtaMax) {
+    if (bitmaps && wide_tier && m > kRowCtaMax) {
         k_u_rows_bitmap<1024>
             <<<(unsigned)std::min<int64_t>(m / kRowCtaMax, 152 * 2), 1024, bitmap_bytes(range), s>>>(
                 off_u, adj_u, g->rank_u, g->rank_l, tier_rows + 2 * (int64_t)r, tier_n + 2, range, gl, gu, num_graphs, uo,
@@ -1395,29 +1535,29 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
     GET(g->mem, g->sbeg, std::max<int64_t>(2 * m, 1));
     GET(g->mem, g->cut, n);
     GET(g->mem, g->work, n);
-    GET(g->mem, g->cursors, 8);
-    GET(g->mem, g->acc, 2);
+    GET(g->mem, g->cursors, 8 + 4);
+    g->acc = reinterpret_cast<unsigned long long *>(g->cursors + 8);   // cleared together
     GET(g->mem, g->pv, n);
+    GET(g->mem, g->warp_items, std::max(n, 1));
     BFC_CUDA(cudaMemsetAsync(g->err, 0, 4 * sizeof(int), s));
 
-    // ---- validation of the caller's CSR (memory safety of everything below)
-    k_check_offsets<<<blocks_for((int64_t)r + 1), kT, 0, s>>>(csr->off_u, r, m, g->err); note_launch();
-    BFC_CUDA(cudaGetLastError());
+    // A batch's start arrays are checked first: its largest layers size what
+    // follows.  Everything else about the caller's arrays is checked by kernels
+    // whose error word stops every later kernel that would index with them, and
+    // reported at the one round trip after the work is known.
     int herr = 0;
-    BFC_CUDA(cudaMemcpyAsync(&herr, g->err, sizeof(int), cudaMemcpyDeviceToHost, s));
-    BFC_CUDA(cudaStreamSynchronize(s));
-    if (herr) { set_last_error("off_u is not a CSR offset array of num_edges entries"); return BFC_ERR_INVALID_GRAPH; }
     int32_t l_range = l;
+    g->max_range = std::max(r, l);
     if (num_graphs > 0) {
-        k_check_starts<<<blocks_for((int64_t)num_graphs + 1), kT, 0, s>>>(graph_u_start, num_graphs, r, g->err); note_launch();
+        k_check_starts<<<blocks_for((int64_t)num_graphs + 1), kT, 0, s>>>(graph_u_start, num_graphs, r, g->err, 0x7fffffff, g->err + 2); note_launch();
         k_check_starts<<<blocks_for((int64_t)num_graphs + 1), kT, 0, s>>>(graph_l_start, num_graphs, l, g->err, 0x7fffffff, g->err + 1); note_launch();
         BFC_CUDA(cudaGetLastError());
-        int hstart[2] = {0, 0};
-        BFC_CUDA(cudaMemcpyAsync(hstart, g->err, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
+        int hstart[3] = {0, 0, 0};
+        BFC_CUDA(cudaMemcpyAsync(hstart, g->err, 3 * sizeof(int), cudaMemcpyDeviceToHost, s));
         BFC_CUDA(cudaStreamSynchronize(s));
-        herr = hstart[0];
+        if (hstart[0]) { set_last_error("graph start arrays are not prefix sums of the layer sizes"); return BFC_ERR_INVALID_GRAPH; }
         l_range = hstart[1];   // the largest L layer of one graph
-        if (herr) { set_last_error("graph start arrays are not prefix sums of the layer sizes"); return BFC_ERR_INVALID_GRAPH; }
+        g->max_range = std::max(hstart[1], hstart[2]);
         g->num_graphs = num_graphs;
         GET(g->mem, g->gstar, std::max<int64_t>(n, 1));
         GET(g->mem, g->vbase, std::max<int64_t>(n, 1));
@@ -1425,14 +1565,16 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
         GET(g->mem, g->gwork, num_graphs);
         BFC_CUDA(cudaMemsetAsync(g->gwork, 0, sizeof(unsigned long long) * num_graphs, s));
     }
+    const int *guard_err = g->err;
 
     // ---- temporaries
     const int64_t nsort = std::max<int64_t>({(int64_t)r, (int64_t)l, m, (int64_t)n, 1});
     uint64_t *k0, *k1;
-    int32_t *v0, *v1, *deg_u, *deg_l, *deg_star, *rows_star, *heads, *big, *n_big;
+    int32_t *v0, *v1, *deg_u, *deg_l, *deg_star, *rows_star, *heads, *big, *n_big, *heavy;
     uint32_t *hist, *hist_tmp;
     int64_t *scan64_tmp, *deg64;
-    int32_t *maxdeg;
+    // [0] W, [1] heaviest start, [2] starts beyond the CTA-hash bin, [3..8) bin
+    // counts, [8] / [9] largest L / U degree
     unsigned long long *red;
     GET(tmp, k0, nsort + 1); GET(tmp, k1, nsort + 1);
     GET(tmp, v0, nsort); GET(tmp, v1, nsort);
@@ -1444,81 +1586,38 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
     GET(tmp, scan64_tmp, std::max(scan_tmp_elems<int64_t>((int64_t)n + 1),
                                   max_scan_tmp_elems(m)));
     GET(tmp, deg64, (int64_t)n + 1);
-    GET(tmp, maxdeg, 4);
-    GET(tmp, red, 8);
+    GET(tmp, red, 10);
+    GET(tmp, heavy, std::max(n, 1));
+    BFC_CUDA(cudaMemsetAsync(red, 0, 10 * sizeof(unsigned long long), s));
 
-    // ---- a1: degrees (and the check of the L ids)
+    // ---- a1: degrees, and the check of the caller's offsets and L ids
     BFC_CUDA(cudaMemsetAsync(deg_l, 0, sizeof(int32_t) * std::max<int64_t>(l, 1), s));
-    if (r > 0) { k_deg_u<<<blocks_for(r), kT, 0, s>>>(csr->off_u, r, deg_u); note_launch(); }
+    k_check_offsets<<<blocks_for((int64_t)r + 1), kT, 0, s>>>(csr->off_u, r, m, deg_u, g->err); note_launch();
     if (m > 0) { k_deg_l<<<grid_stride_blocks(m), kT, 0, s>>>(csr->adj_u, m, l, deg_l, g->err); note_launch(); }
     BFC_CUDA(cudaGetLastError());
-    BFC_CUDA(reduce_max_i32(deg_u, r, maxdeg, s));
-    BFC_CUDA(reduce_max_i32(deg_l, l, maxdeg + 1, s));
-    int32_t hmax[2] = {0, 0};
-    BFC_CUDA(cudaMemcpyAsync(hmax, maxdeg, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-    BFC_CUDA(cudaMemcpyAsync(&herr, g->err, sizeof(int), cudaMemcpyDeviceToHost, s));
-    BFC_CUDA(cudaStreamSynchronize(s));
-    if (herr) { set_last_error("adj_u holds an id outside [0, num_l)"); return BFC_ERR_INVALID_GRAPH; }
-    g->info.max_deg_u = hmax[0];
-    g->info.max_deg_l = hmax[1];
 
-    // ---- a2: per-layer priority ranks by a stable sort on degree
-    int which = 0;
-    if (r > 0) {
-        int bkey = bits_for((uint64_t)hmax[0]);
-        if (num_graphs > 0) {
-            k_iota_keys_batch<<<blocks_for(r), kT, 0, s>>>(deg_u, r, graph_u_start, num_graphs, bkey, k0, v0); note_launch();
-            bkey += bits_for((uint64_t)(num_graphs - 1));
-        } else {
-            k_iota_keys<<<blocks_for(r), kT, 0, s>>>(deg_u, r, k0, v0); note_launch();
-        }
-        BFC_CUDA(cudaGetLastError());
-        BFC_CUDA(radix_sort_pairs(k0, v0, k1, v1, r, 0, bkey, hist,
-                                  hist_tmp, s, &which));
-        const uint64_t *ks = which ? k1 : k0;
-        const int32_t *vs = which ? v1 : v0;
-        k_ranks<<<blocks_for(r), kT, 0, s>>>(ks, vs, r, g->rank_u, deg_star, l, (1ull << bits_for((uint64_t)hmax[0])) - 1); note_launch();
-        BFC_CUDA(cudaGetLastError());
-    }
-    if (l > 0) {
-        int bkey = bits_for((uint64_t)hmax[1]);
-        if (num_graphs > 0) {
-            k_iota_keys_batch<<<blocks_for(l), kT, 0, s>>>(deg_l, l, graph_l_start, num_graphs, bkey, k0, v0); note_launch();
-            bkey += bits_for((uint64_t)(num_graphs - 1));
-        } else {
-            k_iota_keys<<<blocks_for(l), kT, 0, s>>>(deg_l, l, k0, v0); note_launch();
-        }
-        BFC_CUDA(cudaGetLastError());
-        BFC_CUDA(radix_sort_pairs(k0, v0, k1, v1, l, 0, bkey, hist,
-                                  hist_tmp, s, &which));
-        const uint64_t *ks = which ? k1 : k0;
-        const int32_t *vs = which ? v1 : v0;
-        k_ranks<<<blocks_for(l), kT, 0, s>>>(ks, vs, l, g->rank_l, deg_star, 0, (1ull << bits_for((uint64_t)hmax[1])) - 1); note_launch();
-        BFC_CUDA(cudaGetLastError());
+    // ---- a2: per-layer priority ranks by a stable sort on (layer, graph, degree)
+    {
+        int rc = launch_ranks(g, deg_l, deg_u, graph_l_start, graph_u_start, g->max_range, k0, v0, k1, v1, hist,
+                              hist_tmp, deg_star, deg64, red + 8, s, guard_err);
+        if (rc) return rc;
     }
 
     if (num_graphs > 0 && n > 0) {
         k_graph_star<<<grid_stride_blocks(n), kT, 0, s>>>(r, l, graph_u_start, graph_l_start,
-                                                         num_graphs, g->gstar, g->vbase, g->vend); note_launch();
+                                                         num_graphs, g->gstar, g->vbase, g->vend, guard_err); note_launch();
         BFC_CUDA(cudaGetLastError());
     }
 
     // ---- a3: G* offsets and priority-sorted lists
-    if (n > 0) {
-        k_deg_to_i64<<<blocks_for(n), kT, 0, s>>>(deg_star, n, deg64); note_launch();
-        BFC_CUDA(cudaGetLastError());
-    }
     BFC_CUDA(scan_exclusive<int64_t>(deg64, g->off, n, scan64_tmp, s));
     const int bu = bits_for(r > 0 ? (uint64_t)(r - 1) : 0);
     const int bl = bits_for(l > 0 ? (uint64_t)(l - 1) : 0);
     if (m > 0) {
-        if (num_graphs > 0) {
+        if (num_graphs > 0 && (!opt->validate || l_range > kRowBitmapMax)) {
             k_check_batch_rows<<<grid_stride_blocks(r), kT, 0, s>>>(csr->off_u, csr->adj_u, r, graph_u_start,
-                                                                    graph_l_start, num_graphs, g->err); note_launch();
+                                                                    graph_l_start, num_graphs, g->err, guard_err); note_launch();
             BFC_CUDA(cudaGetLastError());
-            BFC_CUDA(cudaMemcpyAsync(&herr, g->err, sizeof(int), cudaMemcpyDeviceToHost, s));
-            BFC_CUDA(cudaStreamSynchronize(s));
-            if (herr) { set_last_error("an edge joins vertices of two different graphs of the batch"); return BFC_ERR_INVALID_GRAPH; }
         }
         // U side row by row (warp / CTA tiers, radix sort for the largest rows);
         // the swapped keys for the L side land in k1
@@ -1528,15 +1627,17 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
         GET(tmp, tier_n, kRowTiers);
         {
             int rc = launch_u_rows(csr->off_u, csr->adj_u, g, l_range, graph_u_start, graph_l_start, num_graphs,
-                                   hmax[0], opt->validate, uo, tier_rows, tier_n, s, nullptr);
+                                   opt->validate, uo, tier_rows, tier_n, s, guard_err);
             if (rc) return rc;
         }
         // rows that no bitmap takes (see the tiers): CTA sorts, and a radix sort
         // of the largest rows' edges
-        if (hmax[0] > kRowWarpSortMax && (!opt->validate || l_range > kRowBitmapMax)) {
+        if (m > kRowWarpSortMax && (!opt->validate || l_range > kRowBitmapMax)) {
             int32_t hn[2] = {0, 0};
             BFC_CUDA(cudaMemcpyAsync(hn, tier_n + 3, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+            BFC_CUDA(cudaMemcpyAsync(&herr, g->err, sizeof(int), cudaMemcpyDeviceToHost, s));
             BFC_CUDA(cudaStreamSynchronize(s));
+            if (int rc = input_error(herr, num_graphs)) return rc;
             if (hn[0] > 0) {
                 k_u_rows_cta<<<(unsigned)std::min<int32_t>(hn[0], 152 * 16), kRowCtaThreads, 0, s>>>(
                     csr->off_u, csr->adj_u, g->rank_u, g->rank_l, tier_rows + 3 * (int64_t)r, hn[0], uo); note_launch();
@@ -1587,41 +1688,46 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
         if (opt->orientation == 0) {
             BFC_CUDA(cudaMemsetAsync(g->plen + m, 0, sizeof(int32_t) * (size_t)m, s));
             k_emit_l_side<true><<<grid_stride_blocks(m), kT, 0, s>>>(k2, v2, m, bu, l, g->off, g->adj, g->eid,
-                                                                      rows_star, g->plen, g->sbeg); note_launch();
+                                                                      rows_star, g->plen, g->sbeg, guard_err); note_launch();
         } else {
             k_emit_l_side<false><<<grid_stride_blocks(m), kT, 0, s>>>(k2, v2, m, bu, l, g->off, g->adj, g->eid,
-                                                                       rows_star, nullptr, nullptr); note_launch();
+                                                                       rows_star, nullptr, nullptr, guard_err); note_launch();
         }
         BFC_CUDA(cudaGetLastError());
-        if (opt->validate) {
-            BFC_CUDA(cudaMemcpyAsync(&herr, g->err, sizeof(int), cudaMemcpyDeviceToHost, s));
-            BFC_CUDA(cudaStreamSynchronize(s));
-            if (herr & kErrDuplicate) { set_last_error("duplicate edge"); return BFC_ERR_INVALID_GRAPH; }
-        }
     }
 
     // ---- a4: cut, per-middle prefix lengths, per-start work, W
-    BFC_CUDA(cudaMemsetAsync(red, 0, 8 * sizeof(unsigned long long), s));
     if (n > 0) {
-        k_cut<<<blocks_for(n), kT, 0, s>>>(g->off, g->adj, deg_star, n, l, g->cut); note_launch();
+        k_cut<<<blocks_for(n), kT, 0, s>>>(g->off, g->adj, deg_star, n, l, g->cut, guard_err); note_launch();
         BFC_CUDA(cudaGetLastError());
     }
     if (m > 0 && opt->orientation == 1) {
         k_slen<<<grid_stride_blocks(2 * m), kT, 0, s>>>(g->off, g->adj, rows_star, g->cut, 2 * m,
-                                                         g->plen, g->sbeg); note_launch();
+                                                         g->plen, g->sbeg, guard_err); note_launch();
         BFC_CUDA(cudaGetLastError());
     }
     const bool core_auto = opt->core_vertices < 0 && opt->orientation == 0 && num_graphs == 0;
     if (n > 0) {
         BFC_CUDA(cudaMemsetAsync(n_big, 0, sizeof(int32_t), s));
-        launch_work(g, big, n_big, num_graphs > 0 ? g->gwork : nullptr, red, s, nullptr);
+        launch_work(g, big, n_big, num_graphs > 0 ? g->gwork : nullptr, red, s, guard_err);
         BFC_CUDA(cudaGetLastError());
     }
-    unsigned long long hred[3] = {0, 0, 0};
-    BFC_CUDA(cudaMemcpyAsync(hred, red, 3 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
+    // the bins without a core, before the round trip (a core, which only large
+    // graphs get, moves its starts to the dense bin: those are binned again)
+    BinBounds bb = bin_bounds(g, opt->warp_max_work, opt->team_max_work, opt->hash_max_work);
+    {
+        int rc = bin_starts(g, s, bb, red + 3, heavy, guard_err);
+        if (rc) return rc;
+    }
+    unsigned long long hred[10] = {0};
+    BFC_CUDA(cudaMemcpyAsync(hred, red, sizeof(hred), cudaMemcpyDeviceToHost, s));
+    BFC_CUDA(cudaMemcpyAsync(&herr, g->err, sizeof(int), cudaMemcpyDeviceToHost, s));
     BFC_CUDA(cudaStreamSynchronize(s));
+    if (int rc = input_error(herr, num_graphs)) return rc;
     g->info.wedges = hred[0];
     g->info.max_start_work = hred[1];
+    g->info.max_deg_l = (int32_t)hred[8];
+    g->info.max_deg_u = (int32_t)hred[9];
 
     // ---- dense-core hybrid (Algorithm 2 single graphs): the requested core
     // size, or (core_vertices = -1) as many vertices as starts heavier than
@@ -1639,8 +1745,16 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
     g->info.core_l = g->core_l;
 
     // ---- a5: heaviest-first order and bins
+    if (g->core_u + g->core_l > 0) {
+        bb = bin_bounds(g, opt->warp_max_work, opt->team_max_work, opt->hash_max_work);
+        int rc = bin_starts(g, s, bb, red + 3, heavy, nullptr);
+        if (rc) return rc;
+        BFC_CUDA(cudaMemcpyAsync(hred + 3, red + 3, 5 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
+        BFC_CUDA(cudaStreamSynchronize(s));
+    }
     {
-        int rc = schedule_graph(g, s, opt->warp_max_work, opt->team_max_work, opt->hash_max_work, rows_star);
+        int rc = schedule_graph(g, s, opt->warp_max_work, opt->team_max_work, opt->hash_max_work, rows_star, bb,
+                                hred + 3, heavy);
         if (rc) return rc;
     }
     g->info.num_u = r; g->info.num_l = l; g->info.num_edges = m;
@@ -1662,15 +1776,26 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
 // ----------------------------------------------------------------------------
 namespace {
 
-// heaviest first by exact work, 32 key bits (work saturated at 2^32 - 1)
-__global__ void k_sched_keys_plan(const uint64_t *__restrict__ work, int32_t n, uint64_t *keys,
-                                  int32_t *vals, const int *guard) {
-    if (aborted(guard)) return;
-    const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= n) return;
-    const uint64_t w = work[x];
-    keys[x] = 0xFFFFFFFFull - (w < 0xFFFFFFFFull ? w : 0xFFFFFFFFull);
-    vals[x] = (int32_t)x;
+// One byte per heavy start, heaviest first inside its bin: the three bins take
+// codes 0..., by quarter octaves of the work (dense starts) or octaves.  Places
+// past the heavy ones get 255.
+__global__ void k_sched_keys_plan(const uint64_t *__restrict__ work, const int32_t *__restrict__ heavy, int32_t n,
+                                  BinBounds bb, const unsigned long long *__restrict__ counts, uint64_t *keys) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    uint64_t key = 255;
+    if (i < (int64_t)counts[4]) {
+        const uint64_t w = work[heavy[i]];
+        const int oct = 63 - __clzll((long long)w);
+        const int bin = bb.of(heavy[i], w);
+        if (bin == 0) {
+            const int q = oct >= 2 ? 4 * oct + (int)((w >> (oct - 2)) & 3) : 4 * oct;
+            key = q < 160 ? 160 - q : 0;          // 1..160; from 2^40 wedges up 0
+        } else {
+            key = (bin == 1 ? 161 : 193) + (31 - min(oct, 31));
+        }
+    }
+    keys[i] = key;
 }
 
 // the item lists from the sorted order and the bin sizes on the device: a
@@ -1678,16 +1803,14 @@ __global__ void k_sched_keys_plan(const uint64_t *__restrict__ work, int32_t n, 
 // counters too), so the lists follow the order directly
 __global__ void k_emit_items_plan(const int32_t *__restrict__ order,
                                   const unsigned long long *__restrict__ counts, int2 *cta_items,
-                                  int32_t *team_items, int32_t *warp_items, const int *guard) {
+                                  int32_t *team_items, const int *guard) {
     if (aborted(guard)) return;
-    const int64_t nd = (int64_t)counts[0], nh = (int64_t)counts[1], nt = (int64_t)counts[2],
-                  nw = (int64_t)counts[3];
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nd + nh + nt + nw;
+    const int64_t nd = (int64_t)counts[0], nh = (int64_t)counts[1], nt = (int64_t)counts[2];
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nd + nh + nt;
          i += (int64_t)gridDim.x * blockDim.x) {
         const int32_t x = order[i];
         if (i < nd + nh) cta_items[i] = make_int2(x, 0);
-        else if (i < nd + nh + nt) team_items[i - nd - nh] = x;
-        else warp_items[i - nd - nh - nt] = x;
+        else team_items[i - nd - nh] = x;
     }
 }
 
@@ -1722,7 +1845,8 @@ int batch_plan_create(BatchPlan *pl, cudaStream_t s) {
     // kept arrays (those of prepare_graph for a batch)
     GET(g->err, 4); GET(g->rank_u, r); GET(g->rank_l, l); GET(g->off, (int64_t)n + 1);
     GET(g->adj, 2 * m); GET(g->eid, 2 * m); GET(g->plen, 2 * m); GET(g->cut, n); GET(g->work, n);
-    GET(g->cursors, 8); GET(g->acc, 2); GET(g->pv, 1); GET(g->sbeg, 2 * m);
+    GET(g->cursors, 8 + 4); GET(g->pv, 1); GET(g->sbeg, 2 * m);
+    g->acc = reinterpret_cast<unsigned long long *>(g->cursors + 8);   // cleared together
     GET(g->gstar, n); GET(g->vbase, n); GET(g->vend, n); GET(g->gwork, G);
     GET(g->cta_items, n); GET(g->team_items, n); GET(g->warp_items, n); GET(g->retry, 1);
     // temporaries, kept with the plan
@@ -1734,7 +1858,7 @@ int batch_plan_create(BatchPlan *pl, cudaStream_t s) {
     GET(pl->hist, radix_hist_elems(nsort));
     GET(pl->hist_tmp, scan_tmp_elems<uint32_t>((int64_t)radix_hist_elems(nsort)));
     GET(pl->scan64_tmp, std::max(scan_tmp_elems<int64_t>((int64_t)n + 1), max_scan_tmp_elems(m)));
-    GET(pl->deg64, (int64_t)n + 1); GET(pl->red, 8);
+    GET(pl->deg64, (int64_t)n + 1); GET(pl->red, 10); GET(pl->heavy, n);
 #undef GET
     // every kept array starts zeroed: a run that stops at the checks leaves
     // arrays that later kernels can still index safely
@@ -1764,37 +1888,21 @@ int batch_plan_run(BatchPlan *pl, const int32_t *off_u, const int32_t *adj_u, co
     const bfc_options *opt = &g->opt;
     BFC_CUDA(cudaMemsetAsync(g->err, 0, 4 * sizeof(int), s));
     // ---- checks: the CSR, the graph start arrays, edges inside their graph
-    k_check_offsets<<<blocks_for((int64_t)r + 1), kT, 0, s>>>(off_u, r, m, g->err); note_launch();
+    k_check_offsets<<<blocks_for((int64_t)r + 1), kT, 0, s>>>(off_u, r, m, pl->deg_u, g->err); note_launch();
     k_check_starts<<<blocks_for((int64_t)G + 1), kT, 0, s>>>(gu, G, r, g->err, pl->max_layer); note_launch();
     k_check_starts<<<blocks_for((int64_t)G + 1), kT, 0, s>>>(gl, G, l, g->err, pl->max_layer); note_launch();
     BFC_CUDA(cudaGetLastError());
     // ---- a1: degrees (and the check of the L ids)
     BFC_CUDA(cudaMemsetAsync(pl->deg_l, 0, sizeof(int32_t) * std::max<int64_t>(l, 1), s));
     if (m > 0) { k_deg_l<<<grid_stride_blocks(m), kT, 0, s>>>(adj_u, m, l, pl->deg_l, g->err); note_launch(); }
-    if (r > 0) { k_deg_u<<<blocks_for(r), kT, 0, s>>>(off_u, r, pl->deg_u, guard); note_launch(); }
     BFC_CUDA(cudaGetLastError());
-    // ---- a2: graph-major ranks; a degree is below 2^bdeg (at most the other layer)
-    const int bdeg = bits_for((uint64_t)pl->max_layer);
-    const int bkey = bdeg + bits_for((uint64_t)(G - 1));
-    const uint64_t dmask = (1ull << bdeg) - 1;
-    int which = 0;
-    for (int side = 0; side < 2; ++side) {
-        const int32_t cnt = side == 0 ? r : l;
-        if (cnt == 0) continue;
-        const int32_t *deg = side == 0 ? pl->deg_u : pl->deg_l;
-        const int32_t *start = side == 0 ? gu : gl;
-        k_iota_keys_batch<<<blocks_for(cnt), kT, 0, s>>>(deg, cnt, start, G, bdeg, pl->k0, pl->v0, guard); note_launch();
-        BFC_CUDA(cudaGetLastError());
-        BFC_CUDA(radix_sort_pairs(pl->k0, pl->v0, pl->k1, pl->v1, cnt, 0, bkey, pl->hist, pl->hist_tmp, s, &which));
-        const uint64_t *ks = which ? pl->k1 : pl->k0;
-        const int32_t *vs = which ? pl->v1 : pl->v0;
-        k_ranks<<<blocks_for(cnt), kT, 0, s>>>(ks, vs, cnt, side == 0 ? g->rank_u : g->rank_l, pl->deg_star,
-                                               side == 0 ? l : 0, dmask, guard); note_launch();
-        BFC_CUDA(cudaGetLastError());
-    }
+    BFC_CUDA(cudaMemsetAsync(pl->red, 0, 10 * sizeof(unsigned long long), s));
+    // ---- a2: graph-major ranks; a degree is below 2^16 (at most the other layer)
+    int rc = launch_ranks(g, pl->deg_l, pl->deg_u, gl, gu, pl->max_layer, pl->k0, pl->v0, pl->k1, pl->v1, pl->hist,
+                          pl->hist_tmp, pl->deg_star, pl->deg64, pl->red + 8, s, guard);
+    if (rc) return rc;
     if (n > 0) {
         k_graph_star<<<grid_stride_blocks(n), kT, 0, s>>>(r, l, gu, gl, G, g->gstar, g->vbase, g->vend, guard); note_launch();
-        k_deg_to_i64<<<blocks_for(n), kT, 0, s>>>(pl->deg_star, n, pl->deg64, guard); note_launch();
         BFC_CUDA(cudaGetLastError());
     }
     BFC_CUDA(scan_exclusive<int64_t>(pl->deg64, g->off, n, pl->scan64_tmp, s));
@@ -1802,10 +1910,8 @@ int batch_plan_run(BatchPlan *pl, const int32_t *off_u, const int32_t *adj_u, co
     const int bu = bits_for(r > 0 ? (uint64_t)(r - 1) : 0);
     const int bl = bits_for(l > 0 ? (uint64_t)(l - 1) : 0);
     if (m > 0) {
-        k_check_batch_rows<<<grid_stride_blocks(r), kT, 0, s>>>(off_u, adj_u, r, gu, gl, G, g->err, guard); note_launch();
         const URowOut uo{m, l, bu, g->off, g->adj, g->eid, pl->rows_star, pl->k1, g->err, opt->validate};
-        int rc = launch_u_rows(off_u, adj_u, g, pl->max_layer, gu, gl, G, pl->max_layer, 1, uo, pl->tier_rows,
-                               pl->tier_n, s, guard);
+        rc = launch_u_rows(off_u, adj_u, g, pl->max_layer, gu, gl, G, 1, uo, pl->tier_rows, pl->tier_n, s, guard);
         if (rc) return rc;
         // L side: stable sort of the swapped keys on their rank_l bits
         int which2 = 0;
@@ -1818,7 +1924,6 @@ int batch_plan_run(BatchPlan *pl, const int32_t *off_u, const int32_t *adj_u, co
         BFC_CUDA(cudaGetLastError());
     }
     // ---- a4: cut, runs, work
-    BFC_CUDA(cudaMemsetAsync(pl->red, 0, 8 * sizeof(unsigned long long), s));
     if (n > 0) { k_cut<<<blocks_for(n), kT, 0, s>>>(g->off, g->adj, pl->deg_star, n, l, g->cut, guard); note_launch(); }
     if (n > 0) {
         BFC_CUDA(cudaMemsetAsync(g->gwork, 0, sizeof(unsigned long long) * G, s));
@@ -1827,23 +1932,26 @@ int batch_plan_run(BatchPlan *pl, const int32_t *off_u, const int32_t *adj_u, co
         BFC_CUDA(cudaGetLastError());
     }
     // ---- a5: heaviest first, bins from device counts
-    unsigned long long *bins = pl->red + 4;
+    // bins by compaction, then the heavy starts heaviest first: how many there
+    // are is not known here, so the sort covers n keys of one byte (the rest
+    // hold the largest key and stay behind), which order them to a quarter octave
+    unsigned long long *bins = pl->red + 3;
     if (n > 0) {
-        k_sched_keys_plan<<<blocks_for(n), kT, 0, s>>>(g->work, n, pl->k0, pl->v0, guard); note_launch();
+        const BinBounds bb{(uint64_t)opt->warp_max_work, pl->team_max, (uint64_t)opt->hash_max_work, l, n, n};
+        rc = bin_starts(g, s, bb, bins, pl->heavy, guard);
+        if (rc) return rc;
+        k_sched_keys_plan<<<blocks_for(n), kT, 0, s>>>(g->work, pl->heavy, n, bb, bins, pl->k0); note_launch();
         BFC_CUDA(cudaGetLastError());
-        BFC_CUDA(radix_sort_pairs(pl->k0, pl->v0, pl->k1, pl->v1, n, 0, 32, pl->hist, pl->hist_tmp, s, &which));
-        const int32_t *order = which ? pl->v1 : pl->v0;
-        k_classify<<<grid_stride_blocks(n), kT, 0, s>>>(g->work, n, (uint64_t)opt->warp_max_work,
-                                                        (uint64_t)pl->team_max, (uint64_t)opt->hash_max_work, l, n, n,
-                                                        bins, guard); note_launch();
-        k_emit_items_plan<<<grid_stride_blocks(n), kT, 0, s>>>(order, bins, g->cta_items, g->team_items,
-                                                               g->warp_items, guard); note_launch();
+        int which = 0;
+        BFC_CUDA(radix_sort_pairs(pl->k0, pl->heavy, pl->k1, pl->v1, n, 0, 8, pl->hist, pl->hist_tmp, s, &which));
+        k_emit_items_plan<<<grid_stride_blocks(n), kT, 0, s>>>(which ? pl->v1 : pl->heavy, bins, g->cta_items,
+                                                               g->team_items, guard); note_launch();
         BFC_CUDA(cudaGetLastError());
     }
     // ---- a6-a7: one persistent count; per-graph totals
     BFC_CUDA(cudaMemsetAsync(totals, 0, sizeof(unsigned long long) * G, s));
     g->item_counts = bins;
-    int rc = launch_count(g, s, kModeBatch, nullptr, nullptr, totals);
+    rc = launch_count(g, s, kModeBatch, nullptr, nullptr, totals);
     if (rc) return rc;
     if (status) {
         k_plan_status<<<1, 1, 0, s>>>(g->err, opt->validate, status); note_launch();

@@ -276,16 +276,6 @@ __global__ void k_index_values(int32_t *v, int64_t n) {
         v[k] = (int32_t)k;
 }
 
-__global__ void k_reduce_max_i32(const int32_t *__restrict__ in, int64_t n, int32_t *out) {
-    int32_t m = 0;
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
-         k += (int64_t)gridDim.x * blockDim.x)
-        m = max(m, in[k]);
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, d));
-    if ((threadIdx.x & 31) == 0 && m > 0) atomicMax(out, m);
-}
-
 }  // namespace
 
 template <typename T>
@@ -380,15 +370,6 @@ cudaError_t radix_sort_pairs(uint64_t *k0, int32_t *v0, uint64_t *k1, int32_t *v
         *which ^= 1;
     }
     return cudaSuccess;
-}
-
-cudaError_t reduce_max_i32(const int32_t *in, int64_t n, int32_t *out, cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(out, 0, sizeof(int32_t), s);
-    if (e != cudaSuccess || n <= 0) return e;
-    int blocks = (int)((n + 255) / 256);
-    if (blocks > 4096) blocks = 4096;
-    k_reduce_max_i32<<<blocks, 256, 0, s>>>(in, n, out); note_launch();
-    return cudaGetLastError();
 }
 
 }  // namespace bfc
