@@ -672,11 +672,11 @@ __global__ void k_slen(const int64_t *__restrict__ off, const int32_t *__restric
 // Algorithm 2, every slot for Algorithm 3).  For Algorithm 2 the U-side middle
 // slots (at or past `fill_from`) also get the start of their run, off[middle].
 // A warp takes 32 starts and each lane walks its own where there are at most
-// 24 slots (neighbouring lists share their sectors); the longer ones go to a
-// queue that k_work_long takes 32 at a time per CTA, one per warp, or one after
-// another by the whole CTA above 4,096 slots.  With one warp per start the
-// millions of one-slot starts of a sparse batch and the longest list of a skewed
-// graph each took 2.5 ms.
+// 24 slots (neighbouring lists share their sectors); the longer ones go to two
+// queues for k_work_long, one per warp up to 4,096 slots and one per CTA above.
+// (Ranks are by degree, so the long lists are neighbours: whatever takes several
+// in a row has them all.)  With one warp per start the millions of one-slot
+// starts of a sparse batch and the longest list of a skewed graph each took 2.5 ms.
 constexpr int kWorkLane = 24;
 constexpr int kWorkWarp = 4096;
 
@@ -708,59 +708,85 @@ __global__ void k_work(const int64_t *__restrict__ off, const int32_t *__restric
             for (int32_t j = 0; j < c; ++j) s += slot_work(off, adj, plen, b + j, fill, sbeg);
             if (x < n) work[x] = s;
         }
-        const uint32_t todo = __ballot_sync(0xffffffffu, c > kWorkLane);
+        // queue[0, n): the warps' from the front, the CTAs' from the back
+        const uint32_t by_warp = __ballot_sync(0xffffffffu, c > kWorkLane && c <= kWorkWarp);
+        const uint32_t by_cta = __ballot_sync(0xffffffffu, c > kWorkWarp);
         int32_t at = 0;
-        if (lane == 0 && todo) at = atomicAdd(queued, __popc(todo));
-        at = __shfl_sync(0xffffffffu, at, 0);
-        if (c > kWorkLane) queue[at + __popc(todo & ((1u << lane) - 1u))] = (int32_t)x;
+        if (lane == 0 && by_warp) at = atomicAdd(queued, __popc(by_warp));
+        if (lane == 1 && by_cta) at = atomicAdd(queued + 1, __popc(by_cta));
+        const int32_t at_w = __shfl_sync(0xffffffffu, at, 0), at_c = __shfl_sync(0xffffffffu, at, 1);
+        const uint32_t lt = (1u << lane) - 1u;
+        if (c > kWorkWarp) queue[n - 1 - at_c - __popc(by_cta & lt)] = (int32_t)x;
+        else if (c > kWorkLane) queue[at_w + __popc(by_warp & lt)] = (int32_t)x;
     }
 }
 
-__global__ void __launch_bounds__(1024) k_work_long(const int64_t *__restrict__ off, const int32_t *__restrict__ adj,
-                                                    const int32_t *__restrict__ cut, const int32_t *__restrict__ plen,
-                                                    int all_slots, int64_t fill_from, int64_t *sbeg, uint64_t *work,
-                                                    const int32_t *__restrict__ queue,
-                                                    const int32_t *__restrict__ queued,
+// Σ plen over slots b + j, b + j + W, ... of a list's first c, four loads at a
+// time, and the runs' starts where `fill`
+template <int W>
+__device__ __forceinline__ unsigned long long walk_slots(const int64_t *__restrict__ off,
+                                                         const int32_t *__restrict__ adj,
+                                                         const int32_t *__restrict__ plen, int64_t b, int32_t j,
+                                                         int32_t c, bool fill, int64_t *__restrict__ sbeg) {
+    unsigned long long t = 0;
+    for (; j < c; j += 4 * W) {
+        unsigned len[4];
+        int32_t mid[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const bool in = j + u * W < c;
+            len[u] = in ? (unsigned)plen[b + j + u * W] : 0u;
+            mid[u] = in && fill ? adj[b + j + u * W] : -1;
+        }
+        if (fill) {
+            int64_t at[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) at[u] = mid[u] >= 0 ? off[mid[u]] : 0;
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (mid[u] >= 0) sbeg[b + j + u * W] = at[u];
+        }
+        t += (unsigned long long)len[0] + len[1] + len[2] + len[3];
+    }
+    return t;
+}
+
+constexpr int kWorkThreads = 512;
+__global__ void __launch_bounds__(kWorkThreads) k_work_long(
+    const int64_t *__restrict__ off, const int32_t *__restrict__ adj, const int32_t *__restrict__ cut,
+    const int32_t *__restrict__ plen, int32_t n, int all_slots, int64_t fill_from, int64_t *sbeg, uint64_t *work,
+    const int32_t *__restrict__ queue, const int32_t *__restrict__ queued,
     const int *guard = nullptr) {
     if (aborted(guard)) return;
-    __shared__ unsigned long long part[32];
-    const int n = *queued, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int i0 = blockIdx.x * 32; i0 < n; i0 += gridDim.x * 32) {
-        if (i0 + warp < n) {
-            const int32_t x = queue[i0 + warp];
-            const int64_t b = off[x];
-            const int32_t c = all_slots ? (int32_t)(off[x + 1] - b) : cut[x];
-            if (c <= kWorkWarp) {
-                const bool fill = b >= fill_from;
-                unsigned long long t = 0;
-#pragma unroll 4
-                for (int32_t j = lane; j < c; j += 32) t += slot_work(off, adj, plen, b + j, fill, sbeg);
+    __shared__ unsigned long long part[kWorkThreads / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int n_warp = queued[0], n_cta = queued[1];
+    for (int i = blockIdx.x; i < n_cta; i += gridDim.x) {
+        const int32_t x = queue[n - 1 - i];
+        const int64_t b = off[x];
+        const int32_t c = all_slots ? (int32_t)(off[x + 1] - b) : cut[x];
+        const bool fill = b >= fill_from;
+        unsigned long long t = walk_slots<kWorkThreads>(off, adj, plen, b, (int32_t)threadIdx.x, c, fill, sbeg);
 #pragma unroll
-                for (int d = 16; d > 0; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
-                if (lane == 0) work[x] = t;
-            }
+        for (int d = 16; d > 0; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
+        if (lane == 0) part[warp] = t;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            t = 0;
+            for (int w = 0; w < kWorkThreads / 32; ++w) t += part[w];
+            work[x] = t;
         }
-        for (int k = 0; k < 32 && i0 + k < n; ++k) {   // uniform over the CTA
-            const int32_t x = queue[i0 + k];
-            const int64_t b = off[x];
-            const int32_t c = all_slots ? (int32_t)(off[x + 1] - b) : cut[x];
-            if (c <= kWorkWarp) continue;
-            const bool fill = b >= fill_from;
-            unsigned long long t = 0;
-#pragma unroll 8
-            for (int32_t j = threadIdx.x; j < c; j += 1024) t += slot_work(off, adj, plen, b + j, fill, sbeg);
+        __syncthreads();
+    }
+    for (int i = blockIdx.x * (kWorkThreads / 32) + warp; i < n_warp; i += gridDim.x * (kWorkThreads / 32)) {
+        const int32_t x = queue[i];
+        const int64_t b = off[x];
+        const int32_t c = all_slots ? (int32_t)(off[x + 1] - b) : cut[x];
+        const bool fill = b >= fill_from;
+        unsigned long long t = walk_slots<32>(off, adj, plen, b, lane, c, fill, sbeg);
 #pragma unroll
-            for (int d = 16; d > 0; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
-            if (lane == 0) part[warp] = t;
-            __syncthreads();
-            if (warp == 0) {
-                t = part[lane];
-#pragma unroll
-                for (int d = 16; d > 0; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
-                if (lane == 0) work[x] = t;
-            }
-            __syncthreads();
-        }
+        for (int d = 16; d > 0; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
+        if (lane == 0) work[x] = t;
     }
 }
 
@@ -1494,8 +1520,8 @@ static void launch_work(Graph *g, int32_t *big, int32_t *n_big, unsigned long lo
     k_work<<<grid_stride_blocks(g->n), kT, 0, s>>>(g->off, g->adj, g->cut, g->plen, g->n, vpp, fill_from, g->sbeg,
                                                    g->work, big, n_big, guard); note_launch();
     if (2 * g->m > kWorkLane) {
-        k_work_long<<<(unsigned)std::min<int64_t>(2 * g->m / kWorkLane / 32 + 1, 152 * 2), 1024, 0, s>>>(
-            g->off, g->adj, g->cut, g->plen, vpp, fill_from, g->sbeg, g->work, big, n_big, guard); note_launch();
+        k_work_long<<<(unsigned)std::min<int64_t>(2 * g->m / kWorkLane / (kWorkThreads / 32) + 1, 152 * 4), kWorkThreads, 0, s>>>(
+            g->off, g->adj, g->cut, g->plen, g->n, vpp, fill_from, g->sbeg, g->work, big, n_big, guard); note_launch();
     }
     k_work_stats<<<(unsigned)std::min<int64_t>(blocks_for(g->n), 152 * 8), kT, 0, s>>>(
         g->work, g->n, (uint64_t)g->opt.hash_max_work, g->gstar, stats, gwork, guard); note_launch();
@@ -1580,7 +1606,7 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
     GET(tmp, v0, nsort); GET(tmp, v1, nsort);
     GET(tmp, deg_u, r); GET(tmp, deg_l, l); GET(tmp, deg_star, n);
     GET(tmp, rows_star, 2 * m);
-    GET(tmp, big, std::min<int64_t>(2 * m / kWorkLane, n) + 1); GET(tmp, n_big, 1);
+    GET(tmp, big, n); GET(tmp, n_big, 2);
     GET(tmp, hist, radix_hist_elems(nsort));
     GET(tmp, hist_tmp, scan_tmp_elems<uint32_t>((int64_t)radix_hist_elems(nsort)));
     GET(tmp, scan64_tmp, std::max(scan_tmp_elems<int64_t>((int64_t)n + 1),
@@ -1708,7 +1734,7 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
     }
     const bool core_auto = opt->core_vertices < 0 && opt->orientation == 0 && num_graphs == 0;
     if (n > 0) {
-        BFC_CUDA(cudaMemsetAsync(n_big, 0, sizeof(int32_t), s));
+        BFC_CUDA(cudaMemsetAsync(n_big, 0, 2 * sizeof(int32_t), s));
         launch_work(g, big, n_big, num_graphs > 0 ? g->gwork : nullptr, red, s, guard_err);
         BFC_CUDA(cudaGetLastError());
     }
@@ -1853,7 +1879,7 @@ int batch_plan_create(BatchPlan *pl, cudaStream_t s) {
     const int64_t nsort = std::max<int64_t>({(int64_t)r, (int64_t)l, m, (int64_t)n, 1});
     GET(pl->k0, nsort + 1); GET(pl->k1, nsort + 1); GET(pl->v0, nsort); GET(pl->v1, nsort);
     GET(pl->deg_u, r); GET(pl->deg_l, l); GET(pl->deg_star, n);
-    GET(pl->rows_star, 2 * m); GET(pl->big, std::min<int64_t>(2 * m / kWorkLane, n) + 1); GET(pl->n_big, 1);
+    GET(pl->rows_star, 2 * m); GET(pl->big, n); GET(pl->n_big, 2);
     GET(pl->tier_rows, kRowTiers * (int64_t)std::max(r, 1)); GET(pl->tier_n, kRowTiers);
     GET(pl->hist, radix_hist_elems(nsort));
     GET(pl->hist_tmp, scan_tmp_elems<uint32_t>((int64_t)radix_hist_elems(nsort)));
@@ -1927,7 +1953,7 @@ int batch_plan_run(BatchPlan *pl, const int32_t *off_u, const int32_t *adj_u, co
     if (n > 0) { k_cut<<<blocks_for(n), kT, 0, s>>>(g->off, g->adj, pl->deg_star, n, l, g->cut, guard); note_launch(); }
     if (n > 0) {
         BFC_CUDA(cudaMemsetAsync(g->gwork, 0, sizeof(unsigned long long) * G, s));
-        BFC_CUDA(cudaMemsetAsync(pl->n_big, 0, sizeof(int32_t), s));
+        BFC_CUDA(cudaMemsetAsync(pl->n_big, 0, 2 * sizeof(int32_t), s));
         launch_work(g, pl->big, pl->n_big, g->gwork, pl->red, s, guard);
         BFC_CUDA(cudaGetLastError());
     }
