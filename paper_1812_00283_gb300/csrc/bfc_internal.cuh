@@ -24,6 +24,7 @@ constexpr int kHashMaxWork = kHashMaxSlots / 4 * 3;       // 24,576 wedges: at m
 constexpr int kWarpRegion = kCounterBytes / kCountWarps;  // 6 KB of counters per warp
 constexpr int kWarpSlots = 512;                           // warp hash: 2 KB keys + 2 KB counts
 constexpr int kWarpMaxWork = kWarpSlots / 4 * 3;          // 384 wedges: at most 3/4 of the slots fill
+constexpr int32_t kTinyMax = 32;                          // wedges and middles of a start counted in one window
 constexpr int kTeamThreads = 256;                         // a team: 8 warps with a named barrier
 constexpr int kTeams = kCountThreads / kTeamThreads;      // 4 teams per CTA
 constexpr int kTeamRegion = kCounterBytes / kTeams;       // 48 KB of shared memory per team
@@ -186,8 +187,8 @@ struct Graph {
     uint64_t *work = nullptr; // [n]
     int2 *cta_items = nullptr;    // (start, chunk) / (start, -1 = hash)
     int32_t *team_items = nullptr;
-    int32_t *warp_items = nullptr;
-    int64_t n_cta_items = 0, n_team_items = 0, n_warp_items = 0;
+    int32_t *warp_items = nullptr;   // [n]: the warp bin from the front, its tiny starts from the back
+    int64_t n_cta_items = 0, n_team_items = 0, n_warp_items = 0, n_tiny_items = 0;
     int32_t team_max = 0;          // effective team bound of the current schedule
     bool may_retry = false;        // the schedule can re-queue starts (retry pass launched)
     int *cursors = nullptr;        // [8] work-queue cursors of the count kernels
@@ -232,7 +233,7 @@ struct Graph {
     int32_t *core_kb_u = nullptr, *core_kb_l = nullptr;
     alignas(64) unsigned char core_map_bytes[4][128];
     // batch plan: the bin sizes in device memory ([0] dense, [1] hash,
-    // [2] team, [3] warp starts; null for graphs prepared by prepare_graph)
+    // [2] team, [3] warp, [5] tiny starts; null for graphs prepared by prepare_graph)
     unsigned long long *item_counts = nullptr;
 };
 
@@ -296,7 +297,7 @@ struct BatchPlan {
     int32_t *heavy = nullptr;
     uint32_t *hist = nullptr, *hist_tmp = nullptr;
     int64_t *scan64_tmp = nullptr, *deg64 = nullptr;
-    unsigned long long *red = nullptr;   // [0] W, [3..8) bin sizes, [8], [9] largest degrees
+    unsigned long long *red = nullptr;   // [0] W, [3..9) bin sizes, [9], [10] largest degrees
 };
 int batch_plan_create(BatchPlan *pl, cudaStream_t s);
 int batch_plan_run(BatchPlan *pl, const int32_t *off_u, const int32_t *adj_u, const int32_t *gu,

@@ -30,7 +30,8 @@
 //      batch's scan, so warps that finish early start the next item's loads.
 //   B. team items: four teams of 256 threads, each with a 48 KB region (a
 //      4,096-slot table and its batch arrays), one start per team.
-//   C. warp items: 32 warps, each with a 512-slot table, one light start each.
+//   C. warp items: 32 warps, each with a table of up to 1,024 slots, one light
+//      start each; then the tiny starts, one window each and no table.
 // A table sized from a bound that can be exceeded (Algorithm 3's ends, or a
 // team bound above 3,072 wedges) detects when it fills up; the start is then
 // re-queued and counted by k_count_retry, first with a CTA table, then if
@@ -45,6 +46,7 @@ namespace bfc {
 namespace {
 
 constexpr int kTeamTableBytes = kTeamSlots * 6;   // 32-bit keys + 16-bit counts
+constexpr int kTeamPackedSlots = 8192;            // (key, count) words: 32 KB
 static_assert(kTeamRegion == (kCountWarps / kTeams) * kWarpRegion,
               "a team's region is exactly the regions of its warps");
 
@@ -61,7 +63,8 @@ struct CountParams {
     int64_t n_cta;
     int64_t n_team;
     int64_t n_warp;
-    int *cursors;                      // [0] CTA, [1] warp, [2] retry pushes, [3] retry, [4] team
+    int64_t n_tiny;                    // at the back of warp_items[n]
+    int *cursors;                      // [0] CTA, [1] warp, [2] retry pushes, [3] retry, [4] team, [5] tiny
     unsigned long long *acc;
     unsigned long long *pv;            // [n] in G* ids
     unsigned long long *pe;            // [2m] by G* slot (each edge has two)
@@ -90,8 +93,8 @@ struct CountParams {
     const int32_t *__restrict__ ccut;      // neighbours outside the other layer's core
     const uint16_t *__restrict__ core_au;  // a(u, w) of the U core
     const uint16_t *__restrict__ core_al;  // a(v, x) of the L core
-    // batch plan: bin sizes in device memory (dense, hash, team, warp
-    // starts; a dense start is one item), and the error word whose check
+    // batch plan: bin sizes in device memory (dense, hash, team, warp, -,
+    // tiny starts; a dense start is one item), and the error word whose check
     // failures stop the launch (null otherwise)
     const unsigned long long *__restrict__ item_counts;
     const int *guard;
@@ -106,6 +109,10 @@ __device__ __forceinline__ int64_t n_team_items(const CountParams &p) {
 }
 __device__ __forceinline__ int64_t n_warp_items(const CountParams &p) {
     return p.item_counts ? (int64_t)p.item_counts[3] : p.n_warp;
+}
+
+__device__ __forceinline__ int64_t n_tiny_items(const CountParams &p) {
+    return p.item_counts ? (int64_t)p.item_counts[5] : p.n_tiny;
 }
 
 // The threads that walk one start together: the whole CTA (barrier 0) or one
@@ -273,7 +280,9 @@ __device__ __forceinline__ uint32_t get4(const uint32_t *w32, int idx) {
     return (w32[idx >> 3] >> sh) & 0xfu;
 }
 
-enum CounterKind { kDenseNarrow = 0, kDenseWide = 1, kHash = 2, kDenseByte = 3, kDenseNibble = 4 };
+enum CounterKind { kDenseNarrow = 0, kDenseWide = 1, kHash = 2, kDenseByte = 3, kDenseNibble = 4, kPacked = 5 };
+// tables: kHash keys and 16-bit counts apart; kPacked (key, count) in one word
+__host__ __device__ constexpr bool is_table(int kind) { return kind == kHash || kind == kPacked; }
 
 // the dense counter kind of a start with at most `bound` middles, its chunk
 // span (dense_chunk_span) and the bytes to clear for `span` counters
@@ -437,6 +446,56 @@ __device__ __forceinline__ unsigned long long hash_group(const CountParams &p, c
         s += d[u];
     }
     return !kSecond && has_second_walk(MODE) ? 0u : s;
+}
+
+// The same for a table of (key, count) words, the count in the low `cb` bits:
+// a start whose keys and counts fit 32 bits together and whose table cannot
+// fill up (at most 3/4 of its slots).  An end's first wedge is one
+// compare-and-swap, a later one that and an addition; the first probes of a
+// group are in flight together.
+constexpr uint32_t kEmpty = 0xffffffffu;   // no key is all ones
+template <int MODE, bool kSecond, int N, typename Pos>
+__device__ __forceinline__ unsigned long long packed_group(const CountParams &p, const int32_t (&w)[N],
+                                                           const Pos (&pos)[N], int32_t lb, uint32_t hmask, int cb,
+                                                           uint32_t *tab, uint32_t (&d)[N]) {
+    const uint32_t cmask = (1u << cb) - 1u;
+    uint32_t e[N];
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+        const uint32_t key = (uint32_t)(w[u] - lb), h = hash_slot((int32_t)key, hmask);
+        e[u] = kEmpty;
+        if (w[u] >= 0) {
+            if (!kSecond) e[u] = atomicCAS(tab + h, kEmpty, (key << cb) | 1u);
+            else e[u] = tab[h];
+        }
+    }
+    uint32_t s = 0;
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+        d[u] = 0;
+        if (kSecond ? w[u] >= 0 : e[u] != kEmpty) {
+            const uint32_t key = (uint32_t)(w[u] - lb);
+            uint32_t h = hash_slot((int32_t)key, hmask), left = hmask;
+            while ((e[u] >> cb) != key && e[u] != kEmpty && left > 0) {
+                h = (h + 1) & hmask;
+                --left;
+                e[u] = kSecond ? tab[h] : atomicCAS(tab + h, kEmpty, (key << cb) | 1u);
+            }
+            if ((e[u] >> cb) == key && e[u] != kEmpty) {
+                if (!kSecond) {
+                    const uint32_t old = atomicAdd(tab + h, 1u);
+                    if (!has_second_walk(MODE)) d[u] = old & cmask;
+                } else {
+                    d[u] = (e[u] & cmask) - 1u;
+                    if (wants_edges(MODE)) red_global_if(p.pe + pos[u], d[u]);
+                }
+            } else if (kSecond || e[u] != kEmpty) {
+                atomicOr(p.err, kErrHashFull);   // cannot happen: every end has its slot
+            }
+        }
+        s += d[u];
+    }
+    return s;
 }
 
 // Adds each lane's x to msum[q], where equal q occupy consecutive lanes (the
@@ -638,7 +697,7 @@ __device__ __forceinline__ unsigned long long batch_windows(const CountParams &p
     constexpr int kSegRuns = 4;
     // segments in flight per warp (eight of the second walk's slots and sums do
     // not fit the registers beside a team's or 64-bit positions)
-    constexpr int kSeg = KIND == kHash || (kSecond && wants_edges(MODE) && (sizeof(Pos) == 8 || kThreads != kCountThreads))
+    constexpr int kSeg = is_table(KIND) || (kSecond && wants_edges(MODE) && (sizeof(Pos) == 8 || kThreads != kCountThreads))
                              ? 4 : 8;
     const int lane = t.tid & 31, warp = t.tid >> 5;
     const uint32_t le_mask = 0xffffffffu >> (31 - lane);
@@ -653,6 +712,8 @@ __device__ __forceinline__ unsigned long long batch_windows(const CountParams &p
         constexpr int N = decltype(n_windows)::value;
         if constexpr (KIND == kHash)
             return hash_group<MODE, kSecond, N, Pos>(p, w, pos, lb, hmask, ctr, &sh.overflow, ins, d);
+        else if constexpr (KIND == kPacked)   // the chunk width holds the count's bits
+            return packed_group<MODE, kSecond, N, Pos>(p, w, pos, lb, hmask, span, reinterpret_cast<uint32_t *>(ctr), d);
         else
             return dense_group<MODE, KIND, kSecond, N, Pos>(p, w, pos, base, (uint32_t)span, ctr32, d);
     };
@@ -777,14 +838,14 @@ __device__ unsigned long long team_walk(const CountParams &p, int32_t x, int32_t
         BatchSlots<Pos, kThreads> bs;
         int32_t total;
         int nnz;
-        batch_runs<KIND != kHash, kSecond, Pos>(p, e0, nmid, mb, lb, lo, hi, flags, ctr, 0, sh, t, bs,
+        batch_runs<!is_table(KIND), kSecond, Pos>(p, e0, nmid, mb, lb, lo, hi, flags, ctr, 0, sh, t, bs,
                                                  &total, &nnz);
         t.sync();
         acc += batch_windows<MODE, KIND, kSecond, Pos>(p, lb, lo, span, hmask, ctr, total, nnz, ins, sh, t);
         // Dense counting needs no join here: the next batch's scan barriers
         // come before its compaction overwrites the run arrays, so warps that
         // finish their windows early already load the next batch's slots.
-        if (KIND == kHash || kSecond) t.sync();
+        if (is_table(KIND) || kSecond) t.sync();
         if (KIND == kHash && !kSecond && sh.overflow) break;   // uniform: read after the barrier
         if (kSecond) middle_sums<MODE, Pos>(p, bs, sh);
     }
@@ -817,7 +878,7 @@ __device__ unsigned long long item_body(const CountParams &p, int32_t x, int32_t
             BatchSlots<Pos, kThreads> bs;
             int32_t total;
             int nnz;
-            batch_runs<KIND != kHash, false, Pos>(p, p.off[x], nmid, 0, lb, lo, hi, flags, ctr, 0, sh, t, bs,
+            batch_runs<!is_table(KIND), false, Pos>(p, p.off[x], nmid, 0, lb, lo, hi, flags, ctr, 0, sh, t, bs,
                                                   &total, &nnz);
             t.sync();
             int *const ins = (KIND == kHash && sh.track) ? &sh.inserts : nullptr;
@@ -862,7 +923,15 @@ template <int MODE, int KIND, int kThreads>
 __device__ __forceinline__ void end_contributions(const CountParams &p, int32_t lb, int32_t lo,
                                                   int32_t hi, uint32_t hmask, const unsigned char *ctr,
                                                   const Team<kThreads> &t) {
-    if (KIND == kHash) {
+    if (KIND == kPacked) {
+        const uint32_t *tab = reinterpret_cast<const uint32_t *>(ctr);
+        const int cb = hi - lo;
+        for (uint32_t s = t.tid; s <= hmask; s += kThreads) {
+            const uint32_t e = tab[s];
+            const unsigned long long b = e != kEmpty ? c2(e & ((1u << cb) - 1u)) : 0ull;
+            if (b) atomicAdd(p.pv + lb + (int32_t)(e >> cb), b);
+        }
+    } else if (KIND == kHash) {
         const int32_t *hkeys = reinterpret_cast<const int32_t *>(ctr);
         const uint32_t *hcnt = reinterpret_cast<const uint32_t *>(ctr + (size_t)(hmask + 1) * 4);
         for (uint32_t s = t.tid; s <= hmask; s += kThreads) {
@@ -942,13 +1011,37 @@ __device__ __forceinline__ int64_t middles(const CountParams &p, int32_t x) {
     return p.orient ? p.off[x + 1] - p.off[x] : (int64_t)p.cut[x];
 }
 
-// A start counted by the team with one hash table of at most `max_slots`
-// slots.  Returns its Σ C(count, 2), or sets sh.overflow.
+// The bits of a packed table's count for start x whose ends are the R vertices
+// below it (Algorithm 2), 0 if keys and counts do not fit one word: a count is
+// at most min(cut[x], degree of the last end, work[x]); keys are below R.
+__device__ __forceinline__ int packed_count_bits(const CountParams &p, int32_t x, int32_t R) {
+    if (p.orient || R <= 0) return 0;
+    const int64_t last = p.off[x] - p.off[x - 1];
+    const uint64_t c = min((uint64_t)min((int64_t)p.cut[x], last), (uint64_t)p.work[x]);
+    const int cb = 64 - __clzll((long long)c), kb = 32 - __clz(R);
+    return cb + kb <= 32 ? cb : 0;
+}
+
+// A start counted by the team with one hash table: of (key, count) words with
+// up to `packed_slots` slots where they fit, else of at most `max_slots` slots
+// with keys and counts apart.  Returns its Σ C(count, 2), or sets sh.overflow.
+// 20M-edge power law: with the tiny starts' windows below, the packed table took
+// prepare and total from 11.09 to 10.54 ms; 16 sparse samples of it (1.9M light
+// starts) 15.1 -> 13.4 ms.
 template <int MODE, typename Pos, int kThreads, class SH>
 __device__ unsigned long long hash_item(const CountParams &p, int32_t x, unsigned char *ctr,
-                                        int max_slots, SH &sh, const Team<kThreads> &t) {
+                                        int max_slots, int packed_slots, SH &sh, const Team<kThreads> &t) {
     const int32_t lb = range_lo(p, x);
     const unsigned long long bound = end_bound(p, x, lb);
+    const int cb = bound <= (unsigned long long)(packed_slots / 4 * 3) ? packed_count_bits(p, x, x - lb) : 0;
+    if (cb > 0) {
+        uint32_t cap = 64;
+        while (cap < 2 * bound && cap < (uint32_t)packed_slots) cap <<= 1;
+        if (t.tid == 0) sh.overflow = 0;
+        team_fill(ctr, (int)cap * 4, kEmpty, t);
+        t.sync();
+        return item_body<MODE, kPacked, Pos>(p, x, lb, 0, cb, 0, cap - 1, ctr, sh, t);
+    }
     uint32_t cap = 64;
     while (cap < 2 * bound && cap < (uint32_t)max_slots) cap <<= 1;
     // hash tables hold 16-bit counts; a count is at most min(middles, work)
@@ -1028,7 +1121,7 @@ __device__ unsigned long long cta_item(const CountParams &p, int2 item, unsigned
             : kind == kDenseByte ? item_body<MODE, kDenseByte, Pos>(p, x, lb, lo, hi, flags, 0, ctr, sh, t)
                                  : item_body<MODE, kDenseNibble, Pos>(p, x, lb, lo, hi, flags, 0, ctr, sh, t);
     } else {
-        acc = hash_item<MODE, Pos>(p, x, ctr, kHashMaxSlots, sh, t);
+        acc = hash_item<MODE, Pos>(p, x, ctr, kHashMaxSlots, kHashMaxSlots, sh, t);
         if (sh.overflow) {
             // the CTA table was too small: dense chunks next
             if (t.tid == 0) push_retry(p, -(x + 1));
@@ -1163,7 +1256,8 @@ __device__ unsigned long long team_item(const CountParams &p, int32_t x, unsigne
         acc = narrow ? item_body<MODE, kDenseNarrow, Pos>(p, x, lb, 0, R, 0, 0, table, sh, t)
                      : item_body<MODE, kDenseByte, Pos>(p, x, lb, 0, R, 0, 0, table, sh, t);
     } else {
-        acc = hash_item<MODE, Pos>(p, x, table, kTeamSlots, sh, t);
+        acc = hash_item<MODE, Pos>(p, x, table, kTeamSlots, p.work[x] <= (uint64_t)kTeamFitWork ? kTeamPackedSlots : 0,
+                                   sh, t);
         if (sh.overflow) {
             // a CTA table next
             if (t.tid == 0) push_retry(p, x);
@@ -1180,8 +1274,10 @@ __device__ unsigned long long team_item(const CountParams &p, int32_t x, unsigne
 // The warp version of team_walk for a light start: batches of 32 middles,
 // compacted runs and the same window masks, with a per-warp hash table that
 // always fits (at most 384 wedges, 512 slots).
+// cb > 0: a table of (key, count) words of 1,024 slots, the count in the low cb
+// bits; cb = 0: keys and counts apart, 512 slots.
 template <int MODE, bool kSecond>
-__device__ unsigned long long warp_walk(const CountParams &p, int32_t x, int32_t lb, uint32_t mask,
+__device__ unsigned long long warp_walk(const CountParams &p, int32_t x, int32_t lb, uint32_t mask, int cb,
                                         int32_t *keys, uint32_t *cnt, uint2 *msum,
                                         int32_t *wstart, long long *wsrc) {
     const int lane = threadIdx.x & 31;
@@ -1232,10 +1328,18 @@ __device__ unsigned long long warp_walk(const CountParams &p, int32_t x, int32_t
                 bool good = true;
                 if (pos < 0 || pos >= p.adj_len) { atomicOr(p.err, kErrBounds); good = false; }
                 const int32_t w = good ? __ldg(p.adj + pos) : 0;
-                const int slot = good ? hash_find(keys, mask, w - lb, !kSecond) : -1;
-                if (good && slot < 0) atomicOr(p.err, kErrHashFull);
-                if (slot >= 0) {
-                    if (!kSecond) {
+                if (good && cb > 0) {
+                    const int32_t w1[1] = {w};
+                    const long long p1[1] = {pos};
+                    uint32_t d1[1];
+                    const uint32_t t = (uint32_t)packed_group<MODE, kSecond, 1, long long>(
+                        p, w1, p1, lb, mask, cb, reinterpret_cast<uint32_t *>(keys), d1);
+                    if (kSecond) delta = t; else acc += t;
+                } else if (good) {
+                    const int slot = hash_find(keys, mask, w - lb, !kSecond);
+                    if (slot < 0) {
+                        atomicOr(p.err, kErrHashFull);
+                    } else if (!kSecond) {
                         const uint32_t old = atomicAdd(cnt + slot, 1u);
                         if (!has_second_walk(MODE)) acc += old;
                     } else {
@@ -1272,25 +1376,36 @@ __device__ unsigned long long warp_item(const CountParams &p, int32_t x, unsigne
     const int lane = threadIdx.x & 31;
     const int32_t lb = range_lo(p, x);
     const unsigned long long bound = end_bound(p, x, lb);
+    const int cb = packed_count_bits(p, x, x - lb);
     uint32_t cap = 32;
-    while (cap < 2 * bound && cap < (uint32_t)kWarpSlots) cap <<= 1;
+    while (cap < 2 * bound && cap < (uint32_t)(cb > 0 ? 2 * kWarpSlots : kWarpSlots)) cap <<= 1;
     int32_t *keys = reinterpret_cast<int32_t *>(region);
     uint32_t *cnt = reinterpret_cast<uint32_t *>(region + kWarpCntOff);
     uint2 *msum = reinterpret_cast<uint2 *>(region + kWarpMsumOff);
     long long *wsrc = reinterpret_cast<long long *>(region + kWarpSrcOff);
     int32_t *wstart = reinterpret_cast<int32_t *>(region + kWarpStartOff);
-    for (uint32_t s = lane; s < cap; s += 32) { keys[s] = -1; cnt[s] = 0; }
+    if (cb > 0) {
+        uint4 *t4 = reinterpret_cast<uint4 *>(region);
+        for (uint32_t s = lane; s < cap / 4; s += 32) t4[s] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
+    } else {
+        for (uint32_t s = lane; s < cap; s += 32) { keys[s] = -1; cnt[s] = 0; }
+    }
     __syncwarp();
-    unsigned long long acc = warp_walk<MODE, false>(p, x, lb, cap - 1, keys, cnt, msum, wstart, wsrc);
+    unsigned long long acc = warp_walk<MODE, false>(p, x, lb, cap - 1, cb, keys, cnt, msum, wstart, wsrc);
     if (has_second_walk(MODE)) {
         __syncwarp();
         if (wants_vertices(MODE)) {
             for (uint32_t s = lane; s < cap; s += 32) {
                 const int32_t k = keys[s];
-                if (k >= 0 && cnt[s] >= 2) atomicAdd(p.pv + lb + k, c2(cnt[s]));
+                if (cb > 0) {
+                    const uint32_t e = (uint32_t)k, c = e & ((1u << cb) - 1u);
+                    if (e != kEmpty && c >= 2) atomicAdd(p.pv + lb + (int32_t)(e >> cb), c2(c));
+                } else if (k >= 0 && cnt[s] >= 2) {
+                    atomicAdd(p.pv + lb + k, c2(cnt[s]));
+                }
             }
         }
-        acc = warp_walk<MODE, true>(p, x, lb, cap - 1, keys, cnt, msum, wstart, wsrc);
+        acc = warp_walk<MODE, true>(p, x, lb, cap - 1, cb, keys, cnt, msum, wstart, wsrc);
         if (wants_vertices(MODE)) {
             unsigned long long t = acc;
 #pragma unroll
@@ -1305,6 +1420,117 @@ __device__ unsigned long long warp_item(const CountParams &p, int32_t x, unsigne
         if (lane == 0 && t) atomicAdd(p.gtot + p.gstar[x], t);
     }
     __syncwarp();
+    return acc;
+}
+
+// Starts of at most 32 wedges (and 32 middles), one window each: equal ends are
+// found by one warp match, with no table.  A warp takes 32 starts, reads their
+// offsets and cuts together, and runs them through two stages, so that the next
+// start's slots and this start's ends load while the one before is counted: a
+// start alone is a chain of five loads of about 700 clocks.
+template <int MODE, typename Pos>
+__device__ unsigned long long tiny_items(const CountParams &p, unsigned char *region) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t le_mask = 0xffffffffu >> (31 - lane), lt_mask = (1u << lane) - 1u;
+    Pos *const wsrc = reinterpret_cast<Pos *>(region);                          // [2][32] by run
+    int32_t *const wslot = reinterpret_cast<int32_t *>(region + 2 * 32 * 8);    // [2][32] lane of a run's middle
+    const int64_t n_tiny = n_tiny_items(p);
+    unsigned long long acc = 0;
+    for (;;) {
+        int it = 0;
+        if (lane == 0) it = atomicAdd(p.cursors + 5, 32);
+        it = __shfl_sync(0xffffffffu, it, 0);
+        if (it >= n_tiny || it < 0) break;
+        const int cnt = (int)min((int64_t)32, n_tiny - it);
+        int32_t x = 0, nm = 0;
+        Pos e0 = 0;
+        if (lane < cnt) {
+            x = p.warp_items[p.n - 1 - it - lane];
+            e0 = (Pos)p.off[x];
+            nm = p.cut[x];
+        }
+        // the slots of start 0
+        int32_t len = 0, v = 0, len_n = 0, v_n = 0;
+        Pos src = 0, src_n = 0;
+        auto slots = [&](int k, int32_t &len_k, int32_t &v_k, Pos &src_k) {
+            const Pos e = __shfl_sync(0xffffffffu, e0, k) + (Pos)lane;
+            const int32_t m = __shfl_sync(0xffffffffu, nm, k);
+            len_k = 0;
+            src_k = 0;
+            v_k = 0;
+            if (lane < m) {
+                len_k = __ldg(p.plen + e);
+                src_k = (Pos)__ldg(p.sbeg + e);
+                if (wants_vertices(MODE)) v_k = __ldg(p.adj + e);
+            }
+        };
+        slots(0, len, v, src);
+        // the start before: its ends, positions, runs and middles
+        int32_t w_p = -1, total_p = 0, q_p = 0, v_p = 0;
+        Pos pos_p = 0;
+        for (int k = 0; k <= cnt; ++k) {
+            int32_t w = -1, total = 0, q = 0;
+            Pos pos = 0;
+            const int par = (k & 1) * 32;
+            if (k < cnt) {   // uniform
+                int32_t incl = len;
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    const int32_t o = __shfl_up_sync(0xffffffffu, incl, d);
+                    if (lane >= d) incl += o;
+                }
+                total = min(__shfl_sync(0xffffffffu, incl, 31), 32);   // at most 32 by its bin
+                const int32_t excl = incl - len;
+                const uint32_t some = __ballot_sync(0xffffffffu, len > 0);
+                // the run starts of the window (a start beyond it would have no bit)
+                const uint32_t m = __reduce_or_sync(0xffffffffu, len > 0 && excl < 32 ? 1u << excl : 0u);
+                const int nz = __popc(some & lt_mask);
+                if (len > 0) {
+                    wsrc[par + nz] = src - (Pos)excl;
+                    wslot[par + nz] = lane;
+                }
+                __syncwarp();
+                q = __popc(m & le_mask) - 1;
+                if (lane < total && q >= 0) {
+                    pos = wsrc[par + q] + (Pos)lane;
+                    if (pos >= 0 && (int64_t)pos < p.adj_len) w = __ldg(p.adj + pos);
+                    else atomicOr(p.err, kErrBounds);
+                }
+                if (k + 1 < cnt) slots(k + 1, len_n, v_n, src_n);
+            }
+            if (k > 0 && total_p > 0) {   // uniform: count start k - 1
+                const uint32_t peers = __match_any_sync(0xffffffffu, w_p >= 0 ? w_p : -1 - lane);
+                const uint32_t c = (uint32_t)__popc(peers), old = (uint32_t)__popc(peers & lt_mask);
+                const bool on = w_p >= 0;
+                const uint32_t d = on ? (has_second_walk(MODE) ? c - 1u : old) : 0u;
+                acc += d;
+                if ((MODE == kModeBatch || has_second_walk(MODE)) && __any_sync(0xffffffffu, d > 0)) {
+                    const int32_t xk = __shfl_sync(0xffffffffu, x, k - 1);
+                    const uint32_t sum = __reduce_add_sync(0xffffffffu, d);
+                    if (MODE == kModeBatch && lane == 0) atomicAdd(p.gtot + p.gstar[xk], (unsigned long long)sum);
+                    if (wants_vertices(MODE)) {
+                        if (lane == 0) atomicAdd(p.pv + xk, (unsigned long long)(sum / 2));
+                        if (on && old == 0 && c >= 2) atomicAdd(p.pv + w_p, c2(c));
+                    }
+                    if (has_second_walk(MODE)) {
+                        const int ml = wslot[(par ^ 32) + max(q_p, 0)] & 31;
+                        const int32_t vm = __shfl_sync(0xffffffffu, v_p, ml);
+                        const int64_t ek = (int64_t)__shfl_sync(0xffffffffu, e0, k - 1) + ml;
+                        if (d > 0) {
+                            if (wants_vertices(MODE)) atomicAdd(p.pv + vm, (unsigned long long)d);
+                            if (wants_edges(MODE)) {
+                                atomicAdd(p.pe + pos_p, (unsigned long long)d);
+                                atomicAdd(p.pe + edge_slot(p, ek), (unsigned long long)d);
+                            }
+                        }
+                    }
+                }
+            }
+            w_p = w; total_p = total; q_p = q; pos_p = pos; v_p = v;
+            len = len_n; src = src_n; v = v_n;
+            __syncwarp();
+        }
+    }
     return acc;
 }
 
@@ -1343,7 +1569,7 @@ __global__ void __launch_bounds__(kCountThreads, kCountCtasPerSm) k_count(CountP
     if (n_team > 0) {
         typedef SharedTeam<MODE, Pos, kTeamThreads> TS;
         constexpr int kDenseBytes = (int)(kTeamRegion - sizeof(TS)) & ~15;
-        static_assert(kTeamTableBytes <= kDenseBytes, "team region overflow");
+        static_assert(kTeamTableBytes <= kDenseBytes && kTeamPackedSlots * 4 <= kDenseBytes, "team region overflow");
         const int k = threadIdx.x / kTeamThreads;
         const Team<kTeamThreads> team{(int)(threadIdx.x % kTeamThreads), 1 + k};
         unsigned char *table = ctr + (size_t)k * kTeamRegion;
@@ -1366,13 +1592,15 @@ __global__ void __launch_bounds__(kCountThreads, kCountCtasPerSm) k_count(CountP
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
         unsigned char *region = ctr + (size_t)warp * kWarpRegion;
         const int64_t n_warp = n_warp_items(p);
+        const int grab = n_warp >= (int64_t)gridDim.x * kCountWarps * 16 ? 4 : 1;
         for (;;) {
             int it = 0;
-            if (lane == 0) it = atomicAdd(p.cursors + 1, 1);
+            if (lane == 0) it = atomicAdd(p.cursors + 1, grab);
             it = __shfl_sync(0xffffffffu, it, 0);
             if (it >= n_warp) break;
-            acc += warp_item<MODE>(p, p.warp_items[it], region);
+            for (int64_t j = it; j < min((int64_t)it + grab, n_warp); ++j) acc += warp_item<MODE>(p, p.warp_items[j], region);
         }
+        if (n_tiny_items(p) > 0) acc += tiny_items<MODE, Pos>(p, region);
     }
     // a7: reduction of the per-thread partial sums (twice ⋈ with a second walk)
     const unsigned long long t = team_sum(acc, sh, cta) / (has_second_walk(MODE) ? 2 : 1);
@@ -1401,7 +1629,7 @@ __global__ void __launch_bounds__(kCountThreads, kCountCtasPerSm) k_count_retry(
         unsigned long long item_acc = 0;
         bool done = false;
         if (entry >= 0) {
-            item_acc = hash_item<MODE, Pos>(p, x, ctr, kHashMaxSlots, sh, cta);
+            item_acc = hash_item<MODE, Pos>(p, x, ctr, kHashMaxSlots, 0, sh, cta);
             done = !sh.overflow;
             __syncthreads();
         }
@@ -1514,6 +1742,7 @@ int launch_count(Graph *g, cudaStream_t s, int mode, unsigned long long *pv_proj
     p.work = g->work; p.cta_items = g->cta_items; p.team_items = g->team_items;
     p.warp_items = g->warp_items;
     p.n_cta = g->n_cta_items; p.n_team = g->n_team_items; p.n_warp = g->n_warp_items;
+    p.n_tiny = g->n_tiny_items;
     p.cursors = g->cursors; p.acc = g->acc; p.pv = pv_proj; p.pe = pe;
     // the chunk-boundary table is relative to the start of each list, which
     // is where Algorithm 2's runs start

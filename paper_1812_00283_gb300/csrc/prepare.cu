@@ -843,71 +843,72 @@ __device__ __forceinline__ bool forced_dense(int32_t x, int32_t l, int32_t core_
 
 // Bins of a6: 0 dense (work > hash_max), 1 CTA hash (team_max < work <=
 // hash_max), 2 team (warp_max < work <= team_max), 3 warp (0 < work <= warp_max).
+// 5: of the warp bin, the starts of at most 32 wedges and 32 middles
+// (Algorithm 2), which take one window and no table.
 struct BinBounds {
     uint64_t warp_max, team_max, hash_max;
     int32_t l, core_lo_u, core_lo_l;
+    const int32_t *cut;   // null: no bin 5
     __device__ __forceinline__ int of(int32_t x, uint64_t w) const {
         if (w > hash_max || forced_dense(x, l, core_lo_u, core_lo_l, w)) return 0;
-        return w > team_max ? 1 : (w > warp_max ? 2 : (w > 0 ? 3 : 4));
+        if (w > warp_max) return w > team_max ? 1 : 2;
+        if (w == 0) return 4;
+        return cut && w <= (uint64_t)kTinyMax && cut[x] <= kTinyMax ? 5 : 3;
     }
 };
 
-// The starts of each bin: counts[b], the warp bin's starts in `warp_items` and
-// the others' in `heavy` (in no order; only the heavy ones, a few per cent of
-// the starts with work, are then sorted).  A CTA takes 2,048 starts and reserves
+// The starts of each bin: counts[b] (and [4]: bins 0 to 2 together), bin 3 from
+// the front of warp_items[n], bin 5 from its back, and the others in `heavy` (in
+// no order; only the heavy ones, a few per cent of the starts with work, are
+// then sorted).  A CTA takes 2,048 starts and reserves
 // their room with one addition per list.
 constexpr int kBinTile = 8 * kT;
 __global__ void __launch_bounds__(kT) k_bin_starts(const uint64_t *__restrict__ work, int32_t n, BinBounds bb,
                                                    unsigned long long *counts, int32_t *heavy, int32_t *warp_items,
     const int *guard = nullptr) {
     if (aborted(guard)) return;
-    __shared__ int32_t cnt[4], at_heavy, at_warp;
+    __shared__ int32_t cnt[6], at[3];   // at: this tile's room in heavy, warp front, warp back
     const int lane = threadIdx.x & 31;
     const uint32_t lt = (1u << lane) - 1u;
     for (int64_t x0 = (int64_t)blockIdx.x * kBinTile; x0 < n; x0 += (int64_t)gridDim.x * kBinTile) {
-        if (threadIdx.x < 4) cnt[threadIdx.x] = 0;
+        if (threadIdx.x < 6) cnt[threadIdx.x] = 0;
         __syncthreads();
-        int bin[8], place[8];   // place: among the tile's heavy, or warp, starts
+        int bin[8], place[8];   // place: among the tile's starts of the same list
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int64_t x = x0 + i * kT + threadIdx.x;
             bin[i] = x < n ? bb.of((int32_t)x, work[x]) : 4;
         }
+        // cnt[0..2]: bins; cnt[3], cnt[5]: lists of their own; cnt[4]: the heavy list
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
 #pragma unroll
-            for (int b = 0; b < 4; ++b) {
+            for (int b = 0; b < 3; ++b) {
                 const uint32_t m = __ballot_sync(0xffffffffu, bin[i] == b);
-                if (b == 3) {
-                    int o = 0;
-                    if (lane == 0 && m) o = atomicAdd(&cnt[3], __popc(m));
-                    o = __shfl_sync(0xffffffffu, o, 0);
-                    if (bin[i] == 3) place[i] = o + __popc(m & lt);
-                } else if (lane == 0 && m) {
-                    atomicAdd(&cnt[b], __popc(m));
-                }
+                if (lane == 0 && m) atomicAdd(&cnt[b], __popc(m));
             }
+            const uint32_t mh = __ballot_sync(0xffffffffu, bin[i] < 3), mw = __ballot_sync(0xffffffffu, bin[i] == 3),
+                           mt = __ballot_sync(0xffffffffu, bin[i] == 5);
+            int o = 0;
+            if (lane == 0 && mh) o = atomicAdd(&cnt[4], __popc(mh));
+            if (lane == 1 && mw) o = atomicAdd(&cnt[3], __popc(mw));
+            if (lane == 2 && mt) o = atomicAdd(&cnt[5], __popc(mt));
+            const int oh = __shfl_sync(0xffffffffu, o, 0), ow = __shfl_sync(0xffffffffu, o, 1),
+                      ot = __shfl_sync(0xffffffffu, o, 2);
+            place[i] = bin[i] < 3 ? oh + __popc(mh & lt) : (bin[i] == 3 ? ow + __popc(mw & lt) : ot + __popc(mt & lt));
         }
         __syncthreads();
-        if (threadIdx.x == 0) {
-            const int32_t h = cnt[0] + cnt[1] + cnt[2];
-            at_heavy = h ? (int32_t)atomicAdd(counts + 4, (unsigned long long)h) : 0;
-            at_warp = cnt[3] ? (int32_t)atomicAdd(counts + 3, (unsigned long long)cnt[3]) : 0;
-            for (int b = 0; b < 3; ++b)
-                if (cnt[b]) atomicAdd(counts + b, (unsigned long long)cnt[b]);
+        if (threadIdx.x < 6 && cnt[threadIdx.x] > 0) {
+            const int32_t o = (int32_t)atomicAdd(counts + threadIdx.x, (unsigned long long)cnt[threadIdx.x]);
+            if (threadIdx.x >= 3) at[threadIdx.x == 4 ? 0 : (threadIdx.x == 3 ? 1 : 2)] = o;
         }
-        __syncthreads();
-        if (threadIdx.x == 0) cnt[0] = 0;   // now the place among the heavy ones
         __syncthreads();
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int32_t x = (int32_t)(x0 + i * kT + threadIdx.x);
-            const uint32_t m = __ballot_sync(0xffffffffu, bin[i] < 3);
-            int o = 0;
-            if (lane == 0 && m) o = atomicAdd(&cnt[0], __popc(m));
-            o = __shfl_sync(0xffffffffu, o, 0);
-            if (bin[i] < 3) heavy[at_heavy + o + __popc(m & lt)] = x;
-            if (bin[i] == 3) warp_items[at_warp + place[i]] = x;
+            if (bin[i] < 3) heavy[at[0] + place[i]] = x;
+            else if (bin[i] == 3) warp_items[at[1] + place[i]] = x;
+            else if (bin[i] == 5) warp_items[n - 1 - at[2] - place[i]] = x;
         }
         __syncthreads();
     }
@@ -1207,14 +1208,15 @@ static BinBounds bin_bounds(const Graph *g, int32_t warp_max_work, int32_t team_
     bb.l = g->l;
     bb.core_lo_u = g->core_u > 0 ? g->core_lo_u : g->n;
     bb.core_lo_l = g->core_l > 0 ? g->core_lo_l : g->n;
+    bb.cut = vpp ? nullptr : g->cut;
     return bb;
 }
 
-// Starts the binning of all starts on s: counts[0..4] (zeroed here) = dense,
-// hash, team, warp, and all but the warp bin together; g->warp_items is filled.
+// Starts the binning of all starts on s: counts[0..5] (zeroed here) = dense,
+// hash, team, warp, the first three together, tiny; g->warp_items is filled.
 static int bin_starts(Graph *g, cudaStream_t s, const BinBounds &bb, unsigned long long *counts, int32_t *heavy,
                       const int *guard) {
-    BFC_CUDA(cudaMemsetAsync(counts, 0, 5 * sizeof(unsigned long long), s));
+    BFC_CUDA(cudaMemsetAsync(counts, 0, 6 * sizeof(unsigned long long), s));
     if (g->n == 0) return BFC_OK;
     k_bin_starts<<<(unsigned)std::min<int64_t>(((int64_t)g->n + kBinTile - 1) / kBinTile, 152 * 8), kT, 0, s>>>(
         g->work, g->n, bb, counts, heavy, g->warp_items, guard); note_launch();
@@ -1226,7 +1228,7 @@ static int bin_starts(Graph *g, cudaStream_t s, const BinBounds &bb, unsigned lo
 // warp, CTA-hash and CTA-dense bins (dense starts into end-range chunks);
 // builds the chunk-boundary table when a dense start has several chunks.
 // `rows_star` (slot -> vertex of G*) may be null; it is rebuilt when needed.
-// hc[0..4] and `heavy` are bin_starts' results with the bounds bb.  Only reads
+// hc[0..5] and `heavy` are bin_starts' results with the bounds bb.  Only reads
 // memory of the library.
 static int schedule_graph(Graph *g, cudaStream_t s, int32_t warp_max_work, int32_t team_max_work,
                           int32_t hash_max_work, const int32_t *rows_star, const BinBounds &bb,
@@ -1246,9 +1248,10 @@ static int schedule_graph(Graph *g, cudaStream_t s, int32_t warp_max_work, int32
         }                                                                             \
     } while (0)
     const uint64_t maxw = g->info.max_start_work, team_max = bb.team_max;
-    int64_t n_dense = 0, n_hash = 0, n_team = 0, n_warp = 0, n_items = 0, h_dense_items = 0;
+    int64_t n_dense = 0, n_hash = 0, n_team = 0, n_warp = 0, n_tiny = 0, n_items = 0, h_dense_items = 0;
     if (n > 0 && g->info.wedges > 0) {
         n_dense = (int64_t)hc[0]; n_hash = (int64_t)hc[1]; n_team = (int64_t)hc[2]; n_warp = (int64_t)hc[3];
+        n_tiny = (int64_t)hc[5];
         const int64_t n_heavy = n_dense + n_hash + n_team;
         uint64_t *k0 = nullptr, *k1 = nullptr;
         int32_t *v1 = nullptr;
@@ -1362,6 +1365,7 @@ static int schedule_graph(Graph *g, cudaStream_t s, int32_t warp_max_work, int32
     g->n_cta_items = n_items;
     g->n_team_items = n_team;
     g->n_warp_items = n_warp;
+    g->n_tiny_items = n_tiny;
     g->team_max = (int32_t)std::min<uint64_t>(team_max, (uint64_t)kTeamMaxWork);
     // each hash start is re-queued at most once per launch
     g->mem.drop(g->retry);
@@ -1380,11 +1384,11 @@ static int schedule_graph(Graph *g, cudaStream_t s, int32_t warp_max_work, int32
     // wedges (4,096 slots) and a CTA start at most 24,576 (32,768 slots)
     g->may_retry = vpp ? (n_hash + n_team > 0) : (n_team > 0 && team_max > (uint64_t)kTeamFitWork);
     g->info.dense_items = h_dense_items;
-    g->info.starts_with_work = n_dense + n_hash + n_team + n_warp;
+    g->info.starts_with_work = n_dense + n_hash + n_team + n_warp + n_tiny;
     g->info.dense_starts = n_dense;
     g->info.hash_starts = n_hash;
     g->info.team_starts = n_team;
-    g->info.warp_starts = n_warp;
+    g->info.warp_starts = n_warp + n_tiny;
     g->opt.warp_max_work = warp_max_work;
     g->opt.team_max_work = team_max_work;
     g->opt.hash_max_work = hash_max_work;
@@ -1403,8 +1407,8 @@ int rebin_graph(Graph *g, cudaStream_t s, int32_t warp_max_work, int32_t team_ma
     tmp.stream = s;
     struct TmpGuard { Allocs *a; ~TmpGuard() { a->release(); } } guard{&tmp};
     int32_t *heavy;
-    unsigned long long *counts, hc[5] = {0, 0, 0, 0, 0};
-    if (tmp.get(&heavy, (size_t)std::max(g->n, 1)) || tmp.get(&counts, 5)) {
+    unsigned long long *counts, hc[6] = {0, 0, 0, 0, 0, 0};
+    if (tmp.get(&heavy, (size_t)std::max(g->n, 1)) || tmp.get(&counts, 6)) {
         set_last_error("device allocation failed: bins");
         return BFC_ERR_OUT_OF_MEMORY;
     }
@@ -1599,8 +1603,8 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
     int32_t *v0, *v1, *deg_u, *deg_l, *deg_star, *rows_star, *heads, *big, *n_big, *heavy;
     uint32_t *hist, *hist_tmp;
     int64_t *scan64_tmp, *deg64;
-    // [0] W, [1] heaviest start, [2] starts beyond the CTA-hash bin, [3..8) bin
-    // counts, [8] / [9] largest L / U degree
+    // [0] W, [1] heaviest start, [2] starts beyond the CTA-hash bin, [3..9) bin
+    // counts, [9] / [10] largest L / U degree
     unsigned long long *red;
     GET(tmp, k0, nsort + 1); GET(tmp, k1, nsort + 1);
     GET(tmp, v0, nsort); GET(tmp, v1, nsort);
@@ -1612,9 +1616,9 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
     GET(tmp, scan64_tmp, std::max(scan_tmp_elems<int64_t>((int64_t)n + 1),
                                   max_scan_tmp_elems(m)));
     GET(tmp, deg64, (int64_t)n + 1);
-    GET(tmp, red, 10);
+    GET(tmp, red, 12);
     GET(tmp, heavy, std::max(n, 1));
-    BFC_CUDA(cudaMemsetAsync(red, 0, 10 * sizeof(unsigned long long), s));
+    BFC_CUDA(cudaMemsetAsync(red, 0, 12 * sizeof(unsigned long long), s));
 
     // ---- a1: degrees, and the check of the caller's offsets and L ids
     BFC_CUDA(cudaMemsetAsync(deg_l, 0, sizeof(int32_t) * std::max<int64_t>(l, 1), s));
@@ -1625,7 +1629,7 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
     // ---- a2: per-layer priority ranks by a stable sort on (layer, graph, degree)
     {
         int rc = launch_ranks(g, deg_l, deg_u, graph_l_start, graph_u_start, g->max_range, k0, v0, k1, v1, hist,
-                              hist_tmp, deg_star, deg64, red + 8, s, guard_err);
+                              hist_tmp, deg_star, deg64, red + 9, s, guard_err);
         if (rc) return rc;
     }
 
@@ -1745,15 +1749,15 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
         int rc = bin_starts(g, s, bb, red + 3, heavy, guard_err);
         if (rc) return rc;
     }
-    unsigned long long hred[10] = {0};
+    unsigned long long hred[12] = {0};
     BFC_CUDA(cudaMemcpyAsync(hred, red, sizeof(hred), cudaMemcpyDeviceToHost, s));
     BFC_CUDA(cudaMemcpyAsync(&herr, g->err, sizeof(int), cudaMemcpyDeviceToHost, s));
     BFC_CUDA(cudaStreamSynchronize(s));
     if (int rc = input_error(herr, num_graphs)) return rc;
     g->info.wedges = hred[0];
     g->info.max_start_work = hred[1];
-    g->info.max_deg_l = (int32_t)hred[8];
-    g->info.max_deg_u = (int32_t)hred[9];
+    g->info.max_deg_l = (int32_t)hred[9];
+    g->info.max_deg_u = (int32_t)hred[10];
 
     // ---- dense-core hybrid (Algorithm 2 single graphs): the requested core
     // size, or (core_vertices = -1) as many vertices as starts heavier than
@@ -1775,7 +1779,7 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
         bb = bin_bounds(g, opt->warp_max_work, opt->team_max_work, opt->hash_max_work);
         int rc = bin_starts(g, s, bb, red + 3, heavy, nullptr);
         if (rc) return rc;
-        BFC_CUDA(cudaMemcpyAsync(hred + 3, red + 3, 5 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
+        BFC_CUDA(cudaMemcpyAsync(hred + 3, red + 3, 6 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
         BFC_CUDA(cudaStreamSynchronize(s));
     }
     {
@@ -1884,7 +1888,7 @@ int batch_plan_create(BatchPlan *pl, cudaStream_t s) {
     GET(pl->hist, radix_hist_elems(nsort));
     GET(pl->hist_tmp, scan_tmp_elems<uint32_t>((int64_t)radix_hist_elems(nsort)));
     GET(pl->scan64_tmp, std::max(scan_tmp_elems<int64_t>((int64_t)n + 1), max_scan_tmp_elems(m)));
-    GET(pl->deg64, (int64_t)n + 1); GET(pl->red, 10); GET(pl->heavy, n);
+    GET(pl->deg64, (int64_t)n + 1); GET(pl->red, 12); GET(pl->heavy, n);
 #undef GET
     // every kept array starts zeroed: a run that stops at the checks leaves
     // arrays that later kernels can still index safely
@@ -1922,10 +1926,10 @@ int batch_plan_run(BatchPlan *pl, const int32_t *off_u, const int32_t *adj_u, co
     BFC_CUDA(cudaMemsetAsync(pl->deg_l, 0, sizeof(int32_t) * std::max<int64_t>(l, 1), s));
     if (m > 0) { k_deg_l<<<grid_stride_blocks(m), kT, 0, s>>>(adj_u, m, l, pl->deg_l, g->err); note_launch(); }
     BFC_CUDA(cudaGetLastError());
-    BFC_CUDA(cudaMemsetAsync(pl->red, 0, 10 * sizeof(unsigned long long), s));
+    BFC_CUDA(cudaMemsetAsync(pl->red, 0, 12 * sizeof(unsigned long long), s));
     // ---- a2: graph-major ranks; a degree is below 2^16 (at most the other layer)
     int rc = launch_ranks(g, pl->deg_l, pl->deg_u, gl, gu, pl->max_layer, pl->k0, pl->v0, pl->k1, pl->v1, pl->hist,
-                          pl->hist_tmp, pl->deg_star, pl->deg64, pl->red + 8, s, guard);
+                          pl->hist_tmp, pl->deg_star, pl->deg64, pl->red + 9, s, guard);
     if (rc) return rc;
     if (n > 0) {
         k_graph_star<<<grid_stride_blocks(n), kT, 0, s>>>(r, l, gu, gl, G, g->gstar, g->vbase, g->vend, guard); note_launch();
@@ -1963,7 +1967,7 @@ int batch_plan_run(BatchPlan *pl, const int32_t *off_u, const int32_t *adj_u, co
     // hold the largest key and stay behind), which order them to a quarter octave
     unsigned long long *bins = pl->red + 3;
     if (n > 0) {
-        const BinBounds bb{(uint64_t)opt->warp_max_work, pl->team_max, (uint64_t)opt->hash_max_work, l, n, n};
+        const BinBounds bb{(uint64_t)opt->warp_max_work, pl->team_max, (uint64_t)opt->hash_max_work, l, n, n, g->cut};
         rc = bin_starts(g, s, bb, bins, pl->heavy, guard);
         if (rc) return rc;
         k_sched_keys_plan<<<blocks_for(n), kT, 0, s>>>(g->work, pl->heavy, n, bb, bins, pl->k0); note_launch();
