@@ -669,9 +669,9 @@ __device__ __forceinline__ void batch_runs(const CountParams &p, int64_t e0, int
 // contiguous range per warp, and a warp takes its range in three ways:
 //   - at least 256 wedges of the current run left: eight windows of 32, no run
 //     lookup, eight end loads in flight per lane;
-//   - else, where the next runs are long enough, eight segments of at most 32
-//     wedges (four of a hash table), each inside one run (the run, its start and its end are the same
-//     in every lane, so no lane searches and a run's δ sum is one reduction);
+//   - else, where the next runs are long enough, segments of at most 32 wedges,
+//     each inside one run (no lane searches and a run's δ sum is one
+//     reduction), eight in flight (four of a hash table);
 //   - else (many runs per 32 wedges) four windows across runs: the run of every
 //     lane is found from a 32-bit mask of run starts (reduce-or + popc).
 // Bound by instruction issue and load latency (53-63% issue, DRAM and L2 below
@@ -690,11 +690,20 @@ __device__ __forceinline__ unsigned long long batch_windows(const CountParams &p
                                                             int *ins, SH &sh, const Team<kThreads> &t) {
     constexpr int kWarps = kThreads / 32;
     constexpr int kU = 4;
-    // four segments against four windows: a window across runs costs about
-    // 17 instructions of lookup (and 25 for the segmented δ sums) that a
-    // segment does not, so segments win from this many wedges in four runs up
-    constexpr int32_t kSegMin = kSecond ? 64 : 96;
-    constexpr int kSegRuns = 4;
+    // A window across runs costs about 17 instructions of lookup (and 25 for the
+    // segmented δ sums) that a segment does not; a segment of n wedges costs
+    // 32 / n times the rest.  So segments are taken where four runs hold this
+    // many wedges.  The second walk of a CTA, whose warps have long ranges,
+    // describes 32 segments at a time in its lanes, where 16 runs hold 20
+    // wedges each (per-edge counts of a 30M-edge shopping graph 7.66 -> 7.24 ms,
+    // per-vertex counts of a 6M-edge graph 3.47 -> 3.39); in the first walk and
+    // for the light starts' tables and teams that was no better (20M-edge power
+    // law 10.53 -> 10.63, 16 sparse samples 13.4 -> 13.5).
+    constexpr bool kLaned = kSecond && !is_table(KIND) && kThreads == kCountThreads;
+    constexpr int kOneRuns = 4;
+    constexpr int32_t kOneMin = kSecond ? 64 : 96;
+    constexpr int kLanedRuns = 16;
+    constexpr int32_t kLanedMin = kLanedRuns * 20;
     // segments in flight per warp (eight of the second walk's slots and sums do
     // not fit the registers beside a team's or 64-bit positions)
     constexpr int kSeg = is_table(KIND) || (kSecond && wants_edges(MODE) && (sizeof(Pos) == 8 || kThreads != kCountThreads))
@@ -717,15 +726,16 @@ __device__ __forceinline__ unsigned long long batch_windows(const CountParams &p
         else
             return dense_group<MODE, KIND, kSecond, N, Pos>(p, w, pos, base, (uint32_t)span, ctr32, d);
     };
-    // the δ sum of one run's lanes goes to middle q
-    auto flush = [&](int q, unsigned long long x) {
-        if (KIND == kDenseWide) {
+    // the sum of a run's lanes, in every lane
+    auto run_sum = [&](auto x) {
+        if constexpr (KIND == kDenseWide) {
+            unsigned long long t = x;
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            return t;
         } else {
-            x = __reduce_add_sync(0xffffffffu, (uint32_t)x);
+            return (unsigned long long)__reduce_add_sync(0xffffffffu, (uint32_t)x);
         }
-        if (lane == 0 && x) msum_add(sh.msum + q, x);
     };
     int q0 = last_le(sh.start, nnz, k0);
     int32_t nxt = min(sh.start[q0 + 1], kend);   // end of the current run (or of this warp's range)
@@ -743,38 +753,98 @@ __device__ __forceinline__ unsigned long long batch_windows(const CountParams &p
             }
             const unsigned long long x = group(std::integral_constant<int, N>(), w, pos, d);
             acc += x;
-            if (kSecond) flush(q0, x);
+            if (kSecond) {   // to middle q0
+                const unsigned long long t = run_sum(x);
+                if (lane == 0 && t) msum_add(sh.msum + q0, t);
+            }
             k0 += 32 * N;
             if (k0 == nxt) { ++q0; nxt = min(sh.start[q0 + 1], kend); }
             continue;
         }
-        if (sh.start[q0 + kSegRuns] - k0 >= kSegMin) {
-            int32_t w[kSeg];
-            Pos pos[kSeg];
-            uint32_t d[kSeg];
-            int q[kSeg];
+        if constexpr (!kLaned) {
+            if (sh.start[q0 + kOneRuns] - k0 >= kOneMin) {
+                int32_t w[kSeg];
+                Pos pos[kSeg];
+                uint32_t d[kSeg];
+                int q[kSeg];
 #pragma unroll
-            for (int u = 0; u < kSeg; ++u) {
-                const int32_t n = min(nxt - k0, 32);   // 0 past the range
-                q[u] = q0;
-                pos[u] = sh.src[q0] + (Pos)(k0 + lane);
-                w[u] = -1;
-                if (lane < n) w[u] = __ldg(p.adj + pos[u]);
-                k0 += n;
-                q0 += k0 == nxt;   // at the range's end: a run past it, never read from
-                nxt = min(sh.start[q0 + 1], kend);
-            }
-            const unsigned long long x = group(std::integral_constant<int, kSeg>(), w, pos, d);
-            acc += x;
-            if (kSecond) {
-                if (q[0] == q[kSeg - 1]) {
-                    flush(q[0], x);
-                } else {
-#pragma unroll
-                    for (int u = 0; u < kSeg; ++u) flush(q[u], d[u]);
+                for (int u = 0; u < kSeg; ++u) {
+                    const int32_t n = min(nxt - k0, 32);   // 0 past the range
+                    q[u] = q0;
+                    pos[u] = sh.src[q0] + (Pos)(k0 + lane);
+                    w[u] = -1;
+                    if (lane < n) w[u] = __ldg(p.adj + pos[u]);
+                    k0 += n;
+                    q0 += k0 == nxt;   // at the range's end: a run past it, never read from
+                    nxt = min(sh.start[q0 + 1], kend);
                 }
+                const unsigned long long x = group(std::integral_constant<int, kSeg>(), w, pos, d);
+                acc += x;
+                if (kSecond) {
+                    auto flush = [&](int qq, auto v) {
+                        const unsigned long long t = run_sum(v);
+                        if (lane == 0 && t) msum_add(sh.msum + qq, t);
+                    };
+                    if (q[0] == q[kSeg - 1]) {
+                        flush(q[0], x);
+                    } else {
+#pragma unroll
+                        for (int u = 0; u < kSeg; ++u) flush(q[u], d[u]);
+                    }
+                }
+                continue;
             }
-            continue;
+        } else {
+            // the next 32 runs in the lanes: [rs, re) of the concatenated wedges
+            const int32_t rs = max(sh.start[q0 + lane], k0);
+            const int32_t re = min(sh.start[q0 + lane + 1], kend);
+            if (__shfl_sync(0xffffffffu, re, kLanedRuns - 1) - k0 >= kLanedMin || sh.start[q0 + kLanedRuns] >= kend) {
+                // up to 32 segments of at most 32 wedges, none across runs: lane i
+                // describes segment i (its run is the last one whose first segment
+                // is at most i), so a segment costs its window two shuffles
+                const int32_t ns = max(re - rs + 31, 0) >> 5;
+                int32_t incl = ns;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += t;
+                }
+                const int32_t excl = incl - ns;
+                const int segs = min(__shfl_sync(0xffffffffu, incl, 31), 32);
+                const uint32_t first = __reduce_or_sync(0xffffffffu, ns > 0 && excl < 32 ? 1u << excl : 0u);
+                const int r = __popc(first & le_mask) - 1;   // runs of no segment lie past the range only
+                const int32_t k = __shfl_sync(0xffffffffu, rs, r) + ((lane - __shfl_sync(0xffffffffu, excl, r)) << 5);
+                const int32_t rend = __shfl_sync(0xffffffffu, re, r);
+                const int32_t n = lane < segs ? min(rend - k, 32) : 0;
+                const Pos at = sh.src[q0 + r] + (Pos)k;
+                unsigned long long mine = 0;   // second walk: Σ δ of this lane's segment
+                for (int s0 = 0; s0 < segs; s0 += kSeg) {   // uniform
+                    int32_t w[kSeg];
+                    Pos pos[kSeg];
+                    uint32_t d[kSeg];
+#pragma unroll
+                    for (int u = 0; u < kSeg; ++u) {
+                        pos[u] = __shfl_sync(0xffffffffu, at, s0 + u) + (Pos)lane;
+                        w[u] = -1;
+                        if (lane < __shfl_sync(0xffffffffu, n, s0 + u)) w[u] = __ldg(p.adj + pos[u]);
+                    }
+                    acc += group(std::integral_constant<int, kSeg>(), w, pos, d);
+                    if (kSecond) {
+#pragma unroll
+                        for (int u = 0; u < kSeg; ++u) {
+                            const unsigned long long x = run_sum(d[u]);
+                            if (lane == s0 + u) mine = x;
+                        }
+                    }
+                }
+                if (kSecond && mine) msum_add(sh.msum + q0 + r, mine);
+                // past the last segment taken
+                const bool whole = k + n == rend;
+                k0 = __shfl_sync(0xffffffffu, k + n, segs - 1);
+                q0 += __shfl_sync(0xffffffffu, r + (whole ? 1 : 0), segs - 1);
+                if (k0 < kend) nxt = min(sh.start[q0 + 1], kend);
+                continue;
+            }
         }
         int32_t w[kU];
         Pos pos[kU];
