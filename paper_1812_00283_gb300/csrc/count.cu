@@ -1494,7 +1494,7 @@ __device__ unsigned long long warp_item(const CountParams &p, int32_t x, unsigne
 }
 
 // Starts of at most 32 wedges (and 32 middles), one window each: equal ends are
-// found by one warp match, with no table.  A warp takes 32 starts, reads their
+// found by one warp match, with no table.  A warp takes up to 32 starts, reads their
 // offsets and cuts together, and runs them through two stages, so that the next
 // start's slots and this start's ends load while the one before is counted: a
 // start alone is a chain of five loads of about 700 clocks.
@@ -1506,12 +1506,14 @@ __device__ unsigned long long tiny_items(const CountParams &p, unsigned char *re
     int32_t *const wslot = reinterpret_cast<int32_t *>(region + 2 * 32 * 8);    // [2][32] lane of a run's middle
     const int64_t n_tiny = n_tiny_items(p);
     unsigned long long acc = 0;
+    // few starts: spread over all warps rather than pipelined in a few of them
+    const int grab = (int)min((int64_t)32, max((int64_t)1, n_tiny / ((int64_t)gridDim.x * kCountWarps)));
     for (;;) {
         int it = 0;
-        if (lane == 0) it = atomicAdd(p.cursors + 5, 32);
+        if (lane == 0) it = atomicAdd(p.cursors + 5, grab);
         it = __shfl_sync(0xffffffffu, it, 0);
         if (it >= n_tiny || it < 0) break;
-        const int cnt = (int)min((int64_t)32, n_tiny - it);
+        const int cnt = (int)min((int64_t)grab, n_tiny - it);
         int32_t x = 0, nm = 0;
         Pos e0 = 0;
         if (lane < cnt) {

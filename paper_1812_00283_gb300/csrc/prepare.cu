@@ -31,26 +31,24 @@ __device__ __forceinline__ bool aborted(const int *guard) {
     return guard && (*(volatile const int *)guard & (kErrBadOffsets | kErrBadId));
 }
 
-// ----- validation (always on: every later index depends on it) -------------
-// (and the U degrees, which are only read once the offsets have passed)
-__global__ void k_check_offsets(const int32_t *__restrict__ off, int32_t r, int64_t m, int32_t *deg_u, int *err) {
-    int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (u > r) return;
-    const int32_t o = off[u];
-    if (u == 0 && o != 0) atomicOr(err, kErrBadOffsets);
-    if (u < r) {
-        const int32_t e = off[u + 1];
-        if (e < o) atomicOr(err, kErrBadOffsets);
-        deg_u[u] = e - o;
+// ----- validation and a1: degrees ----------------------------------------------
+// One pass over the caller's arrays (always on: every later index depends on
+// it): the offsets with the U degrees, and the ids with the L degrees.  An id
+// outside [0, l) is reported and counted nowhere.
+__global__ void k_check_input(const int32_t *__restrict__ off, const int32_t *__restrict__ adj, int32_t r, int32_t l,
+                              int64_t m, int32_t *deg_u, int32_t *deg_l, int *err) {
+    const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t u = i0; u <= r; u += stride) {
+        const int32_t o = off[u];
+        if (u == 0 && o != 0) atomicOr(err, kErrBadOffsets);
+        if (u < r) {
+            const int32_t e = off[u + 1];
+            if (e < o) atomicOr(err, kErrBadOffsets);
+            deg_u[u] = e - o;
+        }
+        if (u == r && (int64_t)o != m) atomicOr(err, kErrBadOffsets);
     }
-    if (u == r && (int64_t)o != m) atomicOr(err, kErrBadOffsets);
-}
-
-// ----- a1: degrees -----------------------------------------------------------
-// L degrees; an id outside [0, l) is reported and counted nowhere
-__global__ void k_deg_l(const int32_t *__restrict__ adj, int64_t m, int32_t l, int32_t *deg_l, int *err) {
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < m;
-         k += (int64_t)gridDim.x * blockDim.x) {
+    for (int64_t k = i0; k < m; k += stride) {
         const int32_t v = adj[k];
         if (v < 0 || v >= l) atomicOr(err, kErrBadId);
         else atomicAdd(&deg_l[v], 1);
@@ -141,6 +139,7 @@ constexpr int kRowCtaMax = 4096;
 constexpr int kRowCtaThreads = 256;
 constexpr int32_t kRowBitmapMax = 1 << 19;   // L ranks of one bitmap
 constexpr int kRowTiers = 5;   // warp sort, bitmap (256 threads), bitmap (1,024), CTA sort, radix
+constexpr int kRedWords = 12 + 4;   // statistics, two queue and five tier counters
 
 struct URowOut {
     int64_t m;
@@ -160,12 +159,14 @@ struct URowOut {
     }
 };
 
-// A warp takes 32 rows (their offsets and ranks are one load per lane), then
-// four rows of at most 8 neighbours at a time, then the longer ones one by one.
+// A warp takes `span` rows (their offsets and ranks are one load per lane; 32
+// where there are enough rows for every warp of the device, else down to 4),
+// then four rows of at most 8 neighbours at a time, then the longer ones one by
+// one.  With 32 rows a warp, 2,000 rows were 63 warps walking 32 rows in turn.
 __global__ void k_u_rows_warp(const int32_t *__restrict__ off_u, const int32_t *__restrict__ adj_u,
                               const int32_t *__restrict__ rank_u, const int32_t *__restrict__ rank_l,
-                              int32_t r, const int32_t *__restrict__ gl, const int32_t *__restrict__ gu,
-                              int32_t num_graphs, URowOut o,
+                              int32_t r, int span, const int32_t *__restrict__ gl,
+                              const int32_t *__restrict__ gu, int32_t num_graphs, URowOut o,
     const int *guard = nullptr) {
     if (aborted(guard)) return;
     const int lane = threadIdx.x & 31;
@@ -173,10 +174,10 @@ __global__ void k_u_rows_warp(const int32_t *__restrict__ off_u, const int32_t *
     bool cross = false;   // a batch: an L rank outside the row's graph
     const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t u0 = w0 * 32; u0 < r; u0 += nw * 32) {
+    for (int64_t u0 = w0 * span; u0 < r; u0 += nw * span) {
         const int64_t u = u0 + lane;
         int32_t b = 0, d = 0, ru = 0, lo = 0, hi = o.l;
-        if (u < r) {
+        if (u < r && lane < span) {
             b = off_u[u];
             d = off_u[u + 1] - b;
             if (d > 0 && d <= kRowWarpMax) {
@@ -589,7 +590,8 @@ __global__ void k_large_emit(const uint64_t *__restrict__ keys, const int32_t *_
 // run through u is the prefix of N(u) before v, which is as long as v's position
 // in that list; where u is the start the run through v is as long as u's
 // position in N(v).  The second kind is scattered to the U-side slot, whose
-// plen the caller has set to zero.  Reads `off` at random (L2-resident: 8 bytes
+// plen the caller has set to zero (the row kernels' scattered stores would cost
+// more than the clear).  Reads `off` at random (L2-resident: 8 bytes
 // per vertex), writes 4 bytes at random for the U starts' middles only; a
 // binary search of the middle's list per slot took 15.8 ms on a 300M-edge
 // shopping graph.
@@ -626,23 +628,25 @@ __global__ void k_emit_l_side(const uint64_t *__restrict__ keys2, const int32_t 
 // the degree of G* ids is non-decreasing inside a layer, so the cut is a
 // lower bound on degree: for x in L a U neighbour of equal degree has higher
 // priority (U ids > L ids); for x in U an L neighbour of equal degree is lower.
+__device__ __forceinline__ int32_t cut_of(const int32_t *__restrict__ adj, const int32_t *__restrict__ deg_star,
+                                          int64_t b, int32_t d, int32_t dx, bool in_u) {
+    int32_t lo = 0, hi = d;
+    while (lo < hi) {
+        const int32_t mid = lo + ((hi - lo) >> 1), dy = deg_star[adj[b + mid]];
+        if (in_u ? dy <= dx : dy < dx) lo = mid + 1; else hi = mid;
+    }
+    return lo;
+}
+
+// (Algorithm 3's run lengths need every cut first; Algorithm 2's k_work finds
+// them as it goes.)
 __global__ void k_cut(const int64_t *__restrict__ off, const int32_t *__restrict__ adj,
-                      const int32_t *__restrict__ deg_star, int32_t n, int32_t l, int32_t *cut,
-    const int *guard = nullptr) {
+                      const int32_t *__restrict__ deg_star, int32_t n, int32_t l, int32_t *cut, const int *guard) {
     if (aborted(guard)) return;
     int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= n) return;
     const int64_t b = off[x];
-    int64_t lo = 0, hi = off[x + 1] - b;
-    const int32_t dx = deg_star[x];
-    const bool in_u = x >= l;
-    while (lo < hi) {
-        int64_t mid = (lo + hi) >> 1;
-        int32_t dy = deg_star[adj[b + mid]];
-        bool lower = in_u ? (dy <= dx) : (dy < dx);
-        if (lower) lo = mid + 1; else hi = mid;
-    }
-    cut[x] = (int32_t)lo;
+    cut[x] = cut_of(adj, deg_star, b, (int32_t)(off[x + 1] - b), deg_star[x], x >= l);
 }
 
 // Algorithm 3: for slot e = (x, v) the ends are the w in N(v) with
@@ -687,8 +691,8 @@ __device__ __forceinline__ unsigned slot_work(const int64_t *off, const int32_t 
 }
 
 __global__ void k_work(const int64_t *__restrict__ off, const int32_t *__restrict__ adj,
-                       const int32_t *__restrict__ cut, const int32_t *__restrict__ plen, int32_t n, int all_slots,
-                       int64_t fill_from, int64_t *sbeg, uint64_t *work, int32_t *queue, int32_t *queued,
+                       const int32_t *__restrict__ deg_star, int32_t l, int32_t *cut,
+                       const int32_t *__restrict__ plen, int32_t n, int all_slots, int64_t fill_from, int64_t *sbeg, uint64_t *work, int32_t *queue, int32_t *queued,
     const int *guard = nullptr) {
     if (aborted(guard)) return;
     const int lane = threadIdx.x & 31;
@@ -700,7 +704,11 @@ __global__ void k_work(const int64_t *__restrict__ off, const int32_t *__restric
         int32_t c = 0;
         if (x < n) {
             b = off[x];
-            c = all_slots ? (int32_t)(off[x + 1] - b) : cut[x];
+            c = (int32_t)(off[x + 1] - b);
+            if (!all_slots) {
+                c = cut_of(adj, deg_star, b, c, deg_star[x], x >= l);
+                cut[x] = c;
+            }
         }
         unsigned long long s = 0;
         if (c <= kWorkLane) {
@@ -790,49 +798,6 @@ __global__ void __launch_bounds__(kWorkThreads) k_work_long(
     }
 }
 
-// stats[0] += Σ work, stats[1] = max work, stats[2] += starts above `heavy`;
-// of a batch, gwork[g] += the work of graph g (one addition per warp where its
-// vertices lie in one graph, which all but a few warps' do)
-__global__ void k_work_stats(const uint64_t *__restrict__ work, int32_t n, uint64_t heavy,
-                             const int32_t *__restrict__ gstar, unsigned long long *stats, unsigned long long *gwork,
-    const int *guard = nullptr) {
-    if (aborted(guard)) return;
-    const int lane = threadIdx.x & 31;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    unsigned long long sum = 0, top = 0, above = 0;
-    for (int64_t x0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); x0 < n; x0 += stride) {
-        const int64_t x = x0 + lane;
-        const unsigned long long w = x < n ? work[x] : 0;
-        sum += w;
-        top = w > top ? w : top;
-        above += w > heavy ? 1 : 0;
-        if (gwork) {
-            const int32_t g = x < n ? gstar[x] : -1;
-            const int32_t g0 = __shfl_sync(0xffffffffu, g, 0);
-            if (__all_sync(0xffffffffu, g == g0)) {
-                unsigned long long t = w;
-#pragma unroll
-                for (int d = 16; d > 0; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
-                if (lane == 0 && t) atomicAdd(gwork + g0, t);
-            } else if (w) {
-                atomicAdd(gwork + g, w);
-            }
-        }
-    }
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-        sum += __shfl_xor_sync(0xffffffffu, sum, d);
-        above += __shfl_xor_sync(0xffffffffu, above, d);
-        const unsigned long long o = __shfl_xor_sync(0xffffffffu, top, d);
-        top = o > top ? o : top;
-    }
-    if (lane == 0) {
-        if (sum) atomicAdd(stats, sum);
-        if (top) atomicMax(stats + 1, top);
-        if (above) atomicAdd(stats + 2, above);
-    }
-}
-
 // ----- a5: bins and schedule ---------------------------------------------------
 // A core start (dense-core hybrid) with wedges is always a dense item: only
 // dense items skip the core wedges and add the core pairs after the walk.
@@ -862,11 +827,19 @@ struct BinBounds {
 // no order; only the heavy ones, a few per cent of the starts with work, are
 // then sorted).  A CTA takes 2,048 starts and reserves
 // their room with one addition per list.
+// With `stats` also: stats[0] += Σ work, stats[1] = max work, stats[2] +=
+// starts above heavy_work, stats[11] = the error word, and of a batch gwork[g] +=
+// the work of graph g (one addition per warp where its vertices lie in one
+// graph, which all but a few warps' do).
 constexpr int kBinTile = 8 * kT;
 __global__ void __launch_bounds__(kT) k_bin_starts(const uint64_t *__restrict__ work, int32_t n, BinBounds bb,
                                                    unsigned long long *counts, int32_t *heavy, int32_t *warp_items,
+                                                   unsigned long long *stats, uint64_t heavy_work,
+                                                   const int32_t *__restrict__ gstar, unsigned long long *gwork,
     const int *guard = nullptr) {
+    if (stats && guard && blockIdx.x == 0 && threadIdx.x == 0) stats[11] = (unsigned long long)*(volatile const int *)guard;
     if (aborted(guard)) return;
+    unsigned long long sum = 0, top = 0, above = 0;
     __shared__ int32_t cnt[6], at[3];   // at: this tile's room in heavy, warp front, warp back
     const int lane = threadIdx.x & 31;
     const uint32_t lt = (1u << lane) - 1u;
@@ -877,7 +850,23 @@ __global__ void __launch_bounds__(kT) k_bin_starts(const uint64_t *__restrict__ 
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int64_t x = x0 + i * kT + threadIdx.x;
-            bin[i] = x < n ? bb.of((int32_t)x, work[x]) : 4;
+            const uint64_t w = x < n ? work[x] : 0;
+            bin[i] = w > 0 ? bb.of((int32_t)x, w) : 4;
+            sum += w;
+            top = w > top ? w : top;
+            above += w > heavy_work ? 1 : 0;
+            if (gwork) {
+                const int32_t g = x < n ? gstar[x] : -1;
+                const int32_t g0 = __shfl_sync(0xffffffffu, g, 0);
+                if (__all_sync(0xffffffffu, g == g0)) {
+                    unsigned long long t = w;
+#pragma unroll
+                    for (int d = 16; d > 0; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
+                    if (lane == 0 && t) atomicAdd(gwork + g0, t);
+                } else if (w) {
+                    atomicAdd(gwork + g, (unsigned long long)w);
+                }
+            }
         }
         // cnt[0..2]: bins; cnt[3], cnt[5]: lists of their own; cnt[4]: the heavy list
 #pragma unroll
@@ -912,6 +901,20 @@ __global__ void __launch_bounds__(kT) k_bin_starts(const uint64_t *__restrict__ 
         }
         __syncthreads();
     }
+    if (stats) {
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) {
+            sum += __shfl_xor_sync(0xffffffffu, sum, d);
+            above += __shfl_xor_sync(0xffffffffu, above, d);
+            const unsigned long long o = __shfl_xor_sync(0xffffffffu, top, d);
+            top = o > top ? o : top;
+        }
+        if (lane == 0) {
+            if (sum) atomicAdd(stats, sum);
+            if (top) atomicMax(stats + 1, top);
+            if (above) atomicAdd(stats + 2, above);
+        }
+    }
 }
 
 // ascending key = descending work; forced dense starts first
@@ -921,6 +924,44 @@ __global__ void k_sched_keys(const uint64_t *__restrict__ work, const int32_t *_
     if (i >= n_heavy) return;
     const int32_t x = heavy[i];
     keys[i] = forced_dense(x, l, core_lo_u, core_lo_l, work[x]) ? 0 : maxw - work[x];
+}
+
+// The same order for at most 4,096 heavy starts, by one CTA: a bitonic sort of
+// (key, place) words in shared memory, one launch for the ten of a radix sort
+// over so few keys.  A pair of elements less than 32 apart is one warp's, so only
+// the wider strides need the CTA's barrier.
+constexpr int kSchedSmall = 4096;
+constexpr int kSchedPlaceBits = 12;
+__global__ void __launch_bounds__(1024) k_sched_small(const uint64_t *__restrict__ work,
+                                                      const int32_t *__restrict__ heavy, int n_heavy, uint64_t maxw,
+                                                      int32_t l, int32_t core_lo_u, int32_t core_lo_l, int32_t *order) {
+    __shared__ uint64_t buf[kSchedSmall];
+    int np = 64;
+    while (np < n_heavy) np <<= 1;
+    for (int i = threadIdx.x; i < np; i += 1024) {
+        uint64_t key = ~0ull;
+        if (i < n_heavy) {
+            const int32_t x = heavy[i];
+            key = (forced_dense(x, l, core_lo_u, core_lo_l, work[x]) ? 0 : maxw - work[x]) << kSchedPlaceBits | (uint64_t)i;
+        }
+        buf[i] = key;
+    }
+    __syncthreads();
+    for (int k = 2; k <= np; k <<= 1) {
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            for (int i = threadIdx.x; i < np; i += 1024) {
+                const int ij = i ^ j;
+                if (ij > i) {
+                    const uint64_t a = buf[i], c = buf[ij];
+                    if ((a > c) == ((i & k) == 0)) { buf[i] = c; buf[ij] = a; }
+                }
+            }
+            // this stride, or the first of the next k, crosses warps
+            if (j >= 32 || (j == 1 && k >= 32)) __syncthreads(); else __syncwarp();
+        }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < n_heavy; i += 1024) order[i] = heavy[buf[i] & ((1u << kSchedPlaceBits) - 1u)];
 }
 
 // the dense chunks of start x (dense_chunk_end from offset 0 up); with `out`,
@@ -1214,12 +1255,14 @@ static BinBounds bin_bounds(const Graph *g, int32_t warp_max_work, int32_t team_
 
 // Starts the binning of all starts on s: counts[0..5] (zeroed here) = dense,
 // hash, team, warp, the first three together, tiny; g->warp_items is filled.
+// With `stats` (zeroed by the caller, counts at stats + 3) the graph's statistics too.
 static int bin_starts(Graph *g, cudaStream_t s, const BinBounds &bb, unsigned long long *counts, int32_t *heavy,
-                      const int *guard) {
-    BFC_CUDA(cudaMemsetAsync(counts, 0, 6 * sizeof(unsigned long long), s));
+                      unsigned long long *stats, const int *guard) {
+    if (!stats) BFC_CUDA(cudaMemsetAsync(counts, 0, 6 * sizeof(unsigned long long), s));
     if (g->n == 0) return BFC_OK;
     k_bin_starts<<<(unsigned)std::min<int64_t>(((int64_t)g->n + kBinTile - 1) / kBinTile, 152 * 8), kT, 0, s>>>(
-        g->work, g->n, bb, counts, heavy, g->warp_items, guard); note_launch();
+        g->work, g->n, bb, counts, heavy, g->warp_items, stats, (uint64_t)g->opt.hash_max_work, g->gstar,
+        stats && g->num_graphs > 0 ? g->gwork : nullptr, guard); note_launch();
     BFC_CUDA(cudaGetLastError());
     return BFC_OK;
 }
@@ -1258,7 +1301,14 @@ static int schedule_graph(Graph *g, cudaStream_t s, int32_t warp_max_work, int32
         uint32_t *hist, *hist_tmp;
         int64_t *scan64_tmp = nullptr, *nch = nullptr;
         const int32_t *order = heavy;
-        if (n_heavy > 0) {
+        if (n_heavy > 0) GET(tmp, scan64_tmp, scan_tmp_elems<int64_t>(std::max<int64_t>(n_dense, n) + 1));
+        if (n_heavy > 1 && n_heavy <= kSchedSmall && maxw < 1ull << (64 - kSchedPlaceBits - 1)) {
+            GET(tmp, v1, n_heavy);
+            k_sched_small<<<1, 1024, 0, s>>>(g->work, heavy, (int)n_heavy, maxw, l, bb.core_lo_u,
+                                                            bb.core_lo_l, v1); note_launch();
+            BFC_CUDA(cudaGetLastError());
+            order = v1;
+        } else if (n_heavy > 1) {
             GET(tmp, k0, n_heavy + 1); GET(tmp, k1, n_heavy + 1); GET(tmp, v1, n_heavy);
             GET(tmp, hist, radix_hist_elems(n_heavy));
             GET(tmp, hist_tmp, scan_tmp_elems<uint32_t>((int64_t)radix_hist_elems(n_heavy)));
@@ -1268,7 +1318,6 @@ static int schedule_graph(Graph *g, cudaStream_t s, int32_t warp_max_work, int32
             BFC_CUDA(cudaGetLastError());
             BFC_CUDA(radix_sort_pairs(k0, heavy, k1, v1, n_heavy, 0, bits_for(maxw), hist, hist_tmp, s, &which));
             order = which ? v1 : heavy;
-            GET(tmp, scan64_tmp, scan_tmp_elems<int64_t>(std::max<int64_t>(n_dense, n) + 1));
         }
         // a layer (a batch's graph's) this small is one chunk of any counters,
         // or of 16-bit ones where no degree can pass 65,535
@@ -1413,7 +1462,7 @@ int rebin_graph(Graph *g, cudaStream_t s, int32_t warp_max_work, int32_t team_ma
         return BFC_ERR_OUT_OF_MEMORY;
     }
     const BinBounds bb = bin_bounds(g, warp_max_work, team_max_work, hash_max_work);
-    int rc = bin_starts(g, s, bb, counts, heavy, nullptr);
+    int rc = bin_starts(g, s, bb, counts, heavy, nullptr, nullptr);
     if (rc) return rc;
     BFC_CUDA(cudaMemcpyAsync(hc, counts, sizeof(hc), cudaMemcpyDeviceToHost, s));
     BFC_CUDA(cudaStreamSynchronize(s));
@@ -1472,7 +1521,7 @@ static int rows_smem_setup(int device) {
     return BFC_OK;
 }
 
-// The U side of G*: every tier that needs no size on the host.  `range`: the L
+// The U side of G*: every tier that needs no size on the host (tier_n is zero).  `range`: the L
 // ranks of a single graph, or of a batch's largest graph.
 static int launch_u_rows(const int32_t *off_u, const int32_t *adj_u, Graph *g, int32_t range, const int32_t *gu,
                          const int32_t *gl, int32_t num_graphs, int bitmaps, const URowOut &uo,
@@ -1481,12 +1530,12 @@ static int launch_u_rows(const int32_t *off_u, const int32_t *adj_u, Graph *g, i
     const int64_t m = g->m;
     int rc = rows_smem_setup(g->device);
     if (rc) return rc;
-    k_u_rows_warp<<<grid_stride_blocks(r), kT, 0, s>>>(off_u, adj_u, g->rank_u, g->rank_l, r, gl, gu,
-                                                       num_graphs, uo, guard); note_launch();
+    const int span = (int)std::min<int64_t>(std::max<int64_t>(r / (152 * 64), 4), 32);
+    k_u_rows_warp<<<grid_stride_blocks((int64_t)(r + span - 1) / span * 32), kT, 0, s>>>(
+        off_u, adj_u, g->rank_u, g->rank_l, r, span, gl, gu, num_graphs, uo, guard); note_launch();
     BFC_CUDA(cudaGetLastError());
     if (m <= kRowWarpMax) return BFC_OK;
     const int wide_tier = range > kRowCtaMax ? 1 : 0;   // a valid row is no longer than the range
-    BFC_CUDA(cudaMemsetAsync(tier_n, 0, kRowTiers * sizeof(int32_t), s));
     k_row_tiers<<<grid_stride_blocks(r), kT, 0, s>>>(off_u, r, range, gu, gl, num_graphs, bitmaps, wide_tier, tier_rows,
                                                      tier_n,
                                                      guard); note_launch();
@@ -1515,20 +1564,18 @@ static int launch_u_rows(const int32_t *off_u, const int32_t *adj_u, Graph *g, i
     return BFC_OK;
 }
 
-// work per start, the runs of the U-side middle slots (Algorithm 2), and
-// stats[0] = W, [1] = the heaviest start, [2] = starts beyond the CTA-hash bin
-static void launch_work(Graph *g, int32_t *big, int32_t *n_big, unsigned long long *gwork, unsigned long long *stats,
-                        cudaStream_t s, const int *guard) {
+// cut (Algorithm 2) and work per start, and the runs of the U-side middle slots
+// (`queued` is zero)
+static void launch_work(Graph *g, const int32_t *deg_star, int32_t *queue, int32_t *queued, cudaStream_t s,
+                        const int *guard) {
     const int vpp = g->opt.orientation;
     const int64_t fill_from = vpp ? 2 * g->m + 1 : g->m;
-    k_work<<<grid_stride_blocks(g->n), kT, 0, s>>>(g->off, g->adj, g->cut, g->plen, g->n, vpp, fill_from, g->sbeg,
-                                                   g->work, big, n_big, guard); note_launch();
+    k_work<<<grid_stride_blocks(g->n), kT, 0, s>>>(g->off, g->adj, deg_star, g->l, g->cut, g->plen, g->n, vpp,
+                                                   fill_from, g->sbeg, g->work, queue, queued, guard); note_launch();
     if (2 * g->m > kWorkLane) {
         k_work_long<<<(unsigned)std::min<int64_t>(2 * g->m / kWorkLane / (kWorkThreads / 32) + 1, 152 * 4), kWorkThreads, 0, s>>>(
-            g->off, g->adj, g->cut, g->plen, g->n, vpp, fill_from, g->sbeg, g->work, big, n_big, guard); note_launch();
+            g->off, g->adj, g->cut, g->plen, g->n, vpp, fill_from, g->sbeg, g->work, queue, queued, guard); note_launch();
     }
-    k_work_stats<<<(unsigned)std::min<int64_t>(blocks_for(g->n), 152 * 8), kT, 0, s>>>(
-        g->work, g->n, (uint64_t)g->opt.hash_max_work, g->gstar, stats, gwork, guard); note_launch();
 }
 
 int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Graph *g,
@@ -1604,26 +1651,28 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
     uint32_t *hist, *hist_tmp;
     int64_t *scan64_tmp, *deg64;
     // [0] W, [1] heaviest start, [2] starts beyond the CTA-hash bin, [3..9) bin
-    // counts, [9] / [10] largest L / U degree
+    // counts, [9] / [10] largest L / U degree, [11] the error word, then the work
+    // queues' and the row tiers' counters: cleared together
     unsigned long long *red;
     GET(tmp, k0, nsort + 1); GET(tmp, k1, nsort + 1);
     GET(tmp, v0, nsort); GET(tmp, v1, nsort);
     GET(tmp, deg_u, r); GET(tmp, deg_l, l); GET(tmp, deg_star, n);
     GET(tmp, rows_star, 2 * m);
-    GET(tmp, big, n); GET(tmp, n_big, 2);
+    GET(tmp, big, n);
     GET(tmp, hist, radix_hist_elems(nsort));
     GET(tmp, hist_tmp, scan_tmp_elems<uint32_t>((int64_t)radix_hist_elems(nsort)));
     GET(tmp, scan64_tmp, std::max(scan_tmp_elems<int64_t>((int64_t)n + 1),
                                   max_scan_tmp_elems(m)));
     GET(tmp, deg64, (int64_t)n + 1);
-    GET(tmp, red, 12);
+    GET(tmp, red, kRedWords);
+    n_big = reinterpret_cast<int32_t *>(red + 12);
     GET(tmp, heavy, std::max(n, 1));
-    BFC_CUDA(cudaMemsetAsync(red, 0, 12 * sizeof(unsigned long long), s));
+    BFC_CUDA(cudaMemsetAsync(red, 0, kRedWords * sizeof(unsigned long long), s));
 
     // ---- a1: degrees, and the check of the caller's offsets and L ids
     BFC_CUDA(cudaMemsetAsync(deg_l, 0, sizeof(int32_t) * std::max<int64_t>(l, 1), s));
-    k_check_offsets<<<blocks_for((int64_t)r + 1), kT, 0, s>>>(csr->off_u, r, m, deg_u, g->err); note_launch();
-    if (m > 0) { k_deg_l<<<grid_stride_blocks(m), kT, 0, s>>>(csr->adj_u, m, l, deg_l, g->err); note_launch(); }
+    k_check_input<<<grid_stride_blocks(std::max<int64_t>(m, (int64_t)r + 1)), kT, 0, s>>>(
+        csr->off_u, csr->adj_u, r, l, m, deg_u, deg_l, g->err); note_launch();
     BFC_CUDA(cudaGetLastError());
 
     // ---- a2: per-layer priority ranks by a stable sort on (layer, graph, degree)
@@ -1652,9 +1701,8 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
         // U side row by row (warp / CTA tiers, radix sort for the largest rows);
         // the swapped keys for the L side land in k1
         const URowOut uo{m, l, bu, g->off, g->adj, g->eid, rows_star, k1, g->err, opt->validate};
-        int32_t *tier_rows = nullptr, *tier_n = nullptr;
+        int32_t *tier_rows = nullptr, *const tier_n = n_big + 2;
         GET(tmp, tier_rows, kRowTiers * std::max<int64_t>(r, 1));
-        GET(tmp, tier_n, kRowTiers);
         {
             int rc = launch_u_rows(csr->off_u, csr->adj_u, g, l_range, graph_u_start, graph_l_start, num_graphs,
                                    opt->validate, uo, tier_rows, tier_n, s, guard_err);
@@ -1727,7 +1775,7 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
     }
 
     // ---- a4: cut, per-middle prefix lengths, per-start work, W
-    if (n > 0) {
+    if (n > 0 && opt->orientation == 1) {
         k_cut<<<blocks_for(n), kT, 0, s>>>(g->off, g->adj, deg_star, n, l, g->cut, guard_err); note_launch();
         BFC_CUDA(cudaGetLastError());
     }
@@ -1738,22 +1786,22 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
     }
     const bool core_auto = opt->core_vertices < 0 && opt->orientation == 0 && num_graphs == 0;
     if (n > 0) {
-        BFC_CUDA(cudaMemsetAsync(n_big, 0, 2 * sizeof(int32_t), s));
-        launch_work(g, big, n_big, num_graphs > 0 ? g->gwork : nullptr, red, s, guard_err);
+        launch_work(g, deg_star, big, n_big, s, guard_err);
         BFC_CUDA(cudaGetLastError());
     }
     // the bins without a core, before the round trip (a core, which only large
     // graphs get, moves its starts to the dense bin: those are binned again)
     BinBounds bb = bin_bounds(g, opt->warp_max_work, opt->team_max_work, opt->hash_max_work);
     {
-        int rc = bin_starts(g, s, bb, red + 3, heavy, guard_err);
+        int rc = bin_starts(g, s, bb, red + 3, heavy, red, guard_err);
         if (rc) return rc;
     }
     unsigned long long hred[12] = {0};
-    BFC_CUDA(cudaMemcpyAsync(hred, red, sizeof(hred), cudaMemcpyDeviceToHost, s));
-    BFC_CUDA(cudaMemcpyAsync(&herr, g->err, sizeof(int), cudaMemcpyDeviceToHost, s));
+    // without a vertex no kernel has copied the error word
+    BFC_CUDA(n > 0 ? cudaMemcpyAsync(hred, red, sizeof(hred), cudaMemcpyDeviceToHost, s)
+                   : cudaMemcpyAsync(&herr, g->err, sizeof(int), cudaMemcpyDeviceToHost, s));
     BFC_CUDA(cudaStreamSynchronize(s));
-    if (int rc = input_error(herr, num_graphs)) return rc;
+    if (int rc = input_error(n > 0 ? (int)hred[11] : herr, num_graphs)) return rc;
     g->info.wedges = hred[0];
     g->info.max_start_work = hred[1];
     g->info.max_deg_l = (int32_t)hred[9];
@@ -1777,7 +1825,7 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
     // ---- a5: heaviest-first order and bins
     if (g->core_u + g->core_l > 0) {
         bb = bin_bounds(g, opt->warp_max_work, opt->team_max_work, opt->hash_max_work);
-        int rc = bin_starts(g, s, bb, red + 3, heavy, nullptr);
+        int rc = bin_starts(g, s, bb, red + 3, heavy, nullptr, nullptr);
         if (rc) return rc;
         BFC_CUDA(cudaMemcpyAsync(hred + 3, red + 3, 6 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
         BFC_CUDA(cudaStreamSynchronize(s));
@@ -1883,12 +1931,14 @@ int batch_plan_create(BatchPlan *pl, cudaStream_t s) {
     const int64_t nsort = std::max<int64_t>({(int64_t)r, (int64_t)l, m, (int64_t)n, 1});
     GET(pl->k0, nsort + 1); GET(pl->k1, nsort + 1); GET(pl->v0, nsort); GET(pl->v1, nsort);
     GET(pl->deg_u, r); GET(pl->deg_l, l); GET(pl->deg_star, n);
-    GET(pl->rows_star, 2 * m); GET(pl->big, n); GET(pl->n_big, 2);
-    GET(pl->tier_rows, kRowTiers * (int64_t)std::max(r, 1)); GET(pl->tier_n, kRowTiers);
+    GET(pl->rows_star, 2 * m); GET(pl->big, n);
+    GET(pl->tier_rows, kRowTiers * (int64_t)std::max(r, 1));
     GET(pl->hist, radix_hist_elems(nsort));
     GET(pl->hist_tmp, scan_tmp_elems<uint32_t>((int64_t)radix_hist_elems(nsort)));
     GET(pl->scan64_tmp, std::max(scan_tmp_elems<int64_t>((int64_t)n + 1), max_scan_tmp_elems(m)));
-    GET(pl->deg64, (int64_t)n + 1); GET(pl->red, 12); GET(pl->heavy, n);
+    GET(pl->deg64, (int64_t)n + 1); GET(pl->red, kRedWords); GET(pl->heavy, n);
+    pl->n_big = reinterpret_cast<int32_t *>(pl->red + 12);
+    pl->tier_n = pl->n_big + 2;
 #undef GET
     // every kept array starts zeroed: a run that stops at the checks leaves
     // arrays that later kernels can still index safely
@@ -1918,15 +1968,15 @@ int batch_plan_run(BatchPlan *pl, const int32_t *off_u, const int32_t *adj_u, co
     const bfc_options *opt = &g->opt;
     BFC_CUDA(cudaMemsetAsync(g->err, 0, 4 * sizeof(int), s));
     // ---- checks: the CSR, the graph start arrays, edges inside their graph
-    k_check_offsets<<<blocks_for((int64_t)r + 1), kT, 0, s>>>(off_u, r, m, pl->deg_u, g->err); note_launch();
     k_check_starts<<<blocks_for((int64_t)G + 1), kT, 0, s>>>(gu, G, r, g->err, pl->max_layer); note_launch();
     k_check_starts<<<blocks_for((int64_t)G + 1), kT, 0, s>>>(gl, G, l, g->err, pl->max_layer); note_launch();
     BFC_CUDA(cudaGetLastError());
     // ---- a1: degrees (and the check of the L ids)
     BFC_CUDA(cudaMemsetAsync(pl->deg_l, 0, sizeof(int32_t) * std::max<int64_t>(l, 1), s));
-    if (m > 0) { k_deg_l<<<grid_stride_blocks(m), kT, 0, s>>>(adj_u, m, l, pl->deg_l, g->err); note_launch(); }
+    k_check_input<<<grid_stride_blocks(std::max<int64_t>(m, (int64_t)r + 1)), kT, 0, s>>>(
+        off_u, adj_u, r, l, m, pl->deg_u, pl->deg_l, g->err); note_launch();
     BFC_CUDA(cudaGetLastError());
-    BFC_CUDA(cudaMemsetAsync(pl->red, 0, 12 * sizeof(unsigned long long), s));
+    BFC_CUDA(cudaMemsetAsync(pl->red, 0, kRedWords * sizeof(unsigned long long), s));
     // ---- a2: graph-major ranks; a degree is below 2^16 (at most the other layer)
     int rc = launch_ranks(g, pl->deg_l, pl->deg_u, gl, gu, pl->max_layer, pl->k0, pl->v0, pl->k1, pl->v1, pl->hist,
                           pl->hist_tmp, pl->deg_star, pl->deg64, pl->red + 9, s, guard);
@@ -1954,11 +2004,9 @@ int batch_plan_run(BatchPlan *pl, const int32_t *off_u, const int32_t *adj_u, co
         BFC_CUDA(cudaGetLastError());
     }
     // ---- a4: cut, runs, work
-    if (n > 0) { k_cut<<<blocks_for(n), kT, 0, s>>>(g->off, g->adj, pl->deg_star, n, l, g->cut, guard); note_launch(); }
     if (n > 0) {
         BFC_CUDA(cudaMemsetAsync(g->gwork, 0, sizeof(unsigned long long) * G, s));
-        BFC_CUDA(cudaMemsetAsync(pl->n_big, 0, 2 * sizeof(int32_t), s));
-        launch_work(g, pl->big, pl->n_big, g->gwork, pl->red, s, guard);
+        launch_work(g, pl->deg_star, pl->big, pl->n_big, s, guard);
         BFC_CUDA(cudaGetLastError());
     }
     // ---- a5: heaviest first, bins from device counts
@@ -1968,7 +2016,7 @@ int batch_plan_run(BatchPlan *pl, const int32_t *off_u, const int32_t *adj_u, co
     unsigned long long *bins = pl->red + 3;
     if (n > 0) {
         const BinBounds bb{(uint64_t)opt->warp_max_work, pl->team_max, (uint64_t)opt->hash_max_work, l, n, n, g->cut};
-        rc = bin_starts(g, s, bb, bins, pl->heavy, guard);
+        rc = bin_starts(g, s, bb, bins, pl->heavy, pl->red, guard);
         if (rc) return rc;
         k_sched_keys_plan<<<blocks_for(n), kT, 0, s>>>(g->work, pl->heavy, n, bb, bins, pl->k0); note_launch();
         BFC_CUDA(cudaGetLastError());
