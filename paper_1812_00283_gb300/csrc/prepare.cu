@@ -386,7 +386,10 @@ __global__ void __launch_bounds__(kRowCtaThreads) k_u_rows_warp_sort(
 __global__ void __launch_bounds__(kRowCtaThreads) k_u_rows_cta(
     const int32_t *__restrict__ off_u, const int32_t *__restrict__ adj_u,
     const int32_t *__restrict__ rank_u, const int32_t *__restrict__ rank_l,
-    const int32_t *__restrict__ rows, int32_t nrows, URowOut o) {
+    const int32_t *__restrict__ rows, const int32_t *__restrict__ nrows_dev, URowOut o,
+    const int *guard = nullptr) {
+    if (aborted(guard)) return;
+    const int32_t nrows = *nrows_dev;
     __shared__ uint64_t buf[kRowCtaMax];
     for (int64_t i0 = blockIdx.x; i0 < nrows; i0 += gridDim.x) {
         const int32_t u = rows[i0];
@@ -423,8 +426,8 @@ __global__ void __launch_bounds__(kRowCtaThreads) k_u_rows_cta(
 // lists of the rows of every tier above 32 neighbours (any order: every row
 // is written to its own slots); one atomic per warp and list.  lists[t * r ...]:
 // tier 0 warp sort, 1 and 2 bitmap, 3 CTA sort, 4 radix.  `range`: the L ranks of
-// a single graph (a batch's row: its graph's); bitmaps only where `bitmaps`, and
-// tier 2 only where `wide_tier`.
+// a single graph (a batch's row: its graph's); bitmaps only where `bitmaps`
+// (2: above 4,096 neighbours only), and tier 2 only where `wide_tier`.
 __global__ void k_row_tiers(const int32_t *__restrict__ off_u, int32_t r, int32_t range,
                             const int32_t *__restrict__ gu, const int32_t *__restrict__ gl, int32_t num_graphs,
                             int bitmaps, int wide_tier, int32_t *lists, int32_t *counts,
@@ -442,7 +445,8 @@ __global__ void k_row_tiers(const int32_t *__restrict__ off_u, int32_t r, int32_
                 const int32_t g = graph_of(gu, num_graphs, (int32_t)u);
                 len = gl[g + 1] - gl[g];
             }
-            tier = (bitmaps && len <= kRowBitmapMax) ? (d <= kRowCtaMax || !wide_tier ? 1 : 2) : (d <= kRowCtaMax ? 3 : 4);
+            tier = (bitmaps && len <= kRowBitmapMax) ? (d <= kRowCtaMax && bitmaps == 2 ? 3 : (d <= kRowCtaMax || !wide_tier ? 1 : 2))
+                                                     : (d <= kRowCtaMax ? 3 : 4);
         }
         if (!__any_sync(0xffffffffu, tier >= 0)) continue;
 #pragma unroll
@@ -595,10 +599,13 @@ __global__ void k_large_emit(const uint64_t *__restrict__ keys, const int32_t *_
 // per vertex), writes 4 bytes at random for the U starts' middles only; a
 // binary search of the middle's list per slot took 15.8 ms on a 300M-edge
 // shopping graph.
+// `dups` (validate = 0, where the caller answers for them): the edges of a
+// duplicate group are neighbours on both sides, and each takes the first one's
+// positions.
 template <bool kRuns>
 __global__ void k_emit_l_side(const uint64_t *__restrict__ keys2, const int32_t *__restrict__ vals2,
                               int64_t m, int bu, int32_t l, const int64_t *__restrict__ off, int32_t *adj_star,
-                              int32_t *eid_star, int32_t *rows_star, int32_t *plen, int64_t *sbeg,
+                              int32_t *eid_star, int32_t *rows_star, int32_t *plen, int64_t *sbeg, int dups,
     const int *guard = nullptr) {
     if (aborted(guard)) return;
     const uint64_t mask_u = (1ull << bu) - 1ull;
@@ -611,13 +618,16 @@ __global__ void k_emit_l_side(const uint64_t *__restrict__ keys2, const int32_t 
         rows_star[i] = v;
         if (kRuns) {
             const int64_t bv = off[v], bu0 = off[u];
+            int64_t first = i;
+            if (dups)
+                while (first > bv && keys2[first - 1] == key) --first;
             // equal degrees: the U vertex has the higher priority
             if (off[u + 1] - bu0 < off[v + 1] - bv) {
-                plen[i] = (int32_t)(m + k - bu0);
+                plen[i] = (int32_t)(m + vals2[first] - bu0);
                 sbeg[i] = bu0;
             } else {
                 plen[i] = 0;
-                plen[m + k] = (int32_t)(i - bv);
+                plen[m + k] = (int32_t)(first - bv);
             }
         }
     }
@@ -1553,6 +1563,10 @@ static int launch_u_rows(const int32_t *off_u, const int32_t *adj_u, Graph *g, i
                 off_u, adj_u, g->rank_u, g->rank_l, tier_rows + r, tier_n + 1, range, gl, gu, num_graphs, uo, guard);
         note_launch();
     }
+    if (bitmaps == 2 && m > kRowWarpSortMax) {
+        k_u_rows_cta<<<(unsigned)std::min<int64_t>(m / kRowWarpSortMax, 152 * 16), kRowCtaThreads, 0, s>>>(
+            off_u, adj_u, g->rank_u, g->rank_l, tier_rows + 3 * (int64_t)r, tier_n + 3, uo, guard); note_launch();
+    }
     if (bitmaps && wide_tier && m > kRowCtaMax) {
         k_u_rows_bitmap<1024>
             <<<(unsigned)std::min<int64_t>(m / kRowCtaMax, 152 * 2), 1024, bitmap_bytes(range), s>>>(
@@ -1718,7 +1732,8 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
             if (int rc = input_error(herr, num_graphs)) return rc;
             if (hn[0] > 0) {
                 k_u_rows_cta<<<(unsigned)std::min<int32_t>(hn[0], 152 * 16), kRowCtaThreads, 0, s>>>(
-                    csr->off_u, csr->adj_u, g->rank_u, g->rank_l, tier_rows + 3 * (int64_t)r, hn[0], uo); note_launch();
+                    csr->off_u, csr->adj_u, g->rank_u, g->rank_l, tier_rows + 3 * (int64_t)r, tier_n + 3,
+                    uo, guard_err); note_launch();
                 BFC_CUDA(cudaGetLastError());
             }
             const int32_t *large_rows = tier_rows + 4 * (int64_t)r;
@@ -1766,10 +1781,11 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
         if (opt->orientation == 0) {
             BFC_CUDA(cudaMemsetAsync(g->plen + m, 0, sizeof(int32_t) * (size_t)m, s));
             k_emit_l_side<true><<<grid_stride_blocks(m), kT, 0, s>>>(k2, v2, m, bu, l, g->off, g->adj, g->eid,
-                                                                      rows_star, g->plen, g->sbeg, guard_err); note_launch();
+                                                                      rows_star, g->plen, g->sbeg, !opt->validate,
+                                                                      guard_err); note_launch();
         } else {
             k_emit_l_side<false><<<grid_stride_blocks(m), kT, 0, s>>>(k2, v2, m, bu, l, g->off, g->adj, g->eid,
-                                                                       rows_star, nullptr, nullptr, guard_err); note_launch();
+                                                                       rows_star, nullptr, nullptr, 0, guard_err); note_launch();
         }
         BFC_CUDA(cudaGetLastError());
     }
@@ -1991,7 +2007,11 @@ int batch_plan_run(BatchPlan *pl, const int32_t *off_u, const int32_t *adj_u, co
     const int bl = bits_for(l > 0 ? (uint64_t)(l - 1) : 0);
     if (m > 0) {
         const URowOut uo{m, l, bu, g->off, g->adj, g->eid, pl->rows_star, pl->k1, g->err, opt->validate};
-        rc = launch_u_rows(off_u, adj_u, g, pl->max_layer, gu, gl, G, 1, uo, pl->tier_rows, pl->tier_n, s, guard);
+        // duplicate edges that the caller answers for keep their order in every row
+        // but the longest
+        if (!opt->validate) { k_check_batch_rows<<<grid_stride_blocks(r), kT, 0, s>>>(off_u, adj_u, r, gu, gl, G, g->err, guard); note_launch(); }
+        rc = launch_u_rows(off_u, adj_u, g, pl->max_layer, gu, gl, G, opt->validate ? 1 : 2, uo, pl->tier_rows, pl->tier_n,
+                           s, guard);
         if (rc) return rc;
         // L side: stable sort of the swapped keys on their rank_l bits
         int which2 = 0;
@@ -2000,7 +2020,7 @@ int batch_plan_run(BatchPlan *pl, const int32_t *off_u, const int32_t *adj_u, co
         const int32_t *v2 = which2 ? pl->v0 : pl->v1;
         BFC_CUDA(cudaMemsetAsync(g->plen + m, 0, sizeof(int32_t) * (size_t)m, s));
         k_emit_l_side<true><<<grid_stride_blocks(m), kT, 0, s>>>(k2, v2, m, bu, l, g->off, g->adj, g->eid,
-                                                                  pl->rows_star, g->plen, g->sbeg, guard); note_launch();
+                                                                  pl->rows_star, g->plen, g->sbeg, !opt->validate, guard); note_launch();
         BFC_CUDA(cudaGetLastError());
     }
     // ---- a4: cut, runs, work

@@ -203,3 +203,42 @@ def test_sparsified_samples_in_two_groups():
     for j in (0, 1, 213, 214, 229):
         ref = oracle.sparsify(g, p, 99, j)
         assert int(kept[j]) == ref.num_edges and int(tot[j]) == oracle.vp(ref)["total"]
+
+
+def test_unchecked_duplicate_edges_count_as_parallel_edges():
+    # validate = 0 leaves duplicates to the caller: they are walked as parallel
+    # edges in Definition 3's order, in rows of every tier
+    from paper_1812_00283_gb300 import bfc
+    rng = np.random.default_rng(5)
+    rows = [np.sort(np.concatenate([rng.choice(340, d, replace=False), rng.integers(0, 340, k)]))
+            for d, k in ((5, 2), (6, 1), (20, 3), (30, 2), (60, 4), (120, 5), (240, 9), (300, 20), (12, 0), (3, 1))]
+    off = np.concatenate([[0], np.cumsum([len(r) for r in rows])]).astype(np.int32)
+    adj = np.concatenate(rows).astype(np.int32)
+    r, l, m = len(rows), 340, adj.size
+    mult = np.zeros((r, l), dtype=np.int64)
+    np.add.at(mult, (np.repeat(np.arange(r), np.diff(off)), adj), 1)
+    deg = np.concatenate([mult.sum(0), mult.sum(1)])
+    pri = np.lexsort((np.arange(r + l), deg)).argsort()
+    full = np.zeros((r + l, r + l), dtype=np.int64)
+    full[l:, :l], full[:l, l:] = mult, mult.T
+    want = 0
+    for x in range(r + l):
+        lower = pri < pri[x]
+        c = ((full[x] * lower) @ full) * lower
+        want += int((c * (c - 1) // 2).sum())
+    o, a = torch.from_numpy(off).cuda(), torch.from_numpy(adj).cuda()
+    s = torch.cuda.current_stream().cuda_stream
+    h = bfc.bfc_prepare(r, l, m, o.data_ptr(), a.data_ptr(), _opts(validate=0), s)
+    tot = torch.zeros(1, dtype=torch.int64, device="cuda")
+    bfc.bfc_count(h, s, tot.data_ptr())
+    bfc.bfc_sync(h, s)
+    bfc.bfc_release(h)
+    assert int(tot.item()) == want
+    start = [torch.tensor(v, dtype=torch.int32, device="cuda") for v in ([0, r], [0, l])]
+    status = torch.full((1,), -1, dtype=torch.int32, device="cuda")
+    plan = bfc.bfc_batch_plan_create(r, l, m, 1, 400, _opts(validate=0), s)
+    bfc.bfc_batch_plan_run(plan, o.data_ptr(), a.data_ptr(), start[0].data_ptr(), start[1].data_ptr(), s, tot.data_ptr(),
+                           status.data_ptr())
+    torch.cuda.synchronize()
+    bfc.bfc_batch_plan_destroy(plan)
+    assert int(status.item()) == 0 and int(tot.item()) == want
