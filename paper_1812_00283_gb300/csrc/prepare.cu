@@ -30,6 +30,16 @@ inline unsigned blocks_for(int64_t n, int t = kT) {
 __device__ __forceinline__ bool aborted(const int *guard) {
     return guard && (*(volatile const int *)guard & (kErrBadOffsets | kErrBadId));
 }
+// The row kernels set the word that they are guarded by (an edge to another
+// graph of the batch), so threads that read it for themselves can differ.  A
+// kernel whose warps or CTAs work together leaves by one decision for all of
+// them: called by every thread of the warp, of the CTA.
+__device__ __forceinline__ bool aborted_warp(const int *guard) {
+    return __any_sync(0xffffffffu, aborted(guard));
+}
+__device__ __forceinline__ bool aborted_cta(const int *guard) {
+    return __syncthreads_or(aborted(guard));
+}
 
 // ----- validation and a1: degrees ----------------------------------------------
 // One pass over the caller's arrays (always on: every later index depends on
@@ -93,7 +103,7 @@ __global__ void __launch_bounds__(kT) k_ranks(const int32_t *__restrict__ order,
                                               int32_t *rank_l, int32_t *rank_u, int32_t *deg_star, int64_t *deg64,
                                               unsigned long long *top,
     const int *guard = nullptr) {
-    if (aborted(guard)) return;
+    if (aborted_cta(guard)) return;
     __shared__ int32_t best[2];
     if (threadIdx.x < 2) best[threadIdx.x] = 0;
     __syncthreads();
@@ -168,7 +178,7 @@ __global__ void k_u_rows_warp(const int32_t *__restrict__ off_u, const int32_t *
                               int32_t r, int span, const int32_t *__restrict__ gl,
                               const int32_t *__restrict__ gu, int32_t num_graphs, URowOut o,
     const int *guard = nullptr) {
-    if (aborted(guard)) return;
+    if (aborted_warp(guard)) return;
     const int lane = threadIdx.x & 31;
     const int g = lane >> 3, j = lane & 7;
     bool cross = false;   // a batch: an L rank outside the row's graph
@@ -313,7 +323,7 @@ __global__ void __launch_bounds__(kRowCtaThreads) k_u_rows_warp_reg(
     const int32_t *__restrict__ rows, const int32_t *__restrict__ nrows_dev,
     const int32_t *__restrict__ gl, const int32_t *__restrict__ gu, int32_t num_graphs, URowOut o,
     const int *guard = nullptr) {
-    if (aborted(guard)) return;
+    if (aborted_warp(guard)) return;
     __shared__ uint32_t buf[kRowCtaThreads / 32][kRowWarpSortMax];
     const int lane = threadIdx.x & 31;
     uint32_t *wb = buf[threadIdx.x >> 5];
@@ -356,7 +366,7 @@ __global__ void __launch_bounds__(kRowCtaThreads) k_u_rows_warp_sort(
     const int32_t *__restrict__ rank_u, const int32_t *__restrict__ rank_l,
     const int32_t *__restrict__ rows, const int32_t *__restrict__ nrows_dev, URowOut o,
     const int *guard = nullptr) {
-    if (aborted(guard)) return;
+    if (aborted_warp(guard)) return;
     const int32_t nrows = *nrows_dev;
     __shared__ uint64_t buf[kRowCtaThreads / 32][kRowWarpSortMax];
     const int lane = threadIdx.x & 31;
@@ -388,7 +398,7 @@ __global__ void __launch_bounds__(kRowCtaThreads) k_u_rows_cta(
     const int32_t *__restrict__ rank_u, const int32_t *__restrict__ rank_l,
     const int32_t *__restrict__ rows, const int32_t *__restrict__ nrows_dev, URowOut o,
     const int *guard = nullptr) {
-    if (aborted(guard)) return;
+    if (aborted_cta(guard)) return;
     const int32_t nrows = *nrows_dev;
     __shared__ uint64_t buf[kRowCtaMax];
     for (int64_t i0 = blockIdx.x; i0 < nrows; i0 += gridDim.x) {
@@ -432,7 +442,7 @@ __global__ void k_row_tiers(const int32_t *__restrict__ off_u, int32_t r, int32_
                             const int32_t *__restrict__ gu, const int32_t *__restrict__ gl, int32_t num_graphs,
                             int bitmaps, int wide_tier, int32_t *lists, int32_t *counts,
     const int *guard = nullptr) {
-    if (aborted(guard)) return;
+    if (aborted_warp(guard)) return;
     const int lane = threadIdx.x & 31;
     const uint32_t lt = (1u << lane) - 1u;
     for (int64_t u0 = (int64_t)blockIdx.x * blockDim.x; u0 < r; u0 += (int64_t)gridDim.x * blockDim.x) {
@@ -474,7 +484,7 @@ __global__ void __launch_bounds__(kThreads) k_u_rows_bitmap(
     const int32_t *__restrict__ rows, const int32_t *__restrict__ nrows_dev, int32_t range,
     const int32_t *__restrict__ gl, const int32_t *__restrict__ gu, int32_t num_graphs, URowOut o,
     const int *guard = nullptr) {
-    if (aborted(guard)) return;
+    if (aborted_cta(guard)) return;
     extern __shared__ __align__(16) uint32_t bm_smem[];   // bits[words], then prefix of each 4 words
     __shared__ int32_t part[kThreads / 32];
     __shared__ int32_t n_dup;
@@ -704,7 +714,7 @@ __global__ void k_work(const int64_t *__restrict__ off, const int32_t *__restric
                        const int32_t *__restrict__ deg_star, int32_t l, int32_t *cut,
                        const int32_t *__restrict__ plen, int32_t n, int all_slots, int64_t fill_from, int64_t *sbeg, uint64_t *work, int32_t *queue, int32_t *queued,
     const int *guard = nullptr) {
-    if (aborted(guard)) return;
+    if (aborted_warp(guard)) return;
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -775,7 +785,7 @@ __global__ void __launch_bounds__(kWorkThreads) k_work_long(
     const int32_t *__restrict__ plen, int32_t n, int all_slots, int64_t fill_from, int64_t *sbeg, uint64_t *work,
     const int32_t *__restrict__ queue, const int32_t *__restrict__ queued,
     const int *guard = nullptr) {
-    if (aborted(guard)) return;
+    if (aborted_cta(guard)) return;
     __shared__ unsigned long long part[kWorkThreads / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int n_warp = queued[0], n_cta = queued[1];
@@ -848,7 +858,7 @@ __global__ void __launch_bounds__(kT) k_bin_starts(const uint64_t *__restrict__ 
                                                    const int32_t *__restrict__ gstar, unsigned long long *gwork,
     const int *guard = nullptr) {
     if (stats && guard && blockIdx.x == 0 && threadIdx.x == 0) stats[11] = (unsigned long long)*(volatile const int *)guard;
-    if (aborted(guard)) return;
+    if (aborted_cta(guard)) return;
     unsigned long long sum = 0, top = 0, above = 0;
     __shared__ int32_t cnt[6], at[3];   // at: this tile's room in heavy, warp front, warp back
     const int lane = threadIdx.x & 31;
@@ -1178,7 +1188,7 @@ __global__ void k_check_batch_rows(const int32_t *__restrict__ off, const int32_
                                    const int32_t *__restrict__ gu, const int32_t *__restrict__ gl,
                                    int32_t num_graphs, int *err,
     const int *guard = nullptr) {
-    if (aborted(guard)) return;
+    if (aborted_warp(guard)) return;
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
