@@ -500,6 +500,7 @@ int bfc_autotune(bfc_graph *h, void *stream, int iters, bfc_options *chosen) {
     BFC_CUDA(cudaEventCreate(&e1));
     float best = 1e30f;
     int32_t bw = g->opt.warp_max_work, bt = g->opt.team_max_work, bh = g->opt.hash_max_work;
+    const Cand before{bw, bt, bh};
     int rc = BFC_OK;
     for (int c = 0; c < nc; ++c) {
         rc = bfc::rebin_graph(g, s, cands[c].w, cands[c].t, cands[c].h);
@@ -519,9 +520,12 @@ int bfc_autotune(bfc_graph *h, void *stream, int iters, bfc_options *chosen) {
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    if (rc) return rc;
-    rc = bfc::rebin_graph(g, s, bw, bt, bh);
-    if (rc) return rc;
+    if (rc == BFC_OK) rc = bfc::rebin_graph(g, s, bw, bt, bh);
+    if (rc) {
+        // back to the bounds that the graph came with, if a rebinning failed
+        if (g->schedule_rc != BFC_OK) bfc::rebin_graph(g, s, before.w, before.t, before.h);
+        return rc;
+    }
     tuned_store(tuned_key(g->opt.orientation, g->num_graphs > 0, g->m, (int64_t)g->n), bw, bt, bh);
     if (chosen) *chosen = g->opt;
     return BFC_OK;

@@ -100,13 +100,15 @@ void pool_free(void *p, cudaStream_t s);
 cudaError_t pool_usage(int64_t *current, int64_t *high, bool reset_high);
 
 // A list of pool allocations released together.  Requests of at most 128 KB
-// are carved from 512 KB slabs (a prepare makes about forty of them, and each
-// pool call costs the host about a microsecond); a carved piece goes back with
-// its slab.
+// are carved from slabs (a prepare makes about forty of them, and each pool
+// call costs the host about a microsecond); a carved piece goes back with its
+// slab.  What is replaced while the list lives is taken by get_own and given back
+// by drop.
 struct Allocs {
     static constexpr size_t kSlab = 512 << 10, kCarve = 128 << 10;
     char *slab = nullptr;
     size_t slab_left = 0;
+    size_t slab_next = kSlab;   // size of the next slab; a smaller first one doubles up to kSlab
     static constexpr int kMax = 64;
     void *ptr[kMax];
     size_t bytes[kMax];
@@ -115,38 +117,32 @@ struct Allocs {
     cudaStream_t stream = nullptr;
     template <typename T>
     cudaError_t get(T **p, size_t count) {
-        if (n >= kMax) return cudaErrorMemoryAllocation;
-        size_t b = count * sizeof(T);
-        if (b == 0) b = 16;
-        b = (b + 255) & ~size_t(255);
-        if (b <= kCarve && b <= slab_left) {
-            *p = reinterpret_cast<T *>(slab);
-            slab += b;
-            slab_left -= b;
-            return cudaSuccess;
+        const size_t b = rounded(count * sizeof(T));
+        if (b > kCarve) return take(reinterpret_cast<void **>(p), b);
+        if (b > slab_left) {
+            const size_t size = slab_next > 2 * b ? slab_next : 2 * b;
+            void *q = nullptr;
+            const cudaError_t e = take(&q, size);
+            if (e != cudaSuccess) return e;
+            slab = static_cast<char *>(q);
+            slab_left = size;
+            slab_next = 2 * size < kSlab ? 2 * size : kSlab;
         }
-        const bool carve = b <= kCarve;
-        const size_t want = b;
-        if (carve) b = kSlab;
-        void *q = nullptr;
-        cudaError_t e = pool_alloc(&q, b, stream);
-        if (e != cudaSuccess) return e;
-        ptr[n] = q;
-        bytes[n] = b;
-        ++n;
-        total += b;
-        if (carve) {
-            slab = static_cast<char *>(q) + want;
-            slab_left = b - want;
-        }
-        *p = static_cast<T *>(q);
+        *p = reinterpret_cast<T *>(slab);
+        slab += b;
+        slab_left -= b;
         return cudaSuccess;
     }
-    // frees one allocation of the list (no-op for null, unknown and carved pointers)
+    // an allocation of its own, which drop gives back
+    template <typename T>
+    cudaError_t get_own(T **p, size_t count) {
+        return take(reinterpret_cast<void **>(p), rounded(count * sizeof(T)));
+    }
+    // frees one allocation of get_own (no-op for null)
     void drop(void *p) {
         if (!p) return;
         for (int i = 0; i < n; ++i)
-            if (ptr[i] == p && bytes[i] != kSlab) {
+            if (ptr[i] == p) {
                 pool_free(p, stream);
                 total -= bytes[i];
                 for (int j = i + 1; j < n; ++j) { ptr[j - 1] = ptr[j]; bytes[j - 1] = bytes[j]; }
@@ -160,6 +156,21 @@ struct Allocs {
         total = 0;
         slab = nullptr;
         slab_left = 0;
+    }
+
+private:
+    static size_t rounded(size_t b) { return ((b == 0 ? 16 : b) + 255) & ~size_t(255); }
+    cudaError_t take(void **p, size_t b) {
+        if (n >= kMax) return cudaErrorMemoryAllocation;
+        void *q = nullptr;
+        const cudaError_t e = pool_alloc(&q, b, stream);
+        if (e != cudaSuccess) return e;
+        ptr[n] = q;
+        bytes[n] = b;
+        ++n;
+        total += b;
+        *p = q;
+        return cudaSuccess;
     }
 };
 
@@ -185,10 +196,13 @@ struct Graph {
     int32_t *plen = nullptr;  // [2m] wedges through each middle slot (0 if not a middle slot)
     int32_t *cut = nullptr;   // [n]
     uint64_t *work = nullptr; // [n]
+    char *lists = nullptr;        // of the current schedule: the next two and `retry` (a plan's are apart)
+    size_t lists_bytes = 0;
     int2 *cta_items = nullptr;    // (start, chunk) / (start, -1 = hash)
     int32_t *team_items = nullptr;
     int32_t *warp_items = nullptr;   // [n]: the warp bin from the front, its tiny starts from the back
     int64_t n_cta_items = 0, n_team_items = 0, n_warp_items = 0, n_tiny_items = 0;
+    int schedule_rc = BFC_ERR_INTERNAL;   // BFC_OK once there is a schedule; else why the last one failed
     int32_t team_max = 0;          // effective team bound of the current schedule
     bool may_retry = false;        // the schedule can re-queue starts (retry pass launched)
     int *cursors = nullptr;        // [8] work-queue cursors of the count kernels
@@ -198,7 +212,6 @@ struct Graph {
     // chunk-boundary table: for vertex v of G*, entry c is the position in
     // N(v) of the first neighbour whose rank in its layer is >= c * kChunkUnit
     int32_t *coff = nullptr;
-    int64_t *coff_start = nullptr;   // a batch's table while it is built: first entry of each vertex
     int32_t *ctb = nullptr;          // a batch's table: first entry of each slot's middle (-1: none)
     int32_t coff_u1 = 0;   // entries per L vertex (its neighbours are U vertices)
     int32_t coff_l1 = 0;   // entries per U vertex

@@ -1807,6 +1807,10 @@ int count_smem_setup(int device) {
 
 int launch_count(Graph *g, cudaStream_t s, int mode, unsigned long long *pv_proj,
                  unsigned long long *pe, unsigned long long *gtot) {
+    if (g->schedule_rc != BFC_OK) {
+        set_last_error("the graph has no schedule: its last rebinning failed");
+        return g->schedule_rc;
+    }
     int rc = count_smem_setup(g->device);
     if (rc) return rc;
     CountParams p;

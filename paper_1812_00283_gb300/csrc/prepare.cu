@@ -1287,6 +1287,32 @@ static int bin_starts(Graph *g, cudaStream_t s, const BinBounds &bb, unsigned lo
     return BFC_OK;
 }
 
+// Room for a schedule's lists in one allocation: CTA items, team items and one
+// place per start that can be re-queued (each at most once per launch).  Another
+// rebinning takes it over where it is large enough, else replaces it.
+static int schedule_lists(Graph *g, int64_t n_items, int64_t n_team, int64_t retry_cap) {
+    n_items = std::max<int64_t>(n_items, 1);
+    n_team = std::max<int64_t>(n_team, 1);
+    retry_cap = std::max<int64_t>(retry_cap, 1);
+    const size_t need = (size_t)n_items * sizeof(int2) + (size_t)(n_team + retry_cap) * sizeof(int32_t);
+    if (need > g->lists_bytes) {
+        g->mem.drop(g->lists);
+        g->lists = nullptr;
+        g->lists_bytes = 0;
+        if (g->mem.get_own(&g->lists, need) != cudaSuccess) {
+            g->lists = nullptr;
+            set_last_error("device allocation failed: schedule lists");
+            return BFC_ERR_OUT_OF_MEMORY;
+        }
+        g->lists_bytes = need;
+    }
+    g->cta_items = reinterpret_cast<int2 *>(g->lists);
+    g->team_items = reinterpret_cast<int32_t *>(g->cta_items + n_items);
+    g->retry = g->team_items + n_team;
+    g->retry_cap = retry_cap;
+    return BFC_OK;
+}
+
 // Step a5: order the starts by descending exact work and split them into the
 // warp, CTA-hash and CTA-dense bins (dense starts into end-range chunks);
 // builds the chunk-boundary table when a dense start has several chunks.
@@ -1355,8 +1381,7 @@ static int schedule_graph(Graph *g, cudaStream_t s, int32_t warp_max_work, int32
             BFC_CUDA(cudaStreamSynchronize(s));
         }
         n_items = h_dense_items + n_hash;
-        GET(g->mem, g->cta_items, std::max<int64_t>(n_items, 1));
-        GET(g->mem, g->team_items, std::max<int64_t>(n_team, 1));
+        if (int rc = schedule_lists(g, n_items, n_team, n_hash + n_team)) return rc;
         if (n_heavy > 0) {
             k_emit_items<<<grid_stride_blocks(n_heavy), kT, 0, s>>>(
                 order, n_dense, n_hash, n_team, nch_scan, l, g->cut, g->off, g->vbase, vpp ? 1 : 0, g->cta_items,
@@ -1372,18 +1397,18 @@ static int schedule_graph(Graph *g, cudaStream_t s, int32_t warp_max_work, int32
             // chunks, as many as the chunks of their graph's neighbour layer
             // (+1), found through a per-vertex start array
             int32_t *mark;
-            int64_t *ecnt;
+            int64_t *ecnt, *cstart;   // cstart: first entry of each vertex
             GET(tmp, mark, n);
             GET(tmp, ecnt, (int64_t)n + 1);
-            GET(g->mem, g->coff_start, (int64_t)n + 1);
+            GET(tmp, cstart, (int64_t)n + 1);
             BFC_CUDA(cudaMemsetAsync(mark, 0, sizeof(int32_t) * (size_t)n, s));
             k_coff_mark<<<grid_stride_blocks(n_dense * 32), kT, 0, s>>>(order, n_dense, nch, g->off, g->adj,
                                                                          g->cut, mark); note_launch();
             k_coff_sizes<<<grid_stride_blocks(n), kT, 0, s>>>(mark, g->off, g->adj, g->vbase, g->vend, n, ecnt); note_launch();
             BFC_CUDA(cudaGetLastError());
-            BFC_CUDA(scan_exclusive<int64_t>(ecnt, g->coff_start, n, scan64_tmp, s));
+            BFC_CUDA(scan_exclusive<int64_t>(ecnt, cstart, n, scan64_tmp, s));
             int64_t ventries = 0;
-            BFC_CUDA(cudaMemcpyAsync(&ventries, g->coff_start + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+            BFC_CUDA(cudaMemcpyAsync(&ventries, cstart + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
             BFC_CUDA(cudaStreamSynchronize(s));
             if (ventries <= kChunkTableMaxEntries) {   // else searches
                 if (!rows_star) {
@@ -1394,21 +1419,19 @@ static int schedule_graph(Graph *g, cudaStream_t s, int32_t warp_max_work, int32
                     rows_star = rs;
                 }
                 GET(g->mem, g->coff, std::max<int64_t>(ventries, 1));
-                k_coff_fill_var<<<grid_stride_blocks(n), kT, 0, s>>>(g->off, g->coff_start, n, g->coff); note_launch();
+                k_coff_fill_var<<<grid_stride_blocks(n), kT, 0, s>>>(g->off, cstart, n, g->coff); note_launch();
                 BFC_CUDA(cudaGetLastError());
                 k_coff_slots_var<<<grid_stride_blocks(2 * m), kT, 0, s>>>(g->off, g->adj, rows_star, 2 * m,
-                                                                          g->vbase, g->coff_start, g->coff); note_launch();
+                                                                          g->vbase, cstart, g->coff); note_launch();
                 BFC_CUDA(cudaGetLastError());
                 // each middle slot of those starts holds its middle's first
                 // entry (-1 elsewhere), read with the slot's other arrays
                 GET(g->mem, g->ctb, 2 * m);
                 BFC_CUDA(cudaMemsetAsync(g->ctb, 0xff, sizeof(int32_t) * (size_t)(2 * m), s));
                 k_coff_slot_bases<<<grid_stride_blocks(n_dense * 32), kT, 0, s>>>(order, n_dense, nch, g->off, g->adj,
-                                                                                   g->cut, g->coff_start, g->ctb); note_launch();
+                                                                                   g->cut, cstart, g->ctb); note_launch();
                 BFC_CUDA(cudaGetLastError());
             }
-            g->mem.drop(g->coff_start);
-            g->coff_start = nullptr;
         }
         if (!g->coff && g->num_graphs == 0 && h_dense_items > n_dense && entries <= kChunkTableMaxEntries) {
             if (!rows_star) {
@@ -1427,21 +1450,15 @@ static int schedule_graph(Graph *g, cudaStream_t s, int32_t warp_max_work, int32
                                                                   g->coff); note_launch();
             BFC_CUDA(cudaGetLastError());
         }
-    } else {
-        GET(g->mem, g->cta_items, 1);
-        GET(g->mem, g->team_items, 1);
+    } else if (int rc = schedule_lists(g, 0, 0, 0)) {
+        return rc;
     }
     g->n_cta_items = n_items;
     g->n_team_items = n_team;
     g->n_warp_items = n_warp;
     g->n_tiny_items = n_tiny;
     g->team_max = (int32_t)std::min<uint64_t>(team_max, (uint64_t)kTeamMaxWork);
-    // each hash start is re-queued at most once per launch
-    g->mem.drop(g->retry);
-    g->retry = nullptr;
     g->retry_static = 0;
-    g->retry_cap = std::max<int64_t>(n_hash + n_team, 1);
-    GET(g->mem, g->retry, g->retry_cap);
     if (vpp && hash_max_work == 0 && n_hash > 0) {
         // every start beyond the warp bin goes to the dense pass directly
         k_items_to_dense_retries<<<blocks_for(n_hash), kT, 0, s>>>(g->cta_items, n_hash, g->retry); note_launch();
@@ -1462,16 +1479,16 @@ static int schedule_graph(Graph *g, cudaStream_t s, int32_t warp_max_work, int32
     g->opt.team_max_work = team_max_work;
     g->opt.hash_max_work = hash_max_work;
 #undef GET
+    g->schedule_rc = BFC_OK;
     return BFC_OK;
 }
 
 int rebin_graph(Graph *g, cudaStream_t s, int32_t warp_max_work, int32_t team_max_work,
                 int32_t hash_max_work) {
+    // no schedule until the new one is whole: a count after a failure reports it
+    // and launches nothing
+    g->schedule_rc = BFC_ERR_OUT_OF_MEMORY;
     g->mem.stream = s;
-    g->mem.drop(g->cta_items);
-    g->mem.drop(g->team_items);
-    g->cta_items = nullptr;
-    g->team_items = nullptr;
     Allocs tmp;
     tmp.stream = s;
     struct TmpGuard { Allocs *a; ~TmpGuard() { a->release(); } } guard{&tmp};
@@ -1487,8 +1504,8 @@ int rebin_graph(Graph *g, cudaStream_t s, int32_t warp_max_work, int32_t team_ma
     BFC_CUDA(cudaMemcpyAsync(hc, counts, sizeof(hc), cudaMemcpyDeviceToHost, s));
     BFC_CUDA(cudaStreamSynchronize(s));
     rc = schedule_graph(g, s, warp_max_work, team_max_work, hash_max_work, nullptr, bb, hc, heavy);
-    if (rc == BFC_OK) BFC_CUDA(cudaStreamSynchronize(s));
     g->info.device_bytes = (int64_t)g->mem.total;
+    if (rc == BFC_OK) BFC_CUDA(cudaStreamSynchronize(s));
     return rc;
 }
 
@@ -1611,6 +1628,7 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
     g->opt = *opt;
     g->stream = s;
     g->mem.stream = s;
+    g->mem.slab_next = 64 << 10;   // many small graphs may be kept: the first slab is no larger than they need
 
     Allocs tmp;
     tmp.stream = s;
@@ -1969,7 +1987,8 @@ int batch_plan_create(BatchPlan *pl, cudaStream_t s) {
     // every kept array starts zeroed: a run that stops at the checks leaves
     // arrays that later kernels can still index safely
     for (int i = 0; i < g->mem.n; ++i) BFC_CUDA(cudaMemsetAsync(g->mem.ptr[i], 0, g->mem.bytes[i], s));
-    g->n_cta_items = 0; g->n_team_items = 0; g->n_warp_items = 0;
+    g->n_cta_items = 0; g->n_team_items = 0; g->n_warp_items = 0;   // a run's are in device memory
+    g->schedule_rc = BFC_OK;
     g->retry_static = 0; g->retry_cap = 1; g->may_retry = false;
     g->info.num_u = r; g->info.num_l = l; g->info.num_edges = m;
     g->info.device_bytes = (int64_t)g->mem.total;
