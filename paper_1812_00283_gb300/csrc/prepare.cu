@@ -1418,19 +1418,22 @@ static int schedule_graph(Graph *g, cudaStream_t s, int32_t warp_max_work, int32
                     BFC_CUDA(cudaGetLastError());
                     rows_star = rs;
                 }
-                GET(g->mem, g->coff, std::max<int64_t>(ventries, 1));
-                k_coff_fill_var<<<grid_stride_blocks(n), kT, 0, s>>>(g->off, cstart, n, g->coff); note_launch();
-                BFC_CUDA(cudaGetLastError());
-                k_coff_slots_var<<<grid_stride_blocks(2 * m), kT, 0, s>>>(g->off, g->adj, rows_star, 2 * m,
-                                                                          g->vbase, cstart, g->coff); note_launch();
-                BFC_CUDA(cudaGetLastError());
                 // each middle slot of those starts holds its middle's first
                 // entry (-1 elsewhere), read with the slot's other arrays
-                GET(g->mem, g->ctb, 2 * m);
-                BFC_CUDA(cudaMemsetAsync(g->ctb, 0xff, sizeof(int32_t) * (size_t)(2 * m), s));
-                k_coff_slot_bases<<<grid_stride_blocks(n_dense * 32), kT, 0, s>>>(order, n_dense, nch, g->off, g->adj,
-                                                                                   g->cut, cstart, g->ctb); note_launch();
+                int32_t *coff, *ctb;
+                GET(g->mem, coff, std::max<int64_t>(ventries, 1));
+                GET(g->mem, ctb, 2 * m);
+                k_coff_fill_var<<<grid_stride_blocks(n), kT, 0, s>>>(g->off, cstart, n, coff); note_launch();
                 BFC_CUDA(cudaGetLastError());
+                k_coff_slots_var<<<grid_stride_blocks(2 * m), kT, 0, s>>>(g->off, g->adj, rows_star, 2 * m,
+                                                                          g->vbase, cstart, coff); note_launch();
+                BFC_CUDA(cudaGetLastError());
+                BFC_CUDA(cudaMemsetAsync(ctb, 0xff, sizeof(int32_t) * (size_t)(2 * m), s));
+                k_coff_slot_bases<<<grid_stride_blocks(n_dense * 32), kT, 0, s>>>(order, n_dense, nch, g->off, g->adj,
+                                                                                   g->cut, cstart, ctb); note_launch();
+                BFC_CUDA(cudaGetLastError());
+                g->coff = coff;   // the two only together
+                g->ctb = ctb;
             }
         }
         if (!g->coff && g->num_graphs == 0 && h_dense_items > n_dense && entries <= kChunkTableMaxEntries) {

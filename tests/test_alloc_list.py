@@ -129,6 +129,16 @@ def test_alloc_list(tmp_path):
     assert r.returncode == 0, r.stdout
 
 
+def test_chunk_table_of_a_batch_is_set_whole():
+    # a count takes a batch's chunk table as two arrays: with only the first one set
+    # (the pool refused the second) it would index the first as a single graph's
+    src = open(os.path.join(ROOT, "paper_1812_00283_gb300", "csrc", "prepare.cu")).read()
+    batch = src[src.index("if (ventries <= kChunkTableMaxEntries)"):]
+    batch = batch[:batch.index("\n            }\n")]
+    last_request = batch.rindex("GET(")
+    assert 0 < last_request < batch.index("g->coff = ") and "&g->coff" not in batch and "g->mem, g->" not in batch
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("orientation", [0, 1])
 @pytest.mark.parametrize("size", [(2000, 3000, 20_000), (48_611, 31_013, 2_000_000)])
