@@ -74,7 +74,14 @@ typedef struct bfc_csr {
  * options pointer means the defaults. */
 typedef struct bfc_options {
     int32_t validate;       /* 1 (default): reject duplicate edges.  Offsets and
-                               id ranges are always checked. */
+                               id ranges are always checked.  0: an edge that
+                               occurs k times counts as k parallel edges (every
+                               count is then one of wedges over parallel edges,
+                               in the order of degrees with multiplicity, and
+                               there is no dense core).  A batch plan holds such
+                               counts in 16 bits: no pair of vertices may have
+                               more than 65,535 wedges, and no list of more than
+                               4,096 neighbours may repeat one. */
     int32_t warp_max_work;  /* starts with at most this many wedges are counted
                                by one warp with a 512-slot shared-memory hash
                                table (default 384, range [0, 384]; a table is at

@@ -51,9 +51,16 @@ __host__ __device__ constexpr int32_t dense_chunk_span(int64_t bound) {
 // min(cut[x], deg(w)), and within a layer G* orders vertices by Definition 3's
 // priority, so degrees do not decrease with the id and the chunk's last end
 // bounds every count of the chunk.  Returns the chunk's end; *bits = 4, 8, 16
-// or 32.  `off` is G*'s offset array.
+// or 32.  `off` is G*'s offset array.  With parallel edges a count is a sum of
+// products, which neither bounds: then `most` is the largest count that x can
+// have (its wedges), else 0.
 __device__ __forceinline__ int32_t dense_chunk_end(int32_t lo, int32_t R, int64_t cut, const int64_t *off,
-                                                   int32_t lb, int *bits) {
+                                                   int32_t lb, uint64_t most, int *bits) {
+    if (most) {
+        *bits = most > kNarrowMaxCut ? 32 : (most > kByteMaxCut ? 16 : 8);
+        const int64_t end = (int64_t)lo + dense_chunk_span((int64_t)most);
+        return end < R ? (int32_t)end : R;
+    }
     int32_t hi = (int32_t)((int64_t)lo + kDense4 < R ? lo + kDense4 : R);
     int64_t top = off[lb + hi] - off[lb + hi - 1];
     if ((cut < top ? cut : top) <= (int64_t)kNibbleMax) { *bits = 4; return hi; }
@@ -75,6 +82,7 @@ constexpr int kErrDuplicate = 4;
 constexpr int kErrHashFull = 8;
 constexpr int kErrBounds = 16;
 constexpr int kErrTimeout = 32;   // a bounded device wait gave up
+constexpr int kErrParallel = 64;  // not an error: parallel edges that the caller answers for (validate = 0)
 
 // ---------------------------------------------------------------------------
 // Host-side error reporting
@@ -180,6 +188,7 @@ private:
 struct Graph {
     int32_t r = 0, l = 0, n = 0;
     int32_t max_range = 0;         // the larger layer (of a batch: of any one graph)
+    bool parallel = false;         // validate = 0 and an edge occurs more than once
     int64_t m = 0;
     bfc_options opt{};
     bfc_info info{};

@@ -98,6 +98,7 @@ struct CountParams {
     // failures stop the launch (null otherwise)
     const unsigned long long *__restrict__ item_counts;
     const int *guard;
+    int32_t parallel;   // 0 no parallel edges, 1 there are, 2 *err says it (a plan with validate = 0)
 };
 
 // item queue lengths: from the host, or from a batch plan's device counts
@@ -1075,9 +1076,20 @@ __device__ __forceinline__ unsigned long long end_bound(const CountParams &p, in
     return w < range ? w : range;
 }
 
+// The bounds on a count_wedge below rest on a simple graph.  With parallel edges a
+// count is a sum of products of multiplicities, which only the wedges of x bound:
+// those, or 0 without parallel edges.  A plan's dense start is one chunk of at
+// most 65,535 ends whatever it holds, so its counters never have more than 16 bits.
+__device__ __forceinline__ uint64_t parallel_bound(const CountParams &p, int32_t x) {
+    if (!p.parallel) return 0;
+    if (p.parallel == 1) return p.work[x];
+    return (*(volatile const int *)p.err & kErrParallel) ? min(p.work[x], (uint64_t)kNarrowMaxCut) : 0;
+}
+
 // A count_wedge is at most the number of middles: cut[x] (Algorithm 2) or
 // deg(x) (Algorithm 3).
 __device__ __forceinline__ int64_t middles(const CountParams &p, int32_t x) {
+    if (const uint64_t most = parallel_bound(p, x)) return (int64_t)most;
     return p.orient ? p.off[x + 1] - p.off[x] : (int64_t)p.cut[x];
 }
 
@@ -1087,7 +1099,8 @@ __device__ __forceinline__ int64_t middles(const CountParams &p, int32_t x) {
 __device__ __forceinline__ int packed_count_bits(const CountParams &p, int32_t x, int32_t R) {
     if (p.orient || R <= 0) return 0;
     const int64_t last = p.off[x] - p.off[x - 1];
-    const uint64_t c = min((uint64_t)min((int64_t)p.cut[x], last), (uint64_t)p.work[x]);
+    const uint64_t most = parallel_bound(p, x);
+    const uint64_t c = most ? most : min((uint64_t)min((int64_t)p.cut[x], last), (uint64_t)p.work[x]);
     const int cb = 64 - __clzll((long long)c), kb = 32 - __clz(R);
     return cb + kb <= 32 ? cb : 0;
 }
@@ -1180,7 +1193,7 @@ __device__ unsigned long long cta_item(const CountParams &p, int2 item, unsigned
         const int32_t R = x - lb;   // the ends are the R vertices below x
         const int32_t lo = item.y;   // the chunk's first end offset
         int bits;
-        const int32_t hi = dense_chunk_end(lo, R, p.cut[x], p.off, lb, &bits);
+        const int32_t hi = dense_chunk_end(lo, R, p.cut[x], p.off, lb, parallel_bound(p, x), &bits);
         const int kind = kind_of_bits(bits);
         const int32_t span = hi - lo;
         const int flags = (lo > 0 ? 1 : 0) | (hi < R ? 2 : 0);
@@ -1225,7 +1238,7 @@ __device__ unsigned long long dense_stream(const CountParams &p, int64_t &it, un
         const int32_t R = x - lb;   // the ends are the R vertices below x
         const int32_t lo = item.y;   // the chunk's first end offset
         int bits;
-        const int32_t hi = dense_chunk_end(lo, R, p.cut[x], p.off, lb, &bits);
+        const int32_t hi = dense_chunk_end(lo, R, p.cut[x], p.off, lb, parallel_bound(p, x), &bits);
         const int kind = kind_of_bits(bits);
         const int32_t span = hi - lo;
         const int flags = (lo > 0 ? 1 : 0) | (hi < R ? 2 : 0);
@@ -1318,7 +1331,8 @@ __device__ unsigned long long team_item(const CountParams &p, int32_t x, unsigne
         lb = range_lo(p, x);
         R = x - lb;
         const int64_t last = R > 0 ? p.off[x] - p.off[x - 1] : 0;
-        narrow = min(min((int64_t)p.cut[x], last), (int64_t)p.work[x]) > (int64_t)kByteMaxCut;
+        const uint64_t most = parallel_bound(p, x);
+        narrow = (most ? (int64_t)most : min(min((int64_t)p.cut[x], last), (int64_t)p.work[x])) > (int64_t)kByteMaxCut;
     }
     if (R > 0 && (narrow ? 2 * (int64_t)R : (int64_t)R) <= dense_bytes) {
         team_fill(table, narrow ? 2 * R : R, 0u, t);
@@ -1837,6 +1851,7 @@ int launch_count(Graph *g, cudaStream_t s, int mode, unsigned long long *pv_proj
     p.ccut = g->ccut; p.core_au = g->core_au; p.core_al = g->core_al;
     p.item_counts = g->item_counts;
     p.guard = g->item_counts ? g->err : nullptr;
+    p.parallel = g->item_counts ? (g->opt.validate ? 0 : 2) : (g->parallel ? 1 : 0);
     if (p.core_on) {
         // the core pairs' a(u, w), on the same stream before the walk
         int rc2 = core_product(g, s);

@@ -70,8 +70,8 @@ __global__ void k_check_input(const int32_t *__restrict__ off, const int32_t *__
 // value the global id (L vertex v -> v, U vertex u -> l + u, ascending before the
 // sort), so the stable sort's positions are the ids of G*: L first, each layer
 // (each graph's part of it) by (degree, id), Definition 3's order.  A degree
-// that does not fit its bits belongs to a row with duplicate edges; it is cut
-// off in the key only.
+// that does not fit its bits belongs to a row with duplicate edges that the
+// validation rejects; it is cut off in the key only.
 __device__ __forceinline__ int32_t graph_of(const int32_t *start, int32_t num_graphs, int32_t id) {
     int32_t lo = 0, hi = num_graphs;   // last g with start[g] <= id
     while (hi - lo > 1) {
@@ -159,7 +159,7 @@ struct URowOut {
     int32_t *adj_star, *eid_star, *rows_star;
     uint64_t *keys2;
     int *err;
-    int check_dup;   // flag duplicate edges (validate)
+    int dup_bit;     // what a duplicate edge sets: kErrDuplicate (validate) or kErrParallel
     __device__ __forceinline__ void put(int32_t ru, int64_t pos, int32_t rl, int32_t slot) const {
         const int64_t k = off_star[l + ru] - m + pos;   // U-side position
         adj_star[m + k] = rl;
@@ -222,7 +222,7 @@ __global__ void k_u_rows_warp(const int32_t *__restrict__ off_u, const int32_t *
                 dup |= ok == rl && k != j;
             }
             if (j < dk) {
-                if (dup && o.check_dup) atomicOr(o.err, kErrDuplicate);
+                if (dup) atomicOr(o.err, o.dup_bit);
                 o.put(rk, pos, rl, bk + j);
             }
         }
@@ -243,7 +243,7 @@ __global__ void k_u_rows_warp(const int32_t *__restrict__ off_u, const int32_t *
                 dup |= ok == rl && k != lane;
             }
             if (lane < dk) {
-                if (dup && o.check_dup) atomicOr(o.err, kErrDuplicate);
+                if (dup) atomicOr(o.err, o.dup_bit);
                 o.put(rk, pos, rl, bk + lane);
             }
         }
@@ -308,7 +308,7 @@ __device__ __forceinline__ void warp_sort_row(const int32_t *adj_u, const int32_
         const int i = r * 32 + lane;
         if (i < d) {
             const uint32_t k = buf[i];
-            if (o.check_dup && i > 0 && (buf[i - 1] >> 8) == (k >> 8)) atomicOr(o.err, kErrDuplicate);
+            if (i > 0 && (buf[i - 1] >> 8) == (k >> 8)) atomicOr(o.err, o.dup_bit);
             o.put(ru, i, base + (int32_t)(k >> 8), b + (int32_t)(k & 0xffu));
         }
     }
@@ -386,7 +386,7 @@ __global__ void __launch_bounds__(kRowCtaThreads) k_u_rows_warp_sort(
         for (int i = lane; i < d; i += 32) {
             const uint64_t vv = wb[i];
             const int32_t rl = (int32_t)(vv >> 32);
-            if (o.check_dup && i > 0 && (int32_t)(wb[i - 1] >> 32) == rl) atomicOr(o.err, kErrDuplicate);
+            if (i > 0 && (int32_t)(wb[i - 1] >> 32) == rl) atomicOr(o.err, o.dup_bit);
             o.put(ru, i, rl, (int32_t)(uint32_t)vv);
         }
         __syncwarp();   // the buffer is reused by the warp's next row
@@ -426,7 +426,7 @@ __global__ void __launch_bounds__(kRowCtaThreads) k_u_rows_cta(
         for (int i = threadIdx.x; i < d; i += kRowCtaThreads) {
             const uint64_t vv = buf[i];
             const int32_t rl = (int32_t)(vv >> 32);
-            if (o.check_dup && i > 0 && (int32_t)(buf[i - 1] >> 32) == rl) atomicOr(o.err, kErrDuplicate);
+            if (i > 0 && (int32_t)(buf[i - 1] >> 32) == rl) atomicOr(o.err, o.dup_bit);
             o.put(ru, i, rl, (int32_t)(uint32_t)vv);
         }
         __syncthreads();   // buf is reused by the next row
@@ -514,7 +514,7 @@ __global__ void __launch_bounds__(kThreads) k_u_rows_bitmap(
             }
             const uint32_t bit = 1u << (k & 31);
             if (atomicOr(&bm_smem[k >> 5], bit) & bit) {
-                if (o.check_dup) atomicOr(o.err, kErrDuplicate);
+                atomicOr(o.err, o.dup_bit);
                 o.put(ru, d - 1 - atomicAdd(&n_dup, 1), rl, b + i);
             }
         }
@@ -593,7 +593,7 @@ __global__ void k_large_emit(const uint64_t *__restrict__ keys, const int32_t *_
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
         const uint64_t key = keys[i];
-        if (o.check_dup && i > 0 && keys[i - 1] == key) atomicOr(o.err, kErrDuplicate);
+        if (i > 0 && keys[i - 1] == key) atomicOr(o.err, o.dup_bit);
         o.put((int32_t)(key >> bl), i - row_first[i], (int32_t)(key & mask_l), vals[i]);
     }
 }
@@ -629,8 +629,13 @@ __global__ void k_emit_l_side(const uint64_t *__restrict__ keys2, const int32_t 
         if (kRuns) {
             const int64_t bv = off[v], bu0 = off[u];
             int64_t first = i;
-            if (dups)
-                while (first > bv && keys2[first - 1] == key) --first;
+            if (dups && i > bv && keys2[i - 1] == key) {   // v's keys ascend from bv on
+                int64_t lo = bv;
+                while (lo < first) {
+                    const int64_t mid = (lo + first) >> 1;
+                    if (keys2[mid] < key) lo = mid + 1; else first = mid;
+                }
+            }
             // equal degrees: the U vertex has the higher priority
             if (off[u + 1] - bu0 < off[v + 1] - bv) {
                 plen[i] = (int32_t)(m + vals2[first] - bu0);
@@ -987,13 +992,13 @@ __global__ void __launch_bounds__(1024) k_sched_small(const uint64_t *__restrict
 // the dense chunks of start x (dense_chunk_end from offset 0 up); with `out`,
 // each chunk's item (x, first end offset) is written there
 __device__ __forceinline__ int32_t dense_chunks(int32_t x, int32_t l, int32_t cut, const int64_t *off,
-                                                const int32_t *vbase, int2 *out = nullptr) {
+                                                const int32_t *vbase, uint64_t most, int2 *out = nullptr) {
     const int32_t lb = vbase ? vbase[x] : (x >= l ? l : 0);
     const int32_t R = x - lb;
     int32_t k = 0;
     for (int32_t lo = 0; lo < R; ++k) {
         int bits;
-        const int32_t hi = dense_chunk_end(lo, R, cut, off, lb, &bits);
+        const int32_t hi = dense_chunk_end(lo, R, cut, off, lb, most, &bits);
         if (out) out[k] = make_int2(x, lo);
         lo = hi;
     }
@@ -1002,11 +1007,11 @@ __device__ __forceinline__ int32_t dense_chunks(int32_t x, int32_t l, int32_t cu
 
 __global__ void k_chunk_counts(const int32_t *__restrict__ order, int64_t n_dense, int32_t l,
                                const int32_t *__restrict__ cut, const int64_t *__restrict__ off,
-                               const int32_t *__restrict__ vbase, int64_t *nch) {
+                               const int32_t *__restrict__ vbase, const uint64_t *__restrict__ most, int64_t *nch) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n_dense) return;
     int32_t x = order[i];
-    nch[i] = dense_chunks(x, l, cut[x], off, vbase);
+    nch[i] = dense_chunks(x, l, cut[x], off, vbase, most ? most[x] : 0);
 }
 
 // A start of the CTA-hash bin whose whole end range is one chunk of dense
@@ -1014,30 +1019,30 @@ __global__ void k_chunk_counts(const int32_t *__restrict__ order, int64_t n_dens
 // 192 KB costs a CTA about 1,500 clocks, a table with as many wedges 70 clocks
 // per 32 of them against about 10.
 __device__ __forceinline__ int2 hash_or_dense_item(int32_t x, int32_t l, int32_t cut, const int64_t *off,
-                                                   const int32_t *vbase) {
+                                                   const int32_t *vbase, uint64_t most) {
     const int32_t lb = vbase ? vbase[x] : (x >= l ? l : 0);
     int bits;
-    return make_int2(x, dense_chunk_end(0, x - lb, cut, off, lb, &bits) == x - lb ? 0 : -1);
+    return make_int2(x, dense_chunk_end(0, x - lb, cut, off, lb, most, &bits) == x - lb ? 0 : -1);
 }
 
 // starts in descending work order: dense (chunked; nch_scan null: one chunk
-// each), CTA hash, team
+// each), CTA hash, team.  `most`: the starts' wedges where edges are parallel, else null
 __global__ void k_emit_items(const int32_t *__restrict__ order, int64_t n_dense, int64_t n_hash,
                              int64_t n_team, const int64_t *__restrict__ nch_scan,
                              int32_t l, const int32_t *__restrict__ cut, const int64_t *__restrict__ off,
-                             const int32_t *__restrict__ vbase, int ends_above, int2 *cta_items,
-                             int32_t *team_items) {
+                             const int32_t *__restrict__ vbase, const uint64_t *__restrict__ most, int ends_above,
+                             int2 *cta_items, int32_t *team_items) {
     const int64_t total_dense = nch_scan ? nch_scan[n_dense] : n_dense;
     const int64_t all = n_dense + n_hash + n_team;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < all;
          i += (int64_t)gridDim.x * blockDim.x) {
         int32_t x = order[i];
         if (i < n_dense) {
-            if (nch_scan) dense_chunks(x, l, cut[x], off, vbase, cta_items + nch_scan[i]);
+            if (nch_scan) dense_chunks(x, l, cut[x], off, vbase, most ? most[x] : 0, cta_items + nch_scan[i]);
             else cta_items[i] = make_int2(x, 0);
         } else if (i < n_dense + n_hash) {
             cta_items[total_dense + (i - n_dense)] =
-                ends_above ? make_int2(x, -1) : hash_or_dense_item(x, l, cut[x], off, vbase);
+                ends_above ? make_int2(x, -1) : hash_or_dense_item(x, l, cut[x], off, vbase, most ? most[x] : 0);
         } else {
             team_items[i - n_dense - n_hash] = x;
         }
@@ -1367,13 +1372,15 @@ static int schedule_graph(Graph *g, cudaStream_t s, int32_t warp_max_work, int32
         }
         // a layer (a batch's graph's) this small is one chunk of any counters,
         // or of 16-bit ones where no degree can pass 65,535
-        const bool one_chunk = g->max_range <= kDense32 || (g->max_range <= kDense16 && g->max_range <= (int32_t)kNarrowMaxCut);
+        const uint64_t *const most = g->parallel ? g->work : nullptr;
+        const bool one_chunk = g->max_range <= kDense32 ||
+                               (!most && g->max_range <= kDense16 && g->max_range <= (int32_t)kNarrowMaxCut);
         int64_t *nch_scan = nullptr;
         h_dense_items = n_dense;
         if (n_dense > 0 && !one_chunk) {
             GET(tmp, nch, n_dense + 1);
             GET(tmp, nch_scan, n_dense + 1);
-            k_chunk_counts<<<blocks_for(n_dense), kT, 0, s>>>(order, n_dense, l, g->cut, g->off, g->vbase, nch); note_launch();
+            k_chunk_counts<<<blocks_for(n_dense), kT, 0, s>>>(order, n_dense, l, g->cut, g->off, g->vbase, most, nch); note_launch();
             BFC_CUDA(cudaGetLastError());
             BFC_CUDA(scan_exclusive<int64_t>(nch, nch_scan, n_dense, scan64_tmp, s));
             BFC_CUDA(cudaMemcpyAsync(&h_dense_items, nch_scan + n_dense, sizeof(int64_t),
@@ -1384,7 +1391,7 @@ static int schedule_graph(Graph *g, cudaStream_t s, int32_t warp_max_work, int32
         if (int rc = schedule_lists(g, n_items, n_team, n_hash + n_team)) return rc;
         if (n_heavy > 0) {
             k_emit_items<<<grid_stride_blocks(n_heavy), kT, 0, s>>>(
-                order, n_dense, n_hash, n_team, nch_scan, l, g->cut, g->off, g->vbase, vpp ? 1 : 0, g->cta_items,
+                order, n_dense, n_hash, n_team, nch_scan, l, g->cut, g->off, g->vbase, most, vpp ? 1 : 0, g->cta_items,
                 g->team_items); note_launch();
             BFC_CUDA(cudaGetLastError());
         }
@@ -1525,15 +1532,21 @@ static int input_error(int err, int32_t num_graphs) {
     return BFC_OK;
 }
 
-// Step a2: one sort of both layers' vertices; `max_range` = the largest layer
-// (of one graph), which bounds every degree of a simple graph.
+// The largest degree that the rank keys have to tell apart: no larger than the
+// largest layer (of one graph) where duplicate edges are rejected; otherwise
+// every edge can be the same one.
+static int64_t degree_bound(const bfc_options *opt, int32_t max_range, int64_t m) {
+    return opt->validate ? max_range : std::max<int64_t>(max_range, m);
+}
+
+// Step a2: one sort of both layers' vertices.
 static int launch_ranks(Graph *g, const int32_t *deg_l, const int32_t *deg_u, const int32_t *gl, const int32_t *gu,
-                        int32_t max_range, uint64_t *k0, int32_t *v0, uint64_t *k1, int32_t *v1, uint32_t *hist,
+                        int64_t max_degree, uint64_t *k0, int32_t *v0, uint64_t *k1, int32_t *v1, uint32_t *hist,
                         uint32_t *hist_tmp, int32_t *deg_star, int64_t *deg64, unsigned long long *top,
                         cudaStream_t s, const int *guard) {
     const int32_t n = g->n;
     if (n == 0) return BFC_OK;
-    const int bdeg = bits_for((uint64_t)max_range);
+    const int bdeg = bits_for((uint64_t)max_degree);
     const int blayer = bdeg + (g->num_graphs > 0 ? bits_for((uint64_t)(g->num_graphs - 1)) : 0);
     k_rank_keys<<<blocks_for(n), kT, 0, s>>>(deg_l, deg_u, g->l, n, gl, gu, g->num_graphs, bdeg, blayer, k0, guard); note_launch();
     BFC_CUDA(cudaGetLastError());
@@ -1722,7 +1735,7 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
 
     // ---- a2: per-layer priority ranks by a stable sort on (layer, graph, degree)
     {
-        int rc = launch_ranks(g, deg_l, deg_u, graph_l_start, graph_u_start, g->max_range, k0, v0, k1, v1, hist,
+        int rc = launch_ranks(g, deg_l, deg_u, graph_l_start, graph_u_start, degree_bound(opt, g->max_range, m), k0, v0, k1, v1, hist,
                               hist_tmp, deg_star, deg64, red + 9, s, guard_err);
         if (rc) return rc;
     }
@@ -1745,7 +1758,7 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
         }
         // U side row by row (warp / CTA tiers, radix sort for the largest rows);
         // the swapped keys for the L side land in k1
-        const URowOut uo{m, l, bu, g->off, g->adj, g->eid, rows_star, k1, g->err, opt->validate};
+        const URowOut uo{m, l, bu, g->off, g->adj, g->eid, rows_star, k1, g->err, opt->validate ? kErrDuplicate : kErrParallel};
         int32_t *tier_rows = nullptr, *const tier_n = n_big + 2;
         GET(tmp, tier_rows, kRowTiers * std::max<int64_t>(r, 1));
         {
@@ -1853,13 +1866,18 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
     g->info.max_start_work = hred[1];
     g->info.max_deg_l = (int32_t)hred[9];
     g->info.max_deg_u = (int32_t)hred[10];
+    if (n > 0 && ((int)hred[11] & kErrParallel)) {   // known from here on: no error of a later count
+        g->parallel = true;
+        BFC_CUDA(cudaMemsetAsync(g->err, 0, sizeof(int), s));
+    }
 
     // ---- dense-core hybrid (Algorithm 2 single graphs): the requested core
     // size, or (core_vertices = -1) as many vertices as starts heavier than
     // the CTA-hash bin, at most kCoreAutoMax
     // (an automatic core below 2 x kCoreAutoMinLayer vertices cannot hold
     // both layers: nothing is launched for it)
-    if (opt->core_vertices != 0 && opt->orientation == 0 && num_graphs == 0 &&
+    // (the product of 0/1 matrices knows no parallel edges)
+    if (opt->core_vertices != 0 && opt->orientation == 0 && num_graphs == 0 && !g->parallel &&
         !(core_auto && hred[2] < 2ull * kCoreAutoMinLayer)) {
         const int32_t k = core_auto ? (int32_t)std::min<unsigned long long>(hred[2], (unsigned long long)kCoreAutoMax)
                                     : opt->core_vertices;
@@ -2025,8 +2043,8 @@ int batch_plan_run(BatchPlan *pl, const int32_t *off_u, const int32_t *adj_u, co
         off_u, adj_u, r, l, m, pl->deg_u, pl->deg_l, g->err); note_launch();
     BFC_CUDA(cudaGetLastError());
     BFC_CUDA(cudaMemsetAsync(pl->red, 0, kRedWords * sizeof(unsigned long long), s));
-    // ---- a2: graph-major ranks; a degree is below 2^16 (at most the other layer)
-    int rc = launch_ranks(g, pl->deg_l, pl->deg_u, gl, gu, pl->max_layer, pl->k0, pl->v0, pl->k1, pl->v1, pl->hist,
+    // ---- a2: graph-major ranks; without duplicates a degree is below 2^16 (at most the other layer)
+    int rc = launch_ranks(g, pl->deg_l, pl->deg_u, gl, gu, degree_bound(opt, pl->max_layer, m), pl->k0, pl->v0, pl->k1, pl->v1, pl->hist,
                           pl->hist_tmp, pl->deg_star, pl->deg64, pl->red + 9, s, guard);
     if (rc) return rc;
     if (n > 0) {
@@ -2038,7 +2056,8 @@ int batch_plan_run(BatchPlan *pl, const int32_t *off_u, const int32_t *adj_u, co
     const int bu = bits_for(r > 0 ? (uint64_t)(r - 1) : 0);
     const int bl = bits_for(l > 0 ? (uint64_t)(l - 1) : 0);
     if (m > 0) {
-        const URowOut uo{m, l, bu, g->off, g->adj, g->eid, pl->rows_star, pl->k1, g->err, opt->validate};
+        const URowOut uo{m, l, bu, g->off, g->adj, g->eid, pl->rows_star, pl->k1, g->err,
+                         opt->validate ? kErrDuplicate : kErrParallel};
         // duplicate edges that the caller answers for keep their order in every row
         // but the longest
         if (!opt->validate) { k_check_batch_rows<<<grid_stride_blocks(r), kT, 0, s>>>(off_u, adj_u, r, gu, gl, G, g->err, guard); note_launch(); }
