@@ -18,6 +18,10 @@ BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libbfc.so")
 SOURCES = ["api.cu", "prepare.cu", "count.cu", "scan_sort.cu", "noalloc.cu", "server.cu", "microbench.cu",
            "derived.cu", "core.cu", "pairs.cu", "sparsify.cu"]
+# (object, source, definitions): the count kernels are an object per mode and position type
+UNITS = [(s[:-3] + ".o", s, []) for s in SOURCES]
+UNITS += [(f"count_{mode}_{pos}.o", "count.cu", [f"-DBFC_COUNT_MODE={mode}", f"-DBFC_COUNT_POS={pos}"])
+          for pos in ("int64_t", "int32_t") for mode in (4, 2, 1, 3, 0)]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -45,11 +49,11 @@ def build(verbose: bool = False, extra_flags=(), force: bool = False) -> str:
     os.makedirs(BUILD, exist_ok=True)
     cc = nvcc()
     jobs = []
-    for s in SOURCES:
-        src = os.path.join(CSRC, s)
-        obj = os.path.join(BUILD, s.replace(".cu", ".o"))
+    for name, source, defs in reversed(UNITS):   # the long ones first
+        src = os.path.join(CSRC, source)
+        obj = os.path.join(BUILD, name)
         if force or _stale(obj, src):
-            jobs.append([cc, *_flags(extra_flags), "-c", src, "-o", obj])
+            jobs.append([cc, *_flags(extra_flags), *defs, "-c", src, "-o", obj])
     if verbose:
         for j in jobs:
             print(" ".join(j))
@@ -60,11 +64,11 @@ def build(verbose: bool = False, extra_flags=(), force: bool = False) -> str:
             raise RuntimeError("nvcc failed:\n" + " ".join(cmd) + "\n" + r.stdout + r.stderr)
         return r.stdout + r.stderr
 
-    with concurrent.futures.ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
+    with concurrent.futures.ThreadPoolExecutor(max_workers=len(UNITS)) as ex:
         for out in ex.map(run, jobs):
             if verbose and out.strip():
                 print(out)
-    objs = [os.path.join(BUILD, s.replace(".cu", ".o")) for s in SOURCES]
+    objs = [os.path.join(BUILD, name) for name, _, _ in UNITS]
     if force or jobs or not os.path.exists(LIB):
         tmp = LIB + f".tmp{os.getpid()}"
         run([cc, *ARCH, "-shared", "-cudart=static", "-Xlinker", "--no-undefined", "-o", tmp, *objs])

@@ -36,19 +36,16 @@
 // team bound above 3,072 wedges) detects when it fills up; the start is then
 // re-queued and counted by k_count_retry, first with a CTA table, then if
 // needed with dense chunks of its end range.
+//
+// The kernels of a mode and a position type are large, so each pair of them is
+// an object of its own (this file with BFC_COUNT_MODE and BFC_COUNT_POS set):
+// they compile side by side.  Without these the file holds the host side.
 #include "bfc_internal.cuh"
 
 #include <algorithm>
 #include <type_traits>
 
 namespace bfc {
-
-namespace {
-
-constexpr int kTeamTableBytes = kTeamSlots * 6;   // 32-bit keys + 16-bit counts
-constexpr int kTeamPackedSlots = 8192;            // (key, count) words: 32 KB
-static_assert(kTeamRegion == (kCountWarps / kTeams) * kWarpRegion,
-              "a team's region is exactly the regions of its warps");
 
 struct CountParams {
     const int64_t *__restrict__ off;
@@ -100,6 +97,21 @@ struct CountParams {
     const int *guard;
     int32_t parallel;   // 0 no parallel edges, 1 there are, 2 *err says it (a plan with validate = 0)
 };
+
+// the count kernels of one mode and position type
+template <int MODE, typename Pos>
+struct CountKernels {
+    static cudaError_t setup();   // once per device
+    static void launch(int grid, cudaStream_t s, const CountParams &p, bool retry);
+};
+
+#ifdef BFC_COUNT_MODE
+namespace {
+
+constexpr int kTeamTableBytes = kTeamSlots * 6;   // 32-bit keys + 16-bit counts
+constexpr int kTeamPackedSlots = 8192;            // (key, count) words: 32 KB
+static_assert(kTeamRegion == (kCountWarps / kTeams) * kWarpRegion,
+              "a team's region is exactly the regions of its warps");
 
 // item queue lengths: from the host, or from a batch plan's device counts
 __device__ __forceinline__ int64_t n_cta_items(const CountParams &p) {
@@ -1728,6 +1740,35 @@ __global__ void __launch_bounds__(kCountThreads, kCountCtasPerSm) k_count_retry(
     if (threadIdx.x == 0 && t) atomicAdd(p.acc, t);
 }
 
+}  // namespace
+
+template <int MODE, typename Pos>
+cudaError_t CountKernels<MODE, Pos>::setup() {
+    cudaError_t e = cudaFuncSetAttribute(k_count<MODE, Pos>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kCounterBytes);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_count<MODE, Pos>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 cudaSharedmemCarveoutMaxShared);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_count_retry<MODE, Pos>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, kCounterBytes);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_count_retry<MODE, Pos>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 cudaSharedmemCarveoutMaxShared);
+    return e;
+}
+
+template <int MODE, typename Pos>
+void CountKernels<MODE, Pos>::launch(int grid, cudaStream_t s, const CountParams &p, bool retry) {
+    if (retry) k_count_retry<MODE, Pos><<<grid, kCountThreads, kCounterBytes, s>>>(p);
+    else k_count<MODE, Pos><<<grid, kCountThreads, kCounterBytes, s>>>(p);
+}
+
+template struct CountKernels<BFC_COUNT_MODE, BFC_COUNT_POS>;
+
+#else   // the host side
+namespace {
+
 __global__ void k_gather_vertices(const unsigned long long *__restrict__ pv,
                                   const int32_t *__restrict__ rank_u,
                                   const int32_t *__restrict__ rank_l, int32_t r, int32_t l,
@@ -1765,56 +1806,33 @@ __global__ void k_export_eid(const int32_t *__restrict__ eid, int64_t m, int32_t
         out[i] = i < m ? eid[m + eid[i]] : eid[i];
 }
 
-template <int MODE, typename Pos>
-cudaError_t setup_one() {
-    cudaError_t e = cudaFuncSetAttribute(k_count<MODE, Pos>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kCounterBytes);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_count<MODE, Pos>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 cudaSharedmemCarveoutMaxShared);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_count_retry<MODE, Pos>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, kCounterBytes);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_count_retry<MODE, Pos>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 cudaSharedmemCarveoutMaxShared);
-    return e;
-}
+}  // namespace
 
+namespace {
 template <typename Pos>
-void launch_main(int mode, int grid, cudaStream_t s, const CountParams &p) {
-    if (mode == kModeTotal) k_count<kModeTotal, Pos><<<grid, kCountThreads, kCounterBytes, s>>>(p);
-    else if (mode == kModeBatch) k_count<kModeBatch, Pos><<<grid, kCountThreads, kCounterBytes, s>>>(p);
-    else if (mode == kModeVertices) k_count<kModeVertices, Pos><<<grid, kCountThreads, kCounterBytes, s>>>(p);
-    else if (mode == kModeAll) k_count<kModeAll, Pos><<<grid, kCountThreads, kCounterBytes, s>>>(p);
-    else k_count<kModeEdges, Pos><<<grid, kCountThreads, kCounterBytes, s>>>(p);
+void launch_kernels(int mode, int grid, cudaStream_t s, const CountParams &p, bool retry) {
+    if (mode == kModeTotal) CountKernels<kModeTotal, Pos>::launch(grid, s, p, retry);
+    else if (mode == kModeBatch) CountKernels<kModeBatch, Pos>::launch(grid, s, p, retry);
+    else if (mode == kModeVertices) CountKernels<kModeVertices, Pos>::launch(grid, s, p, retry);
+    else if (mode == kModeAll) CountKernels<kModeAll, Pos>::launch(grid, s, p, retry);
+    else CountKernels<kModeEdges, Pos>::launch(grid, s, p, retry);
 }
-
-template <typename Pos>
-void launch_retry(int mode, int grid, cudaStream_t s, const CountParams &p) {
-    if (mode == kModeTotal) k_count_retry<kModeTotal, Pos><<<grid, kCountThreads, kCounterBytes, s>>>(p);
-    else if (mode == kModeBatch) k_count_retry<kModeBatch, Pos><<<grid, kCountThreads, kCounterBytes, s>>>(p);
-    else if (mode == kModeVertices) k_count_retry<kModeVertices, Pos><<<grid, kCountThreads, kCounterBytes, s>>>(p);
-    else if (mode == kModeAll) k_count_retry<kModeAll, Pos><<<grid, kCountThreads, kCounterBytes, s>>>(p);
-    else k_count_retry<kModeEdges, Pos><<<grid, kCountThreads, kCounterBytes, s>>>(p);
-}
-
 }  // namespace
 
 int count_smem_setup(int device) {
     static bool done[64] = {false};
     if (device < 0 || device >= 64) return BFC_ERR_INVALID_ARGUMENT;
     if (done[device]) return BFC_OK;
-    BFC_CUDA((setup_one<kModeTotal, int32_t>()));
-    BFC_CUDA((setup_one<kModeVertices, int32_t>()));
-    BFC_CUDA((setup_one<kModeEdges, int32_t>()));
-    BFC_CUDA((setup_one<kModeBatch, int32_t>()));
-    BFC_CUDA((setup_one<kModeTotal, long long>()));
-    BFC_CUDA((setup_one<kModeVertices, long long>()));
-    BFC_CUDA((setup_one<kModeEdges, long long>()));
-    BFC_CUDA((setup_one<kModeBatch, long long>()));
-    BFC_CUDA((setup_one<kModeAll, int32_t>()));
-    BFC_CUDA((setup_one<kModeAll, long long>()));
+    BFC_CUDA((CountKernels<kModeTotal, int32_t>::setup()));
+    BFC_CUDA((CountKernels<kModeVertices, int32_t>::setup()));
+    BFC_CUDA((CountKernels<kModeEdges, int32_t>::setup()));
+    BFC_CUDA((CountKernels<kModeBatch, int32_t>::setup()));
+    BFC_CUDA((CountKernels<kModeAll, int32_t>::setup()));
+    BFC_CUDA((CountKernels<kModeTotal, int64_t>::setup()));
+    BFC_CUDA((CountKernels<kModeVertices, int64_t>::setup()));
+    BFC_CUDA((CountKernels<kModeEdges, int64_t>::setup()));
+    BFC_CUDA((CountKernels<kModeBatch, int64_t>::setup()));
+    BFC_CUDA((CountKernels<kModeAll, int64_t>::setup()));
     done[device] = true;
     return BFC_OK;
 }
@@ -1861,14 +1879,14 @@ int launch_count(Graph *g, cudaStream_t s, int mode, unsigned long long *pv_proj
     const int grid = g->grid;
     // 32-bit adjacency positions whenever G* has fewer than 2^31 slots
     const bool narrow_pos = 2 * g->m <= 0x7fffffffll && !g->opt.wide_positions;
-    if (narrow_pos) launch_main<int32_t>(mode, grid, s, p);
-    else launch_main<long long>(mode, grid, s, p);
+    if (narrow_pos) launch_kernels<int32_t>(mode, grid, s, p, false);
+    else launch_kernels<int64_t>(mode, grid, s, p, false);
     note_launch();
     BFC_CUDA(cudaGetLastError());
     if (g->may_retry) {
         // the retry pass reads how many starts the first launch re-queued
-        if (narrow_pos) launch_retry<int32_t>(mode, grid, s, p);
-        else launch_retry<long long>(mode, grid, s, p);
+        if (narrow_pos) launch_kernels<int32_t>(mode, grid, s, p, true);
+        else launch_kernels<int64_t>(mode, grid, s, p, true);
         note_launch();
         BFC_CUDA(cudaGetLastError());
     }
@@ -1905,5 +1923,7 @@ int gather_vertices(Graph *g, cudaStream_t s, uint64_t *per_u, uint64_t *per_l) 
     BFC_CUDA(cudaGetLastError());
     return BFC_OK;
 }
+
+#endif  // BFC_COUNT_MODE
 
 }  // namespace bfc
