@@ -166,8 +166,9 @@ struct Allocs {
         slab_left = 0;
     }
 
-private:
     static size_t rounded(size_t b) { return ((b == 0 ? 16 : b) + 255) & ~size_t(255); }
+
+private:
     cudaError_t take(void **p, size_t b) {
         if (n >= kMax) return cudaErrorMemoryAllocation;
         void *q = nullptr;

@@ -1644,7 +1644,15 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
     g->opt = *opt;
     g->stream = s;
     g->mem.stream = s;
-    g->mem.slab_next = 64 << 10;   // many small graphs may be kept: the first slab is no larger than they need
+    {
+        // many small graphs may be kept: one slab that just holds a small graph's arrays
+        auto small = [](size_t bytes) { return bytes <= Allocs::kCarve ? Allocs::rounded(bytes) : 0; };
+        const size_t nn = (size_t)n, mm = (size_t)m, per_n = num_graphs > 0 ? 6 : 3;
+        const size_t sum = small(4 * (size_t)r) + small(4 * (size_t)l) + 2 * small(8 * nn) + small(8 * (nn + 1)) +
+                           per_n * small(4 * nn) + 3 * small(8 * mm) + small(16 * mm) +
+                           (num_graphs > 0 ? small(8 * (size_t)num_graphs) : 0) + 2 * 256;
+        g->mem.slab_next = std::min(sum, Allocs::kSlab);
+    }
 
     Allocs tmp;
     tmp.stream = s;
