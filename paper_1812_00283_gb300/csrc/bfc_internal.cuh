@@ -51,16 +51,9 @@ __host__ __device__ constexpr int32_t dense_chunk_span(int64_t bound) {
 // min(cut[x], deg(w)), and within a layer G* orders vertices by Definition 3's
 // priority, so degrees do not decrease with the id and the chunk's last end
 // bounds every count of the chunk.  Returns the chunk's end; *bits = 4, 8, 16
-// or 32.  `off` is G*'s offset array.  With parallel edges a count is a sum of
-// products, which neither bounds: then `most` is the largest count that x can
-// have (its wedges), else 0.
+// or 32.  `cut` and `off` are the graph's bcut[x] and boff (see Graph).
 __device__ __forceinline__ int32_t dense_chunk_end(int32_t lo, int32_t R, int64_t cut, const int64_t *off,
-                                                   int32_t lb, uint64_t most, int *bits) {
-    if (most) {
-        *bits = most > kNarrowMaxCut ? 32 : (most > kByteMaxCut ? 16 : 8);
-        const int64_t end = (int64_t)lo + dense_chunk_span((int64_t)most);
-        return end < R ? (int32_t)end : R;
-    }
+                                                   int32_t lb, int *bits) {
     int32_t hi = (int32_t)((int64_t)lo + kDense4 < R ? lo + kDense4 : R);
     int64_t top = off[lb + hi] - off[lb + hi - 1];
     if ((cut < top ? cut : top) <= (int64_t)kNibbleMax) { *bits = 4; return hi; }
@@ -73,6 +66,19 @@ __device__ __forceinline__ int32_t dense_chunk_end(int32_t lo, int32_t R, int64_
     *bits = 32;
     return (int32_t)((int64_t)lo + kDense32 < R ? lo + kDense32 : R);
 }
+// A dense item's y: the chunk's first end offset in units, and its counters' width.
+__host__ __device__ constexpr int32_t dense_item_y(int32_t lo, int bits) {
+    return lo / kChunkUnit * 4 + (bits == 4 ? 0 : (bits == 8 ? 1 : (bits == 16 ? 2 : 3)));
+}
+__device__ __forceinline__ void dense_item_range(int32_t y, int32_t R, int32_t *lo, int32_t *hi, int *bits) {
+    const int32_t at = (y >> 2) * kChunkUnit;
+    const int32_t span = kChunkUnit << (3 - (y & 3));
+    *lo = at;
+    *hi = span < R - at ? at + span : R;   // as dense_chunk_end has it
+    *bits = 4 << (y & 3);
+}
+static_assert(kDense32 == kChunkUnit && kDense16 == 2 * kChunkUnit && kDense8 == 4 * kChunkUnit &&
+                  kDense4 == 8 * kChunkUnit, "a chunk's span follows from its counters' width");
 constexpr int64_t kChunkTableMaxEntries = 1ll << 29;      // 2 GB of int32 at most
 
 // device error bits (graph-owned error word)
@@ -190,6 +196,12 @@ struct Graph {
     int32_t r = 0, l = 0, n = 0;
     int32_t max_range = 0;         // the larger layer (of a batch: of any one graph)
     bool parallel = false;         // validate = 0 and an edge occurs more than once
+    // what bounds a count_wedge(x, w): bcut[x] and boff[w + 1] - boff[w].  The
+    // graph's own cut and off, except with parallel edges: a count is then a sum
+    // of products of multiplicities, which only the wedges of x bound, and the two
+    // are arrays of their own (work[x], and differences past any count).
+    const int32_t *bcut = nullptr;
+    const int64_t *boff = nullptr;
     int64_t m = 0;
     bfc_options opt{};
     bfc_info info{};
@@ -208,7 +220,7 @@ struct Graph {
     uint64_t *work = nullptr; // [n]
     char *lists = nullptr;        // of the current schedule: the next two and `retry` (a plan's are apart)
     size_t lists_bytes = 0;
-    int2 *cta_items = nullptr;    // (start, chunk) / (start, -1 = hash)
+    int2 *cta_items = nullptr;    // (start, dense_item_y) / (start, -1 = hash)
     int32_t *team_items = nullptr;
     int32_t *warp_items = nullptr;   // [n]: the warp bin from the front, its tiny starts from the back
     int64_t n_cta_items = 0, n_team_items = 0, n_warp_items = 0, n_tiny_items = 0;
@@ -318,6 +330,8 @@ struct BatchPlan {
     int32_t *v0 = nullptr, *v1 = nullptr, *deg_u = nullptr, *deg_l = nullptr, *deg_star = nullptr;
     int32_t *rows_star = nullptr, *tier_rows = nullptr, *tier_n = nullptr, *big = nullptr, *n_big = nullptr;
     int32_t *heavy = nullptr;
+    int32_t *bcut = nullptr;       // the graph's, where validate = 0
+    int64_t *boff = nullptr;
     uint32_t *hist = nullptr, *hist_tmp = nullptr;
     int64_t *scan64_tmp = nullptr, *deg64 = nullptr;
     unsigned long long *red = nullptr;   // [0] W, [3..9) bin sizes, [9], [10] largest degrees

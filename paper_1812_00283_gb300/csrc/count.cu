@@ -15,8 +15,8 @@
 // shared memory.  Three phases, each fed by its own queue, heaviest first
 // (Section 6.2's dynamic scheduling with the exact per-start work):
 //   A. CTA items, the whole CTA on one item:
-//      dense (u, lo) count_wedge is a dense array over the chunk of u's end
-//                    range that starts at offset lo: 4-bit counts when
+//      dense (u, y)  count_wedge is a dense array over the chunk of u's end
+//                    range that y names (dense_item_y): 4-bit counts when
 //                    every count of the chunk is at most 15, 8-bit when at
 //                    most 255, 16-bit when at most 65,535, else 32-bit (the
 //                    same shared memory holds 393,216, 196,608, 98,304 or
@@ -95,7 +95,8 @@ struct CountParams {
     // failures stop the launch (null otherwise)
     const unsigned long long *__restrict__ item_counts;
     const int *guard;
-    int32_t parallel;   // 0 no parallel edges, 1 there are, 2 *err says it (a plan with validate = 0)
+    const int32_t *__restrict__ bcut;   // what bounds a count (see Graph)
+    const int64_t *__restrict__ boff;
 };
 
 // the count kernels of one mode and position type
@@ -1088,21 +1089,10 @@ __device__ __forceinline__ unsigned long long end_bound(const CountParams &p, in
     return w < range ? w : range;
 }
 
-// The bounds on a count_wedge below rest on a simple graph.  With parallel edges a
-// count is a sum of products of multiplicities, which only the wedges of x bound:
-// those, or 0 without parallel edges.  A plan's dense start is one chunk of at
-// most 65,535 ends whatever it holds, so its counters never have more than 16 bits.
-__device__ __forceinline__ uint64_t parallel_bound(const CountParams &p, int32_t x) {
-    if (!p.parallel) return 0;
-    if (p.parallel == 1) return p.work[x];
-    return (*(volatile const int *)p.err & kErrParallel) ? min(p.work[x], (uint64_t)kNarrowMaxCut) : 0;
-}
-
 // A count_wedge is at most the number of middles: cut[x] (Algorithm 2) or
 // deg(x) (Algorithm 3).
 __device__ __forceinline__ int64_t middles(const CountParams &p, int32_t x) {
-    if (const uint64_t most = parallel_bound(p, x)) return (int64_t)most;
-    return p.orient ? p.off[x + 1] - p.off[x] : (int64_t)p.cut[x];
+    return p.orient ? p.boff[x + 1] - p.boff[x] : (int64_t)p.bcut[x];
 }
 
 // The bits of a packed table's count for start x whose ends are the R vertices
@@ -1110,9 +1100,8 @@ __device__ __forceinline__ int64_t middles(const CountParams &p, int32_t x) {
 // at most min(cut[x], degree of the last end, work[x]); keys are below R.
 __device__ __forceinline__ int packed_count_bits(const CountParams &p, int32_t x, int32_t R) {
     if (p.orient || R <= 0) return 0;
-    const int64_t last = p.off[x] - p.off[x - 1];
-    const uint64_t most = parallel_bound(p, x);
-    const uint64_t c = most ? most : min((uint64_t)min((int64_t)p.cut[x], last), (uint64_t)p.work[x]);
+    const int64_t last = p.boff[x] - p.boff[x - 1];
+    const uint64_t c = min((uint64_t)min((int64_t)p.bcut[x], last), (uint64_t)p.work[x]);
     const int cb = 64 - __clzll((long long)c), kb = 32 - __clz(R);
     return cb + kb <= 32 ? cb : 0;
 }
@@ -1203,9 +1192,9 @@ __device__ unsigned long long cta_item(const CountParams &p, int2 item, unsigned
     if (item.y >= 0) {          // dense items exist only for Algorithm 2
         const int32_t lb = range_lo(p, x);
         const int32_t R = x - lb;   // the ends are the R vertices below x
-        const int32_t lo = item.y;   // the chunk's first end offset
+        int32_t lo, hi;
         int bits;
-        const int32_t hi = dense_chunk_end(lo, R, p.cut[x], p.off, lb, parallel_bound(p, x), &bits);
+        dense_item_range(item.y, R, &lo, &hi, &bits);
         const int kind = kind_of_bits(bits);
         const int32_t span = hi - lo;
         const int flags = (lo > 0 ? 1 : 0) | (hi < R ? 2 : 0);
@@ -1248,9 +1237,9 @@ __device__ unsigned long long dense_stream(const CountParams &p, int64_t &it, un
         const int32_t x = item.x;
         const int32_t lb = range_lo(p, x);
         const int32_t R = x - lb;   // the ends are the R vertices below x
-        const int32_t lo = item.y;   // the chunk's first end offset
+        int32_t lo, hi;
         int bits;
-        const int32_t hi = dense_chunk_end(lo, R, p.cut[x], p.off, lb, parallel_bound(p, x), &bits);
+        dense_item_range(item.y, R, &lo, &hi, &bits);
         const int kind = kind_of_bits(bits);
         const int32_t span = hi - lo;
         const int flags = (lo > 0 ? 1 : 0) | (hi < R ? 2 : 0);
@@ -1342,9 +1331,8 @@ __device__ unsigned long long team_item(const CountParams &p, int32_t x, unsigne
     if (!p.orient && p.work[x] <= (uint64_t)kTeamFitWork) {
         lb = range_lo(p, x);
         R = x - lb;
-        const int64_t last = R > 0 ? p.off[x] - p.off[x - 1] : 0;
-        const uint64_t most = parallel_bound(p, x);
-        narrow = (most ? (int64_t)most : min(min((int64_t)p.cut[x], last), (int64_t)p.work[x])) > (int64_t)kByteMaxCut;
+        const int64_t last = R > 0 ? p.boff[x] - p.boff[x - 1] : 0;
+        narrow = min(min((int64_t)p.bcut[x], last), (int64_t)p.work[x]) > (int64_t)kByteMaxCut;
     }
     if (R > 0 && (narrow ? 2 * (int64_t)R : (int64_t)R) <= dense_bytes) {
         team_fill(table, narrow ? 2 * R : R, 0u, t);
@@ -1869,7 +1857,8 @@ int launch_count(Graph *g, cudaStream_t s, int mode, unsigned long long *pv_proj
     p.ccut = g->ccut; p.core_au = g->core_au; p.core_al = g->core_al;
     p.item_counts = g->item_counts;
     p.guard = g->item_counts ? g->err : nullptr;
-    p.parallel = g->item_counts ? (g->opt.validate ? 0 : 2) : (g->parallel ? 1 : 0);
+    p.bcut = g->bcut;
+    p.boff = g->boff;
     if (p.core_on) {
         // the core pairs' a(u, w), on the same stream before the walk
         int rc2 = core_product(g, s);

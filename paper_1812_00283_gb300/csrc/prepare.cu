@@ -990,28 +990,37 @@ __global__ void __launch_bounds__(1024) k_sched_small(const uint64_t *__restrict
 }
 
 // the dense chunks of start x (dense_chunk_end from offset 0 up); with `out`,
-// each chunk's item (x, first end offset) is written there
+// each chunk's item is written there
 __device__ __forceinline__ int32_t dense_chunks(int32_t x, int32_t l, int32_t cut, const int64_t *off,
-                                                const int32_t *vbase, uint64_t most, int2 *out = nullptr) {
+                                                const int32_t *vbase, int2 *out = nullptr) {
     const int32_t lb = vbase ? vbase[x] : (x >= l ? l : 0);
     const int32_t R = x - lb;
     int32_t k = 0;
     for (int32_t lo = 0; lo < R; ++k) {
         int bits;
-        const int32_t hi = dense_chunk_end(lo, R, cut, off, lb, most, &bits);
-        if (out) out[k] = make_int2(x, lo);
+        const int32_t hi = dense_chunk_end(lo, R, cut, off, lb, &bits);
+        if (out) out[k] = make_int2(x, dense_item_y(lo, bits));
         lo = hi;
     }
     return k;
 }
 
+// the only dense chunk of a start whose layer is no larger than one
+__device__ __forceinline__ int2 one_dense_item(int32_t x, int32_t l, int32_t cut, const int64_t *off,
+                                               const int32_t *vbase) {
+    const int32_t lb = vbase ? vbase[x] : (x >= l ? l : 0);
+    int bits = 4;
+    if (x > lb) dense_chunk_end(0, x - lb, cut, off, lb, &bits);
+    return make_int2(x, dense_item_y(0, bits));
+}
+
 __global__ void k_chunk_counts(const int32_t *__restrict__ order, int64_t n_dense, int32_t l,
                                const int32_t *__restrict__ cut, const int64_t *__restrict__ off,
-                               const int32_t *__restrict__ vbase, const uint64_t *__restrict__ most, int64_t *nch) {
+                               const int32_t *__restrict__ vbase, int64_t *nch) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n_dense) return;
     int32_t x = order[i];
-    nch[i] = dense_chunks(x, l, cut[x], off, vbase, most ? most[x] : 0);
+    nch[i] = dense_chunks(x, l, cut[x], off, vbase);
 }
 
 // A start of the CTA-hash bin whose whole end range is one chunk of dense
@@ -1019,33 +1028,45 @@ __global__ void k_chunk_counts(const int32_t *__restrict__ order, int64_t n_dens
 // 192 KB costs a CTA about 1,500 clocks, a table with as many wedges 70 clocks
 // per 32 of them against about 10.
 __device__ __forceinline__ int2 hash_or_dense_item(int32_t x, int32_t l, int32_t cut, const int64_t *off,
-                                                   const int32_t *vbase, uint64_t most) {
+                                                   const int32_t *vbase) {
     const int32_t lb = vbase ? vbase[x] : (x >= l ? l : 0);
     int bits;
-    return make_int2(x, dense_chunk_end(0, x - lb, cut, off, lb, most, &bits) == x - lb ? 0 : -1);
+    return make_int2(x, dense_chunk_end(0, x - lb, cut, off, lb, &bits) == x - lb ? dense_item_y(0, bits) : -1);
 }
 
 // starts in descending work order: dense (chunked; nch_scan null: one chunk
-// each), CTA hash, team.  `most`: the starts' wedges where edges are parallel, else null
+// each), CTA hash, team.  Here and above `cut` and `off` are the graph's bcut and boff.
 __global__ void k_emit_items(const int32_t *__restrict__ order, int64_t n_dense, int64_t n_hash,
                              int64_t n_team, const int64_t *__restrict__ nch_scan,
                              int32_t l, const int32_t *__restrict__ cut, const int64_t *__restrict__ off,
-                             const int32_t *__restrict__ vbase, const uint64_t *__restrict__ most, int ends_above,
-                             int2 *cta_items, int32_t *team_items) {
+                             const int32_t *__restrict__ vbase, int ends_above, int2 *cta_items,
+                             int32_t *team_items) {
     const int64_t total_dense = nch_scan ? nch_scan[n_dense] : n_dense;
     const int64_t all = n_dense + n_hash + n_team;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < all;
          i += (int64_t)gridDim.x * blockDim.x) {
         int32_t x = order[i];
         if (i < n_dense) {
-            if (nch_scan) dense_chunks(x, l, cut[x], off, vbase, most ? most[x] : 0, cta_items + nch_scan[i]);
-            else cta_items[i] = make_int2(x, 0);
+            if (nch_scan) dense_chunks(x, l, cut[x], off, vbase, cta_items + nch_scan[i]);
+            else cta_items[i] = one_dense_item(x, l, cut[x], off, vbase);
         } else if (i < n_dense + n_hash) {
             cta_items[total_dense + (i - n_dense)] =
-                ends_above ? make_int2(x, -1) : hash_or_dense_item(x, l, cut[x], off, vbase, most ? most[x] : 0);
+                ends_above ? make_int2(x, -1) : hash_or_dense_item(x, l, cut[x], off, vbase);
         } else {
             team_items[i - n_dense - n_hash] = x;
         }
+    }
+}
+
+// bcut and boff (see Graph).  With `err` only where the word tells of parallel
+// edges, else copies of cut and off; `most` caps bcut.
+__global__ void k_count_bounds(const uint64_t *__restrict__ work, const int32_t *__restrict__ cut,
+                               const int64_t *__restrict__ off, int32_t n, int32_t most, const int *err,
+                               int32_t *bcut, int64_t *boff) {
+    const bool parallel = !err || (*err & kErrParallel);
+    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x <= n; x += (int64_t)gridDim.x * blockDim.x) {
+        boff[x] = parallel ? x << 31 : off[x];
+        if (x < n) bcut[x] = parallel ? (int32_t)(work[x] < (uint64_t)most ? work[x] : (uint64_t)most) : cut[x];
     }
 }
 
@@ -1372,15 +1393,14 @@ static int schedule_graph(Graph *g, cudaStream_t s, int32_t warp_max_work, int32
         }
         // a layer (a batch's graph's) this small is one chunk of any counters,
         // or of 16-bit ones where no degree can pass 65,535
-        const uint64_t *const most = g->parallel ? g->work : nullptr;
         const bool one_chunk = g->max_range <= kDense32 ||
-                               (!most && g->max_range <= kDense16 && g->max_range <= (int32_t)kNarrowMaxCut);
+                               (!g->parallel && g->max_range <= kDense16 && g->max_range <= (int32_t)kNarrowMaxCut);
         int64_t *nch_scan = nullptr;
         h_dense_items = n_dense;
         if (n_dense > 0 && !one_chunk) {
             GET(tmp, nch, n_dense + 1);
             GET(tmp, nch_scan, n_dense + 1);
-            k_chunk_counts<<<blocks_for(n_dense), kT, 0, s>>>(order, n_dense, l, g->cut, g->off, g->vbase, most, nch); note_launch();
+            k_chunk_counts<<<blocks_for(n_dense), kT, 0, s>>>(order, n_dense, l, g->bcut, g->boff, g->vbase, nch); note_launch();
             BFC_CUDA(cudaGetLastError());
             BFC_CUDA(scan_exclusive<int64_t>(nch, nch_scan, n_dense, scan64_tmp, s));
             BFC_CUDA(cudaMemcpyAsync(&h_dense_items, nch_scan + n_dense, sizeof(int64_t),
@@ -1391,7 +1411,7 @@ static int schedule_graph(Graph *g, cudaStream_t s, int32_t warp_max_work, int32
         if (int rc = schedule_lists(g, n_items, n_team, n_hash + n_team)) return rc;
         if (n_heavy > 0) {
             k_emit_items<<<grid_stride_blocks(n_heavy), kT, 0, s>>>(
-                order, n_dense, n_hash, n_team, nch_scan, l, g->cut, g->off, g->vbase, most, vpp ? 1 : 0, g->cta_items,
+                order, n_dense, n_hash, n_team, nch_scan, l, g->bcut, g->boff, g->vbase, vpp ? 1 : 0, g->cta_items,
                 g->team_items); note_launch();
             BFC_CUDA(cudaGetLastError());
         }
@@ -1682,6 +1702,8 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
     g->acc = reinterpret_cast<unsigned long long *>(g->cursors + 8);   // cleared together
     GET(g->mem, g->pv, n);
     GET(g->mem, g->warp_items, std::max(n, 1));
+    g->bcut = g->cut;
+    g->boff = g->off;
     BFC_CUDA(cudaMemsetAsync(g->err, 0, 4 * sizeof(int), s));
 
     // A batch's start arrays are checked first: its largest layers size what
@@ -1877,6 +1899,15 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
     if (n > 0 && ((int)hred[11] & kErrParallel)) {   // known from here on: no error of a later count
         g->parallel = true;
         BFC_CUDA(cudaMemsetAsync(g->err, 0, sizeof(int), s));
+        int32_t *bcut;
+        int64_t *boff;
+        GET(g->mem, bcut, n);
+        GET(g->mem, boff, (int64_t)n + 1);
+        k_count_bounds<<<grid_stride_blocks((int64_t)n + 1), kT, 0, s>>>(g->work, g->cut, g->off, n, 0x7fffffff,
+                                                                         nullptr, bcut, boff); note_launch();
+        BFC_CUDA(cudaGetLastError());
+        g->bcut = bcut;
+        g->boff = boff;
     }
 
     // ---- dense-core hybrid (Algorithm 2 single graphs): the requested core
@@ -1953,14 +1984,15 @@ __global__ void k_sched_keys_plan(const uint64_t *__restrict__ work, const int32
 // dense start is one chunk (and so is one of the CTA-hash bin, which gets dense
 // counters too), so the lists follow the order directly
 __global__ void k_emit_items_plan(const int32_t *__restrict__ order,
-                                  const unsigned long long *__restrict__ counts, int2 *cta_items,
+                                  const unsigned long long *__restrict__ counts, const int32_t *__restrict__ cut,
+                                  const int64_t *__restrict__ off, const int32_t *__restrict__ vbase, int2 *cta_items,
                                   int32_t *team_items, const int *guard) {
     if (aborted(guard)) return;
     const int64_t nd = (int64_t)counts[0], nh = (int64_t)counts[1], nt = (int64_t)counts[2];
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nd + nh + nt;
          i += (int64_t)gridDim.x * blockDim.x) {
         const int32_t x = order[i];
-        if (i < nd + nh) cta_items[i] = make_int2(x, 0);
+        if (i < nd + nh) cta_items[i] = one_dense_item(x, 0, cut[x], off, vbase);
         else team_items[i - nd - nh] = x;
     }
 }
@@ -1999,6 +2031,13 @@ int batch_plan_create(BatchPlan *pl, cudaStream_t s) {
     GET(g->cursors, 8 + 4); GET(g->pv, 1); GET(g->sbeg, 2 * m);
     g->acc = reinterpret_cast<unsigned long long *>(g->cursors + 8);   // cleared together
     GET(g->gstar, n); GET(g->vbase, n); GET(g->vend, n); GET(g->gwork, G);
+    g->bcut = g->cut;
+    g->boff = g->off;
+    if (!g->opt.validate) {
+        GET(pl->bcut, n); GET(pl->boff, (int64_t)n + 1);
+        g->bcut = pl->bcut;
+        g->boff = pl->boff;
+    }
     GET(g->cta_items, n); GET(g->team_items, n); GET(g->warp_items, n); GET(g->retry, 1);
     // temporaries, kept with the plan
     const int64_t nsort = std::max<int64_t>({(int64_t)r, (int64_t)l, m, (int64_t)n, 1});
@@ -2101,8 +2140,14 @@ int batch_plan_run(BatchPlan *pl, const int32_t *off_u, const int32_t *adj_u, co
         BFC_CUDA(cudaGetLastError());
         int which = 0;
         BFC_CUDA(radix_sort_pairs(pl->k0, pl->heavy, pl->k1, pl->v1, n, 0, 8, pl->hist, pl->hist_tmp, s, &which));
-        k_emit_items_plan<<<grid_stride_blocks(n), kT, 0, s>>>(which ? pl->v1 : pl->heavy, bins, g->cta_items,
-                                                               g->team_items, guard); note_launch();
+        if (!opt->validate) {
+            // a dense start is one chunk of up to 65,535 ends, so of 16-bit counters
+            k_count_bounds<<<grid_stride_blocks((int64_t)n + 1), kT, 0, s>>>(
+                g->work, g->cut, g->off, n, (int32_t)kNarrowMaxCut, g->err, pl->bcut, pl->boff); note_launch();
+            BFC_CUDA(cudaGetLastError());
+        }
+        k_emit_items_plan<<<grid_stride_blocks(n), kT, 0, s>>>(which ? pl->v1 : pl->heavy, bins, g->bcut, g->boff,
+                                                               g->vbase, g->cta_items, g->team_items, guard); note_launch();
         BFC_CUDA(cudaGetLastError());
     }
     // ---- a6-a7: one persistent count; per-graph totals
