@@ -153,7 +153,11 @@ struct SharedTeam {
     static constexpr int kB = Batch<Pos, kThreads>::kSize;
     int32_t start[kB + 33];             // compacted batch: exclusive prefix of run lengths, then
                                         // the total and 32 sentinels (INT_MAX)
-    Pos src[kB + 1];                    // compacted batch: adjacency position of a run minus its prefix
+    // compacted batch: adjacency position of a run minus its prefix.  A group of
+    // segments that ends before its last one takes the next entries for those
+    // left over (of no wedges), up to kPast past the last run.
+    static constexpr int kPast = 7;
+    Pos src[kB + kPast];
     uint2 msum[has_second_walk(MODE) ? kB : 1];  // second walk: Σ δ per compacted middle (low, high half)
     long long wtot[kThreads / 32];
     unsigned long long red[kThreads / 32];
@@ -722,6 +726,7 @@ __device__ __forceinline__ unsigned long long batch_windows(const CountParams &p
     // not fit the registers beside a team's or 64-bit positions)
     constexpr int kSeg = is_table(KIND) || (kSecond && wants_edges(MODE) && (sizeof(Pos) == 8 || kThreads != kCountThreads))
                              ? 4 : 8;
+    static_assert(kSeg - 1 <= SH::kPast, "a group's last segment lies past the run array");
     const int lane = t.tid & 31, warp = t.tid >> 5;
     const uint32_t le_mask = 0xffffffffu >> (31 - lane);
     const uint32_t ctr32 = (uint32_t)__cvta_generic_to_shared(ctr);
@@ -789,7 +794,7 @@ __device__ __forceinline__ unsigned long long batch_windows(const CountParams &p
                     w[u] = -1;
                     if (lane < n) w[u] = __ldg(p.adj + pos[u]);
                     k0 += n;
-                    q0 += k0 == nxt;   // at the range's end: a run past it, never read from
+                    q0 += k0 == nxt;   // past the range's end: a run of which no wedge is taken
                     nxt = min(sh.start[q0 + 1], kend);
                 }
                 const unsigned long long x = group(std::integral_constant<int, kSeg>(), w, pos, d);
