@@ -516,7 +516,7 @@ int bfc_count_all_host(int32_t num_u, int32_t num_l, int64_t num_edges, const in
  * status_dev is not NULL, BFC_OK or BFC_ERR_INVALID_GRAPH (offsets not a CSR
  * of num_edges entries, or an id out of range) into *status_dev (one int32,
  * device memory); *total_dev is 0 for an invalid graph.  Duplicate edges are
- * not detected.  Asynchronous on `stream`; one cooperative kernel launch.
+ * not rejected: they count as parallel edges.  Asynchronous on `stream`; one cooperative kernel launch.
  *
  * Limits: num_u <= 49,152, num_l <= 49,152, num_u + num_l <= 65,536,
  * num_edges <= 1,048,576; larger graphs return BFC_ERR_INVALID_ARGUMENT

@@ -17,7 +17,10 @@
 // writes both sides' lists as 16-bit ranks (the filter p(w) < p(x) is then one
 // comparison, with no degree lookup per wedge) and counts with Algorithm 2:
 // a start with at most 768 possible wedges by one warp with a hash table, a
-// heavier one by a CTA with dense 16-bit counters.
+// heavier one by a CTA with dense 16-bit counters.  A count of a simple graph
+// is at most 49,152; edges that occur more than once can take one past 16 bits,
+// which the counter's own increments show: the heavy starts are then counted
+// again with 32-bit counters over halves of the ranks.
 #include <cooperative_groups.h>
 
 #include <mutex>
@@ -45,6 +48,7 @@ constexpr int32_t kNaLightWork = kNaSlots / 4 * 3;
 constexpr int kNaBigList = 512;                   // a middle's list above this is read by the whole CTA
 constexpr int kNaMaxBig = (int)(2 * kNaMaxEdges / kNaBigList);
 constexpr int kNaCntBytes = kNaMaxVertices * 2;   // 16-bit counters by rank
+constexpr int32_t kNaWide = kNaCntBytes / 4;      // ranks per 32-bit pass
 static_assert(kNaCntBytes + kNaMaxBig * 2 <= kNaSmemBytes, "counters and big-list queue");
 static_assert(kNaWarps * kNaSlots * 4 <= kNaSmemBytes, "warp tables");
 static_assert(16384 * 8 <= kNaSmemBytes && kNaMaxHigh <= 16384, "high-degree sort");
@@ -67,7 +71,7 @@ namespace {
 // Where the scratch's parts begin.
 struct NaScratch {
     unsigned long long *acc;
-    int32_t *err, *cursor, *n_heavy, *n_light, *q_heavy, *q_light;
+    int32_t *err, *cursor, *n_heavy, *n_light, *q_heavy, *q_light, *q_again;
     int32_t *deg;      // [n] by global id (L vertex v -> v, U vertex u -> l + u)
     int32_t *rank;     // [n] by global id: position in Definition 3's order
     int32_t *vstart;   // [n] by rank: where the vertex's list starts in `adj`
@@ -78,8 +82,8 @@ struct NaScratch {
     int32_t *high;     // vertices of degree 255 or more, ascending global id
     uint16_t *adj;     // [2m] neighbours' ranks: L lists, then U lists at m + off_u
     __device__ NaScratch(int32_t *s, int32_t n, int32_t l) {
-        acc = reinterpret_cast<unsigned long long *>(s);
-        err = s + 2; cursor = s + 3; n_heavy = s + 4; n_light = s + 5; q_heavy = s + 6; q_light = s + 7;
+        acc = reinterpret_cast<unsigned long long *>(s);   // [4]: light starts, heavy ones, the same again, -
+        err = s + 8; cursor = s + 9; n_heavy = s + 10; n_light = s + 11; q_heavy = s + 12; q_light = s + 13; q_again = s + 14;
         deg = s + kNaHeader;
         rank = deg + n;
         vstart = rank + n;
@@ -134,7 +138,7 @@ k_count_noalloc(int32_t r, int32_t l, int32_t m, const int32_t *__restrict__ off
                 unsigned long long *total_out, int32_t *status_out) {
     cg::grid_group grid = cg::this_grid();
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ unsigned long long red[32];
+    __shared__ unsigned long long red[64];
     __shared__ int32_t sh_item, sh_nbig, sh_part[32], sh_base[kNaDigits];
 
     const int32_t n = r + l;
@@ -316,46 +320,64 @@ k_count_noalloc(int32_t r, int32_t l, int32_t m, const int32_t *__restrict__ off
     }
     grid.sync();
 
-    // Algorithm 2: Σ old over the increments of count_wedge(w) = Σ C(count, 2)
-    unsigned long long acc = 0;
+    // Algorithm 2: Σ old over the increments of count_wedge(w) = Σ C(count, 2),
+    // the heavy starts' apart from the light ones'
+    unsigned long long acc = 0, acc_light = 0;
     const int32_t n_heavy = *((volatile int32_t *)S.n_heavy), n_light = *((volatile int32_t *)S.n_light);
-    {
-        uint32_t *const cnt = reinterpret_cast<uint32_t *>(smem_raw);   // 16-bit counters, two per word
+    // the wedges of heavy start x, by the whole CTA (sh_nbig is zero); flush()
+    // follows at most 1,024 calls of op(w) by a thread, unless more long lists
+    // are met than a simple graph has
+    auto heavy_walk = [&](int32_t x, auto op, auto flush) {
         uint16_t *const big = reinterpret_cast<uint16_t *>(smem_raw + kNaCntBytes);
-        for (;;) {
+        const int32_t s = S.vstart[x], d = S.vdeg[x];
+        for (int32_t j0 = warp * 32; j0 < d; j0 += kNaThreads) {
+            const int32_t v = j0 + lane < d ? (int32_t)S.adj[s + j0 + lane] : 0x7fffffff;
+            int32_t vs = 0, vd = 0;
+            if (v < x) { vs = S.vstart[v]; vd = S.vdeg[v]; }
+            if (vd > kNaBigList) {
+                const int at = atomicAdd(&sh_nbig, 1);
+                if (at < kNaMaxBig) { big[at] = (uint16_t)v; vd = 0; }   // else this warp reads it
+            }
+            na_middles(S.adj, vs, vd, x, lane, op);
+            flush();
+        }
+        __syncthreads();
+        const int nbig = min(sh_nbig, kNaMaxBig);
+        for (int b = 0; b < nbig; ++b) {
+            const int32_t v = big[b], vs = S.vstart[v], vd = S.vdeg[v];
+            for (int32_t k = tid; k < vd; k += kNaThreads) {
+                const int32_t w = S.adj[vs + k];
+                if (w < x) op(w);
+            }
+            flush();
+        }
+    };
+    uint32_t *const cnt = reinterpret_cast<uint32_t *>(smem_raw);
+    auto clear = [&](int32_t words) {
+        uint4 *const c4 = reinterpret_cast<uint4 *>(smem_raw);
+        for (int32_t i = tid; i < (words + 3) / 4; i += kNaThreads) c4[i] = make_uint4(0, 0, 0, 0);
+    };
+    {
+        uint32_t sum = 0;   // Σ old since the last flush: below 2^26
+        uint32_t top = 0;   // the largest count that this thread has added to
+        for (;;) {          // 16-bit counters, two per word
             __syncthreads();
             if (tid == 0) { sh_item = atomicAdd(S.q_heavy, 1); sh_nbig = 0; }
             __syncthreads();
             const int32_t it = sh_item;
             if (it >= n_heavy) break;
-            const int32_t x = S.items[it], s = S.vstart[x], d = S.vdeg[x];
-            uint4 *const c4 = reinterpret_cast<uint4 *>(smem_raw);
-            for (int32_t i = tid; i < (x + 7) / 8; i += kNaThreads) c4[i] = make_uint4(0, 0, 0, 0);
+            const int32_t x = S.items[it];
+            clear((x + 1) / 2);
             __syncthreads();
-            auto op = [&](int32_t w) {
+            heavy_walk(x, [&](int32_t w) {
                 const uint32_t sh = (uint32_t)(w & 1) << 4;
-                acc += (atomicAdd(cnt + (w >> 1), 1u << sh) >> sh) & 0xffffu;
-            };
-            for (int32_t j0 = warp * 32; j0 < d; j0 += kNaThreads) {
-                const int32_t v = j0 + lane < d ? (int32_t)S.adj[s + j0 + lane] : 0x7fffffff;
-                int32_t vs = 0, vd = 0;
-                if (v < x) { vs = S.vstart[v]; vd = S.vdeg[v]; }
-                if (vd > kNaBigList) {
-                    const int at = atomicAdd(&sh_nbig, 1);
-                    if (at < kNaMaxBig) { big[at] = (uint16_t)v; vd = 0; }   // else this warp reads it
-                }
-                na_middles(S.adj, vs, vd, x, lane, op);
-            }
-            __syncthreads();
-            const int nbig = min(sh_nbig, kNaMaxBig);
-            for (int b = 0; b < nbig; ++b) {
-                const int32_t v = big[b], vs = S.vstart[v], vd = S.vdeg[v];
-                for (int32_t k = tid; k < vd; k += kNaThreads) {
-                    const int32_t w = S.adj[vs + k];
-                    if (w < x) op(w);
-                }
-            }
+                const uint32_t old = (atomicAdd(cnt + (w >> 1), 1u << sh) >> sh) & 0xffffu;
+                top = max(top, old);
+                sum += old;
+            }, [&]() { acc += sum; sum = 0; });
+            if (sh_nbig > kNaMaxBig) top = 0xffffu;   // those lists were read by one warp each
         }
+        if (top == 0xffffu) atomicOr(S.err, 8);   // a counter wrapped, or a sum may have
     }
     {
         // light starts: a table of (rank, count) words per warp; a rank below
@@ -380,7 +402,7 @@ k_count_noalloc(int32_t r, int32_t l, int32_t m, const int32_t *__restrict__ off
                         if (e == ~0u) return;
                     }
                     if ((e >> 16) == (uint32_t)w) {
-                        acc += atomicAdd(tab + h, 1u) & 0xffffu;
+                        acc_light += atomicAdd(tab + h, 1u) & 0xffffu;
                         return;
                     }
                     h = (h + 1) & (kNaSlots - 1);
@@ -396,20 +418,50 @@ k_count_noalloc(int32_t r, int32_t l, int32_t m, const int32_t *__restrict__ off
             __syncwarp();
         }
     }
+    // two sums over the grid, added to to[0] and to[1]
+    auto grid_sums = [&](unsigned long long v, unsigned long long v1, unsigned long long *to) {
 #pragma unroll
-    for (int d = 16; d > 0; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
-    if (lane == 0) red[warp] = acc;
-    __syncthreads();
-    if (warp == 0) {
-        unsigned long long t = red[lane];
+        for (int d = 16; d > 0; d >>= 1) {
+            v += __shfl_xor_sync(0xffffffffu, v, d);
+            v1 += __shfl_xor_sync(0xffffffffu, v1, d);
+        }
+        if (lane == 0) { red[warp] = v; red[32 + warp] = v1; }
+        __syncthreads();
+        if (warp < 2) {
+            unsigned long long t = red[32 * warp + lane];
 #pragma unroll
-        for (int d = 16; d > 0; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
-        if (lane == 0 && t) atomicAdd(S.acc, t);
-    }
+            for (int d = 16; d > 0; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
+            if (lane == 0 && t) atomicAdd(to + warp, t);
+        }
+    };
+    grid_sums(acc_light, acc, S.acc);
     grid.sync();
+    const bool again = (*((volatile int32_t *)S.err) & 8) != 0;   // the same in every thread of the grid
+    if (again) {   // the heavy starts with 32-bit counters, kNaWide ranks at a time
+        acc = 0;
+        for (;;) {
+            __syncthreads();
+            if (tid == 0) sh_item = atomicAdd(S.q_again, 1);
+            __syncthreads();
+            const int32_t it = sh_item;
+            if (it >= n_heavy) break;
+            const int32_t x = S.items[it];
+            for (int32_t lo = 0; lo < x; lo += kNaWide) {
+                __syncthreads();
+                if (tid == 0) sh_nbig = 0;
+                clear(min(x - lo, kNaWide));
+                __syncthreads();
+                heavy_walk(x, [&](int32_t w) {
+                    if ((uint32_t)(w - lo) < (uint32_t)kNaWide) acc += atomicAdd(cnt + (w - lo), 1u);
+                }, []() {});
+            }
+        }
+        grid_sums(acc, 0, S.acc + 2);
+        grid.sync();
+    }
     if (gtid == 0) {
         const bool full = (*((volatile int32_t *)S.err) & 4) != 0;
-        *total_out = *((volatile unsigned long long *)S.acc);
+        *total_out = *((volatile unsigned long long *)S.acc) + *((volatile unsigned long long *)(S.acc + (again ? 2 : 1)));
         if (status_out) *status_out = full ? BFC_ERR_INTERNAL : BFC_OK;
     }
 }

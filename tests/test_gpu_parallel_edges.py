@@ -177,3 +177,50 @@ def test_one_edge_many_times():
     bfc.bfc_release(h)
     c = 3 * k
     assert int(t.item()) == c * (c - 1) // 2
+
+
+@pytest.mark.parametrize("extra", [0, 16_000, 32_000])
+@pytest.mark.parametrize("case", CASES + ["two_pairs"])
+def test_parallel_edges_without_allocation(case, extra):
+    # "two_pairs": counts above 16 bits at neighbouring ranks and at 65,535 exactly;
+    # extra vertices move the ends' ranks into the upper half of the 32-bit pass
+    from paper_1812_00283_gb300 import bfc
+    rng = np.random.default_rng(len(case))
+    if case == "two_pairs":
+        mult = np.zeros((4, 5), dtype=np.int64)
+        mult[:, 0] = 255, 257, 258, 257
+        mult[3, 1:] = 300
+    else:
+        mult = _mult(case, rng)
+    total = _reference(mult)[0]
+    off, adj = _csr(mult, rng)
+    off = np.concatenate([off, np.full(extra, adj.size, dtype=np.int32)])
+    o, a = torch.from_numpy(off).cuda(), torch.from_numpy(adj).cuda()
+    out = torch.full((1,), -1, dtype=torch.int64, device="cuda")
+    status = torch.full((1,), -1, dtype=torch.int32, device="cuda")
+    s = torch.cuda.current_stream().cuda_stream
+    for _ in range(2):
+        bfc.bfc_count_small_noalloc(mult.shape[0] + extra, mult.shape[1] + extra, adj.size, o.data_ptr(), a.data_ptr(), s,
+                                    out.data_ptr(), status.data_ptr())
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0 and int(out.item()) == total
+
+
+def test_many_long_middles_without_allocation():
+    # one start with 5,000 copies of edges to middles of more than 512 neighbours each:
+    # more long lists in one start than a simple graph of this size can have
+    from paper_1812_00283_gb300 import bfc
+    mult = np.zeros((602, 4), dtype=np.int64)
+    mult[:600, :3] = 1
+    mult[600, :3] = 1700
+    mult[601, 3] = 6000
+    rng = np.random.default_rng(3)
+    total = _reference(mult)[0]
+    off, adj = _csr(mult, rng)
+    o, a = torch.from_numpy(off).cuda(), torch.from_numpy(adj).cuda()
+    out = torch.full((1,), -1, dtype=torch.int64, device="cuda")
+    status = torch.full((1,), -1, dtype=torch.int32, device="cuda")
+    bfc.bfc_count_small_noalloc(602, 4, adj.size, o.data_ptr(), a.data_ptr(), torch.cuda.current_stream().cuda_stream,
+                                out.data_ptr(), status.data_ptr())
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0 and int(out.item()) == total > 0
