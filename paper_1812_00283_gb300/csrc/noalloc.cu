@@ -181,13 +181,17 @@ k_count_noalloc(int32_t r, int32_t l, int32_t m, const int32_t *__restrict__ off
 
     // ranks: vertices in (degree, global id) order.  One stable counting pass
     // over 256 classes (degrees 0..254 exactly, the rest in the last class),
-    // 1,024 vertices per CTA; then the few vertices of the last class are
-    // sorted by one CTA.
+    // in tiles of 1,024 vertices, one per CTA where there are 64 CTAs; then the
+    // few vertices of the last class are sorted by one CTA.
     uint32_t *const wcnt = reinterpret_cast<uint32_t *>(smem_raw);   // [32 warps][256]
     const int tiles = (n + kNaThreads - 1) / kNaThreads;
-    int32_t digit = 0, before = 0;   // this thread's class and its place among its warp's
-    const int32_t id = (int32_t)blockIdx.x * kNaThreads + tid;
-    if ((int)blockIdx.x < tiles) {
+    int32_t digit = 0, before = 0, id = 0;   // this thread's class and its place among its warp's, its vertex
+    // wcnt[w][c] = how many of class c the tile's warps before w hold; returns
+    // (for c = tid) how many the tile holds
+    auto tile_classes = [&](int tile) {
+        id = tile * kNaThreads + tid;
+        uint32_t run = 0;
+        __syncthreads();
         for (int i = tid; i < kNaWarps * kNaDigits; i += kNaThreads) wcnt[i] = 0;
         __syncthreads();
         digit = id < n ? min(S.deg[id], kNaDigits - 1) : kNaDigits;
@@ -195,15 +199,18 @@ k_count_noalloc(int32_t r, int32_t l, int32_t m, const int32_t *__restrict__ off
         before = __popc(peers & lt);
         if (id < n && before == 0) wcnt[warp * kNaDigits + digit] = __popc(peers);
         __syncthreads();
-        if (tid < kNaDigits) {   // prefix over the warps, tile totals
-            uint32_t run = 0;
+        if (tid < kNaDigits) {
             for (int w = 0; w < kNaWarps; ++w) {
                 const uint32_t c = wcnt[w * kNaDigits + tid];
                 wcnt[w * kNaDigits + tid] = run;
                 run += c;
             }
-            S.thist[blockIdx.x * kNaDigits + tid] = (int32_t)run;
         }
+        return run;
+    };
+    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const uint32_t run = tile_classes(tile);
+        if (tid < kNaDigits) S.thist[tile * kNaDigits + tid] = (int32_t)run;
     }
     // L lists: 32 at a time take their room from one cursor (any order)
     for (int32_t v0 = gwarp * 32; v0 < l; v0 += gwarps * 32) {
@@ -220,13 +227,14 @@ k_count_noalloc(int32_t r, int32_t l, int32_t m, const int32_t *__restrict__ off
         if (v < l) S.lpos[v] = at;
     }
     grid.sync();
-    if ((int)blockIdx.x < tiles) {
+    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        if (tiles > (int)gridDim.x) tile_classes(tile);   // a CTA's only tile keeps what it counted
         // class starts: all tiles of the lower classes, and the lower tiles of this one
         int32_t all = 0, mine = 0;
         if (tid < kNaDigits)
             for (int t = 0; t < tiles; ++t) {
                 const int32_t c = S.thist[t * kNaDigits + tid];
-                if (t < (int)blockIdx.x) mine += c;
+                if (t < tile) mine += c;
                 all += c;
             }
         int32_t incl = all;
@@ -491,7 +499,7 @@ int noalloc_setup(int dev, int32_t **ptr, int *grid) {
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_count_noalloc, kNaThreads,
                                                           kNaSmemBytes);
         if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
-        if (per_sm < 1 || sms * per_sm < kNaTiles) { set_last_error("k_count_noalloc does not fit on the device"); return BFC_ERR_CUDA; }
+        if (per_sm < 1) { set_last_error("k_count_noalloc does not fit on an SM"); return BFC_ERR_CUDA; }
         g_na_grid[dev] = sms * per_sm;
         g_na_ptr[dev] = static_cast<int32_t *>(p);
     }
