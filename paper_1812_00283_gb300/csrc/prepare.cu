@@ -133,12 +133,18 @@ __global__ void __launch_bounds__(kT) k_ranks(const int32_t *__restrict__ order,
 //   256 < d            one CTA (256 threads up to 4,096 neighbours, 1,024 above),
 //                      a bitmap of the L ranks of the row's graph, whose prefix
 //                      popcounts are the positions, where that range is at most
-//                      524,288 ranks (64 KB) and duplicate edges are rejected
-//                      anyway (a repeated bit has no position of its own).
-// Otherwise (wider ranges, validate = 0):
-//   32 < d <= 256      one warp, bitonic sort of (rank, slot) in its shared memory;
-//   256 < d <= 4,096   one CTA, bitonic sort of (rank, slot) in shared memory;
-//   d > 4,096          (a few hundred rows) one radix sort of their edges.
+//                      524,288 ranks (80 KB with the prefixes: two CTAs share an
+//                      SM; wider bitmaps have not been measured) and duplicate
+//                      edges are rejected anyway (a repeated bit has no position
+//                      of its own).
+// Otherwise:
+//   32 < d <= 256      (ranges above 2^24 ranks) one warp, bitonic sort of
+//                      (rank, slot) in its shared memory;
+//   256 < d <= 4,096   (ranges above 524,288, validate = 0) one CTA, bitonic sort
+//                      of (rank, slot) in shared memory;
+//   d > 4,096          (likewise; a few hundred rows) one radix sort of their
+//                      edges.  A plan, which cannot read their number, takes the
+//                      bitmap with validate = 0 too.
 // Each tier also writes the swapped key (rank_l, rank_u) at the U-side
 // position; U-side order is ascending in rank_u, so the stable sort of those
 // keys on the rank_l bits yields the L side.  The sort carries each key's
