@@ -363,7 +363,9 @@ void bfc_batch_plan_destroy(bfc_batch_plan *plan);
  * (BFC_ERR_INVALID_ARGUMENT otherwise); offsets that are not a CSR of
  * num_edges slots, or L ids outside [0, num_l), give BFC_ERR_INVALID_GRAPH
  * before any sample is written.  Synchronises `stream`; the sampled union is
- * transient (freed in stream order once prepared). */
+ * transient (freed in stream order once prepared), and so are the keep masks
+ * beside it: num_samples · num_edges / 4 bytes, at most 2 GB or one sample's
+ * share. */
 int bfc_prepare_sparsified(int32_t num_u, int32_t num_l, int64_t num_edges, const int32_t *off_u_dev,
                            const int32_t *adj_u_dev, double p, uint64_t seed, int32_t num_samples,
                            const bfc_options *opt, void *stream, uint64_t *sample_edges_dev,

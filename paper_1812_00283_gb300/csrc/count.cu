@@ -692,8 +692,8 @@ __device__ __forceinline__ void batch_runs(const CountParams &p, int64_t e0, int
 //     reduction), eight in flight (four of a hash table);
 //   - else (many runs per 32 wedges) four windows across runs: the run of every
 //     lane is found from a 32-bit mask of run starts (reduce-or + popc).
-// Bound by instruction issue and load latency (53-63% issue, DRAM and L2 below
-// 20%).  Against windows across runs everywhere with a branch per wedge:
+// Bound by instruction issue and load latency: DRAM, L2 and the shared atomic
+// pipe stay far below their rates.  Against windows across runs everywhere with a branch per wedge:
 // per-edge counts of a 30M-edge shopping graph 10.69 -> 8.83 ms, per-vertex
 // counts of a 6M-edge power-law graph 4.70 -> 3.92, prepare and total of a
 // 20M-edge power-law graph 13.25 -> 12.38.
