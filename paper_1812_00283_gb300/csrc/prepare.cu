@@ -1540,6 +1540,7 @@ int rebin_graph(Graph *g, cudaStream_t s, int32_t warp_max_work, int32_t team_ma
     BFC_CUDA(cudaMemcpyAsync(hc, counts, sizeof(hc), cudaMemcpyDeviceToHost, s));
     BFC_CUDA(cudaStreamSynchronize(s));
     rc = schedule_graph(g, s, warp_max_work, team_max_work, hash_max_work, nullptr, bb, hc, heavy);
+    if (rc != BFC_OK) g->schedule_rc = rc;
     g->info.device_bytes = (int64_t)g->mem.total;
     if (rc == BFC_OK) BFC_CUDA(cudaStreamSynchronize(s));
     return rc;
