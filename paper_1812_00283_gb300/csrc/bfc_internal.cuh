@@ -147,6 +147,12 @@ struct Allocs {
         slab_left -= b;
         return cudaSuccess;
     }
+    // a piece of what is left of the current slab, or false
+    template <typename T>
+    bool carve(T **p, size_t count) {
+        const size_t b = rounded(count * sizeof(T));
+        return b <= kCarve && b <= slab_left && get(p, count) == cudaSuccess;
+    }
     // an allocation of its own, which drop gives back
     template <typename T>
     cudaError_t get_own(T **p, size_t count) {
@@ -220,11 +226,12 @@ struct Graph {
     uint64_t *work = nullptr; // [n]
     char *lists = nullptr;        // of the current schedule: the next two and `retry` (a plan's are apart)
     size_t lists_bytes = 0;
+    bool lists_own = false;       // by get_own
     int2 *cta_items = nullptr;    // (start, dense_item_y) / (start, -1 = hash)
     int32_t *team_items = nullptr;
     int32_t *warp_items = nullptr;   // [n]: the warp bin from the front, its tiny starts from the back
     int64_t n_cta_items = 0, n_team_items = 0, n_warp_items = 0, n_tiny_items = 0;
-    int schedule_rc = BFC_ERR_INTERNAL;   // BFC_OK once there is a schedule; else why the last one failed
+    int schedule_rc = BFC_ERR_INTERNAL;   // BFC_OK once there is a schedule; else the last attempt's status
     int32_t team_max = 0;          // effective team bound of the current schedule
     bool may_retry = false;        // the schedule can re-queue starts (retry pass launched)
     int *cursors = nullptr;        // [8] work-queue cursors of the count kernels

@@ -1320,19 +1320,24 @@ static int bin_starts(Graph *g, cudaStream_t s, const BinBounds &bb, unsigned lo
 }
 
 // Room for a schedule's lists in one allocation: CTA items, team items and one
-// place per start that can be re-queued (each at most once per launch).  Another
-// rebinning takes it over where it is large enough, else replaces it.
+// place per start that can be re-queued (each at most once per launch): the rest
+// of the first slab where they fit (the one schedule that most graphs have), else
+// an allocation of its own.  Another rebinning takes it over where it is large
+// enough, else replaces it.
 static int schedule_lists(Graph *g, int64_t n_items, int64_t n_team, int64_t retry_cap) {
     n_items = std::max<int64_t>(n_items, 1);
     n_team = std::max<int64_t>(n_team, 1);
     retry_cap = std::max<int64_t>(retry_cap, 1);
     const size_t need = (size_t)n_items * sizeof(int2) + (size_t)(n_team + retry_cap) * sizeof(int32_t);
     if (need > g->lists_bytes) {
-        g->mem.drop(g->lists);
+        const bool first = !g->lists;
+        if (g->lists_own) g->mem.drop(g->lists);
         g->lists = nullptr;
         g->lists_bytes = 0;
-        if (g->mem.get_own(&g->lists, need) != cudaSuccess) {
+        g->lists_own = !(first && g->mem.carve(&g->lists, need));
+        if (g->lists_own && g->mem.get_own(&g->lists, need) != cudaSuccess) {
             g->lists = nullptr;
+            g->lists_own = false;
             set_last_error("device allocation failed: schedule lists");
             return BFC_ERR_OUT_OF_MEMORY;
         }
@@ -1677,7 +1682,8 @@ int prepare_graph(const bfc_csr *csr, const bfc_options *opt, cudaStream_t s, Gr
         const size_t nn = (size_t)n, mm = (size_t)m, per_n = num_graphs > 0 ? 6 : 3;
         const size_t sum = small(4 * (size_t)r) + small(4 * (size_t)l) + 2 * small(8 * nn) + small(8 * (nn + 1)) +
                            per_n * small(4 * nn) + 3 * small(8 * mm) + small(16 * mm) +
-                           (num_graphs > 0 ? small(8 * (size_t)num_graphs) : 0) + 2 * 256;
+                           (num_graphs > 0 ? small(8 * (size_t)num_graphs) : 0) + 2 * 256 +
+                           small(4 * nn);   // the schedule's lists, where few starts are heavy
         g->mem.slab_next = std::min(sum, Allocs::kSlab);
     }
 

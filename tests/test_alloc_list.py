@@ -88,6 +88,12 @@ int main() {
         }
         a.drop(nullptr);
         CHECK(inside(kept, 1000));
+
+        // a piece of the current slab only where it fits
+        const size_t held = in_use, rest = a.slab_left;
+        char *c = nullptr;
+        CHECK(!a.carve(&c, rest + 1) && c == nullptr && in_use == held);
+        CHECK(a.carve(&c, rest < Allocs::kCarve ? rest : Allocs::kCarve) && inside(c, 256) && in_use == held);
         a.release();
         CHECK(in_use == 0);
 
