@@ -130,7 +130,7 @@ __device__ __forceinline__ void na_middles(const uint16_t *adj, int32_t s, int32
 
 // What bounds it: latency.  A small graph is a chain of dependent passes over a
 // few hundred KB with a grid barrier between them, then starts of a few
-// microseconds each.  On 12,007 x 8,001 vertices with 150,001 edges 129 us; 521 us
+// microseconds each.  On 12,007 x 8,001 vertices with 150,001 edges 132 us; 521 us
 // when each row's list was built by one thread and every start took a CTA.
 __global__ void __launch_bounds__(kNaThreads, 1)
 k_count_noalloc(int32_t r, int32_t l, int32_t m, const int32_t *__restrict__ off_u,
